@@ -112,9 +112,11 @@ typedef struct {
                          second, low-priority stream, overlapping the B build and the
                          Davidson; the first gradient / coupling call waits for them.
                          0: computed by the first derivative call */
-  int emu_f64;        /* mixed precision: 1 (default) runs the Coulomb B transforms
-                         (the two MO transforms of (mu nu|P)_J) as FP64-accurate products
-                         on the FP16 tensor cores by exact operand splitting; 0: FP64 */
+  int emu_f64;        /* 1 (default): FP64-accurate products on the FP16 tensor cores by exact
+                         operand splitting.  Mixed precision: the Coulomb B transforms (the
+                         two MO transforms of (mu nu|P)_J).  RIS_FP64: the exchange products
+                         (B^K build, the exchange part of the A products and of Gamma) of all
+                         but the smallest systems.  0: on the FP64 pipe */
   int eig_fp32;       /* mixed precision: 1 solves the Davidson subspace eigenproblem in FP32
                          (FP64 Rayleigh quotients, close pairs and restarts re-orthonormalised
                          in FP64, back to FP64 if the residuals stall); 0 (default): FP64 */
@@ -369,6 +371,16 @@ int ris_debug_gemm_tf32x3(int M, int N, int K, const double* A, const double* B,
  * RIS_ERR_TIMEOUT if a pipeline wait timed out, or another ris_status.
  */
 int ris_debug_gemm_f64emu(int M, int N, int K, const double* A, const double* B, double* C);
+
+/*
+ * Test hook: the same with nine balanced 7-bit digit slices per row frame
+ * (the form behind the exchange products of RIS_FP64): operands rounded to
+ * 62 bits of the frame, sums kept in integers over the whole contraction and
+ * rounded once.  Error per element below K 2^-57 max_k|A_rk|
+ * max_k|B_ck| plus one FP64 rounding of the result; rows that hold an
+ * infinity or a NaN give NaN.
+ */
+int ris_debug_gemm_f64emu97(int M, int N, int K, const double* A, const double* B, double* C);
 
 /*
  * Test hook: C = alpha A op(B) + beta C with the library's double-FP32 GEMM

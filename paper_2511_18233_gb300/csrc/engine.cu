@@ -127,6 +127,7 @@ void Engine::trim() {
   FBuf* fbs[] = {&BooH, &BooL, &BvvH, &BvvL, &XtH, &XtL, &YH, &YL, &cvvH, &cvvL,
                  &cooH, &cooL, &CoH, &CoL, &CvH, &CvL, &Df};
   for (FBuf* b : fbs) b->release();
+  release_emu_ops();
   aoPtr.release();
   aoList.release();
   axPtr.release();
@@ -718,6 +719,35 @@ __global__ void k_build_W(const double* __restrict__ C, int nmo, const double* _
   if (t >= nao * 2 * nocc) return;
   const int nu = t / (2 * nocc), k = t % (2 * nocc);
   W[t] = k < nocc ? C[(size_t)nu * nmo + k] : Q[(size_t)(k - nocc) * nao + nu];
+}
+
+// W[s][nu][k'] (k' < kw) for every state: blocks of columns [C_o | Q_0^T | C_o | Q_1^T | C_o]
+// (kw = 2 o, one comb; kw = 5 o, two combs and the trailing C_o); Q_c = q0, q1 [s][i][nu]
+__global__ void k_build_W_states(const double* __restrict__ C, int nmo, const double* __restrict__ q0,
+                                 const double* __restrict__ q1, int nao, int nocc, int kw,
+                                 double* __restrict__ W) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (long long)nao * kw) return;
+  const int s = blockIdx.y, nu = (int)(t / kw), k = (int)(t % kw), blk = k / nocc, i = k % nocc;
+  const double* q = (blk == 3 ? q1 : q0) + (size_t)s * nocc * nao;
+  W[(size_t)s * nao * kw + t] = (blk & 1) ? q[(size_t)i * nao + nu] : C[(size_t)nu * nmo + i];
+}
+
+// out[P][x][y] = E[x][off + y][P] (transposed: E[y][off + x][P]); E has row length ld
+__global__ void k_pick_E(const double* __restrict__ E, int o, int ld, int off, int nK, bool tr,
+                         double* __restrict__ out) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (long long)o * o * nK) return;
+  const int P = (int)(t % nK);
+  const long long xy = t / nK;
+  int x = (int)(xy / o), y = (int)(xy % o);
+  const double e = E[((size_t)x * ld + off + y) * nK + P];
+  if (tr) {
+    const int z = x;
+    x = y;
+    y = z;
+  }
+  out[((size_t)P * o + x) * o + y] = e;
 }
 
 constexpr int kCBatch = 8;  // states (or pairs) sharing one pass over the derivative integrals
@@ -1440,6 +1470,15 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   } else {
     dgemm(true, false, o, n * nK, n, 1.0, Co, nmo, TK.p, n * nK, 0.0, w2.p, n * nK, st);
   }
+  release_emu_ops();
+  if (emu_exchange()) {
+    w4.ensure((size_t)v * v * nK, st);
+    build_K_emu(HK, w4.p);
+    BKvvD.ensure((size_t)v * v * nK, st);
+    transpose_last2(w4.p, v, v, nK, BKvvD.p, st);  // [b][R][a]
+    stage = 2;
+    return;
+  }
   {
     GemmBatch bt;
     bt.nb1 = o;
@@ -1492,6 +1531,165 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   transpose_last2(w4.p, v, v, nK, BKvvD.p, st);  // [b][R][a]
   if (opt.precision == RIS_MIXED) prepare_mixed();
   stage = 2;
+}
+
+// The FP64 form's exchange products run emulated on the tensor cores (option
+// emu_f64) unless the system is so small that the FP64 pipe finishes a
+// product before the emulation's extra passes (slicing, about ten launches)
+// would: kEmuMinFlops is the exchange work of one A product there.
+constexpr double kEmuMinFlops = 2.0e7;
+bool Engine::emu_exchange() const {
+  return opt.precision == RIS_FP64 && opt.emu_f64 && !streamed &&
+         2.0 * nocc * (double)nvir * nvir * nK >= kEmuMinFlops;
+}
+
+void Engine::emu97(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep) {
+  if (!d_tcerr) {
+    RIS_ALLOC(cudaMallocAsync((void**)&d_tcerr, sizeof(int), st));
+    RIS_CUDA(cudaMemsetAsync(d_tcerr, 0, sizeof(int), st));
+  }
+  emu_gemm(kEmu9x7, M, N, A, B, ep, d_tcerr, st);
+}
+
+void Engine::check_tcerr() {
+  if (!d_tcerr) return;
+  int h_err = 0;
+  RIS_CUDA(cudaMemcpyAsync(&h_err, d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, st));
+  RIS_CUDA(cudaStreamSynchronize(st));
+  RIS_REQUIRE(h_err == 0, RIS_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
+}
+
+void Engine::release_emu_ops() {
+  emu_ready = false;
+  for (EmuMat* m : {&ebBoo, &ebBvv, &ebBov, &ebBovT}) m->release();
+}
+
+static EmuSource emu_src(const double* p, long long rs, long long ks, int rin = 0, long long rld = 0) {
+  EmuSource s;
+  s.p = p;
+  s.rs = rs;
+  s.ks = ks;
+  s.rin = rin;
+  s.rld = rld;
+  return s;
+}
+// element (r, c) at c[(r / rin) rld + (r % rin) rs + (c / cin) cld + (c % cin) cs]
+static EmuEpilogue emu_out(double* c, long long rs, long long cs, int rin = 0, long long rld = 0,
+                           int cin = 0, long long cld = 0) {
+  EmuEpilogue e;
+  e.c64 = c;
+  e.rs = rs;
+  e.cs = cs;
+  e.rin = rin;
+  e.rld = rld;
+  e.cin = cin;
+  e.cld = cld;
+  return e;
+}
+
+// Exchange part of the FP64 B build on the tensor cores: B^K_oo, c^K_oo, the
+// vv block (into Bvv, [a][b][R]), c^K_vv and, for RPA, the ov blocks, from
+// HK[i][nu][P] = C_o^T T^K and T^K.  P runs fastest everywhere, so the
+// operands are cut with lanes along (index, P) and every product writes
+// consecutive rows (index, P) to consecutive addresses.
+void Engine::build_K_emu(const double* HK, double* Bvv) {
+  const int o = nocc, v = nvir, n = nao;
+  const long long nov = (long long)o * v;
+  const double* Cv = C.p + o;
+  const EmuForm f = kEmu9x7;
+  EmuMat cv, co, li, lt, a;
+  cv.slice(f, emu_src(Cv, 1, nmo), v, n, st);            // rows a over mu
+  li.slice(f, emu_src(LKinv.p, nK, 1), nK, nK, st);      // rows R over P
+  lt.slice(f, emu_src(LKinv.p, 1, nK), nK, nK, st);      // rows Q over R
+  // [x][y][P] -> B = . L^-T -> c = B L^-1, rows (x, y)
+  auto metric = [&](const double* g, long long rows, double* B, double* c) {
+    a.slice(f, emu_src(g, nK, 1), rows, nK, st);
+    emu97((int)rows, nK, a.op, li.op, emu_out(B, nK, 1));
+    a.slice(f, emu_src(B, nK, 1), rows, nK, st);
+    emu97((int)rows, nK, a.op, lt.op, emu_out(c, nK, 1));
+  };
+  {  // rows (i,P) of HK over nu
+    EmuMat h;
+    h.slice(f, emu_src(HK, 1, nK, nK, (long long)n * nK), (long long)o * nK, n, st);
+    co.slice(f, emu_src(C.p, 1, nmo), o, n, st);
+    w3.ensure((size_t)std::max(nov, (long long)o * o) * nK, st);
+    emu97(o * nK, o, h.op, co.op, emu_out(w3.p, 1, nK, nK, (long long)o * nK));
+    BKoo.ensure((size_t)o * o * nK, st);
+    cKoo.ensure((size_t)o * o * nK, st);
+    metric(w3.p, (long long)o * o, BKoo.p, cKoo.p);
+    if (opt.rpa) {
+      emu97(o * nK, v, h.op, cv.op, emu_out(w3.p, 1, nK, nK, (long long)v * nK));
+      SBuf<double> Bia((size_t)nov * nK, st);  // [i][a][R]
+      cKov.ensure((size_t)nov * nK, st);
+      metric(w3.p, nov, Bia.p, cKov.p);
+      BKovR.ensure((size_t)nov * nK, st);
+      transpose_last2(Bia.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]
+    }
+  }
+  // rows (nu,P) over mu (T^K symmetric in mu, nu), then rows (a,P) over nu
+  w2.ensure((size_t)v * n * nK, st);
+  w3.ensure((size_t)v * v * nK, st);
+  {
+    EmuMat t;
+    t.slice(f, emu_src(TK.p, 1, (long long)n * nK), (long long)n * nK, n, st);
+    emu97(n * nK, v, t.op, cv.op, emu_out(w2.p, 1, (long long)n * nK));  // H[a][nu][P]
+  }
+  a.slice(f, emu_src(w2.p, 1, nK, nK, (long long)n * nK), (long long)v * nK, n, st);
+  emu97(v * nK, v, a.op, cv.op, emu_out(w3.p, 1, nK, nK, (long long)v * nK));  // [a][b][P]
+  cKvv.ensure((size_t)v * v * nK, st);
+  metric(w3.p, (long long)v * v, Bvv, cKvv.p);
+}
+
+void Engine::ensure_emu_ops() {
+  const int o = nocc, v = nvir;
+  if (!emu_ready) {
+    ebBoo.slice(kEmu9x7, emu_src(BKoo.p, 1, nK, nK, (long long)o * nK), (long long)o * nK, o, st);
+    ebBvv.slice(kEmu9x7, emu_src(BKvvD.p, (long long)nK * v, 1), v, nK * v, st);
+    emu_ready = true;
+  }
+}
+
+// Exchange contractions of exchange_terms for nvec vectors, as products over
+// long rows on the tensor cores:
+//   Y[(vec,i)][(R,b)] = sum_j B^K_oo[(i,R)][j] Z[vec][j][b]
+//   K1[(vec,i)][a]    = sum_(R,b) Y[(vec,i)][(R,b)] B^K_vv[a][(R,b)]
+//   Y1[(vec,i)][(R,j)] = sum_b B^K_ov[(R,i)][b] Z[vec][j][b]
+//   K2[(vec,i)][a]     = sum_(R,j) Y1[(vec,i)][(R,j)] B^K_ov[(R,j)][a]
+// The second product of each is the work (o v^2 nK against o^2 v nK); this
+// order keeps its outputs few and its contraction long.  Vectors run in
+// blocks of about 1280 rows (vec,i): ten row tiles reuse each slice of B^K,
+// and Y with its slices stays a few GB on the largest dense systems.
+void Engine::exchange_emu(const double* Z, int nvec, double* K1, double alpha, double beta,
+                          double* K2) {
+  const int o = nocc, v = nvir;
+  const long long nov = (long long)o * v;
+  const EmuForm f = kEmu9x7;
+  ensure_emu_ops();
+  if (K2 && !ebBov.op.rows) {
+    ebBov.slice(f, emu_src(BKovR.p, v, 1), (long long)nK * o, v, st);
+    ebBovT.slice(f, emu_src(BKovR.p, 1, v), v, nK * o, st);
+  }
+  const int nblk = cdiv((long long)nvec * o, 1280 + o), per = cdiv(nvec, nblk);
+  EmuMat x, y;
+  for (int s0 = 0; s0 < nvec; s0 += per) {
+    const int nb = std::min(per, nvec - s0);
+    const double* z = Z + s0 * nov;
+    w6.ensure((size_t)std::min(per, nvec) * o * nK * std::max(v, K2 ? o : 0), st);
+    x.slice(f, emu_src(z, 1, v, v, nov), (long long)nb * v, o, st);  // rows (vec,b) over j
+    emu97(nb * v, o * nK, x.op, ebBoo.op, emu_out(w6.p, 1, v, v, (long long)o * nK * v));
+    y.slice(f, emu_src(w6.p, (long long)nK * v, 1), (long long)nb * o, nK * v, st);
+    EmuEpilogue e = emu_out(K1 + s0 * nov, v, 1);
+    e.alpha = alpha;
+    e.beta = beta;
+    emu97(nb * o, v, y.op, ebBvv.op, e);
+    if (!K2) continue;
+    x.slice(f, emu_src(z, v, 1), (long long)nb * o, v, st);  // rows (vec,j) over b
+    // rows (vec,j), columns (R,i): Y1[vec][i][R][j]
+    emu97(nb * o, nK * o, x.op, ebBov.op,
+          emu_out(w6.p, 1, (long long)nK * o, o, (long long)o * nK * o, o, o));
+    y.slice(f, emu_src(w6.p, (long long)nK * o, 1), (long long)nb * o, nK * o, st);
+    emu97(nb * o, v, y.op, ebBovT.op, emu_out(K2 + s0 * nov, v, 1));
+  }
 }
 
 // FP32 hi/lo operands of the exchange products (Eq. A_matrix, (ij|ab) term)
@@ -1580,15 +1778,17 @@ void Engine::emu_abt(int M, int N, int K, const double* A, long long rsA, long l
     RIS_ALLOC(cudaMallocAsync((void**)&d_tcerr, sizeof(int), st));
     RIS_CUDA(cudaMemsetAsync(d_tcerr, 0, sizeof(int), st));
   }
-  const int lk = ld8(K);
-  SBuf<__half> sA((size_t)kEmuSlices * M * lk, st), sB((size_t)kEmuSlices * N * lk, st);
+  SBuf<__half> sA(emu_size(kEmu10x6, M, K), st), sB(emu_size(kEmu10x6, N, K), st);
   SBuf<int> eA(M, st), eB(N, st);
   EmuOperand a, b;
   a.s = sA.p; a.e = eA.p;
   b.s = sB.p; b.e = eB.p;
-  emu_slice(A, M, K, rsA, ksA, a, st);
-  emu_slice(B, N, K, rsB, ksB, b, st);
-  emu_gemm(M, N, a, b, ep, d_tcerr, st);
+  EmuSource xa, xb;
+  xa.p = A; xa.rs = rsA; xa.ks = ksA;
+  xb.p = B; xb.rs = rsB; xb.ks = ksB;
+  emu_slice(kEmu10x6, xa, M, K, a, st);
+  emu_slice(kEmu10x6, xb, N, K, b, st);
+  emu_gemm(kEmu10x6, M, N, a, b, ep, d_tcerr, st);
 }
 
 // Mixed precision: (ab|P)_K = sum_mu,nu C_mu,a C_nu,b (mu nu|P) by two
@@ -1774,6 +1974,12 @@ void Engine::apply_A_tda(const double* Xin, int nvec, double* out) {
   w5.ensure((size_t)nvec * std::max(nJ, 1), st);
   dgemm(false, false, nvec, nJ, (int)nov, 1.0, Xin, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
   dgemm(false, true, nvec, (int)nov, nJ, 2.0, w5.p, nJ, BJ.p, nJ, 0.0, out, (int)nov, st);
+  if (emu_exchange()) {
+    exchange_emu(Xin, nvec, out, -opt.cx, 1.0, nullptr);
+    k_add_diag<<<cdiv(nov * nvec, 256), 256, 0, st>>>(de.p, Xin, nov, nvec, out);
+    RIS_CHECK_LAUNCH();
+    return;
+  }
   w6.ensure((size_t)nvec * o * nK * v, st);
   {
     GemmBatch bt;
@@ -1803,12 +2009,14 @@ void Engine::apply(int nvec, const double* Xh, double* out, double* out2) {
   if (opt.rpa) {
     z.ensure(n, st);
     apply_ApB_AmB(x.p, nvec, y.p, z.p);
+    if (emu_exchange()) check_tcerr();
     copy_out(out2, z.p, n, st);
   } else if (opt.precision == RIS_MIXED) {
     apply_A_mixed(x.p, nvec, y.p);
   } else {
     apply_A_tda(x.p, nvec, y.p);
   }
+  if (emu_exchange()) check_tcerr();
   copy_out(out, y.p, n, st);
   RIS_CUDA(cudaStreamSynchronize(st));
 }
@@ -1819,6 +2027,10 @@ void Engine::apply(int nvec, const double* Xh, double* out, double* out2) {
 void Engine::exchange_terms(const double* Z, int nvec, double* K1, double* K2, bool mixed) {
   const int o = nocc, v = nvir;
   const long long nov = (long long)o * v;
+  if (emu_exchange()) {
+    exchange_emu(Z, nvec, K1, 1.0, 0.0, K2);
+    return;
+  }
   if (mixed) {
     apply_exchange_mixed(Z, nvec, K1, 1.0, 0.0);
   } else {
@@ -1869,6 +2081,7 @@ void Engine::apply_ApB_AmB(const double* Z, int nvec, double* outP, double* outM
 void Engine::davidson_tda(int ns, const double* guess) {
   if (opt.precision != RIS_MIXED) {
     dav_core(ns, guess, guess ? ns : 0, false, opt.conv_tol, true);
+    if (emu_exchange()) check_tcerr();
     return;
   }
   bool ok = true;
@@ -1903,10 +2116,7 @@ void Engine::davidson_tda(int ns, const double* guess) {
     stats[4] += s4;
     stats[5] += s5;
   }
-  int h_err = 0;
-  RIS_CUDA(cudaMemcpyAsync(&h_err, d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, st));
-  RIS_CUDA(cudaStreamSynchronize(st));
-  RIS_REQUIRE(h_err == 0, RIS_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
+  check_tcerr();
 }
 
 // M = D - s + f B^J B^J^T (orbital-energy differences plus the Coulomb part
@@ -2464,12 +2674,7 @@ void Engine::davidson_rpa(int ns) {
   RIS_CHECK_LAUNCH();
   k_phase<<<ns, 256, 0, st>>>(X.p, Y.p, n);
   RIS_CHECK_LAUNCH();
-  if (mixed) {
-    int h_err = 0;
-    RIS_CUDA(cudaMemcpyAsync(&h_err, d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, st));
-    RIS_CUDA(cudaStreamSynchronize(st));
-    RIS_REQUIRE(h_err == 0, RIS_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
-  }
+  if (mixed || emu_exchange()) check_tcerr();
 }
 
 // ------------------------------------------------------------------ derivatives
@@ -2506,6 +2711,105 @@ void Engine::ensure_D() {
   start_D(st);
   have_D = true;
 }
+
+// Exchange densities of pairs in the FP64 form on the tensor cores.  For each
+// comb c of (R_I,R_J), (L_I,L_J) (TDA: the first alone):
+//   Z[j][b][P] = sum_a U[j][a] c^vv[a][b][P],  G[j][k][P] = sum_b V[k][b] Z[j][b][P]
+//   M[mu][k'][P]: k' < o   sum_j C_o[mu][j] G[j][k][P]
+//                 k' >= o  sum_i Q_U[i][mu] c^oo[i][k][P]
+//   Gamma[mu][nu][P] = f sum_k' W_V[nu][k'] M[mu][k'][P],  W_V = [C_o | Q_V^T]
+// and for RPA the (ib|ja) terms, E1_c = U c^ov^T, E2_c = V c^ov^T (o x o per P):
+//   M[mu][4o + k][P] = sum_k' (E1_0 Q_V0 + E2_0 Q_U0 - E1_1 Q_V1 - E2_1 Q_U1)[k][mu]
+// against a further C_o block of W, so that Gamma is written once by one
+// product over all k'.  P runs fastest in every array.
+struct GammaEmu {
+  EmuMat cvv, coo, cov, Co, U[2], QT[2], W;
+  SBuf<double> Z, G, M, Wd, EE, QW, e1, e2;
+  EmuMat zs, gs, ms, qs;
+  int nc = 1, kw = 0;
+  const double* Q[2] = {nullptr, nullptr};
+
+  void setup(Engine& e, int nsu, const double* R, const double* L, const double* QR, const double* QL) {
+    const int o = e.nocc, v = e.nvir, n = e.nao, nK = e.nK;
+    const EmuForm f = kEmu9x7;
+    cudaStream_t st = e.st;
+    nc = L ? 2 : 1;
+    kw = (L ? 5 : 2) * o;
+    Q[0] = QR;
+    Q[1] = QL;
+    cvv.slice(f, emu_src(e.cKvv.p, 1, (long long)v * nK), (long long)v * nK, v, st);  // rows (b,P) over a
+    coo.slice(f, emu_src(e.cKoo.p, 1, (long long)o * nK), (long long)o * nK, o, st);  // rows (k,P) over i
+    Co.slice(f, emu_src(e.C.p, e.nmo, 1), n, o, st);                                   // rows mu over j
+    if (L)  // rows (k,P) over a
+      cov.slice(f, emu_src(e.cKov.p, 1, nK, nK, (long long)v * nK), (long long)o * nK, v, st);
+    for (int c = 0; c < nc; c++) {
+      U[c].slice(f, emu_src(c ? L : R, v, 1), (long long)nsu * o, v, st);  // rows (s,j) over a
+      QT[c].slice(f, emu_src(Q[c], 1, n, n, (long long)o * n), (long long)nsu * n, o, st);  // (s,mu) over i
+    }
+    Wd.ensure((size_t)nsu * n * kw, st);
+    k_build_W_states<<<dim3(cdiv((long long)n * kw, 256), nsu), 256, 0, st>>>(e.C.p, e.nmo, QR, QL, n, o,
+                                                                              kw, Wd.p);
+    RIS_CHECK_LAUNCH();
+    W.slice(f, emu_src(Wd.p, kw, 1), (long long)nsu * n, kw, st);  // rows (s,nu) over k'
+    Z.ensure((size_t)o * v * nK, st);
+    G.ensure((size_t)o * o * nK, st);
+    M.ensure((size_t)n * kw * nK, st);
+    if (L) {
+      EE.ensure((size_t)o * 4 * o * nK, st);
+      QW.ensure((size_t)4 * o * n, st);
+      e1.ensure((size_t)o * o * nK, st);
+      e2.ensure((size_t)o * o * nK, st);
+    }
+  }
+
+  // Gam written, Om (nU x nU) added to
+  void pair(Engine& e, int sI, int sJ, double* Gam, double* Om) {
+    const int o = e.nocc, v = e.nvir, n = e.nao, nK = e.nK, nU = e.nU;
+    const EmuForm f = kEmu9x7;
+    cudaStream_t st = e.st;
+    const double w = nc == 2 ? -0.5 * e.opt.cx : -e.opt.cx;
+    const long long kP = (long long)kw * nK;
+    for (int c = 0; c < nc; c++) {
+      e.emu97(v * nK, o, cvv.op, U[c].op.sub((long long)sI * o, o), emu_out(Z.p, 1, (long long)v * nK));
+      zs.slice(f, emu_src(Z.p, 1, nK, nK, (long long)v * nK), (long long)o * nK, v, st);  // (j,P) over b
+      e.emu97(o * nK, o, zs.op, U[c].op.sub((long long)sJ * o, o),
+              emu_out(G.p, 1, nK, nK, (long long)o * nK));
+      gs.slice(f, emu_src(G.p, 1, (long long)o * nK), (long long)o * nK, o, st);  // (k,P) over j
+      double* m = M.p + (size_t)2 * c * o * nK;
+      e.emu97(o * nK, n, gs.op, Co.op, emu_out(m, 1, kP));
+      e.emu97(o * nK, n, coo.op, QT[c].op.sub((long long)sI * n, n),
+              emu_out(m + (size_t)o * nK, 1, kP));
+      // Omega[P][Q] += w sum_ij c^oo_ij,P G_ij,Q   (K functions are union 0..nK-1)
+      dgemm(true, false, nK, nK, o * o, w, e.cKoo.p, nK, G.p, nK, 1.0, Om, nU, st);
+    }
+    if (nc == 2) {
+      const size_t oo = (size_t)o * nK, on = (size_t)o * n;
+      for (int c = 0; c < 2; c++) {
+        const double sg = c ? -1.0 : 1.0;
+        for (int h = 0; h < 2; h++) {  // E1 from U paired with Q_V, E2 from V paired with Q_U
+          const int s = h ? sJ : sI, t = h ? sI : sJ, blk = 2 * c + h;
+          e.emu97(o * nK, o, cov.op, U[c].op.sub((long long)s * o, o),
+                  emu_out(EE.p + blk * oo, 1, 4LL * o * nK));
+          axpby((long long)on, sg, Q[c] + t * on, 0.0, nullptr, QW.p + blk * on, st);
+        }
+        // Omega[A][B] += w_c sum_ki E2_A[k][i] E1_B[i][k]
+        const int nt = cdiv((long long)o * o * nK, 256);
+        k_pick_E<<<nt, 256, 0, st>>>(EE.p, o, 4 * o, (2 * c + 1) * o, nK, false, e2.p);
+        RIS_CHECK_LAUNCH();
+        k_pick_E<<<nt, 256, 0, st>>>(EE.p, o, 4 * o, 2 * c * o, nK, true, e1.p);
+        RIS_CHECK_LAUNCH();
+        dgemm(false, true, nK, nK, o * o, sg * w, e2.p, o * o, e1.p, o * o, 1.0, Om, nU, st);
+      }
+      gs.slice(f, emu_src(EE.p, 1, nK, nK, 4LL * o * nK), (long long)o * nK, 4 * o, st);  // (k,P) over k'
+      qs.slice(f, emu_src(QW.p, 1, n), n, 4 * o, st);                                     // mu over k'
+      e.emu97(o * nK, n, gs.op, qs.op, emu_out(M.p + 4 * oo, 1, kP));
+    }
+    ms.slice(f, emu_src(M.p, 1, nK, nK, kP), (long long)n * nK, kw, st);  // rows (mu,P) over k'
+    EmuEpilogue ep = emu_out(Gam, 1, nK, nK, (long long)n * nK);
+    ep.alpha = w;
+    e.emu97(n * nK, n, ms.op, W.op.sub((long long)sJ * n, n), ep);
+  }
+};
 
 void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in,
                          const double* Y_in, double* out) {
@@ -2607,14 +2911,15 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   }
   if (!mixed || rpa) {
     QR.ensure((size_t)nsu * o * nn, st);
-    QL.ensure((size_t)nsu * o * nn, st);
+    if (rpa) QL.ensure((size_t)nsu * o * nn, st);
     for (int s = 0; s < nsu; s++) {
       if (!mixed) {
         dgemm(false, false, nn, v, o, 1.0, Co, nmo, Rs.p + s * nov, v, 0.0, t1.p, v, st);
         dgemm(false, true, nn, nn, v, 1.0, t1.p, v, Cv, nmo, 0.0, DR.p + (size_t)s * nn * nn, nn, st);
       }
       dgemm(false, true, o, nn, v, 1.0, Rs.p + s * nov, v, Cv, nmo, 0.0, QR.p + (size_t)s * o * nn, nn, st);
-      dgemm(false, true, o, nn, v, 1.0, Ls.p + s * nov, v, Cv, nmo, 0.0, QL.p + (size_t)s * o * nn, nn, st);
+      if (rpa)
+        dgemm(false, true, o, nn, v, 1.0, Ls.p + s * nov, v, Cv, nmo, 0.0, QL.p + (size_t)s * o * nn, nn, st);
     }
   }
   // u_s = R_s . B^J (nJ), c_s = u_s L^-1 (row vector)
@@ -2672,17 +2977,20 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   const int slK = pick_slices((long long)nn * nK, nbAvg);
   SBuf<double> partK((size_t)slK * NB * 3 * nn * nK, st);
   SBuf<int> pst(2 * NB, st);
-  if (opt.precision != RIS_MIXED) {
+  if (opt.precision != RIS_MIXED && !emu_exchange()) {
     Z.ensure((size_t)o * v * nK, st);
     Goo.ensure((size_t)o * o * nK, st);
     M1.ensure((size_t)nn * 2 * o * nK, st);
     WV.ensure((size_t)nn * 2 * o, st);
   }
   const double cx = opt.cx;
+  GammaEmu ge;
+  const bool emu = emu_exchange();
+  if (emu) ge.setup(*this, nsu, Rs.p, rpa ? Ls.p : nullptr, QR.p, rpa ? QL.p : nullptr);
   for (int g0 = 0; g0 < npair; g0 += NB) {
     const int nb = std::min(NB, npair - g0);
-    // (in mixed TDA the single exchange GEMM writes every element of G^K)
-    if (!gk32) RIS_CUDA(cudaMemsetAsync(GK.p, 0, sizeof(double) * nb * gk, st));
+    // (in mixed TDA and in the emulated form one exchange GEMM writes every element of G^K)
+    if (!gk32 && !emu) RIS_CUDA(cudaMemsetAsync(GK.p, 0, sizeof(double) * nb * gk, st));
     RIS_CUDA(cudaMemsetAsync(OmB.p, 0, sizeof(double) * nb * nU * nU, st));
     std::vector<int> h_pst(2 * nb);
     for (int b = 0; b < nb; b++) {
@@ -2696,6 +3004,10 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
       k_omega_J<<<cdiv(nJ * nJ, 256), 256, 0, st>>>(cJ.p + (size_t)sI * nJ, cJ.p + (size_t)sJ * nJ,
                                                      d_jU, nJ, nU, 2.0, Om);
       RIS_CHECK_LAUNCH();
+      if (emu) {
+        ge.pair(*this, sI, sJ, Gam, Om);
+        continue;
+      }
       // exchange (ij|ab) for (R_I,R_J) and (L_I,L_J), each with weight -c_x/2;
       // with Y = 0 both combinations coincide, so one pass with -c_x.
       const int ncomb = rpa ? 2 : 1;
@@ -2808,12 +3120,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
     RIS_CHECK_LAUNCH();
     RIS_CUDA(cudaStreamSynchronize(st));  // h_pst goes out of scope
   }
-  if (opt.precision == RIS_MIXED) {
-    int h_err = 0;
-    RIS_CUDA(cudaMemcpyAsync(&h_err, d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, st));
-    RIS_CUDA(cudaStreamSynchronize(st));
-    RIS_REQUIRE(h_err == 0, RIS_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
-  }
+  if (opt.precision == RIS_MIXED || emu_exchange()) check_tcerr();
 }
 
 
@@ -2829,6 +3136,22 @@ void Engine::ensure_Kov() {
   const double* Co = C.p;
   const double* Cv = C.p + o;
   SBuf<double> H((size_t)o * n * nK, st), Bia((size_t)nov * nK, st), Bm((size_t)nov * nK, st);
+  if (emu_exchange()) {
+    const EmuForm f = kEmu9x7;
+    EmuMat t, c, li;
+    t.slice(f, emu_src(TK.p, 1, (long long)n * nK), (long long)n * nK, n, st);  // rows (nu,P) over mu
+    c.slice(f, emu_src(Co, 1, nmo), o, n, st);
+    emu97(n * nK, o, t.op, c.op, emu_out(H.p, 1, (long long)n * nK));  // H[i][nu][P]
+    t.slice(f, emu_src(H.p, 1, nK, nK, (long long)n * nK), (long long)o * nK, n, st);
+    c.slice(f, emu_src(Cv, 1, nmo), v, n, st);
+    emu97(o * nK, v, t.op, c.op, emu_out(Bia.p, 1, nK, nK, (long long)v * nK));  // [i][a][P]
+    t.slice(f, emu_src(Bia.p, nK, 1), nov, nK, st);
+    li.slice(f, emu_src(LKinv.p, nK, 1), nK, nK, st);
+    emu97((int)nov, nK, t.op, li.op, emu_out(Bm.p, nK, 1));
+    BKovR.ensure((size_t)nov * nK, st);
+    transpose_last2(Bm.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]
+    return;
+  }
   dgemm(true, false, o, n * nK, n, 1.0, Co, nmo, TK.p, n * nK, 0.0, H.p, n * nK, st);
   GemmBatch bt;
   bt.nb1 = o;
@@ -2929,12 +3252,7 @@ void Engine::zvector(int nr, const double* rhs_in, double* Z_out) {
   stats[7] = worst;
   RIS_REQUIRE(converged, RIS_ERR_NOT_CONVERGED,
               "Z-vector CG did not converge in " + std::to_string(it) + " iterations");
-  if (opt.precision == RIS_MIXED) {
-    int h_err = 0;
-    RIS_CUDA(cudaMemcpyAsync(&h_err, d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, st));
-    RIS_CUDA(cudaStreamSynchronize(st));
-    RIS_REQUIRE(h_err == 0, RIS_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
-  }
+  if (opt.precision == RIS_MIXED || emu_exchange()) check_tcerr();
   copy_out(Z_out, x.p, sz, st);
   RIS_CUDA(cudaStreamSynchronize(st));
 }
@@ -3546,12 +3864,7 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
     RIS_CHECK_LAUNCH();
     RIS_CUDA(cudaStreamSynchronize(st));  // h_pst goes out of scope
   }
-  if (mixed) {
-    int h_err = 0;
-    RIS_CUDA(cudaMemcpyAsync(&h_err, d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, st));
-    RIS_CUDA(cudaStreamSynchronize(st));
-    RIS_REQUIRE(h_err == 0, RIS_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
-  }
+  if (mixed || emu_exchange()) check_tcerr();
 }
 
 // ------------------------------------------------------------------ time couplings

@@ -63,6 +63,26 @@ struct FBuf {
   ~FBuf() { release(); }
 };
 
+// A sliced operand of the emulated FP64 products (gemm_emu.cuh) and its
+// storage.
+struct EmuMat {
+  SBuf<__half> s;
+  SBuf<int> e;
+  EmuOperand op;
+  void slice(EmuForm f, const EmuSource& src, long long rows, int K, cudaStream_t st) {
+    s.ensure(emu_size(f, rows, K), st);
+    e.ensure((size_t)rows, st);
+    op.s = s.p;
+    op.e = e.p;
+    emu_slice(f, src, (int)rows, K, op, st);
+  }
+  void release() {
+    s.release();
+    e.release();
+    op = EmuOperand();
+  }
+};
+
 // The context's stream; a base class so that it outlives every buffer
 // member, whose stream-ordered frees are queued on it.
 struct StreamOwner {
@@ -155,6 +175,14 @@ struct Engine : StreamOwner {
   FBuf CvH, CvL;    // C_v as [mu][a] (a padded)
   int* d_tcerr = nullptr;
 
+  // FP64 form with emulated exchange products (emu_exchange): sliced B^K,
+  // made on first use after a B build
+  bool emu_ready = false;
+  EmuMat ebBoo;   // rows (i,R) over j
+  EmuMat ebBvv;   // rows a over (R,b)
+  EmuMat ebBov;   // rows (R,i) over b         (RPA and Z-vector products)
+  EmuMat ebBovT;  // rows a over (R,j)
+
   // excitations
   int nstates = 0;
   DBuf omega, X, Y;
@@ -209,6 +237,16 @@ struct Engine : StreamOwner {
   // FP64-accurate product on the tensor cores
   void emu_abt(int M, int N, int K, const double* A, long long rsA, long long ksA, const double* B,
                long long rsB, long long ksB, const EmuEpilogue& ep);
+  // FP64 form: the exchange products (B^K build, A products, exchange
+  // densities) as FP64-accurate products on the FP16 tensor cores
+  bool emu_exchange() const;
+  void ensure_emu_ops();
+  void release_emu_ops();
+  void check_tcerr();  // throws if a tensor-core pipeline wait timed out (synchronises)
+  void emu97(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep);
+  void build_K_emu(const double* HK, double* Bvv);
+  // K1 (alpha, beta into out) and, when K2 is given, K2 of exchange_terms
+  void exchange_emu(const double* Z, int nvec, double* K1, double alpha, double beta, double* K2);
   // exchange part of Gamma / Omega for one (U,V) pair with weight f (3xTF32);
   // US/VS: splits of U, V [i][a]; WU/WV: [Q^T | C_o] splits of U and V;
   // Gamma accumulated in FP64 (Gam) or, when Gam32 is given, written in FP32

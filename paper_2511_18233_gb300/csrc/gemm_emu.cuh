@@ -7,31 +7,56 @@
 
 namespace ris {
 
-// Slicing: bits per slice and slices per operand.  A row r of an operand
-// (contraction index k) is written in one fixed-point frame per row,
-//   x_rk = 2^(E_r) * sum_{p=1..kEmuSlices} d_p(r,k) 2^(-kEmuBeta p),
-// |d_p| < 2^kEmuBeta, E_r set by the row's largest magnitude; the digits
-// are the first kEmuSlices * kEmuBeta bits of x_rk in that frame.
-constexpr int kEmuBeta = 6;
-constexpr int kEmuSlices = 10;
-// Largest contraction length of one tensor-core pass: a sum of eight digit
-// products over K stays below 2^24 (K * 63^2 * 8 < 2^24), so it is exact in
-// the FP32 accumulators.  Longer contractions run as several passes.
-constexpr int kEmuKChunk = 512;
+// Slicing forms.  A row r of an operand (contraction index k) is written in
+// one fixed-point frame per row, 2^(E_r) above its largest magnitude, and cut
+// into digits:
+//   kEmu10x6  ten 6-bit slices, digits 0 .. 63 with the element's sign (60
+//             bits, truncated): the Coulomb transforms of the mixed form
+//   kEmu9x7   nine 7-bit slices, balanced digits -64 .. 64 (62 bits and sign,
+//             rounded to nearest): the exchange products of the FP64 form.
+//             45 slice products instead of 55, and a frame 9 bits finer than
+//             an FP64 significand, so that a row's small elements beside one
+//             nine bits larger still keep FP64's relative precision
+enum EmuForm { kEmu10x6 = 0, kEmu9x7 = 1 };
+constexpr int emu_slices(EmuForm f) { return f == kEmu10x6 ? 10 : 9; }
 
-// A sliced operand: digits as FP16 integers [kEmuSlices][rows][ldk] (K
-// contiguous, ldk % 8 == 0, zero past K) and the row exponents E[rows].
+// A sliced operand: digits as FP16 integers [slices][rows][ldk] (K
+// contiguous, ldk % 8 == 0, zero past K) and the row exponents E[rows]
+// (kEmuNonFinite for a row that holds an infinity or a NaN: every product
+// with it is NaN).
+constexpr int kEmuNonFinite = 1 << 20;
 struct EmuOperand {
   __half* s = nullptr;
   int* e = nullptr;
   int rows = 0, K = 0, ldk = 0;
+  long long plane = 0;  // elements between slices
+  // rows r0 .. r0 + n - 1
+  EmuOperand sub(long long r0, int n) const {
+    EmuOperand o = *this;
+    o.s += r0 * ldk;
+    o.e += r0;
+    o.rows = n;
+    return o;
+  }
 };
 
-// Slices src with element (r, k) at src[r * rs + k * ks], r < rows, k < K,
-// into op (op.s / op.e must hold kEmuSlices * rows * ldk halves and rows
-// ints; ldk = ld8(K)).
-void emu_slice(const double* src, int rows, int K, long long rs, long long ks, EmuOperand& op,
-               cudaStream_t st);
+inline int ld8(int k) { return (k + 7) & ~7; }
+// halves an operand of the form needs (ints: rows)
+inline size_t emu_size(EmuForm f, long long rows, int K) {
+  return (size_t)emu_slices(f) * rows * ld8(K);
+}
+
+// Source placement: element (r, k) of an operand at src[row(r) + k * ks] with
+// row(r) = (r / rin) * rld + (r % rin) * rs (rin = 0: r * rs).
+struct EmuSource {
+  const double* p = nullptr;
+  long long rs = 0, ks = 1;
+  int rin = 0;
+  long long rld = 0;
+};
+
+// Slices src (rows x K) into op (op.s / op.e hold emu_size / rows elements).
+void emu_slice(EmuForm f, const EmuSource& src, int rows, int K, EmuOperand& op, cudaStream_t st);
 
 // Output placement: element (r, c) goes to
 //   c64[(r / rin) * rld + (r % rin) * rs + (c / cin) * cld + (c % cin) * cs]
@@ -43,11 +68,9 @@ struct EmuEpilogue {
   double alpha = 1.0, beta = 0.0;
 };
 
-// C (M x N) = A (M x K) . B (N x K)^T from sliced operands; *d_err (device
-// int) is set non-zero if a pipeline wait timed out.
-void emu_gemm(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep,
-              int* d_err, cudaStream_t st);
-
-inline int ld8(int k) { return (k + 7) & ~7; }
+// C (M x N) = A (M x K) . B (N x K)^T from operands sliced in form f; *d_err
+// (device int) is set non-zero if a pipeline wait timed out.
+void emu_gemm(EmuForm f, int M, int N, const EmuOperand& A, const EmuOperand& B,
+              const EmuEpilogue& ep, int* d_err, cudaStream_t st);
 
 }  // namespace ris

@@ -23,7 +23,7 @@ STATUS = {0: "RIS_OK", -1: "RIS_ERR_ARG", -2: "RIS_ERR_OOM", -3: "RIS_ERR_METRIC
 FP64, MIXED = 0, 1
 
 EXPORTS = ["ris_options_default", "ris_create", "ris_build_aux", "ris_build_B", "ris_excite",
-           "ris_apply", "ris_excite_guess", "ris_trim", "ris_zvector", "ris_phase_align", "ris_time_coupling", "ris_get_mo_window", "ris_debug_gemm_tf32x3", "ris_debug_gemm_f64emu", "ris_debug_gemm_ff", "ris_debug_sym_eig", "ris_debug_sym_eig_f32", "ris_debug_dgemm",
+           "ris_apply", "ris_excite_guess", "ris_trim", "ris_zvector", "ris_phase_align", "ris_time_coupling", "ris_get_mo_window", "ris_debug_gemm_tf32x3", "ris_debug_gemm_f64emu", "ris_debug_gemm_f64emu97", "ris_debug_gemm_ff", "ris_debug_sym_eig", "ris_debug_sym_eig_f32", "ris_debug_dgemm",
            "ris_gemm_tf32x3_noalloc", "ris_debug_alloc_count", "ris_debug_peak_probe",
            "ris_gradient", "ris_nac", "ris_get_dims", "ris_get_stats", "ris_debug_boys",
            "ris_last_error", "ris_destroy"]
@@ -84,6 +84,7 @@ def load(path: str = LIB_PATH):
     L.ris_debug_boys.argtypes = [i, P, P, P]
     L.ris_debug_gemm_tf32x3.argtypes = [i, i, i, P, P, P]
     L.ris_debug_gemm_f64emu.argtypes = [i, i, i, P, P, P]
+    L.ris_debug_gemm_f64emu97.argtypes = [i, i, i, P, P, P]
     L.ris_debug_gemm_ff.argtypes = [i, i, i, i, ctypes.c_double, P, P, ctypes.c_double, P,
                                     ctypes.POINTER(i)]
     L.ris_debug_sym_eig.argtypes = [i, i, P, P, P]
@@ -313,16 +314,17 @@ def debug_gemm_tf32x3(A, B):
     return C_t.cpu().numpy()
 
 
-def debug_gemm_f64emu(A, B):
+def debug_gemm_f64emu(A, B, form="10x6"):
     """C = A B^T through the library's FP64-emulating tensor-core GEMM
-    (numpy in/out)."""
+    (numpy in/out); form "10x6" or "9x7" (slices x bits)."""
     import torch
     A_t = torch.as_tensor(np.ascontiguousarray(A, dtype=np.float64), device="cuda")
     B_t = torch.as_tensor(np.ascontiguousarray(B, dtype=np.float64), device="cuda")
     M, K = A_t.shape
     N = B_t.shape[0]
     C_t = torch.zeros((M, N), dtype=torch.float64, device="cuda")
-    st = load().ris_debug_gemm_f64emu(M, N, K, A_t.data_ptr(), B_t.data_ptr(), C_t.data_ptr())
+    fn = load().ris_debug_gemm_f64emu97 if form == "9x7" else load().ris_debug_gemm_f64emu
+    st = fn(M, N, K, A_t.data_ptr(), B_t.data_ptr(), C_t.data_ptr())
     torch.cuda.synchronize()
     if st != 0:
         raise RisError(st, "ris_debug_gemm_f64emu failed")
