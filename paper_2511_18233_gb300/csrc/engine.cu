@@ -1564,8 +1564,10 @@ void Engine::release_emu_ops() {
   for (EmuMat* m : {&ebBoo, &ebBvv, &ebBov, &ebBovT}) m->release();
 }
 
-static EmuSource emu_src(const double* p, long long rs, long long ks, int rin = 0, long long rld = 0) {
+static EmuSource emu_src(const double* p, long long rs, long long ks, int rin = 0, long long rld = 0,
+                         int rvalid = 0) {
   EmuSource s;
+  s.rvalid = rvalid;
   s.p = p;
   s.rs = rs;
   s.ks = ks;
@@ -1643,22 +1645,23 @@ void Engine::build_K_emu(const double* HK, double* Bvv) {
 void Engine::ensure_emu_ops() {
   const int o = nocc, v = nvir;
   if (!emu_ready) {
-    ebBoo.slice(kEmu9x7, emu_src(BKoo.p, 1, nK, nK, (long long)o * nK), (long long)o * nK, o, st);
-    ebBvv.slice(kEmu9x7, emu_src(BKvvD.p, (long long)nK * v, 1), v, nK * v, st);
+    ebBvv.slice(kEmu9x7, emu_src(BKvvD.p, 1, (long long)nK * v), (long long)nK * v, v, st);
+    ebBoo.slice(kEmu9x7, emu_src(BKoo.p, (long long)o * nK, 1), o, o * nK, st);
     emu_ready = true;
   }
 }
 
-// Exchange contractions of exchange_terms for nvec vectors, as products over
-// long rows on the tensor cores:
-//   Y[(vec,i)][(R,b)] = sum_j B^K_oo[(i,R)][j] Z[vec][j][b]
-//   K1[(vec,i)][a]    = sum_(R,b) Y[(vec,i)][(R,b)] B^K_vv[a][(R,b)]
+// Exchange contractions of exchange_terms for nvec vectors on the tensor cores:
+//   W[(vec,j)][(R,a)]  = sum_b Z[vec][j][b] B^K_vv[(R,a)][b]
+//   K1[vec][i][a]      = sum_(j,R) B^K_oo[i][(j,R)] W[vec][(j,R)][a]
 //   Y1[(vec,i)][(R,j)] = sum_b B^K_ov[(R,i)][b] Z[vec][j][b]
 //   K2[(vec,i)][a]     = sum_(R,j) Y1[(vec,i)][(R,j)] B^K_ov[(R,j)][a]
-// The second product of each is the work (o v^2 nK against o^2 v nK); this
-// order keeps its outputs few and its contraction long.  Vectors run in
-// blocks of about 1280 rows (vec,i): ten row tiles reuse each slice of B^K,
-// and Y with its slices stays a few GB on the largest dense systems.
+// The long product comes first (o v^2 nK multiply-adds; over j first it would
+// be o^2 v nK): the intermediate has as many elements either way, and after a
+// contraction of length v its rounding and stores hide under the tensor cores
+// (at length o they are the time: 186 us for ten C20H22 vectors).  Vectors run
+// in blocks of about 1280 rows (vec,j), so that the intermediate and its
+// slices stay a few GB on the largest dense systems.
 void Engine::exchange_emu(const double* Z, int nvec, double* K1, double alpha, double beta,
                           double* K2) {
   const int o = nocc, v = nvir;
@@ -1675,19 +1678,25 @@ void Engine::exchange_emu(const double* Z, int nvec, double* K1, double alpha, d
     const int nb = std::min(per, nvec - s0);
     const double* z = Z + s0 * nov;
     w6.ensure((size_t)std::min(per, nvec) * o * nK * std::max(v, K2 ? o : 0), st);
-    x.slice(f, emu_src(z, 1, v, v, nov), (long long)nb * v, o, st);  // rows (vec,b) over j
-    emu97(nb * v, o * nK, x.op, ebBoo.op, emu_out(w6.p, 1, v, v, (long long)o * nK * v));
-    y.slice(f, emu_src(w6.p, (long long)nK * v, 1), (long long)nb * o, nK * v, st);
-    EmuEpilogue e = emu_out(K1 + s0 * nov, v, 1);
+    x.slice(f, emu_src(z, v, 1), (long long)nb * o, v, st);  // rows (vec,j) over b
+    EmuEpilogue e = emu_out(w6.p, 1, (long long)nK * v);
+    e.lead = y.clear_lead((long long)nb * v, st);  // row (vec,a) of W from (R,a) and (vec,j)
+    e.lead_rows(1, v, 1);
+    e.lead_cols(o, nb, v);
+    emu97(nK * v, nb * o, ebBvv.op, x.op, e);
+    y.slice(f, emu_src(w6.p, 1, v, v, (long long)o * nK * v), (long long)nb * v, o * nK, st, true);
+    e = emu_out(K1 + s0 * nov, 1, v, v, nov);
     e.alpha = alpha;
     e.beta = beta;
-    emu97(nb * o, v, y.op, ebBvv.op, e);
+    emu97(nb * v, o, y.op, ebBoo.op, e);
     if (!K2) continue;
-    x.slice(f, emu_src(z, v, 1), (long long)nb * o, v, st);  // rows (vec,j) over b
     // rows (vec,j), columns (R,i): Y1[vec][i][R][j]
-    emu97(nb * o, nK * o, x.op, ebBov.op,
-          emu_out(w6.p, 1, (long long)nK * o, o, (long long)o * nK * o, o, o));
-    y.slice(f, emu_src(w6.p, (long long)nK * o, 1), (long long)nb * o, nK * o, st);
+    e = emu_out(w6.p, 1, (long long)nK * o, o, (long long)o * nK * o, o, o);
+    e.lead = y.clear_lead((long long)nb * o, st);  // row (vec,i) from (vec,j) and (R,i)
+    e.lead_rows(o, nb, o);
+    e.lead_cols(1, o, 1);
+    emu97(nb * o, nK * o, x.op, ebBov.op, e);
+    y.slice(f, emu_src(w6.p, (long long)nK * o, 1), (long long)nb * o, nK * o, st, true);
     emu97(nb * o, v, y.op, ebBovT.op, emu_out(K2 + s0 * nov, v, 1));
   }
 }
@@ -2726,7 +2735,7 @@ struct GammaEmu {
   EmuMat cvv, coo, cov, Co, U[2], QT[2], W;
   SBuf<double> Z, G, M, Wd, EE, QW, e1, e2;
   EmuMat zs, gs, ms, qs;
-  int nc = 1, kw = 0;
+  int nc = 1, kw = 0, o8 = 0, n8 = 0;
   const double* Q[2] = {nullptr, nullptr};
 
   void setup(Engine& e, int nsu, const double* R, const double* L, const double* QR, const double* QL) {
@@ -2735,6 +2744,8 @@ struct GammaEmu {
     cudaStream_t st = e.st;
     nc = L ? 2 : 1;
     kw = (L ? 5 : 2) * o;
+    o8 = ld8(o);
+    n8 = ld8(n);
     Q[0] = QR;
     Q[1] = QL;
     cvv.slice(f, emu_src(e.cKvv.p, 1, (long long)v * nK), (long long)v * nK, v, st);  // rows (b,P) over a
@@ -2743,14 +2754,15 @@ struct GammaEmu {
     if (L)  // rows (k,P) over a
       cov.slice(f, emu_src(e.cKov.p, 1, nK, nK, (long long)v * nK), (long long)o * nK, v, st);
     for (int c = 0; c < nc; c++) {
-      U[c].slice(f, emu_src(c ? L : R, v, 1), (long long)nsu * o, v, st);  // rows (s,j) over a
-      QT[c].slice(f, emu_src(Q[c], 1, n, n, (long long)o * n), (long long)nsu * n, o, st);  // (s,mu) over i
+      // rows (s,j) over a and (s,mu) over i, a state's rows padded to whole groups
+      U[c].slice(f, emu_src(c ? L : R, v, 1, o8, (long long)o * v, o), (long long)nsu * o8, v, st);
+      QT[c].slice(f, emu_src(Q[c], 1, n, n8, (long long)o * n, n), (long long)nsu * n8, o, st);
     }
     Wd.ensure((size_t)nsu * n * kw, st);
     k_build_W_states<<<dim3(cdiv((long long)n * kw, 256), nsu), 256, 0, st>>>(e.C.p, e.nmo, QR, QL, n, o,
                                                                               kw, Wd.p);
     RIS_CHECK_LAUNCH();
-    W.slice(f, emu_src(Wd.p, kw, 1), (long long)nsu * n, kw, st);  // rows (s,nu) over k'
+    W.slice(f, emu_src(Wd.p, kw, 1, n8, (long long)n * kw, n), (long long)nsu * n8, kw, st);  // (s,nu) over k'
     Z.ensure((size_t)o * v * nK, st);
     G.ensure((size_t)o * o * nK, st);
     M.ensure((size_t)n * kw * nK, st);
@@ -2770,14 +2782,14 @@ struct GammaEmu {
     const double w = nc == 2 ? -0.5 * e.opt.cx : -e.opt.cx;
     const long long kP = (long long)kw * nK;
     for (int c = 0; c < nc; c++) {
-      e.emu97(v * nK, o, cvv.op, U[c].op.sub((long long)sI * o, o), emu_out(Z.p, 1, (long long)v * nK));
+      e.emu97(v * nK, o, cvv.op, U[c].op.sub((long long)sI * o8, o), emu_out(Z.p, 1, (long long)v * nK));
       zs.slice(f, emu_src(Z.p, 1, nK, nK, (long long)v * nK), (long long)o * nK, v, st);  // (j,P) over b
-      e.emu97(o * nK, o, zs.op, U[c].op.sub((long long)sJ * o, o),
+      e.emu97(o * nK, o, zs.op, U[c].op.sub((long long)sJ * o8, o),
               emu_out(G.p, 1, nK, nK, (long long)o * nK));
       gs.slice(f, emu_src(G.p, 1, (long long)o * nK), (long long)o * nK, o, st);  // (k,P) over j
       double* m = M.p + (size_t)2 * c * o * nK;
       e.emu97(o * nK, n, gs.op, Co.op, emu_out(m, 1, kP));
-      e.emu97(o * nK, n, coo.op, QT[c].op.sub((long long)sI * n, n),
+      e.emu97(o * nK, n, coo.op, QT[c].op.sub((long long)sI * n8, n),
               emu_out(m + (size_t)o * nK, 1, kP));
       // Omega[P][Q] += w sum_ij c^oo_ij,P G_ij,Q   (K functions are union 0..nK-1)
       dgemm(true, false, nK, nK, o * o, w, e.cKoo.p, nK, G.p, nK, 1.0, Om, nU, st);
@@ -2788,7 +2800,7 @@ struct GammaEmu {
         const double sg = c ? -1.0 : 1.0;
         for (int h = 0; h < 2; h++) {  // E1 from U paired with Q_V, E2 from V paired with Q_U
           const int s = h ? sJ : sI, t = h ? sI : sJ, blk = 2 * c + h;
-          e.emu97(o * nK, o, cov.op, U[c].op.sub((long long)s * o, o),
+          e.emu97(o * nK, o, cov.op, U[c].op.sub((long long)s * o8, o),
                   emu_out(EE.p + blk * oo, 1, 4LL * o * nK));
           axpby((long long)on, sg, Q[c] + t * on, 0.0, nullptr, QW.p + blk * on, st);
         }
@@ -2807,7 +2819,7 @@ struct GammaEmu {
     ms.slice(f, emu_src(M.p, 1, nK, nK, kP), (long long)n * nK, kw, st);  // rows (mu,P) over k'
     EmuEpilogue ep = emu_out(Gam, 1, nK, nK, (long long)n * nK);
     ep.alpha = w;
-    e.emu97(n * nK, n, ms.op, W.op.sub((long long)sJ * n, n), ep);
+    e.emu97(n * nK, n, ms.op, W.op.sub((long long)sJ * n8, n), ep);
   }
 };
 

@@ -69,12 +69,19 @@ struct EmuMat {
   SBuf<__half> s;
   SBuf<int> e;
   EmuOperand op;
-  void slice(EmuForm f, const EmuSource& src, long long rows, int K, cudaStream_t st) {
+  void slice(EmuForm f, const EmuSource& src, long long rows, int K, cudaStream_t st,
+             bool have_lead = false) {
     s.ensure(emu_size(f, rows, K), st);
     e.ensure((size_t)rows, st);
     op.s = s.p;
     op.e = e.p;
-    emu_slice(f, src, (int)rows, K, op, st);
+    emu_slice(f, src, (int)rows, K, op, st, have_lead);
+  }
+  // the row exponents of the rows to come, for an EmuEpilogue that fills them
+  int* clear_lead(long long rows, cudaStream_t st) {
+    e.ensure((size_t)rows, st);
+    RIS_CUDA(cudaMemsetAsync(e.p, 0x80, sizeof(int) * rows, st));
+    return e.p;
   }
   void release() {
     s.release();
@@ -178,8 +185,8 @@ struct Engine : StreamOwner {
   // FP64 form with emulated exchange products (emu_exchange): sliced B^K,
   // made on first use after a B build
   bool emu_ready = false;
-  EmuMat ebBoo;   // rows (i,R) over j
-  EmuMat ebBvv;   // rows a over (R,b)
+  EmuMat ebBvv;   // rows (R,a) over b
+  EmuMat ebBoo;   // rows i over (j,R)
   EmuMat ebBov;   // rows (R,i) over b         (RPA and Z-vector products)
   EmuMat ebBovT;  // rows a over (R,j)
 

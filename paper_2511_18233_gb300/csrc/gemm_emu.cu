@@ -20,10 +20,14 @@
 // form keeps adding integers over all chunks (also over the CTAs of a split
 // contraction) and rounds once at the end.
 //
-// Kernel (one 128 x BN output tile per CTA, 320 threads, one CTA per SM):
-//   warp 0 / lane 0 : TMA producer, 4-stage ring; a stage is K = 16 of all
-//                     slices of A (128 rows) and of B (BN rows), two 3-D
-//                     loads with 32-byte swizzle
+// Kernel (persistent, one CTA of 576 threads per SM looping over 128 x BN
+// output tiles):
+//   warp 0 / lane 0 : producer, 4-stage ring; a stage is K = 16 of all slices
+//                     of A (128 rows) and of B (BN rows), two contiguous bulk
+//                     copies per slice (the slicing writes the operands in the
+//                     layout of the stages: as 32-byte rows of a tensor map
+//                     the copies took 1.6 cycles a row and held the loop at
+//                     0.43 of the tensor pipe)
 //   warp 1          : allocates 512 TMEM columns (S accumulators of BN
 //                     columns); lane 0 issues the slice products.  The B
 //                     slices of a stage lie one after the other, and so do
@@ -31,18 +35,19 @@
 //                     tcgen05.mma of N = (up to 256 / BN) BN multiplies A
 //                     slice p with several B slices at once: the 128-row A
 //                     slice is read from shared memory once per such group
-//                     instead of once per product (15 instructions a stage
-//                     instead of 55 at 10 x 6, BN = 48)
-//   warps 2-9       : epilogue, one output row and every other block of 8
-//                     columns per thread
+//                     instead of once per product (13 instructions a stage
+//                     instead of 45 at 9 x 7, BN = 48)
+//   warps 2-17      : epilogue, one output row and a quarter of the columns
+//                     per thread.  A chunk's accumulators are read into
+//                     integers first and handed back, so that the next chunk
+//                     or tile runs on the tensor cores while the results are
+//                     rounded and stored
 // FP64 arithmetic is kept out of the epilogue (GB300 issues about 1.7 FP64
 // operations per clock per SM, so five per output would cost a 128 x 48 tile
-// 18k cycles, the time of 500 values of k): the result is rounded to FP64
+// 18k cycles, the time of 270 values of k): the result is rounded to FP64
 // with integer operations, bit for bit what the FP64 combination gives.
 // Every mbarrier wait is bounded; a timeout sets the error flag, drains what
 // the CTA has in flight and frees its tensor memory.
-#include <cuda.h>
-
 #include <algorithm>
 
 #include "gemm_emu.cuh"
@@ -56,7 +61,7 @@ using namespace tcx;
 constexpr int EBM = 128, EBK = 16, ESTAGES = 4;
 constexpr int A_SLICE = EBM * EBK * 2;  // 4 KB
 constexpr int TMEM_COLS = 512;
-constexpr int EPI_WARPS = 8, ETHREADS = 64 + 32 * EPI_WARPS;
+constexpr int EPI_WARPS = 16, ETHREADS = 64 + 32 * EPI_WARPS;
 
 struct Form10x6 {
   static constexpr int S = 10, kFrac = 60, kChunk = 512, kMaxBN = 48;
@@ -75,22 +80,6 @@ struct Tile {
   static_assert(F::S * F::kMaxBN <= TMEM_COLS, "accumulators exceed tensor memory");
   static_assert(kSmem <= 232448, "pipeline exceeds shared memory");
 };
-
-// 3-D map {K, rows, slice} of FP16 digits, box {16, box_rows, S}, 32-byte swizzle.
-CUtensorMap make_map(const EmuOperand& op, int slices, int box_rows) {
-  RIS_REQUIRE(((uintptr_t)op.s & 15) == 0, RIS_ERR_ARG, "emu_gemm: slices not 16-byte aligned");
-  RIS_REQUIRE(op.ldk % 8 == 0 && op.ldk >= op.K, RIS_ERR_ARG, "emu_gemm: ldk must be a multiple of 8");
-  CUtensorMap m;
-  cuuint64_t dims[3] = {(cuuint64_t)op.K, (cuuint64_t)op.rows, (cuuint64_t)slices};
-  cuuint64_t strides[2] = {(cuuint64_t)op.ldk * 2, (cuuint64_t)op.plane * 2};
-  cuuint32_t box[3] = {EBK, (cuuint32_t)box_rows, (cuuint32_t)slices};
-  cuuint32_t es[3] = {1, 1, 1};
-  CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, (void*)op.s, dims, strides, box, es,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
-                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  RIS_REQUIRE(r == CUDA_SUCCESS, RIS_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
-  return m;
-}
 
 // K-major operand tile, rows of 32 bytes with 32-byte swizzle: start
 // address, leading offset unused (1), 256 B between 8-row groups,
@@ -127,18 +116,56 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
 }
 
 struct EmuArgs {
-  int M, N, K, bn;
-  int ntn;         // column tiles (fastest on grid.x)
-  int nchunk, cps; // chunks of the contraction, chunks per slice of it (blockIdx.y)
+  int M, N, K;
+  int ntn, tiles;       // column tiles (fastest), all tiles
+  int nchunk, cps, ns;  // chunks of the contraction, chunks per slice of it, slices
+  const __half* sa;     // digits; elements between row groups' planes
+  const __half* sb;
+  long long pa, pb;
+  int ra, rb;           // rows the operands hold
   const int* ea;
   const int* eb;
-  longlong2* ws;   // split contraction: [blockIdx.y][M][N] integer partial sums
+  longlong2* ws;   // split contraction: [slice][M][N] integer partial sums
   EmuEpilogue ep;
+  int mode;        // 0: C = x, 1: C = alpha x, 2: C = alpha x + beta C
   int* err;
 };
 
+// bulk copy of contiguous bytes into shared memory (16-byte aligned, a
+// multiple of 16 bytes), completing on bar
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(sa(dst)),
+      "l"(src), "r"(bytes), "r"(sa(bar))
+      : "memory");
+}
+
+// Row exponent -> row frame: E_r = 1 + exponent of the largest magnitude, so
+// that every |x_rk| < 2^(E_r) (0 for a row of zeros).
+__device__ __forceinline__ int row_frame(int lead) { return lead == kEmuNoLead ? 0 : lead + 1; }
+__device__ __forceinline__ bool row_bad(int lead) { return lead >= kEmuLeadBad; }
+__device__ __forceinline__ int lead_exp(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ef = (int)((b >> 52) & 0x7FF);
+  if (ef) return ef - 1023;
+  const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+  return m ? -1011 - __clzll(m) : kEmuNoLead;  // -1074 + (63 - clz)
+}
+
 __device__ __forceinline__ long long emu_off(int i, int in, long long ld, long long s) {
   return in > 0 ? (long long)(i / in) * ld + (long long)(i % in) * s : (long long)i * s;
+}
+
+// C = x, or out of line C = alpha x (+ beta C), so that no FP64 operation is
+// predicated into the plain store
+__device__ __noinline__ void store_scaled(double* p, double x, int mode, double alpha, double beta) {
+  *p = mode == 2 ? fma(alpha, x, beta * *p) : alpha * x;
+}
+__device__ __forceinline__ void store_out(double* p, double x, int mode, double alpha, double beta) {
+  if (mode == 0)
+    *p = x;
+  else
+    store_scaled(p, x, mode, alpha, beta);
 }
 
 // (hi 2^sh + lo) 2^e rounded to the nearest FP64 (ties to even), 0 < sh < 64,
@@ -234,11 +261,10 @@ struct EmuAcc<Form10x6> {
   __device__ __forceinline__ double result(int) const { return s; }
 };
 
-template <class F>
-__global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(const __grid_constant__ CUtensorMap mA,
-                                                           const __grid_constant__ CUtensorMap mB,
-                                                           EmuArgs args) {
+template <class F, int bn>
+__global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
   constexpr int S = F::S;
+  constexpr int kSteps = F::kChunk / EBK;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + ESTAGES * Tile<F>::kStage);
@@ -249,12 +275,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(const __grid_constant_
   uint32_t* tmem_slot = (uint32_t*)(done + 1);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int bn = args.bn;
-  const int n0 = (int)(blockIdx.x % args.ntn) * bn, m0 = (int)(blockIdx.x / args.ntn) * EBM;
-  const int c0 = blockIdx.y * args.cps, c1 = min(args.nchunk, c0 + args.cps);
-  const int kbeg = c0 * F::kChunk, kend = min(args.K, c1 * F::kChunk);
-  const int nk = (kend - kbeg + EBK - 1) / EBK;  // stages (kChunk is a multiple of EBK)
-  const uint32_t stage_tx = (uint32_t)(Tile<F>::kABytes + S * bn * EBK * 2);
+  const int items = args.tiles * args.ns;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < ESTAGES; s++) {
@@ -278,140 +299,191 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(const __grid_constant_
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
+  // work item w: tile w % tiles, contraction slice w / tiles
   if (warp == 0) {
     if (lane == 0) {
       // producer
-      int issued = 0;
-      for (int i = 0; i < nk; i++) {
-        const int s = i % ESTAGES;
-        if (i >= ESTAGES && !mbar_wait(&empty[s], ((i / ESTAGES) - 1) & 1)) {
-          *abort_flag = 1;
-          break;
+      int it = 0;  // stages issued
+      for (int w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
+        const int t = w % args.tiles, c0 = (w / args.tiles) * args.cps;
+        const int n0 = (t % args.ntn) * bn, m0 = (t / args.ntn) * EBM;
+        const int s0 = c0 * kSteps;
+        const int s1 = min((args.K + EBK - 1) / EBK, (c0 + args.cps) * kSteps);
+        const uint32_t ba = (uint32_t)(min(EBM, (args.ra - m0 + 7) & ~7) * 32);
+        const uint32_t bb = (uint32_t)(min(bn, (args.rb - n0 + 7) & ~7) * 32);
+        const __half* ga = args.sa + (size_t)s0 * S * args.pa + (size_t)m0 * 16;
+        const __half* gb = args.sb + (size_t)s0 * S * args.pb + (size_t)n0 * 16;
+        for (int i = s0; i < s1; i++, it++) {
+          const int s = it % ESTAGES;
+          if (it >= ESTAGES && !mbar_wait(&empty[s], ((it / ESTAGES) - 1) & 1)) *abort_flag = 1;
+          if (*abort_flag) break;
+          uint8_t* st = smem + s * Tile<F>::kStage;
+          mbar_expect_tx(&full[s], S * (ba + bb));
+#pragma unroll
+          for (int p = 0; p < S; p++) {
+            bulk_load(st + p * A_SLICE, ga, ba, &full[s]);
+            bulk_load(st + Tile<F>::kABytes + p * bn * EBK * 2, gb, bb, &full[s]);
+            ga += args.pa;
+            gb += args.pb;
+          }
         }
-        if (*abort_flag) break;
-        uint8_t* st = smem + s * Tile<F>::kStage;
-        mbar_expect_tx(&full[s], stage_tx);
-        tma_load(st, &mA, &full[s], kbeg + i * EBK, m0, 0);
-        tma_load(st + Tile<F>::kABytes, &mB, &full[s], kbeg + i * EBK, n0, 0);
-        issued = i + 1;
       }
-      for (int i = (issued > ESTAGES ? issued - ESTAGES : 0); i < issued; i++)
+      // no copy is left in flight
+      for (int i = (it > ESTAGES ? it - ESTAGES : 0); i < it; i++)
         mbar_wait(&full[i % ESTAGES], (i / ESTAGES) & 1);
     }
   } else if (warp == 1) {
     if (lane == 0) {
       // MMA issuer: slice products p + q < S into accumulator p + q
-      const int per = 256 / bn;  // B slices per instruction
-      constexpr int kSteps = F::kChunk / EBK;
-      for (int i = 0; i < nk; i++) {
-        const int s = i % ESTAGES, in = i % kSteps, ch = i / kSteps;
-        // a new chunk: the epilogue must have read the previous one
-        if (in == 0 && ch > 0 && !mbar_wait(acc_empty, (ch - 1) & 1)) {
-          *abort_flag = 1;
-          break;
-        }
-        if (!mbar_wait(&full[s], (i / ESTAGES) & 1)) {
-          *abort_flag = 1;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        uint8_t* st = smem + s * Tile<F>::kStage;
-#pragma unroll 1
-        for (int p = 0; p < S; p++) {
-          const uint64_t da = desc_sw32(st + p * A_SLICE);
-          for (int q = 0; q < S - p; q += per) {
-            const int nq = min(per, S - p - q);
-            const uint64_t db = desc_sw32(st + Tile<F>::kABytes + q * bn * EBK * 2);
-            mma_f16(tmem + (uint32_t)((p + q) * bn), da, db, idesc_f16(nq * bn),
-                    (in > 0 || p > 0) ? 1u : 0u);
+      constexpr int per = 256 / bn;  // B slices per instruction
+      int it = 0, nch = 0;       // stages, chunks issued
+      for (int w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
+        const int c0 = (w / args.tiles) * args.cps;
+        const int s0 = c0 * kSteps;
+        const int s1 = min((args.K + EBK - 1) / EBK, (c0 + args.cps) * kSteps);
+        for (int i = s0; i < s1; i++, it++) {
+          const int s = it % ESTAGES, in = i % kSteps;
+          // a new chunk: the epilogue must have read the previous one
+          if (in == 0) {
+            if (nch > 0 && !mbar_wait(acc_empty, (nch - 1) & 1)) *abort_flag = 1;
+            nch++;
           }
+          if (*abort_flag || !mbar_wait(&full[s], (it / ESTAGES) & 1)) {
+            *abort_flag = 1;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          // (fully unrolled: descriptors, columns and shapes are the stage's
+          // base plus constants.  One thread feeds the tensor core, and an
+          // instruction of N = 240 lasts about 120 cycles)
+          const uint64_t d0 = desc_sw32(smem + s * Tile<F>::kStage);
+          const uint32_t acc = in > 0 ? 1u : 0u;
+#pragma unroll
+          for (int p = 0; p < S; p++) {
+#pragma unroll
+            for (int q = 0; q < S - p; q += per) {
+              const int nq = per < S - p - q ? per : S - p - q;
+              mma_f16(tmem + (uint32_t)((p + q) * bn), d0 + (p * A_SLICE >> 4),
+                      d0 + ((Tile<F>::kABytes + q * bn * EBK * 2) >> 4), idesc_f16(nq * bn),
+                      p > 0 ? 1u : acc);
+            }
+          }
+          mma_commit(&empty[s]);
+          if (in == kSteps - 1 || i == s1 - 1) mma_commit(acc_full);
         }
-        mma_commit(&empty[s]);
-        if (in == kSteps - 1 || i == nk - 1) mma_commit(acc_full);
       }
       // nothing is left in flight when the tensor memory is freed, whatever happened
       mma_commit(done);
       if (!mbar_wait(done, 0)) *abort_flag = 1;
     }
   } else {
-    // epilogue: row = TMEM lane of this warp's quadrant, column blocks of 8
-    // shared between the two warps of a quadrant
-    constexpr int NB = F::kMaxBN / 16;
-    EmuAcc<F> acc[NB][8];
-#pragma unroll
-    for (int b = 0; b < NB; b++)
-#pragma unroll
-      for (int j = 0; j < 8; j++) acc[b][j].zero();
-    const int quad = warp & 3, half = (warp - 2) >> 2;
-    const int row = m0 + quad * 32 + lane;
-    const bool live = row < args.M;
-    const int er = live ? args.ea[row] : 0;
-    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
+    // epilogue: row = TMEM lane of this warp's quadrant; the four warps of a
+    // quadrant take bn / 4 columns each, read four at a time
+    constexpr int ncol = bn / 4, NB = ncol / 4;  // blocks of four columns
+    const int quad = warp & 3, cg = (warp - 2) >> 2;
+    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(cg * ncol);
+    const EmuEpilogue& ep = args.ep;
+    int nch = 0;
     bool good = true;
-    for (int ch = 0; ch < c1 - c0; ch++) {
-      if (!mbar_wait(acc_full, ch & 1) || *abort_flag) {
-        good = false;
-        break;
+    for (int w = blockIdx.x; w < items && good; w += gridDim.x) {
+      const int t = w % args.tiles, z = w / args.tiles, c0 = z * args.cps;
+      const int nc = min(args.nchunk, c0 + args.cps) - c0;
+      const int n0 = (t % args.ntn) * bn + cg * ncol;
+      const int row = (t / args.ntn) * EBM + quad * 32 + lane;
+      const bool live = row < args.M;
+      const int lr = live ? args.ea[row] : kEmuNoLead;
+      const int er = row_frame(lr);
+      // lane j < ncol holds column j's exponent and output offset
+      const int mc = n0 + lane;
+      const int lc = (lane < ncol && mc < args.N) ? args.eb[mc] : kEmuNoLead;
+      long long coff = 0;
+      int lidx = 0;
+      if (lane < ncol && mc < args.N) {
+        coff = emu_off(mc, ep.cin, ep.cld, ep.cs);
+        if (ep.lead) lidx = ((mc / ep.lcd) % ep.lcm) * ep.lcs;
       }
-      __syncwarp();
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      EmuAcc<F> acc[NB][4];
 #pragma unroll
-      for (int b = 0; b < NB; b++) {
-        const int cb = b * 16 + half * 8;
-        if (cb < bn) {
+      for (int b = 0; b < NB; b++)
 #pragma unroll
-          for (int h = 0; h < 2; h++) {
-            float v[S][4];
+        for (int j = 0; j < 4; j++) acc[b][j].zero();
+      for (int ch = 0; ch < nc; ch++, nch++) {
+        if (!mbar_wait(acc_full, nch & 1) || *abort_flag) {
+          good = false;
+          break;
+        }
+        __syncwarp();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-            for (int g = 0; g < S; g++) tmem_ld4(lane_base + (uint32_t)(g * bn + cb + 4 * h), v[g]);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        for (int b = 0; b < NB; b++) {
+          float v[S][4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-              float u[S];
+          for (int g = 0; g < S; g++) tmem_ld4(lane_base + (uint32_t)(g * bn + 4 * b), v[g]);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-              for (int g = 0; g < S; g++) u[g] = v[g][j];
-              int e = 0;
-              if (!F::kBalanced) e = er + args.eb[min(n0 + cb + 4 * h + j, args.N - 1)];
-              acc[b][4 * h + j].add(u, e, ch == 0);
-            }
+          for (int j = 0; j < 4; j++) {
+            float u[S];
+#pragma unroll
+            for (int g = 0; g < S; g++) u[g] = v[g][j];
+            int e = 0;
+            if (!F::kBalanced) e = er + row_frame(__shfl_sync(0xffffffffu, lc, 4 * b + j));
+            acc[b][j].add(u, e, ch == 0);
           }
         }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty);
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(acc_empty);
-    }
-    if (!good) *abort_flag = 1;
-    const EmuEpilogue& ep = args.ep;
-    if (good && live) {
-      const long long roff = emu_off(row, ep.rin, ep.rld, ep.rs);
+      if (!good) break;
+      double* prow = ep.c64 + emu_off(row, ep.rin, ep.rld, ep.rs);
+      const int lrow = ep.lead ? ((row / ep.lrd) % ep.lrm) * ep.lrs : 0;
+      const bool one_row = __all_sync(0xffffffffu, lrow == __shfl_sync(0xffffffffu, lrow, 0) && live);
+      int lcur = -1, lmax = kEmuNoLead;
+      auto flush = [&] {  // the running exponent of lead column lcur
+        if (lcur < 0) return;
+        if (one_row) {
+          const int m = __reduce_max_sync(0xffffffffu, lmax);
+          if (lane == 0) atomicMax(ep.lead + lrow + lcur, m);
+        } else if (live) {
+          atomicMax(ep.lead + lrow + lcur, lmax);
+        }
+        lmax = kEmuNoLead;
+      };
 #pragma unroll
       for (int b = 0; b < NB; b++) {
-        const int cb = b * 16 + half * 8;
 #pragma unroll
-        for (int j = 0; j < 8; j++) {
-          const int col = n0 + cb + j;
-          if (cb >= bn || col >= args.N) continue;
+        for (int j = 0; j < 4; j++) {
+          const int jc = 4 * b + j;
+          if (n0 + jc >= args.N) continue;  // warp-uniform
+          const int lcj = __shfl_sync(0xffffffffu, lc, jc);
+          const long long cj = __shfl_sync(0xffffffffu, coff, jc);
           if constexpr (F::kBalanced) {
             if (args.ws) {  // one slice of the contraction: integer partial sums
-              longlong2 t;
-              t.x = acc[b][j].hi;
-              t.y = acc[b][j].lo;
-              args.ws[((size_t)blockIdx.y * args.M + row) * args.N + col] = t;
+              longlong2 s;
+              s.x = acc[b][j].hi;
+              s.y = acc[b][j].lo;
+              if (live) args.ws[((size_t)z * args.M + row) * args.N + n0 + jc] = s;
               continue;
             }
           }
-          const int ec = args.eb[col];
-          double x = acc[b][j].result(er + ec);
-          if (er >= kEmuNonFinite / 2 || ec >= kEmuNonFinite / 2) x = __longlong_as_double(0x7ff8000000000000ll);
-          double* p = ep.c64 + roff + emu_off(col, ep.cin, ep.cld, ep.cs);
-          if (ep.beta != 0.0)
-            *p = fma(ep.alpha, x, ep.beta * *p);
-          else
-            *p = ep.alpha == 1.0 ? x : ep.alpha * x;
+          double x = acc[b][j].result(er + row_frame(lcj));
+          if (row_bad(lr) || row_bad(lcj)) x = __longlong_as_double(0x7ff8000000000000ll);
+          if (ep.lead) {
+            const int li = __shfl_sync(0xffffffffu, lidx, jc);
+            if (li != lcur) {
+              flush();
+              lcur = li;
+            }
+            lmax = max(lmax, lead_exp(x));
+          }
+          if (!live) continue;
+          double* p = prow + cj;
+          store_out(p, x, args.mode, ep.alpha, ep.beta);
         }
       }
+      if (ep.lead) flush();
     }
+    if (!good) *abort_flag = 1;
   }
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -437,201 +509,231 @@ __global__ void __launch_bounds__(256) k_emu_finish(EmuArgs args, int nsplit) {
     lo += w.y;
   }
   const int row = (int)(t / args.N), col = (int)(t % args.N);
-  const int er = args.ea[row], ec = args.eb[col];
-  double x = EmuAcc<Form9x7>::value(hi, lo, er + ec);
-  if (er >= kEmuNonFinite / 2 || ec >= kEmuNonFinite / 2) x = __longlong_as_double(0x7ff8000000000000ll);
+  const int lr = args.ea[row], lc = args.eb[col];
+  double x = EmuAcc<Form9x7>::value(hi, lo, row_frame(lr) + row_frame(lc));
+  if (row_bad(lr) || row_bad(lc)) x = __longlong_as_double(0x7ff8000000000000ll);
   const EmuEpilogue& ep = args.ep;
+  if (ep.lead)
+    atomicMax(ep.lead + ((row / ep.lrd) % ep.lrm) * ep.lrs + ((col / ep.lcd) % ep.lcm) * ep.lcs,
+              lead_exp(x));
   double* p = ep.c64 + emu_off(row, ep.rin, ep.rld, ep.rs) + emu_off(col, ep.cin, ep.cld, ep.cs);
-  if (ep.beta != 0.0)
-    *p = fma(ep.alpha, x, ep.beta * *p);
-  else
-    *p = ep.alpha == 1.0 ? x : ep.alpha * x;
+  store_out(p, x, args.mode, ep.alpha, ep.beta);
 }
 
 // ------------------------------------------------------------------ slicing
-// Row exponents: E_r = 1 + max_k floor(log2 |x_rk|) (subnormals included;
-// 0 for a row of zeros), so that every |x_rk| < 2^(E_r).
-constexpr int kNoLead = -4096;
-constexpr int kLeadBad = 1024;  // lead_exp of an infinity or a NaN
-__device__ __forceinline__ int lead_exp(double x) {
+// Digits of elements in their row frame, on the integer pipe: a fixed-point
+// number per element, then word(p) = digits p of two of them as an FP16 pair.
+// A digit u + bias is turned into FP16 by or-ing it into the significand of
+// 1024 and subtracting 1024 + bias.
+__device__ __forceinline__ unsigned sub_half2(unsigned w, unsigned short bias) {
+  const __half2 b = __halves2half2(__ushort_as_half(bias), __ushort_as_half(bias));
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), b);
+  return *reinterpret_cast<const unsigned*>(&h);
+}
+// |x| = m 2^q
+__device__ __forceinline__ unsigned long long split_double(double x, int& q) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int ef = (int)((b >> 52) & 0x7FF);
-  if (ef) return ef - 1023;
   const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-  return m ? -1011 - __clzll(m) : kNoLead;  // -1074 + (63 - clz)
+  q = ef ? ef - 1075 : -1074;
+  return ef ? m | (1ull << 52) : m;
 }
-__device__ __forceinline__ int row_frame(int lead) {
-  return lead == kNoLead ? 0 : lead >= kLeadBad ? kEmuNonFinite : lead + 1;
-}
-
-// Digits of two elements in their row frame as FP16 pairs d[p] = (digit p of
-// x0, digit p of x1), on the integer pipe.  A digit u + bias is turned into
-// FP16 by or-ing it into the significand of 1024 and subtracting 1024 + bias.
 template <class F>
-struct Digits;
+struct Fixed;
 template <>
-struct Digits<Form10x6> {
+struct Fixed<Form10x6> {
   // X = floor(|x| 2^(60 - E)), d_p = its bits [60 - 6(p+1), 60 - 6p), signed like x
-  static __device__ __forceinline__ unsigned long long fixed(double x, int E, unsigned& neg) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int ef = (int)((b >> 52) & 0x7FF);
-    unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-    int q = -1074;  // |x| = m 2^q
-    if (ef) {
-      m |= 1ull << 52;
-      q = ef - 1075;
-    }
-    neg = (unsigned)(b >> 63);
+  unsigned long long X;
+  unsigned sign;
+  __device__ __forceinline__ void set(double x, int E) {
+    int q;
+    const unsigned long long m = split_double(x, q);
+    sign = (unsigned)((unsigned long long)__double_as_longlong(x) >> 63) << 15;
     const int sh = q + Form10x6::kFrac - E;
-    return sh >= 0 ? (m << sh) : (sh <= -64 ? 0ull : (m >> -sh));
+    X = sh >= 0 ? (m << sh) : (sh <= -64 ? 0ull : (m >> -sh));
   }
-  static __device__ __forceinline__ void cut(double x0, double x1, int E, unsigned (&d)[10]) {
-    unsigned n0, n1;
-    const unsigned long long X0 = fixed(x0, E, n0), X1 = fixed(x1, E, n1);
-    const unsigned sign = (n0 << 15) | (n1 << 31);
-    const __half2 bias = __halves2half2(__ushort_as_half(0x6400), __ushort_as_half(0x6400));
-#pragma unroll
-    for (int p = 0; p < 10; p++) {
-      const int sh = 60 - 6 * (p + 1);
-      const unsigned w = ((unsigned)(X0 >> sh) & 63u) | (((unsigned)(X1 >> sh) & 63u) << 16) | 0x64006400u;
-      const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), bias);
-      d[p] = *reinterpret_cast<const unsigned*>(&h) ^ sign;
-    }
+  static __device__ __forceinline__ unsigned word(const Fixed& a, const Fixed& b, int p) {
+    const int sh = 60 - 6 * (p + 1);
+    const unsigned w = ((unsigned)(a.X >> sh) & 63u) | (((unsigned)(b.X >> sh) & 63u) << 16) | 0x64006400u;
+    return sub_half2(w, 0x6400) ^ (a.sign | (b.sign << 16));
   }
 };
 template <>
-struct Digits<Form9x7> {
-  // X = round(x 2^(62 - E)), |X| <= 2^62; with 64 added to each of the eight
-  // lower digits, digit p is a 7-bit field less 64 and the top digit, in
+struct Fixed<Form9x7> {
+  // X = round(x 2^(62 - E)), |X| <= 2^62, plus 64 in each of the eight lower
+  // digits: digit p is then a 7-bit field less 64 and the top digit, in
   // [-64, 64], what is left above
-  static __device__ __forceinline__ long long fixed(double x, int E) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int ef = (int)((b >> 52) & 0x7FF);
-    unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-    int q = -1074;
-    if (ef) {
-      m |= 1ull << 52;
-      q = ef - 1075;
-    }
+  long long X;
+  __device__ __forceinline__ void set(double x, int E) {
+    constexpr long long kBias = 64ll * (((1ll << 56) - 1) / 127);
+    int q;
+    const unsigned long long m = split_double(x, q);
     const int sh = q + Form9x7::kFrac - E;
-    const unsigned long long X =
+    const unsigned long long a =
         sh >= 0 ? (m << sh) : (sh <= -60 ? 0ull : ((m >> (-sh - 1)) + 1) >> 1);
-    return (b >> 63) ? -(long long)X : (long long)X;
+    X = (__double_as_longlong(x) < 0 ? -(long long)a : (long long)a) + kBias;
   }
-  static __device__ __forceinline__ void cut(double x0, double x1, int E, unsigned (&d)[9]) {
-    constexpr long long kBias = 64ll * ((1ll << 56) - 1) / 127;  // 64 in each of eight 7-bit fields
-    const long long X0 = fixed(x0, E) + kBias, X1 = fixed(x1, E) + kBias;
-    const __half2 bias = __halves2half2(__ushort_as_half(0x6440), __ushort_as_half(0x6440));  // 1088
-    const unsigned t0 = (unsigned)((int)(X0 >> 56) + 64), t1 = (unsigned)((int)(X1 >> 56) + 64);
-    unsigned w = t0 | (t1 << 16) | 0x64006400u;
-    __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), bias);
-    d[0] = *reinterpret_cast<const unsigned*>(&h);
-#pragma unroll
-    for (int p = 1; p < 9; p++) {
+  static __device__ __forceinline__ unsigned word(const Fixed& a, const Fixed& b, int p) {
+    unsigned w;
+    if (p == 0) {
+      w = (unsigned)((int)(a.X >> 56) + 64) | ((unsigned)((int)(b.X >> 56) + 64) << 16);
+    } else {
       const int sh = 7 * (8 - p);
-      w = ((unsigned)(X0 >> sh) & 127u) | (((unsigned)(X1 >> sh) & 127u) << 16) | 0x64006400u;
-      h = __hsub2(*reinterpret_cast<const __half2*>(&w), bias);
-      d[p] = *reinterpret_cast<const unsigned*>(&h);
+      w = ((unsigned)(a.X >> sh) & 127u) | (((unsigned)(b.X >> sh) & 127u) << 16);
     }
+    return sub_half2(w | 0x64006400u, 0x6440);  // 1024 + 64
   }
 };
 
-// four consecutive digits per slice of one row, 8-byte stores
+// eight consecutive digits per slice of one row (half of a K step): 16-byte
+// stores, o = the K step's first slice
 template <class F>
-__device__ __forceinline__ void put4(const double (&x)[4], int E, __half* o, size_t plane) {
-  unsigned a[F::S], b[F::S];
-  if (E == kEmuNonFinite) E = 0;  // digits are not used
-  Digits<F>::cut(x[0], x[1], E, a);
-  Digits<F>::cut(x[2], x[3], E, b);
+__device__ __forceinline__ void put8(const double (&x)[8], int lead, __half* o, long long groups, int r,
+                                     int half) {
+  Fixed<F> f[8];
+  const int E = row_bad(lead) ? 0 : row_frame(lead);  // digits of a bad row are not used
 #pragma unroll
-  for (int p = 0; p < F::S; p++) *reinterpret_cast<uint2*>(o + (size_t)p * plane) = make_uint2(a[p], b[p]);
+  for (int i = 0; i < 8; i++) f[i].set(row_bad(lead) ? 0.0 : x[i], E);
+  o += (size_t)(r >> 3) * 128 + (r & 7) * 16 + ((half ^ ((r >> 2) & 1)) << 3);
+#pragma unroll
+  for (int p = 0; p < F::S; p++)
+    *reinterpret_cast<uint4*>(o + (size_t)p * groups * 128) =
+        make_uint4(Fixed<F>::word(f[0], f[1], p), Fixed<F>::word(f[2], f[3], p),
+                   Fixed<F>::word(f[4], f[5], p), Fixed<F>::word(f[6], f[7], p));
 }
 
-// Rows contiguous in k: TPR threads per row find the row's exponent, then cut
-// it (the second read comes from L2: one pass over DRAM instead of two).
-template <class F, int TPR>
+__device__ __forceinline__ bool src_row(const EmuSource& src, int r, int rows, long long& off) {
+  if (r >= rows) return false;
+  off = emu_off(r, src.rin, src.rld, src.rs);
+  return src.rvalid == 0 || r % src.rin < src.rvalid;
+}
+
+// Row exponents of rows contiguous in k, one CTA per row.
+__global__ void __launch_bounds__(256) k_emu_lead(EmuSource src, int rows, int K, int* __restrict__ E) {
+  __shared__ int red[8];
+  long long off = 0;
+  const int r = blockIdx.x;
+  int m = kEmuNoLead;
+  if (src_row(src, r, rows, off))
+    for (int k = threadIdx.x; k < K; k += 256) m = max(m, lead_exp(src.p[off + k]));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) m = max(m, red[w]);
+    E[r] = m;
+  }
+}
+
+// Rows contiguous in k: 16 rows per CTA; lane = (row, half of a K step), one K
+// step per warp, so that a warp's stores fill two row groups of a slice.  With
+// LEAD the CTA first finds its rows' exponents (two rows per warp; the second
+// read comes from L2: one pass over DRAM) and takes every K step; otherwise E
+// holds them and the K steps are spread over blockIdx.y.
+template <class F, bool LEAD>
 __global__ void __launch_bounds__(256) k_emu_slice_rows(EmuSource src, int rows, int K,
                                                         int* __restrict__ E, __half* __restrict__ out,
-                                                        int ldk) {
-  __shared__ int red[8];
-  const int r = blockIdx.x * (256 / TPR) + threadIdx.x / TPR;
-  const int t = threadIdx.x % TPR;
-  const bool on = r < rows;
-  const double* x = on ? src.p + emu_off(r, src.rin, src.rld, src.rs) : src.p;
-  int m = kNoLead;
-  if (on)
-    for (int k = t; k < K; k += TPR) m = max(m, lead_exp(x[k]));
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (TPR > 32) {
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    for (int w = 0; w < 8; w++) m = max(m, red[w]);
-  }
-  if (!on) return;
-  const int e = row_frame(m);
-  if (t == 0) E[r] = e;
-  const size_t plane = (size_t)rows * ldk;
-  for (int k = 4 * t; k < ldk; k += 4 * TPR) {
-    double v[4];
+                                                        long long groups) {
+  __shared__ int ex[16];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r0 = blockIdx.x * 16;
+  if (LEAD) {
 #pragma unroll
-    for (int i = 0; i < 4; i++) v[i] = k + i < K ? x[k + i] : 0.0;
-    put4<F>(v, e, out + (size_t)r * ldk + k, plane);
+    for (int h = 0; h < 2; h++) {
+      const int r = r0 + 2 * warp + h;
+      long long off = 0;
+      int m = kEmuNoLead;
+      if (src_row(src, r, rows, off))
+        for (int k = lane; k < K; k += 32) m = max(m, lead_exp(src.p[off + k]));
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0) {
+        ex[2 * warp + h] = m;
+        if (r < rows) E[r] = m;
+      }
+    }
+    __syncthreads();
+  }
+  const int r = r0 + (lane >> 1), half = lane & 1;
+  if ((r >> 3) >= groups) return;
+  long long off = 0;
+  const bool on = src_row(src, r, rows, off);
+  const int lead = LEAD ? ex[lane >> 1] : (r < rows ? E[r] : kEmuNoLead);
+  const double* x = src.p + off;
+  const int nk = (K + 15) / 16;
+  for (int s = blockIdx.y * 8 + warp; s < nk; s += gridDim.y * 8) {
+    const int k = s * 16 + half * 8;
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) v[i] = (on && k + i < K) ? x[k + i] : 0.0;
+    put8<F>(v, lead, out + (size_t)s * F::S * groups * 128, groups, r, half);
   }
 }
 
 // Rows strided in k (consecutive rows adjacent in memory): 32 rows per CTA,
-// lanes along the rows for the reads, transposed through shared memory.
-template <class F>
+// lanes along the rows for the reads, transposed through shared memory.  LEAD
+// and blockIdx.y as in k_emu_slice_rows.
+template <class F, bool LEAD>
 __global__ void __launch_bounds__(256) k_emu_slice_cols(EmuSource src, int rows, int K,
                                                         int* __restrict__ E, __half* __restrict__ out,
-                                                        int ldk) {
+                                                        long long groups) {
   __shared__ double tile[64][33];  // [k][r]
   __shared__ int red[8][32];
   const int r0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const bool on = r0 + tx < rows;
-  const double* x = src.p + (on ? emu_off(r0 + tx, src.rin, src.rld, src.rs) : 0);
-  int m = kNoLead;
-  if (on)
+  long long off = 0;
+  const bool on = src_row(src, r0 + tx, rows, off);
+  const double* x = src.p + off;
+  if (LEAD) {
+    int m = kEmuNoLead;
+    if (on)
 #pragma unroll 4
-    for (int k = ty; k < K; k += 8) m = max(m, lead_exp(x[(size_t)k * src.ks]));
-  red[ty][tx] = m;
-  __syncthreads();
-  if (ty == 0) {
-    for (int y = 1; y < 8; y++) m = max(m, red[y][tx]);
-    m = row_frame(m);
-    red[0][tx] = m;
-    if (on) E[r0 + tx] = m;
+      for (int k = ty; k < K; k += 8) m = max(m, lead_exp(x[(size_t)k * src.ks]));
+    red[ty][tx] = m;
+    __syncthreads();
+    if (ty == 0) {
+      for (int y = 1; y < 8; y++) m = max(m, red[y][tx]);
+      red[0][tx] = m;
+      if (r0 + tx < rows) E[r0 + tx] = m;
+    }
+  } else if (ty == 0) {
+    red[0][tx] = r0 + tx < rows ? E[r0 + tx] : kEmuNoLead;
   }
-  const size_t plane = (size_t)rows * ldk;
-  const int q = threadIdx.x & 15, rr0 = threadIdx.x >> 4;  // 16 threads x 4 digits per row
-  for (int k0 = 0; k0 < ldk; k0 += 64) {
+  // warp = (K step of the tile, rows 0-15 / 16-31), lane = (row, half of the K step)
+  const int rr = (ty & 1) * 16 + (tx >> 1), ks = ty >> 1, half = tx & 1;
+  const int nk = (K + 15) / 16;
+  for (int s0 = blockIdx.y * 4; s0 < nk; s0 += gridDim.y * 4) {
     __syncthreads();
 #pragma unroll
     for (int kk = ty; kk < 64; kk += 8)
-      tile[kk][tx] = (on && k0 + kk < K) ? x[(size_t)(k0 + kk) * src.ks] : 0.0;
+      tile[kk][tx] = (on && s0 * 16 + kk < K) ? x[(size_t)(s0 * 16 + kk) * src.ks] : 0.0;
     __syncthreads();
+    if (s0 + ks >= nk || ((r0 + rr) >> 3) >= groups) continue;
+    double v[8];
 #pragma unroll
-    for (int rr = rr0; rr < 32; rr += 16) {
-      const int k = k0 + 4 * q;
-      if (r0 + rr >= rows || k >= ldk) continue;
-      double v[4];
-#pragma unroll
-      for (int i = 0; i < 4; i++) v[i] = tile[4 * q + i][rr];
-      put4<F>(v, red[0][rr], out + (size_t)(r0 + rr) * ldk + k, plane);
-    }
+    for (int i = 0; i < 8; i++) v[i] = tile[ks * 16 + half * 8 + i][rr];
+    put8<F>(v, red[0][rr], out + (size_t)(s0 + ks) * F::S * groups * 128, groups, r0 + rr, half);
   }
 }
 
 template <class F>
-void slice_form(const EmuSource& src, int rows, int K, EmuOperand& op, cudaStream_t st) {
-  if (src.ks == 1) {
-    // long rows take a CTA each so that a few hundred rows fill the device
-    if (K >= 2048)
-      k_emu_slice_rows<F, 256><<<rows, 256, 0, st>>>(src, rows, K, op.e, op.s, op.ldk);
-    else
-      k_emu_slice_rows<F, 32><<<cdiv(rows, 8), 256, 0, st>>>(src, rows, K, op.e, op.s, op.ldk);
+void slice_form(const EmuSource& src, int rows, int K, EmuOperand& op, cudaStream_t st, bool have_lead) {
+  const int nk = cdiv(K, 16);
+  if (src.ks != 1) {
+    if (have_lead) {
+      const int ny = std::min(cdiv(nk, 4), std::max(1, cdiv(8 * 152, cdiv(rows, 32))));
+      k_emu_slice_cols<F, false><<<dim3(cdiv(rows, 32), ny), 256, 0, st>>>(src, rows, K, op.e, op.s, op.groups);
+    } else {
+      k_emu_slice_cols<F, true><<<cdiv(rows, 32), 256, 0, st>>>(src, rows, K, op.e, op.s, op.groups);
+    }
+  } else if (have_lead || K >= 2048) {
+    // few long rows: exponents first, one row per CTA, so that a few hundred
+    // rows fill the device
+    if (!have_lead) {
+      k_emu_lead<<<rows, 256, 0, st>>>(src, rows, K, op.e);
+      RIS_CHECK_LAUNCH();
+    }
+    const int ny = std::min(cdiv(nk, 8), std::max(1, cdiv(8 * 152, cdiv(rows, 16))));
+    k_emu_slice_rows<F, false><<<dim3(cdiv(rows, 16), ny), 256, 0, st>>>(src, rows, K, op.e, op.s, op.groups);
   } else {
-    k_emu_slice_cols<F><<<cdiv(rows, 32), 256, 0, st>>>(src, rows, K, op.e, op.s, op.ldk);
+    k_emu_slice_rows<F, true><<<cdiv(rows, 16), 256, 0, st>>>(src, rows, K, op.e, op.s, op.groups);
   }
   RIS_CHECK_LAUNCH();
 }
@@ -649,21 +751,29 @@ int pick_bn(int N, int max_bn) {
 template <class F>
 void gemm_pass(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep,
                int* d_err, cudaStream_t st) {
-  ensure_smem_attr((const void*)k_emu_gemm<F>, Tile<F>::kSmem);
   EmuArgs a;
   a.M = M;
   a.N = N;
   a.K = A.K;
-  a.bn = pick_bn(N, F::kMaxBN);
-  a.ntn = cdiv(N, a.bn);
+  const int bn = pick_bn(N, F::kMaxBN);
+  a.ntn = cdiv(N, bn);
   a.nchunk = cdiv(A.K, F::kChunk);
+  RIS_REQUIRE((((uintptr_t)A.s | (uintptr_t)B.s) & 15) == 0, RIS_ERR_ARG, "emu_gemm: slices not 16-byte aligned");
+  a.sa = A.s;
+  a.sb = B.s;
+  a.pa = A.groups * 128;
+  a.pb = B.groups * 128;
+  a.ra = A.rows;
+  a.rb = B.rows;
   a.ea = A.e;
   a.eb = B.e;
   a.ws = nullptr;
   a.ep = ep;
+  a.mode = ep.beta != 0.0 ? 2 : ep.alpha != 1.0 ? 1 : 0;
   a.err = d_err;
   const long long tiles = (long long)a.ntn * cdiv(M, EBM);
-  RIS_REQUIRE(tiles < (1LL << 31), RIS_ERR_ARG, "emu_gemm: too many tiles");
+  RIS_REQUIRE(tiles * 64 < (1LL << 31), RIS_ERR_ARG, "emu_gemm: too many tiles");
+  a.tiles = (int)tiles;
   // slices of a long contraction: the number of chunk rounds of the busiest
   // SM, plus about a chunk's time for each CTA's start and end
   int ns = 1;
@@ -681,12 +791,13 @@ void gemm_pass(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
     }
   }
   a.cps = cdiv(a.nchunk, ns);
+  a.ns = ns;
   MemTrack* tr = nullptr;
   const size_t wsb = (size_t)ns * M * N * sizeof(longlong2);
   if (ns > 1) a.ws = (longlong2*)dev_alloc(wsb, st, &tr);
-  const CUtensorMap mA = make_map(A, F::S, EBM);
-  const CUtensorMap mB = make_map(B, F::S, a.bn);
-  k_emu_gemm<F><<<dim3((unsigned)tiles, ns), ETHREADS, Tile<F>::kSmem, st>>>(mA, mB, a);
+  auto kern = bn == 48 ? k_emu_gemm<F, 48> : bn == 32 ? k_emu_gemm<F, 32> : k_emu_gemm<F, 16>;
+  ensure_smem_attr((const void*)kern, Tile<F>::kSmem);
+  kern<<<(unsigned)std::min<long long>(tiles * ns, 152), ETHREADS, Tile<F>::kSmem, st>>>(a);
   RIS_CHECK_LAUNCH();
   if (ns > 1) {
     k_emu_finish<<<cdiv((long long)M * N, 256), 256, 0, st>>>(a, ns);
@@ -706,8 +817,8 @@ void gemm_form(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
   for (int k0 = 0; k0 < A.K; k0 += kPass) {
     EmuOperand a = A, b = B;
     EmuEpilogue e = ep;
-    a.s = A.s + k0;
-    b.s = B.s + k0;
+    a.s = A.s + (size_t)(k0 / EBK) * F::S * A.groups * 128;
+    b.s = B.s + (size_t)(k0 / EBK) * F::S * B.groups * 128;
     a.K = b.K = std::min(kPass, A.K - k0);
     if (k0 > 0) e.beta = 1.0;
     gemm_pass<F>(M, N, a, b, e, d_err, st);
@@ -717,16 +828,16 @@ void gemm_form(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
 
 }  // namespace
 
-void emu_slice(EmuForm f, const EmuSource& src, int rows, int K, EmuOperand& op, cudaStream_t st) {
+void emu_slice(EmuForm f, const EmuSource& src, int rows, int K, EmuOperand& op, cudaStream_t st,
+               bool have_lead) {
   RIS_REQUIRE(rows > 0 && K > 0 && op.s && op.e, RIS_ERR_ARG, "emu_slice: bad operand");
   op.rows = rows;
   op.K = K;
-  op.ldk = ld8(K);
-  op.plane = (long long)rows * op.ldk;
+  op.groups = (rows + 7) / 8;
   if (f == kEmu10x6)
-    slice_form<Form10x6>(src, rows, K, op, st);
+    slice_form<Form10x6>(src, rows, K, op, st, have_lead);
   else
-    slice_form<Form9x7>(src, rows, K, op, st);
+    slice_form<Form9x7>(src, rows, K, op, st, have_lead);
 }
 
 void emu_gemm(EmuForm f, int M, int N, const EmuOperand& A, const EmuOperand& B,

@@ -20,20 +20,25 @@ namespace ris {
 enum EmuForm { kEmu10x6 = 0, kEmu9x7 = 1 };
 constexpr int emu_slices(EmuForm f) { return f == kEmu10x6 ? 10 : 9; }
 
-// A sliced operand: digits as FP16 integers [slices][rows][ldk] (K
-// contiguous, ldk % 8 == 0, zero past K) and the row exponents E[rows]
-// (kEmuNonFinite for a row that holds an infinity or a NaN: every product
-// with it is NaN).
-constexpr int kEmuNonFinite = 1 << 20;
+// A sliced operand: FP16 integer digits in the layout in which the GEMM's
+// stages lie in shared memory, so that a stage is a few contiguous copies:
+//   [K step of 16][slice][row group of 8][8 rows x 32 bytes]
+// with the two 16-byte halves of rows 4..7 of a group exchanged (the 32-byte
+// swizzle of the tensor core's operand tiles), zero past K; and per row the
+// exponent of its largest magnitude (kEmuNoLead for a row of zeros; at least
+// kEmuLeadBad for a row that holds an infinity or a NaN: every product with it
+// is NaN).
+constexpr int kEmuNoLead = (int)0x80808080;  // set by a byte fill of 0x80
+constexpr int kEmuLeadBad = 1024;
 struct EmuOperand {
   __half* s = nullptr;
   int* e = nullptr;
-  int rows = 0, K = 0, ldk = 0;
-  long long plane = 0;  // elements between slices
-  // rows r0 .. r0 + n - 1
+  int rows = 0, K = 0;
+  long long groups = 0;  // row groups per slice
+  // rows r0 .. r0 + n - 1, r0 a multiple of 8
   EmuOperand sub(long long r0, int n) const {
     EmuOperand o = *this;
-    o.s += r0 * ldk;
+    o.s += r0 * 16;
     o.e += r0;
     o.rows = n;
     return o;
@@ -43,20 +48,24 @@ struct EmuOperand {
 inline int ld8(int k) { return (k + 7) & ~7; }
 // halves an operand of the form needs (ints: rows)
 inline size_t emu_size(EmuForm f, long long rows, int K) {
-  return (size_t)emu_slices(f) * rows * ld8(K);
+  return (size_t)((K + 15) / 16) * emu_slices(f) * ((rows + 7) / 8) * 128;
 }
 
 // Source placement: element (r, k) of an operand at src[row(r) + k * ks] with
-// row(r) = (r / rin) * rld + (r % rin) * rs (rin = 0: r * rs).
+// row(r) = (r / rin) * rld + (r % rin) * rs (rin = 0: r * rs); rows with
+// r % rin >= rvalid are zero (rvalid = 0: none).
 struct EmuSource {
   const double* p = nullptr;
   long long rs = 0, ks = 1;
   int rin = 0;
   long long rld = 0;
+  int rvalid = 0;
 };
 
 // Slices src (rows x K) into op (op.s / op.e hold emu_size / rows elements).
-void emu_slice(EmuForm f, const EmuSource& src, int rows, int K, EmuOperand& op, cudaStream_t st);
+// have_lead: op.e already holds the row exponents (EmuEpilogue::lead).
+void emu_slice(EmuForm f, const EmuSource& src, int rows, int K, EmuOperand& op, cudaStream_t st,
+               bool have_lead = false);
 
 // Output placement: element (r, c) goes to
 //   c64[(r / rin) * rld + (r % rin) * rs + (c / cin) * cld + (c % cin) * cs]
@@ -66,6 +75,15 @@ struct EmuEpilogue {
   int rin = 0, cin = 0;
   long long rld = 0, rs = 0, cld = 0, cs = 1;
   double alpha = 1.0, beta = 0.0;
+  // lead: also the largest exponent of the outputs that the next product reads
+  // as one row, by atomic maximum into
+  //   lead[((r / lrd) % lrm) * lrs + ((c / lcd) % lcm) * lcs]
+  // (filled with kEmuNoLead before), so that slicing them needs no pass of its
+  // own for the row exponents
+  int* lead = nullptr;
+  int lrd = 1, lrm = 1, lrs = 0, lcd = 1, lcm = 1, lcs = 0;
+  void lead_rows(int d, int m, int s) { lrd = d; lrm = m; lrs = s; }
+  void lead_cols(int d, int m, int s) { lcd = d; lcm = m; lcs = s; }
 };
 
 // C (M x N) = A (M x K) . B (N x K)^T from operands sliced in form f; *d_err

@@ -48,10 +48,13 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sa(b)) : "memory");
 }
-__device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
+// try_wait suspends the thread in hardware for a while instead of polling: a
+// polling warp takes issue slots from the one thread that feeds the tensor
+// core (sixteen polling epilogue warps cost k_emu_gemm 20% of its main loop)
+__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
   uint32_t ok;
   asm volatile(
-      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
       " selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(ok)
       : "r"(sa(b)), "r"(parity)
@@ -60,8 +63,9 @@ __device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
 }
 // bounded wait; false on timeout
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity) {
+  if (mbar_try(b, parity)) return true;
   const long long t0 = clock64();
-  while (!mbar_test(b, parity)) {
+  while (!mbar_try(b, parity)) {
     if (clock64() - t0 > kWaitCycles) return false;
   }
   return true;
