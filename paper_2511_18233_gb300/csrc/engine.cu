@@ -1600,20 +1600,20 @@ void Engine::build_K_emu(const double* HK, double* Bvv) {
   const double* Cv = C.p + o;
   const EmuForm f = kEmu9x7;
   EmuMat cv, co, li, lt, a;
-  cv.slice(f, emu_src(Cv, 1, nmo), v, n, st);            // rows a over mu
-  li.slice(f, emu_src(LKinv.p, nK, 1), nK, nK, st);      // rows R over P
-  lt.slice(f, emu_src(LKinv.p, 1, nK), nK, nK, st);      // rows Q over R
+  cv.slice(f, emu_cols(v), emu_src(Cv, 1, nmo), v, n, st);            // rows a over mu
+  li.slice(f, emu_cols(nK), emu_src(LKinv.p, nK, 1), nK, nK, st);      // rows R over P
+  lt.slice(f, emu_cols(nK), emu_src(LKinv.p, 1, nK), nK, nK, st);      // rows Q over R
   // [x][y][P] -> B = . L^-T -> c = B L^-1, rows (x, y)
   auto metric = [&](const double* g, long long rows, double* B, double* c) {
-    a.slice(f, emu_src(g, nK, 1), rows, nK, st);
+    a.slice(f, kEmuRowsA, emu_src(g, nK, 1), rows, nK, st);
     emu97((int)rows, nK, a.op, li.op, emu_out(B, nK, 1));
-    a.slice(f, emu_src(B, nK, 1), rows, nK, st);
+    a.slice(f, kEmuRowsA, emu_src(B, nK, 1), rows, nK, st);
     emu97((int)rows, nK, a.op, lt.op, emu_out(c, nK, 1));
   };
   {  // rows (i,P) of HK over nu
     EmuMat h;
-    h.slice(f, emu_src(HK, 1, nK, nK, (long long)n * nK), (long long)o * nK, n, st);
-    co.slice(f, emu_src(C.p, 1, nmo), o, n, st);
+    h.slice(f, kEmuRowsA, emu_src(HK, 1, nK, nK, (long long)n * nK), (long long)o * nK, n, st);
+    co.slice(f, emu_cols(o), emu_src(C.p, 1, nmo), o, n, st);
     w3.ensure((size_t)std::max(nov, (long long)o * o) * nK, st);
     emu97(o * nK, o, h.op, co.op, emu_out(w3.p, 1, nK, nK, (long long)o * nK));
     BKoo.ensure((size_t)o * o * nK, st);
@@ -1633,10 +1633,10 @@ void Engine::build_K_emu(const double* HK, double* Bvv) {
   w3.ensure((size_t)v * v * nK, st);
   {
     EmuMat t;
-    t.slice(f, emu_src(TK.p, 1, (long long)n * nK), (long long)n * nK, n, st);
+    t.slice(f, kEmuRowsA, emu_src(TK.p, 1, (long long)n * nK), (long long)n * nK, n, st);
     emu97(n * nK, v, t.op, cv.op, emu_out(w2.p, 1, (long long)n * nK));  // H[a][nu][P]
   }
-  a.slice(f, emu_src(w2.p, 1, nK, nK, (long long)n * nK), (long long)v * nK, n, st);
+  a.slice(f, kEmuRowsA, emu_src(w2.p, 1, nK, nK, (long long)n * nK), (long long)v * nK, n, st);
   emu97(v * nK, v, a.op, cv.op, emu_out(w3.p, 1, nK, nK, (long long)v * nK));  // [a][b][P]
   cKvv.ensure((size_t)v * v * nK, st);
   metric(w3.p, (long long)v * v, Bvv, cKvv.p);
@@ -1645,8 +1645,8 @@ void Engine::build_K_emu(const double* HK, double* Bvv) {
 void Engine::ensure_emu_ops() {
   const int o = nocc, v = nvir;
   if (!emu_ready) {
-    ebBvv.slice(kEmu9x7, emu_src(BKvvD.p, 1, (long long)nK * v), (long long)nK * v, v, st);
-    ebBoo.slice(kEmu9x7, emu_src(BKoo.p, (long long)o * nK, 1), o, o * nK, st);
+    ebBvv.slice(kEmu9x7, kEmuRowsA, emu_src(BKvvD.p, 1, (long long)nK * v), (long long)nK * v, v, st);
+    ebBoo.slice(kEmu9x7, emu_cols(o), emu_src(BKoo.p, (long long)o * nK, 1), o, o * nK, st);
     emu_ready = true;
   }
 }
@@ -1669,8 +1669,8 @@ void Engine::exchange_emu(const double* Z, int nvec, double* K1, double alpha, d
   const EmuForm f = kEmu9x7;
   ensure_emu_ops();
   if (K2 && !ebBov.op.rows) {
-    ebBov.slice(f, emu_src(BKovR.p, v, 1), (long long)nK * o, v, st);
-    ebBovT.slice(f, emu_src(BKovR.p, 1, v), v, nK * o, st);
+    ebBov.slice(f, kEmuRowsA, emu_src(BKovR.p, v, 1), (long long)nK * o, v, st);
+    ebBovT.slice(f, emu_cols(v), emu_src(BKovR.p, 1, v), v, nK * o, st);
   }
   const int nblk = cdiv((long long)nvec * o, 1280 + o), per = cdiv(nvec, nblk);
   EmuMat x, y;
@@ -1678,25 +1678,26 @@ void Engine::exchange_emu(const double* Z, int nvec, double* K1, double alpha, d
     const int nb = std::min(per, nvec - s0);
     const double* z = Z + s0 * nov;
     w6.ensure((size_t)std::min(per, nvec) * o * nK * std::max(v, K2 ? o : 0), st);
-    x.slice(f, emu_src(z, v, 1), (long long)nb * o, v, st);  // rows (vec,j) over b
+    x.slice(f, emu_cols(nb * o), emu_src(z, v, 1), (long long)nb * o, v, st);  // rows (vec,j) over b
     EmuEpilogue e = emu_out(w6.p, 1, (long long)nK * v);
     e.lead = y.clear_lead((long long)nb * v, st);  // row (vec,a) of W from (R,a) and (vec,j)
     e.lead_rows(1, v, 1);
     e.lead_cols(o, nb, v);
     emu97(nK * v, nb * o, ebBvv.op, x.op, e);
-    y.slice(f, emu_src(w6.p, 1, v, v, (long long)o * nK * v), (long long)nb * v, o * nK, st, true);
+    y.slice(f, kEmuRowsA, emu_src(w6.p, 1, v, v, (long long)o * nK * v), (long long)nb * v, o * nK, st, true);
     e = emu_out(K1 + s0 * nov, 1, v, v, nov);
     e.alpha = alpha;
     e.beta = beta;
     emu97(nb * v, o, y.op, ebBoo.op, e);
     if (!K2) continue;
-    // rows (vec,j), columns (R,i): Y1[vec][i][R][j]
-    e = emu_out(w6.p, 1, (long long)nK * o, o, (long long)o * nK * o, o, o);
-    e.lead = y.clear_lead((long long)nb * o, st);  // row (vec,i) from (vec,j) and (R,i)
-    e.lead_rows(o, nb, o);
-    e.lead_cols(1, o, 1);
-    emu97(nb * o, nK * o, x.op, ebBov.op, e);
-    y.slice(f, emu_src(w6.p, (long long)nK * o, 1), (long long)nb * o, nK * o, st, true);
+    // rows (R,i), columns (vec,j): Y1[vec][R][j][i]
+    const long long noo = (long long)nK * o * o;
+    e = emu_out(w6.p, 1, o, o, (long long)o * o, o, noo);
+    e.lead = y.clear_lead((long long)nb * o, st);  // row (vec,i) from (R,i) and (vec,j)
+    e.lead_rows(1, o, 1);
+    e.lead_cols(o, nb, o);
+    emu97(nK * o, nb * o, ebBov.op, x.op, e);
+    y.slice(f, kEmuRowsA, emu_src(w6.p, 1, o, o, noo), (long long)nb * o, nK * o, st, true);
     emu97(nb * o, v, y.op, ebBovT.op, emu_out(K2 + s0 * nov, v, 1));
   }
 }
@@ -1787,17 +1788,10 @@ void Engine::emu_abt(int M, int N, int K, const double* A, long long rsA, long l
     RIS_ALLOC(cudaMallocAsync((void**)&d_tcerr, sizeof(int), st));
     RIS_CUDA(cudaMemsetAsync(d_tcerr, 0, sizeof(int), st));
   }
-  SBuf<__half> sA(emu_size(kEmu10x6, M, K), st), sB(emu_size(kEmu10x6, N, K), st);
-  SBuf<int> eA(M, st), eB(N, st);
-  EmuOperand a, b;
-  a.s = sA.p; a.e = eA.p;
-  b.s = sB.p; b.e = eB.p;
-  EmuSource xa, xb;
-  xa.p = A; xa.rs = rsA; xa.ks = ksA;
-  xb.p = B; xb.rs = rsB; xb.ks = ksB;
-  emu_slice(kEmu10x6, xa, M, K, a, st);
-  emu_slice(kEmu10x6, xb, N, K, b, st);
-  emu_gemm(kEmu10x6, M, N, a, b, ep, d_tcerr, st);
+  EmuMat a, b;
+  a.slice(kEmu10x6, kEmuRowsA, emu_src(A, rsA, ksA), M, K, st);
+  b.slice(kEmu10x6, emu_cols(N), emu_src(B, rsB, ksB), N, K, st);
+  emu_gemm(kEmu10x6, M, N, a.op, b.op, ep, d_tcerr, st);
 }
 
 // Mixed precision: (ab|P)_K = sum_mu,nu C_mu,a C_nu,b (mu nu|P) by two
@@ -2744,25 +2738,25 @@ struct GammaEmu {
     cudaStream_t st = e.st;
     nc = L ? 2 : 1;
     kw = (L ? 5 : 2) * o;
-    o8 = ld8(o);
-    n8 = ld8(n);
+    o8 = emu_pad(o, emu_cols(o));
+    n8 = emu_pad(n, emu_cols(n));
     Q[0] = QR;
     Q[1] = QL;
-    cvv.slice(f, emu_src(e.cKvv.p, 1, (long long)v * nK), (long long)v * nK, v, st);  // rows (b,P) over a
-    coo.slice(f, emu_src(e.cKoo.p, 1, (long long)o * nK), (long long)o * nK, o, st);  // rows (k,P) over i
-    Co.slice(f, emu_src(e.C.p, e.nmo, 1), n, o, st);                                   // rows mu over j
+    cvv.slice(f, kEmuRowsA, emu_src(e.cKvv.p, 1, (long long)v * nK), (long long)v * nK, v, st);  // rows (b,P) over a
+    coo.slice(f, kEmuRowsA, emu_src(e.cKoo.p, 1, (long long)o * nK), (long long)o * nK, o, st);  // rows (k,P) over i
+    Co.slice(f, emu_cols(n), emu_src(e.C.p, e.nmo, 1), n, o, st);                                   // rows mu over j
     if (L)  // rows (k,P) over a
-      cov.slice(f, emu_src(e.cKov.p, 1, nK, nK, (long long)v * nK), (long long)o * nK, v, st);
+      cov.slice(f, kEmuRowsA, emu_src(e.cKov.p, 1, nK, nK, (long long)v * nK), (long long)o * nK, v, st);
     for (int c = 0; c < nc; c++) {
-      // rows (s,j) over a and (s,mu) over i, a state's rows padded to whole groups
-      U[c].slice(f, emu_src(c ? L : R, v, 1, o8, (long long)o * v, o), (long long)nsu * o8, v, st);
-      QT[c].slice(f, emu_src(Q[c], 1, n, n8, (long long)o * n, n), (long long)nsu * n8, o, st);
+      // rows (s,j) over a and (s,mu) over i, a state's rows padded to whole blocks
+      U[c].slice(f, emu_cols(o), emu_src(c ? L : R, v, 1, o8, (long long)o * v, o), (long long)nsu * o8, v, st);
+      QT[c].slice(f, emu_cols(n), emu_src(Q[c], 1, n, n8, (long long)o * n, n), (long long)nsu * n8, o, st);
     }
     Wd.ensure((size_t)nsu * n * kw, st);
     k_build_W_states<<<dim3(cdiv((long long)n * kw, 256), nsu), 256, 0, st>>>(e.C.p, e.nmo, QR, QL, n, o,
                                                                               kw, Wd.p);
     RIS_CHECK_LAUNCH();
-    W.slice(f, emu_src(Wd.p, kw, 1, n8, (long long)n * kw, n), (long long)nsu * n8, kw, st);  // (s,nu) over k'
+    W.slice(f, emu_cols(n), emu_src(Wd.p, kw, 1, n8, (long long)n * kw, n), (long long)nsu * n8, kw, st);  // (s,nu) over k'
     Z.ensure((size_t)o * v * nK, st);
     G.ensure((size_t)o * o * nK, st);
     M.ensure((size_t)n * kw * nK, st);
@@ -2783,10 +2777,10 @@ struct GammaEmu {
     const long long kP = (long long)kw * nK;
     for (int c = 0; c < nc; c++) {
       e.emu97(v * nK, o, cvv.op, U[c].op.sub((long long)sI * o8, o), emu_out(Z.p, 1, (long long)v * nK));
-      zs.slice(f, emu_src(Z.p, 1, nK, nK, (long long)v * nK), (long long)o * nK, v, st);  // (j,P) over b
+      zs.slice(f, kEmuRowsA, emu_src(Z.p, 1, nK, nK, (long long)v * nK), (long long)o * nK, v, st);  // (j,P) over b
       e.emu97(o * nK, o, zs.op, U[c].op.sub((long long)sJ * o8, o),
               emu_out(G.p, 1, nK, nK, (long long)o * nK));
-      gs.slice(f, emu_src(G.p, 1, (long long)o * nK), (long long)o * nK, o, st);  // (k,P) over j
+      gs.slice(f, kEmuRowsA, emu_src(G.p, 1, (long long)o * nK), (long long)o * nK, o, st);  // (k,P) over j
       double* m = M.p + (size_t)2 * c * o * nK;
       e.emu97(o * nK, n, gs.op, Co.op, emu_out(m, 1, kP));
       e.emu97(o * nK, n, coo.op, QT[c].op.sub((long long)sI * n8, n),
@@ -2812,11 +2806,11 @@ struct GammaEmu {
         RIS_CHECK_LAUNCH();
         dgemm(false, true, nK, nK, o * o, sg * w, e2.p, o * o, e1.p, o * o, 1.0, Om, nU, st);
       }
-      gs.slice(f, emu_src(EE.p, 1, nK, nK, 4LL * o * nK), (long long)o * nK, 4 * o, st);  // (k,P) over k'
-      qs.slice(f, emu_src(QW.p, 1, n), n, 4 * o, st);                                     // mu over k'
+      gs.slice(f, kEmuRowsA, emu_src(EE.p, 1, nK, nK, 4LL * o * nK), (long long)o * nK, 4 * o, st);  // (k,P) over k'
+      qs.slice(f, emu_cols(n), emu_src(QW.p, 1, n), n, 4 * o, st);                                     // mu over k'
       e.emu97(o * nK, n, gs.op, qs.op, emu_out(M.p + 4 * oo, 1, kP));
     }
-    ms.slice(f, emu_src(M.p, 1, nK, nK, kP), (long long)n * nK, kw, st);  // rows (mu,P) over k'
+    ms.slice(f, kEmuRowsA, emu_src(M.p, 1, nK, nK, kP), (long long)n * nK, kw, st);  // rows (mu,P) over k'
     EmuEpilogue ep = emu_out(Gam, 1, nK, nK, (long long)n * nK);
     ep.alpha = w;
     e.emu97(n * nK, n, ms.op, W.op.sub((long long)sJ * n8, n), ep);
@@ -2869,7 +2863,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   }
   ensure_D();
   // per state: R, L, D^R = C_o R C_v^T, c^J, Q_R = R C_v^T, Q_L = L C_v^T
-  SBuf<double> Rs((size_t)nsu * nov, st), Ls((size_t)nsu * nov, st), DR, cJ, QR, QL, t1;
+  SBuf<double> Rs((size_t)nsu * nov, st), Ls((size_t)nsu * nov, st), DR, cJ, QR, QL;
   for (int s = 0; s < nsu; s++) {
     const double* xs = Xa + (size_t)su[s] * nov;
     const double* ys = rpa ? Ya + (size_t)su[s] * nov : nullptr;
@@ -2877,7 +2871,6 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
     axpby(nov, 1.0, xs, -1.0, ys, Ls.p + s * nov, st);
   }
   DR.ensure((size_t)nsu * nn * nn, st);
-  t1.ensure((size_t)nn * v, st);
   cJ.ensure((size_t)nsu * nJ, st);
   w5.ensure((size_t)nsu * nJ, st);
   const double* Co = C.p;
@@ -2921,17 +2914,35 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
       RIS_CHECK_LAUNCH();
     }
   }
+  // Q_s[i][nu] = sum_a R_s[i][a] C_v[nu][a] for every state, and from it
+  // D^R_s[mu][nu] = sum_i C_o[mu][i] Q_s[i][nu] (o n^2 multiply-adds; forming
+  // C_o R_s first would take o n v + n^2 v)
+  const bool emu = emu_exchange();
   if (!mixed || rpa) {
     QR.ensure((size_t)nsu * o * nn, st);
     if (rpa) QL.ensure((size_t)nsu * o * nn, st);
-    for (int s = 0; s < nsu; s++) {
-      if (!mixed) {
-        dgemm(false, false, nn, v, o, 1.0, Co, nmo, Rs.p + s * nov, v, 0.0, t1.p, v, st);
-        dgemm(false, true, nn, nn, v, 1.0, t1.p, v, Cv, nmo, 0.0, DR.p + (size_t)s * nn * nn, nn, st);
+    EmuMat c, r;
+    if (emu) c.slice(kEmu9x7, kEmuRowsA, emu_src(Cv, nmo, 1), nn, v, st);  // rows nu over a
+    for (int w = 0; w < (rpa ? 2 : 1); w++) {
+      const double* u = w ? Ls.p : Rs.p;
+      double* q = w ? QL.p : QR.p;
+      if (emu) {  // columns (s,i) over a
+        r.slice(kEmu9x7, emu_cols(nsu * o), emu_src(u, v, 1), (long long)nsu * o, v, st);
+        emu97(nn, nsu * o, c.op, r.op, emu_out(q, 1, nn));
+      } else {
+        dgemm(false, true, nsu * o, nn, v, 1.0, u, v, Cv, nmo, 0.0, q, nn, st);
       }
-      dgemm(false, true, o, nn, v, 1.0, Rs.p + s * nov, v, Cv, nmo, 0.0, QR.p + (size_t)s * o * nn, nn, st);
-      if (rpa)
-        dgemm(false, true, o, nn, v, 1.0, Ls.p + s * nov, v, Cv, nmo, 0.0, QL.p + (size_t)s * o * nn, nn, st);
+    }
+    if (emu) {  // rows (s,nu) over i, columns mu
+      c.slice(kEmu9x7, kEmuRowsA, emu_src(QR.p, 1, nn, nn, (long long)o * nn), (long long)nsu * nn, o, st);
+      r.slice(kEmu9x7, emu_cols(nn), emu_src(Co, nmo, 1), nn, o, st);
+      emu97(nsu * nn, nn, c.op, r.op, emu_out(DR.p, 1, nn, nn, (long long)nn * nn));
+    } else if (!mixed) {
+      GemmBatch bt;
+      bt.nb1 = nsu;
+      bt.sB1 = (long long)o * nn;
+      bt.sC1 = (long long)nn * nn;
+      dgemm(false, false, nn, nn, o, 1.0, Co, nmo, QR.p, nn, 0.0, DR.p, nn, st, bt);
     }
   }
   // u_s = R_s . B^J (nJ), c_s = u_s L^-1 (row vector)
@@ -2989,7 +3000,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   const int slK = pick_slices((long long)nn * nK, nbAvg);
   SBuf<double> partK((size_t)slK * NB * 3 * nn * nK, st);
   SBuf<int> pst(2 * NB, st);
-  if (opt.precision != RIS_MIXED && !emu_exchange()) {
+  if (opt.precision != RIS_MIXED && !emu) {
     Z.ensure((size_t)o * v * nK, st);
     Goo.ensure((size_t)o * o * nK, st);
     M1.ensure((size_t)nn * 2 * o * nK, st);
@@ -2997,7 +3008,6 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   }
   const double cx = opt.cx;
   GammaEmu ge;
-  const bool emu = emu_exchange();
   if (emu) ge.setup(*this, nsu, Rs.p, rpa ? Ls.p : nullptr, QR.p, rpa ? QL.p : nullptr);
   for (int g0 = 0; g0 < npair; g0 += NB) {
     const int nb = std::min(NB, npair - g0);
@@ -3151,14 +3161,14 @@ void Engine::ensure_Kov() {
   if (emu_exchange()) {
     const EmuForm f = kEmu9x7;
     EmuMat t, c, li;
-    t.slice(f, emu_src(TK.p, 1, (long long)n * nK), (long long)n * nK, n, st);  // rows (nu,P) over mu
-    c.slice(f, emu_src(Co, 1, nmo), o, n, st);
+    t.slice(f, kEmuRowsA, emu_src(TK.p, 1, (long long)n * nK), (long long)n * nK, n, st);  // rows (nu,P) over mu
+    c.slice(f, emu_cols(o), emu_src(Co, 1, nmo), o, n, st);
     emu97(n * nK, o, t.op, c.op, emu_out(H.p, 1, (long long)n * nK));  // H[i][nu][P]
-    t.slice(f, emu_src(H.p, 1, nK, nK, (long long)n * nK), (long long)o * nK, n, st);
-    c.slice(f, emu_src(Cv, 1, nmo), v, n, st);
+    t.slice(f, kEmuRowsA, emu_src(H.p, 1, nK, nK, (long long)n * nK), (long long)o * nK, n, st);
+    c.slice(f, emu_cols(v), emu_src(Cv, 1, nmo), v, n, st);
     emu97(o * nK, v, t.op, c.op, emu_out(Bia.p, 1, nK, nK, (long long)v * nK));  // [i][a][P]
-    t.slice(f, emu_src(Bia.p, nK, 1), nov, nK, st);
-    li.slice(f, emu_src(LKinv.p, nK, 1), nK, nK, st);
+    t.slice(f, kEmuRowsA, emu_src(Bia.p, nK, 1), nov, nK, st);
+    li.slice(f, emu_cols(nK), emu_src(LKinv.p, nK, 1), nK, nK, st);
     emu97((int)nov, nK, t.op, li.op, emu_out(Bm.p, nK, 1));
     BKovR.ensure((size_t)nov * nK, st);
     transpose_last2(Bm.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]

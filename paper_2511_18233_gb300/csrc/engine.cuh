@@ -64,17 +64,18 @@ struct FBuf {
 };
 
 // A sliced operand of the emulated FP64 products (gemm_emu.cuh) and its
-// storage.
+// storage; rb: kEmuRowsA (left operand) or emu_cols(N) (right operand).
 struct EmuMat {
   SBuf<__half> s;
   SBuf<int> e;
   EmuOperand op;
-  void slice(EmuForm f, const EmuSource& src, long long rows, int K, cudaStream_t st,
+  void slice(EmuForm f, int rb, const EmuSource& src, long long rows, int K, cudaStream_t st,
              bool have_lead = false) {
-    s.ensure(emu_size(f, rows, K), st);
+    s.ensure(emu_size(f, rows, K, rb), st);
     e.ensure((size_t)rows, st);
     op.s = s.p;
     op.e = e.p;
+    op.rb = rb;
     emu_slice(f, src, (int)rows, K, op, st, have_lead);
   }
   // the row exponents of the rows to come, for an EmuEpilogue that fills them

@@ -22,14 +22,12 @@
 //
 // Kernel (persistent, one CTA of 576 threads per SM looping over 128 x BN
 // output tiles):
-//   warp 0 / lane 0 : producer, 4-stage ring; a stage is K = 16 of all slices
-//                     of A (128 rows) and of B (BN rows), two contiguous bulk
-//                     copies per slice (the slicing writes the operands in the
-//                     layout of the stages: as 32-byte rows of a tensor map
-//                     the copies took 1.6 cycles a row and held the loop at
-//                     0.43 of the tensor pipe)
+//   warp 0          : producer, 4-stage ring; a stage is K = 16 of all slices
+//                     of A (128 rows) and of B (BN rows), one contiguous bulk
+//                     copy each (the slicing writes the operands in the layout
+//                     of the stages)
 //   warp 1          : allocates 512 TMEM columns (S accumulators of BN
-//                     columns); lane 0 issues the slice products.  The B
+//                     columns) and issues the slice products.  The B
 //                     slices of a stage lie one after the other, and so do
 //                     the accumulators g = p, p + 1, ..., so one
 //                     tcgen05.mma of N = (up to 256 / BN) BN multiplies A
@@ -119,10 +117,9 @@ struct EmuArgs {
   int M, N, K;
   int ntn, tiles;       // column tiles (fastest), all tiles
   int nchunk, cps, ns;  // chunks of the contraction, chunks per slice of it, slices
-  const __half* sa;     // digits; elements between row groups' planes
+  const __half* sa;     // digits; elements between K steps
   const __half* sb;
   long long pa, pb;
-  int ra, rb;           // rows the operands hold
   const int* ea;
   const int* eb;
   longlong2* ws;   // split contraction: [slice][M][N] integer partial sums
@@ -300,82 +297,97 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
   const uint32_t tmem = *tmem_slot;
 
   // work item w: tile w % tiles, contraction slice w / tiles
+  // (the two feeding warps run their loops with all lanes and elect one for
+  // the copies and products: counters and descriptors then live in uniform
+  // registers, where those instructions take them from)
   if (warp == 0) {
-    if (lane == 0) {
-      // producer
-      int it = 0;  // stages issued
-      for (int w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
-        const int t = w % args.tiles, c0 = (w / args.tiles) * args.cps;
-        const int n0 = (t % args.ntn) * bn, m0 = (t / args.ntn) * EBM;
-        const int s0 = c0 * kSteps;
-        const int s1 = min((args.K + EBK - 1) / EBK, (c0 + args.cps) * kSteps);
-        const uint32_t ba = (uint32_t)(min(EBM, (args.ra - m0 + 7) & ~7) * 32);
-        const uint32_t bb = (uint32_t)(min(bn, (args.rb - n0 + 7) & ~7) * 32);
-        const __half* ga = args.sa + (size_t)s0 * S * args.pa + (size_t)m0 * 16;
-        const __half* gb = args.sb + (size_t)s0 * S * args.pb + (size_t)n0 * 16;
-        for (int i = s0; i < s1; i++, it++) {
-          const int s = it % ESTAGES;
-          if (it >= ESTAGES && !mbar_wait(&empty[s], ((it / ESTAGES) - 1) & 1)) *abort_flag = 1;
-          if (*abort_flag) break;
+    // producer
+    int it = 0;  // stages issued
+    bool stop = false;  // warp-uniform
+    for (int w = blockIdx.x; w < items && !stop; w += gridDim.x) {
+      const int t = w % args.tiles, c0 = (w / args.tiles) * args.cps;
+      const int n0 = (t % args.ntn) * bn, m0 = (t / args.ntn) * EBM;
+      const int s0 = c0 * kSteps;
+      const int s1 = min((args.K + EBK - 1) / EBK, (c0 + args.cps) * kSteps);
+      const __half* ga = args.sa + (size_t)s0 * args.pa + (size_t)m0 * (16 * S);
+      const __half* gb = args.sb + (size_t)s0 * args.pb + (size_t)n0 * (16 * S);
+      for (int i = s0; i < s1; i++, it++) {
+        const int s = it % ESTAGES;
+        if (it >= ESTAGES && !mbar_wait(&empty[s], ((it / ESTAGES) - 1) & 1)) *abort_flag = 1;
+        stop = __any_sync(0xffffffffu, *abort_flag);
+        if (stop) break;
+        if (elect_one()) {
           uint8_t* st = smem + s * Tile<F>::kStage;
-          mbar_expect_tx(&full[s], S * (ba + bb));
-#pragma unroll
-          for (int p = 0; p < S; p++) {
-            bulk_load(st + p * A_SLICE, ga, ba, &full[s]);
-            bulk_load(st + Tile<F>::kABytes + p * bn * EBK * 2, gb, bb, &full[s]);
-            ga += args.pa;
-            gb += args.pb;
-          }
+          mbar_expect_tx(&full[s], Tile<F>::kABytes + S * bn * EBK * 2);
+          bulk_load(st, ga, Tile<F>::kABytes, &full[s]);
+          bulk_load(st + Tile<F>::kABytes, gb, S * bn * EBK * 2, &full[s]);
         }
+        __syncwarp();
+        ga += args.pa;
+        gb += args.pb;
       }
-      // no copy is left in flight
-      for (int i = (it > ESTAGES ? it - ESTAGES : 0); i < it; i++)
-        mbar_wait(&full[i % ESTAGES], (i / ESTAGES) & 1);
     }
+    // no copy is left in flight
+    for (int i = (it > ESTAGES ? it - ESTAGES : 0); i < it; i++)
+      mbar_wait(&full[i % ESTAGES], (i / ESTAGES) & 1);
   } else if (warp == 1) {
-    if (lane == 0) {
-      // MMA issuer: slice products p + q < S into accumulator p + q
-      constexpr int per = 256 / bn;  // B slices per instruction
-      int it = 0, nch = 0;       // stages, chunks issued
-      for (int w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
-        const int c0 = (w / args.tiles) * args.cps;
-        const int s0 = c0 * kSteps;
-        const int s1 = min((args.K + EBK - 1) / EBK, (c0 + args.cps) * kSteps);
-        for (int i = s0; i < s1; i++, it++) {
-          const int s = it % ESTAGES, in = i % kSteps;
-          // a new chunk: the epilogue must have read the previous one
-          if (in == 0) {
-            if (nch > 0 && !mbar_wait(acc_empty, (nch - 1) & 1)) *abort_flag = 1;
-            nch++;
-          }
-          if (*abort_flag || !mbar_wait(&full[s], (it / ESTAGES) & 1)) {
-            *abort_flag = 1;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          // (fully unrolled: descriptors, columns and shapes are the stage's
-          // base plus constants.  One thread feeds the tensor core, and an
-          // instruction of N = 240 lasts about 120 cycles)
-          const uint64_t d0 = desc_sw32(smem + s * Tile<F>::kStage);
-          const uint32_t acc = in > 0 ? 1u : 0u;
+    // MMA issuer: slice products p + q < S into accumulator p + q
+    constexpr int per = 256 / bn;  // B slices per instruction
+    int it = 0, nch = 0;           // stages, chunks issued
+    bool stop = false;             // warp-uniform
+    for (int w = blockIdx.x; w < items && !stop; w += gridDim.x) {
+      const int c0 = (w / args.tiles) * args.cps;
+      const int s0 = c0 * kSteps;
+      const int s1 = min((args.K + EBK - 1) / EBK, (c0 + args.cps) * kSteps);
+      for (int i = s0; i < s1; i++, it++) {
+        const int s = it % ESTAGES, in = i % kSteps;
+        // a new chunk: the epilogue must have read the previous one
+        if (in == 0) {
+          if (nch > 0 && !mbar_wait(acc_empty, (nch - 1) & 1)) *abort_flag = 1;
+          nch++;
+        }
+        stop = __any_sync(0xffffffffu, *abort_flag);
+        if (!stop && !mbar_wait(&full[s], (it / ESTAGES) & 1)) *abort_flag = 1;
+        stop = __any_sync(0xffffffffu, *abort_flag);
+        if (stop) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        // (fully unrolled: descriptors, columns and shapes are the stage's
+        // base plus constants.  One thread feeds the tensor core, and an
+        // instruction of N = 240 lasts about 120 cycles)
+        const uint64_t d0 = desc_sw32(smem + s * Tile<F>::kStage);
+        const uint32_t acc = in > 0 ? 1u : 0u;
+        if (elect_one()) {
+          auto mma = [&](int p, int g0, int g1, uint32_t on) {  // accumulators g0 .. g1 - 1
+            mma_f16(tmem + (uint32_t)(g0 * bn), d0 + (p * A_SLICE >> 4),
+                    d0 + ((Tile<F>::kABytes + (g0 - p) * bn * EBK * 2) >> 4), idesc_f16((g1 - g0) * bn), on);
+          };
+          if (per < S && acc) {
+            // accumulators below and above `per` in turn, so that an
+            // instruction does not start on columns that the one before it is
+            // still writing (3% of the loop)
 #pragma unroll
-          for (int p = 0; p < S; p++) {
+            for (int x = 0; x < S; x++) {
+              const int p = S - 1 - x;
+              mma(p, p > per ? p : per, S, 1u);
+              if (x < per) mma(x, x, per, 1u);
+            }
+          } else {  // the first step clears the accumulators
 #pragma unroll
-            for (int q = 0; q < S - p; q += per) {
-              const int nq = per < S - p - q ? per : S - p - q;
-              mma_f16(tmem + (uint32_t)((p + q) * bn), d0 + (p * A_SLICE >> 4),
-                      d0 + ((Tile<F>::kABytes + q * bn * EBK * 2) >> 4), idesc_f16(nq * bn),
-                      p > 0 ? 1u : acc);
+            for (int p = 0; p < S; p++) {
+#pragma unroll
+              for (int g = p; g < S; g += per) mma(p, g, g + per < S ? g + per : S, p > 0 ? 1u : acc);
             }
           }
           mma_commit(&empty[s]);
           if (in == kSteps - 1 || i == s1 - 1) mma_commit(acc_full);
         }
+        __syncwarp();
       }
-      // nothing is left in flight when the tensor memory is freed, whatever happened
-      mma_commit(done);
-      if (!mbar_wait(done, 0)) *abort_flag = 1;
     }
+    // nothing is left in flight when the tensor memory is freed, whatever happened
+    if (elect_one()) mma_commit(done);
+    __syncwarp();
+    if (!mbar_wait(done, 0)) *abort_flag = 1;
   } else {
     // epilogue: row = TMEM lane of this warp's quadrant; the four warps of a
     // quadrant take bn / 4 columns each, read four at a time
@@ -408,11 +420,9 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
 #pragma unroll
         for (int j = 0; j < 4; j++) acc[b][j].zero();
       for (int ch = 0; ch < nc; ch++, nch++) {
-        if (!mbar_wait(acc_full, nch & 1) || *abort_flag) {
-          good = false;
-          break;
-        }
-        __syncwarp();
+        if (!mbar_wait(acc_full, nch & 1)) *abort_flag = 1;
+        good = !__any_sync(0xffffffffu, *abort_flag);
+        if (!good) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
         for (int b = 0; b < NB; b++) {
@@ -483,7 +493,6 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
       }
       if (ep.lead) flush();
     }
-    if (!good) *abort_flag = 1;
   }
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -586,18 +595,19 @@ struct Fixed<Form9x7> {
 };
 
 // eight consecutive digits per slice of one row (half of a K step): 16-byte
-// stores, o = the K step's first slice
+// stores, o = the K step's digits
 template <class F>
-__device__ __forceinline__ void put8(const double (&x)[8], int lead, __half* o, long long groups, int r,
+__device__ __forceinline__ void put8(const double (&x)[8], int lead, __half* o, int rb, int r,
                                      int half) {
   Fixed<F> f[8];
   const int E = row_bad(lead) ? 0 : row_frame(lead);  // digits of a bad row are not used
 #pragma unroll
   for (int i = 0; i < 8; i++) f[i].set(row_bad(lead) ? 0.0 : x[i], E);
-  o += (size_t)(r >> 3) * 128 + (r & 7) * 16 + ((half ^ ((r >> 2) & 1)) << 3);
+  const int b = r / rb, i = r - b * rb;
+  o += (size_t)b * (F::S * 16 * rb) + (i >> 3) * 128 + (i & 7) * 16 + ((half ^ ((i >> 2) & 1)) << 3);
 #pragma unroll
   for (int p = 0; p < F::S; p++)
-    *reinterpret_cast<uint4*>(o + (size_t)p * groups * 128) =
+    *reinterpret_cast<uint4*>(o + p * (16 * rb)) =
         make_uint4(Fixed<F>::word(f[0], f[1], p), Fixed<F>::word(f[2], f[3], p),
                    Fixed<F>::word(f[4], f[5], p), Fixed<F>::word(f[6], f[7], p));
 }
@@ -633,7 +643,7 @@ __global__ void __launch_bounds__(256) k_emu_lead(EmuSource src, int rows, int K
 template <class F, bool LEAD>
 __global__ void __launch_bounds__(256) k_emu_slice_rows(EmuSource src, int rows, int K,
                                                         int* __restrict__ E, __half* __restrict__ out,
-                                                        long long groups) {
+                                                        int rb, int prows) {
   __shared__ int ex[16];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r0 = blockIdx.x * 16;
   if (LEAD) {
@@ -653,7 +663,7 @@ __global__ void __launch_bounds__(256) k_emu_slice_rows(EmuSource src, int rows,
     __syncthreads();
   }
   const int r = r0 + (lane >> 1), half = lane & 1;
-  if ((r >> 3) >= groups) return;
+  if (r >= prows) return;
   long long off = 0;
   const bool on = src_row(src, r, rows, off);
   const int lead = LEAD ? ex[lane >> 1] : (r < rows ? E[r] : kEmuNoLead);
@@ -664,7 +674,7 @@ __global__ void __launch_bounds__(256) k_emu_slice_rows(EmuSource src, int rows,
     double v[8];
 #pragma unroll
     for (int i = 0; i < 8; i++) v[i] = (on && k + i < K) ? x[k + i] : 0.0;
-    put8<F>(v, lead, out + (size_t)s * F::S * groups * 128, groups, r, half);
+    put8<F>(v, lead, out + (size_t)s * F::S * 16 * prows, rb, r, half);
   }
 }
 
@@ -674,7 +684,7 @@ __global__ void __launch_bounds__(256) k_emu_slice_rows(EmuSource src, int rows,
 template <class F, bool LEAD>
 __global__ void __launch_bounds__(256) k_emu_slice_cols(EmuSource src, int rows, int K,
                                                         int* __restrict__ E, __half* __restrict__ out,
-                                                        long long groups) {
+                                                        int rb, int prows) {
   __shared__ double tile[64][33];  // [k][r]
   __shared__ int red[8][32];
   const int r0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -705,23 +715,23 @@ __global__ void __launch_bounds__(256) k_emu_slice_cols(EmuSource src, int rows,
     for (int kk = ty; kk < 64; kk += 8)
       tile[kk][tx] = (on && s0 * 16 + kk < K) ? x[(size_t)(s0 * 16 + kk) * src.ks] : 0.0;
     __syncthreads();
-    if (s0 + ks >= nk || ((r0 + rr) >> 3) >= groups) continue;
+    if (s0 + ks >= nk || r0 + rr >= prows) continue;
     double v[8];
 #pragma unroll
     for (int i = 0; i < 8; i++) v[i] = tile[ks * 16 + half * 8 + i][rr];
-    put8<F>(v, red[0][rr], out + (size_t)(s0 + ks) * F::S * groups * 128, groups, r0 + rr, half);
+    put8<F>(v, red[0][rr], out + (size_t)(s0 + ks) * F::S * 16 * prows, rb, r0 + rr, half);
   }
 }
 
 template <class F>
 void slice_form(const EmuSource& src, int rows, int K, EmuOperand& op, cudaStream_t st, bool have_lead) {
-  const int nk = cdiv(K, 16);
+  const int nk = cdiv(K, 16), prows = (int)op.blocks * op.rb;  // padded rows are cut as zeros
   if (src.ks != 1) {
     if (have_lead) {
-      const int ny = std::min(cdiv(nk, 4), std::max(1, cdiv(8 * 152, cdiv(rows, 32))));
-      k_emu_slice_cols<F, false><<<dim3(cdiv(rows, 32), ny), 256, 0, st>>>(src, rows, K, op.e, op.s, op.groups);
+      const int ny = std::min(cdiv(nk, 4), std::max(1, cdiv(8 * 152, cdiv(prows, 32))));
+      k_emu_slice_cols<F, false><<<dim3(cdiv(prows, 32), ny), 256, 0, st>>>(src, rows, K, op.e, op.s, op.rb, prows);
     } else {
-      k_emu_slice_cols<F, true><<<cdiv(rows, 32), 256, 0, st>>>(src, rows, K, op.e, op.s, op.groups);
+      k_emu_slice_cols<F, true><<<cdiv(prows, 32), 256, 0, st>>>(src, rows, K, op.e, op.s, op.rb, prows);
     }
   } else if (have_lead || K >= 2048) {
     // few long rows: exponents first, one row per CTA, so that a few hundred
@@ -730,22 +740,12 @@ void slice_form(const EmuSource& src, int rows, int K, EmuOperand& op, cudaStrea
       k_emu_lead<<<rows, 256, 0, st>>>(src, rows, K, op.e);
       RIS_CHECK_LAUNCH();
     }
-    const int ny = std::min(cdiv(nk, 8), std::max(1, cdiv(8 * 152, cdiv(rows, 16))));
-    k_emu_slice_rows<F, false><<<dim3(cdiv(rows, 16), ny), 256, 0, st>>>(src, rows, K, op.e, op.s, op.groups);
+    const int ny = std::min(cdiv(nk, 8), std::max(1, cdiv(8 * 152, cdiv(prows, 16))));
+    k_emu_slice_rows<F, false><<<dim3(cdiv(prows, 16), ny), 256, 0, st>>>(src, rows, K, op.e, op.s, op.rb, prows);
   } else {
-    k_emu_slice_rows<F, true><<<cdiv(rows, 16), 256, 0, st>>>(src, rows, K, op.e, op.s, op.groups);
+    k_emu_slice_rows<F, true><<<cdiv(prows, 16), 256, 0, st>>>(src, rows, K, op.e, op.s, op.rb, prows);
   }
   RIS_CHECK_LAUNCH();
-}
-
-// Tile width: a stage brings (128 + BN) rows of digits through shared memory
-// whatever the products, so the total over the column tiles is taken least;
-// ties go to the wider tile.
-int pick_bn(int N, int max_bn) {
-  int bn = max_bn;
-  for (int c = max_bn; c >= 16; c -= 16)
-    if ((long long)cdiv(N, c) * (EBM + c) < (long long)cdiv(N, bn) * (EBM + bn)) bn = c;
-  return bn;
 }
 
 template <class F>
@@ -755,16 +755,14 @@ void gemm_pass(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
   a.M = M;
   a.N = N;
   a.K = A.K;
-  const int bn = pick_bn(N, F::kMaxBN);
+  const int bn = B.rb;
   a.ntn = cdiv(N, bn);
   a.nchunk = cdiv(A.K, F::kChunk);
   RIS_REQUIRE((((uintptr_t)A.s | (uintptr_t)B.s) & 15) == 0, RIS_ERR_ARG, "emu_gemm: slices not 16-byte aligned");
   a.sa = A.s;
   a.sb = B.s;
-  a.pa = A.groups * 128;
-  a.pb = B.groups * 128;
-  a.ra = A.rows;
-  a.rb = B.rows;
+  a.pa = A.blocks * A.rb * (16 * F::S);
+  a.pb = B.blocks * B.rb * (16 * F::S);
   a.ea = A.e;
   a.eb = B.e;
   a.ws = nullptr;
@@ -817,8 +815,8 @@ void gemm_form(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
   for (int k0 = 0; k0 < A.K; k0 += kPass) {
     EmuOperand a = A, b = B;
     EmuEpilogue e = ep;
-    a.s = A.s + (size_t)(k0 / EBK) * F::S * A.groups * 128;
-    b.s = B.s + (size_t)(k0 / EBK) * F::S * B.groups * 128;
+    a.s = A.s + (size_t)(k0 / EBK) * F::S * 16 * A.blocks * A.rb;
+    b.s = B.s + (size_t)(k0 / EBK) * F::S * 16 * B.blocks * B.rb;
     a.K = b.K = std::min(kPass, A.K - k0);
     if (k0 > 0) e.beta = 1.0;
     gemm_pass<F>(M, N, a, b, e, d_err, st);
@@ -828,12 +826,24 @@ void gemm_form(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
 
 }  // namespace
 
+// Tile width for N columns: a stage brings (128 + BN) rows of digits through
+// shared memory whatever the products, so the total over the column tiles is
+// taken least; ties go to the wider tile.
+int emu_cols(int N) {
+  int bn = 48;
+  for (int c = 48; c >= 16; c -= 16)
+    if ((long long)cdiv(N, c) * (EBM + c) < (long long)cdiv(N, bn) * (EBM + bn)) bn = c;
+  return bn;
+}
+
 void emu_slice(EmuForm f, const EmuSource& src, int rows, int K, EmuOperand& op, cudaStream_t st,
                bool have_lead) {
   RIS_REQUIRE(rows > 0 && K > 0 && op.s && op.e, RIS_ERR_ARG, "emu_slice: bad operand");
   op.rows = rows;
   op.K = K;
-  op.groups = (rows + 7) / 8;
+  RIS_REQUIRE(op.rb > 0 && op.rb % 8 == 0, RIS_ERR_ARG, "emu_slice: row block");
+  op.blocks = cdiv(rows, op.rb);
+  op.slices = emu_slices(f);
   if (f == kEmu10x6)
     slice_form<Form10x6>(src, rows, K, op, st, have_lead);
   else
@@ -845,6 +855,9 @@ void emu_gemm(EmuForm f, int M, int N, const EmuOperand& A, const EmuOperand& B,
   if (M <= 0 || N <= 0) return;
   RIS_REQUIRE(A.K == B.K && A.K > 0, RIS_ERR_ARG, "emu_gemm: contraction lengths differ");
   RIS_REQUIRE(A.rows >= M && B.rows >= N, RIS_ERR_ARG, "emu_gemm: operand rows");
+  RIS_REQUIRE(A.rb == kEmuRowsA && (B.rb == 48 || B.rb == 32 || B.rb == 16), RIS_ERR_ARG,
+              "emu_gemm: operand row blocks");
+  RIS_REQUIRE(A.slices == emu_slices(f) && B.slices == A.slices, RIS_ERR_ARG, "emu_gemm: operand form");
   if (f == kEmu10x6)
     gemm_form<Form10x6>(M, N, A, B, ep, d_err, st);
   else
@@ -863,8 +876,10 @@ int debug_emu(ris::EmuForm f, int M, int N, int K, const double* A, const double
     cudaStream_t st = 0;
     EmuOperand a, b;
     int* err;
-    RIS_ALLOC(cudaMalloc(&a.s, sizeof(__half) * emu_size(f, M, K)));
-    RIS_ALLOC(cudaMalloc(&b.s, sizeof(__half) * emu_size(f, N, K)));
+    a.rb = kEmuRowsA;
+    b.rb = emu_cols(N);
+    RIS_ALLOC(cudaMalloc(&a.s, sizeof(__half) * emu_size(f, M, K, a.rb)));
+    RIS_ALLOC(cudaMalloc(&b.s, sizeof(__half) * emu_size(f, N, K, b.rb)));
     RIS_ALLOC(cudaMalloc(&a.e, sizeof(int) * (size_t)M));
     RIS_ALLOC(cudaMalloc(&b.e, sizeof(int) * (size_t)N));
     RIS_ALLOC(cudaMalloc(&err, sizeof(int)));

@@ -21,34 +21,40 @@ enum EmuForm { kEmu10x6 = 0, kEmu9x7 = 1 };
 constexpr int emu_slices(EmuForm f) { return f == kEmu10x6 ? 10 : 9; }
 
 // A sliced operand: FP16 integer digits in the layout in which the GEMM's
-// stages lie in shared memory, so that a stage is a few contiguous copies:
-//   [K step of 16][slice][row group of 8][8 rows x 32 bytes]
+// stages lie in shared memory, so that a stage is one contiguous copy per
+// operand:
+//   [K step of 16][block of rb rows][slice][group of 8 rows][8 rows x 32 bytes]
 // with the two 16-byte halves of rows 4..7 of a group exchanged (the 32-byte
-// swizzle of the tensor core's operand tiles), zero past K; and per row the
-// exponent of its largest magnitude (kEmuNoLead for a row of zeros; at least
-// kEmuLeadBad for a row that holds an infinity or a NaN: every product with it
-// is NaN).
+// swizzle of the tensor core's operand tiles), zero past K and past the rows;
+// and per row the exponent of its largest magnitude (kEmuNoLead for a row of
+// zeros; at least kEmuLeadBad for a row that holds an infinity or a NaN: every
+// product with it is NaN).  rb is the GEMM's tile edge: kEmuRowsA for the left
+// operand, emu_cols(N) for the right one.
 constexpr int kEmuNoLead = (int)0x80808080;  // set by a byte fill of 0x80
 constexpr int kEmuLeadBad = 1024;
+constexpr int kEmuRowsA = 128;
+int emu_cols(int N);
 struct EmuOperand {
   __half* s = nullptr;
   int* e = nullptr;
   int rows = 0, K = 0;
-  long long groups = 0;  // row groups per slice
-  // rows r0 .. r0 + n - 1, r0 a multiple of 8
+  int rb = 0;
+  long long blocks = 0;  // row blocks
+  int slices = 0;
+  // rows r0 .. r0 + n - 1, r0 a multiple of rb
   EmuOperand sub(long long r0, int n) const {
     EmuOperand o = *this;
-    o.s += r0 * 16;
+    o.s += r0 * 16 * slices;
     o.e += r0;
     o.rows = n;
     return o;
   }
 };
 
-inline int ld8(int k) { return (k + 7) & ~7; }
+inline int emu_pad(int n, int rb) { return (n + rb - 1) / rb * rb; }
 // halves an operand of the form needs (ints: rows)
-inline size_t emu_size(EmuForm f, long long rows, int K) {
-  return (size_t)((K + 15) / 16) * emu_slices(f) * ((rows + 7) / 8) * 128;
+inline size_t emu_size(EmuForm f, long long rows, int K, int rb) {
+  return (size_t)((K + 15) / 16) * emu_slices(f) * ((rows + rb - 1) / rb * rb) * 16;
 }
 
 // Source placement: element (r, k) of an operand at src[row(r) + k * ks] with
@@ -62,7 +68,8 @@ struct EmuSource {
   int rvalid = 0;
 };
 
-// Slices src (rows x K) into op (op.s / op.e hold emu_size / rows elements).
+// Slices src (rows x K) into op (op.rb set; op.s / op.e hold emu_size / rows
+// elements).
 // have_lead: op.e already holds the row exponents (EmuEpilogue::lead).
 void emu_slice(EmuForm f, const EmuSource& src, int rows, int K, EmuOperand& op, cudaStream_t st,
                bool have_lead = false);
