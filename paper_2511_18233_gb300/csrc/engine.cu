@@ -1437,11 +1437,12 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   // Coulomb: H[i][nu][P] = sum_mu C_mu,i T[mu][nu][P]; B[i][a][P]; B L^-T
   // (mixed form: H as [nu][i][P], both transforms FP64-accurate on the
   // tensor cores)
-  const bool emu = opt.precision == RIS_MIXED && opt.emu_f64;
+  const bool emu = opt.precision == RIS_MIXED && opt.emu_f64, emuJ = emu || emu_exchange();
+  const EmuForm fJ = emu ? kEmu10x6 : kEmu9x7;
   w2.ensure((size_t)o * n * std::max(nJ, nK), st);
   w3.ensure((size_t)std::max(nov, (long long)o * o) * std::max(nJ, nK), st);
-  if (emu) {
-    coulomb_emu(w2.p, w3.p);
+  if (emuJ) {
+    coulomb_emu(fJ, w2.p, w3.p);
   } else {
     dgemm(true, false, o, n * nJ, n, 1.0, Co, nmo, TJ.p, n * nJ, 0.0, w2.p, n * nJ, st);
     GemmBatch bt;
@@ -1451,10 +1452,10 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     dgemm(true, false, v, nJ, n, 1.0, Cv, nmo, w2.p, nJ, 0.0, w3.p, nJ, st, bt);
   }
   BJ.ensure((size_t)nov * nJ, st);
-  if (emu) {  // B[(i,a)][R] = sum_P W[(i,a)][P] L_J^-1[R][P]
+  if (emuJ) {  // B[(i,a)][R] = sum_P W[(i,a)][P] L_J^-1[R][P]
     EmuEpilogue e;
     e.c64 = BJ.p; e.rs = nJ; e.cs = 1;
-    emu_abt((int)nov, nJ, nJ, w3.p, nJ, 1, LJinv.p, nJ, 1, e);
+    emu_abt(fJ, (int)nov, nJ, nJ, w3.p, nJ, 1, LJinv.p, nJ, 1, e);
   } else {
     dgemm(false, true, (int)nov, nJ, nJ, 1.0, w3.p, nJ, LJinv.p, nJ, 0.0, BJ.p, nJ, st);
   }
@@ -1464,7 +1465,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     w5.ensure((size_t)o * n * nK, st);
     const long long rows = (long long)o * n;
     k_gather_cols<<<(unsigned)cdiv(rows * nK, 256), 256, 0, st>>>(w2.p, rows, nJ, d_kJ, nK, w5.p,
-                                                                  emu ? n : 0, o);
+                                                                  emuJ ? n : 0, o);
     RIS_CHECK_LAUNCH();
     HK = w5.p;
   } else {
@@ -1523,7 +1524,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   if (emu) {  // c[(a,b)][Q] = sum_R B[(a,b)][R] L_K^-1[R][Q]
     EmuEpilogue e;
     e.c64 = cKvv.p; e.rs = nK; e.cs = 1;
-    emu_abt(v * v, nK, nK, w4.p, nK, 1, LKinv.p, 1, nK, e);
+    emu_abt(kEmu10x6, v * v, nK, nK, w4.p, nK, 1, LKinv.p, 1, nK, e);
   } else {
     dgemm(false, false, v * v, nK, nK, 1.0, w4.p, nK, LKinv.p, nK, 0.0, cKvv.p, nK, st);
   }
@@ -1760,38 +1761,42 @@ static TcEpilogue ep_f64(double* c, long long rs, long long bsc = 0, double alph
   return e;
 }
 
-// Mixed precision, Coulomb transforms (ia|P)_J = sum_mu,nu C_mu,i C_nu,a
-// (mu nu|P) as FP64-accurate products on the FP16 tensor cores (exact
-// operand splitting, gemm_emu.cu).  The J metric is ill-conditioned and the
+// Coulomb transforms (ia|P)_J = sum_mu,nu C_mu,i C_nu,a (mu nu|P) as
+// FP64-accurate products on the FP16 tensor cores (exact operand splitting,
+// gemm_emu.cu; 10 x 6 bits in the mixed form, 9 x 7 in the FP64 form).  The J metric is ill-conditioned and the
 // MO transforms cancel heavily, so these stay at FP64 accuracy.
 // Transform 1: H[(nu,P)][i] = sum_mu T[(nu,P)][mu] C_o[mu][i], stored as
 // H[nu][i][P] (T symmetric in mu, nu; read through (mu nu|P) = T[mu][nu][P]);
 // transform 2: W[(i,P)][a] = sum_nu H[(i,P)][nu] C_v[nu][a], stored as
 // W[i][a][P].
-void Engine::coulomb_emu(double* H, double* W) {
+void Engine::coulomb_emu(EmuForm f, double* H, double* W) {
   const int o = nocc, v = nvir, n = nao;
   const long long rT = (long long)n * nJ, rH = (long long)o * nJ;
-  RIS_REQUIRE(rT < (1ll << 31), RIS_ERR_ARG, "Coulomb transform too large for one product");
-  // H[(nu,P)][i]: A[(nu,P)][mu] = T[mu][(nu,P)], B[i][mu] = C[mu][i]
-  EmuEpilogue e1;
-  e1.c64 = H; e1.rin = nJ; e1.rld = rH; e1.rs = 1; e1.cs = nJ;
-  emu_abt((int)rT, o, n, TJ.p, 1, rT, C.p, 1, nmo, e1);
+  // H[(nu,P)][i]: A[(nu,P)][mu] = T[mu][(nu,P)], B[i][mu] = C[mu][i]; blocks
+  // of nu, so that the digits of T stay below about 4 GB on any system
+  const int per = (int)std::max(1LL, std::min((long long)n, (1LL << 31) / ((long long)emu_slices(f) * n * nJ)));
+  for (int nu = 0; nu < n; nu += per) {
+    const int nn = std::min(per, n - nu);
+    EmuEpilogue e1;
+    e1.c64 = H + nu * rH; e1.rin = nJ; e1.rld = rH; e1.rs = 1; e1.cs = nJ;
+    emu_abt(f, nn * nJ, o, n, TJ.p + (long long)nu * nJ, 1, rT, C.p, 1, nmo, e1);
+  }
   // W[(i,P)][a]: A[(i,P)][nu] = H[nu][(i,P)], B[a][nu] = C[nu][o + a]
   EmuEpilogue e2;
   e2.c64 = W; e2.rin = nJ; e2.rld = (long long)v * nJ; e2.rs = 1; e2.cs = nJ;
-  emu_abt((int)rH, v, n, H, 1, rH, C.p + o, 1, nmo, e2);
+  emu_abt(f, (int)rH, v, n, H, 1, rH, C.p + o, 1, nmo, e2);
 }
 
-void Engine::emu_abt(int M, int N, int K, const double* A, long long rsA, long long ksA,
+void Engine::emu_abt(EmuForm f, int M, int N, int K, const double* A, long long rsA, long long ksA,
                      const double* B, long long rsB, long long ksB, const EmuEpilogue& ep) {
   if (!d_tcerr) {
     RIS_ALLOC(cudaMallocAsync((void**)&d_tcerr, sizeof(int), st));
     RIS_CUDA(cudaMemsetAsync(d_tcerr, 0, sizeof(int), st));
   }
   EmuMat a, b;
-  a.slice(kEmu10x6, kEmuRowsA, emu_src(A, rsA, ksA), M, K, st);
-  b.slice(kEmu10x6, emu_cols(N), emu_src(B, rsB, ksB), N, K, st);
-  emu_gemm(kEmu10x6, M, N, a.op, b.op, ep, d_tcerr, st);
+  a.slice(f, kEmuRowsA, emu_src(A, rsA, ksA), M, K, st);
+  b.slice(f, emu_cols(N), emu_src(B, rsB, ksB), N, K, st);
+  emu_gemm(f, M, N, a.op, b.op, ep, d_tcerr, st);
 }
 
 // Mixed precision: (ab|P)_K = sum_mu,nu C_mu,a C_nu,b (mu nu|P) by two
@@ -3441,10 +3446,10 @@ void Engine::setup_streamed() {
     if (opt.precision == RIS_MIXED && opt.emu_f64) {
       EmuEpilogue e;
       e.c64 = BJao.p; e.rs = nJ; e.cs = 1;
-      emu_abt((int)nfp, nJ, nU, Ts.p, nU, 1, LJu.p, nU, 1, e);
+      emu_abt(kEmu10x6, (int)nfp, nJ, nU, Ts.p, nU, 1, LJu.p, nU, 1, e);
       EmuEpilogue e2;
       e2.c64 = BKao.p; e2.rs = nK; e2.cs = 1;
-      emu_abt((int)nfp, nK, nK, Ts.p, nU, 1, LKinv.p, nK, 1, e2);
+      emu_abt(kEmu10x6, (int)nfp, nK, nK, Ts.p, nU, 1, LKinv.p, nK, 1, e2);
     } else {
       dgemm(false, true, (int)nfp, nJ, nU, 1.0, Ts.p, nU, LJu.p, nU, 0.0, BJao.p, nJ, st);
       dgemm(false, true, (int)nfp, nK, nK, 1.0, Ts.p, nU, LKinv.p, nK, 0.0, BKao.p, nK, st);
@@ -3511,10 +3516,10 @@ void Engine::build_B_streamed() {
         const long long rT = (long long)n * rw, rH = (long long)o * rw;
         EmuEpilogue e1;
         e1.c64 = H.p; e1.rin = rw; e1.rld = rH; e1.rs = 1; e1.cs = rw;
-        emu_abt((int)rT, o, n, Tb.p, 1, rT, C.p, 1, nmo, e1);
+        emu_abt(kEmu10x6, (int)rT, o, n, Tb.p, 1, rT, C.p, 1, nmo, e1);
         EmuEpilogue e2;
         e2.c64 = BJ.p + r0; e2.rin = rw; e2.rld = (long long)v * nJ; e2.rs = 1; e2.cs = nJ;
-        emu_abt((int)rH, v, n, H.p, 1, rH, C.p + o, 1, nmo, e2);
+        emu_abt(kEmu10x6, (int)rH, v, n, H.p, 1, rH, C.p + o, 1, nmo, e2);
       } else {  // H[i][nu][r], then per i: B[i][a][r0 + r]
         dgemm(true, false, o, n * rw, n, 1.0, Co, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
         GemmBatch bt;

@@ -240,10 +240,10 @@ struct Engine : StreamOwner {
   void apply_exchange_mixed(const double* Z, int nvec, double* out, double alpha, double beta);
   void prepare_mixed();
   void build_Kvv_tc(double* out);
-  void coulomb_emu(double* H, double* W);  // H [nu][i][P], W [i][a][P] (mixed form)
+  void coulomb_emu(EmuForm f, double* H, double* W);  // H [nu][i][P], W [i][a][P]
   // C = A B^T, element (r, k) of A at A[r rsA + k ksA] (B likewise), as an
   // FP64-accurate product on the tensor cores
-  void emu_abt(int M, int N, int K, const double* A, long long rsA, long long ksA, const double* B,
+  void emu_abt(EmuForm f, int M, int N, int K, const double* A, long long rsA, long long ksA, const double* B,
                long long rsB, long long ksB, const EmuEpilogue& ep);
   // FP64 form: the exchange products (B^K build, A products, exchange
   // densities) as FP64-accurate products on the FP16 tensor cores
