@@ -144,6 +144,20 @@ __host__ __device__ constexpr int hidx(int t, int u, int v) {
   return (t + u + v) * (t + u + v + 1) * (t + u + v + 2) / 6 +
          (u + v) * (u + v + 1) / 2 + v;
 }
+// hidx as a table for the rolled loops (its indices are uniform over a warp)
+constexpr int kHL = 2 * kMaxLAO + kMaxLAux + 2;  // t, u, v <= LA + LB + LC + 1
+struct HTab {
+  unsigned char h[kHL][kHL][kHL];
+  static constexpr HTab make() {
+    HTab r{};
+    for (int t = 0; t < kHL; t++)
+      for (int u = 0; u < kHL; u++)
+        for (int v = 0; v < kHL; v++)
+          r.h[t][u][v] = t + u + v < kHL ? (unsigned char)hidx(t, u, v) : 0;
+    return r;
+  }
+};
+__constant__ HTab c_h = HTab::make();
 template <int L>
 struct NH {
   static constexpr int n = (L + 1) * (L + 2) * (L + 3) / 6;
@@ -186,13 +200,41 @@ __device__ __forceinline__ void hermite_E(double p, const double (&PA)[3], const
   }
 }
 
-// R[hidx(t,u,v)] = R^{(0)}_{tuv}(rho, X,Y,Z) for t+u+v <= L, built in place
-// from n = L down to 0.
+// E[i][j][t] of one axis for i <= IA, j <= JB (rows of IA + JB + 1; entries
+// past t = i + j are not written).
+template <int IA, int JB>
+__device__ void hermite_E(double o2p, double PA, double PB, double* E) {
+  constexpr int NT = IA + JB + 1;
+  auto at = [&](int i, int j) { return E + (i * (JB + 1) + j) * NT; };
+  E[0] = 1.0;
+  for (int i = 1; i <= IA; i++) {
+    const double* lo = at(i - 1, 0);
+    for (int t = 0; t <= i; t++) {
+      double v = t < i ? PA * lo[t] : 0.0;
+      if (t > 0) v += o2p * lo[t - 1];
+      if (t + 1 < i) v += (t + 1) * lo[t + 1];
+      at(i, 0)[t] = v;
+    }
+  }
+  for (int j = 1; j <= JB; j++)
+    for (int i = 0; i <= IA; i++) {
+      const double* lo = at(i, j - 1);
+      for (int t = 0; t <= i + j; t++) {
+        double v = t < i + j ? PB * lo[t] : 0.0;
+        if (t > 0) v += o2p * lo[t - 1];
+        if (t + 1 < i + j) v += (t + 1) * lo[t + 1];
+        at(i, j)[t] = v;
+      }
+    }
+}
+
+// R[hidx(t,u,v)] = pref R^{(0)}_{tuv}(rho, X,Y,Z) for t+u+v <= L, built in
+// place from n = L down to 0.
 template <int L>
-__device__ __forceinline__ void hermite_R(double rho, double X, double Y, double Z,
+__device__ __forceinline__ void hermite_R(double pref, double rho, double X, double Y, double Z,
                                           const double (&F)[L + 1], double (&R)[NH<L>::n]) {
   double pw[L + 1];
-  pw[0] = 1.0;
+  pw[0] = pref;
 #pragma unroll
   for (int n = 1; n <= L; n++) pw[n] = pw[n - 1] * (-2.0 * rho);
   R[0] = pw[L] * F[L];
@@ -233,6 +275,10 @@ __host__ __device__ constexpr int cy_(int l, int c) {
 }
 __host__ __device__ constexpr int cz_(int l, int c) {
   return l - cx_(l, c) - cy_(l, c);
+}
+// exponent of axis d
+__host__ __device__ constexpr int cxyz(int l, int c, int d) {
+  return d == 0 ? cx_(l, c) : d == 1 ? cy_(l, c) : cz_(l, c);
 }
 // 1/sqrt((2lx-1)!!(2ly-1)!!(2lz-1)!!) for the normalisation of component c
 __host__ __device__ constexpr double cfac(int l, int c) {
@@ -310,7 +356,7 @@ __global__ void __launch_bounds__(128) k_int3c(const int* __restrict__ pa, const
   double F[L + 1];
   boys<L>(rho * (X * X + Y * Y + Z * Z), boys_tab, F);
   double R[NH<L>::n];
-  hermite_R<L>(rho, X, Y, Z, F, R);
+  hermite_R<L>(1.0, rho, X, Y, Z, F, R);
   double E[3][LA + 1][LB + 1][LA + LB + 1];
   hermite_E<LA, LB>(g.p, g.PA, g.PB, E);
   const double pref = 2.0 * 17.493418327624862 /* pi^2.5 */ / (g.p * gam * sqrt(g.p + gam)) *
@@ -371,101 +417,219 @@ __global__ void __launch_bounds__(128) k_int3c(const int* __restrict__ pa, const
   }
 }
 
-// d(mu nu|P)/dA_x (A = centre of mu) and d(mu nu|P)/dB_x, written as
-// D[x][mu][nu][P] and D[x][nu][mu][P] (computed in FP64, stored as T).
-template <int LA, int LB, int LC, class T>
-__global__ void __launch_bounds__(128) k_int3c_deriv(
-    const int* __restrict__ pa, const int* __restrict__ pb, int p0, int np,
-    const int* __restrict__ auxl, int nax, const int* __restrict__ sh_atom,
-    const int* __restrict__ sh_off, const double* __restrict__ sh_ex,
-    const double* __restrict__ sh_nb, const int* __restrict__ ax_atom,
-    const int* __restrict__ ax_off, const double* __restrict__ ax_ex,
-    const double* __restrict__ ax_nb, const double* __restrict__ xyz,
-    const double* __restrict__ boys_tab, int nao, int naux, T* __restrict__ D) {
-  constexpr int L = LA + LB + LC + 1;
-  long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= (long long)np * nax) return;
-  const int ip = p0 + (int)(tid / nax);
-  const int sc = auxl[(int)(tid % nax)];
-  const int sa = pa[ip], sb = pb[ip];
-  const double* A = xyz + 3 * sh_atom[sa];
-  const double* B = xyz + 3 * sh_atom[sb];
-  const double* Cc = xyz + 3 * ax_atom[sc];
-  PairGeom g;
-  const double alpha = sh_ex[sa], beta = sh_ex[sb];
-  pair_geom(alpha, A, beta, B, sh_nb[sa], sh_nb[sb], g);
-  const double gam = ax_ex[sc];
-  const double rho = g.p * gam / (g.p + gam);
-  const double X = g.P[0] - Cc[0], Y = g.P[1] - Cc[1], Z = g.P[2] - Cc[2];
-  double F[L + 1];
-  boys<L>(rho * (X * X + Y * Y + Z * Z), boys_tab, F);
-  double R[NH<L>::n];
-  hermite_R<L>(rho, X, Y, Z, F, R);
-  double E[3][LA + 2][LB + 2][LA + LB + 3];
-  hermite_E<LA + 1, LB + 1>(g.p, g.PA, g.PB, E);
-  const double pref = 2.0 * 17.493418327624862 / (g.p * gam * sqrt(g.p + gam)) * g.pref_ab *
-                      ax_nb[sc];
-  const int oa = sh_off[sa], ob = sh_off[sb], oc = ax_off[sc];
-  const size_t plane = (size_t)nao * nao * naux;
-#pragma unroll 1
-  for (int ia = 0; ia < (LA + 1) * (LA + 2) / 2; ia++) {
-    const int a_[3] = {cx_(LA, ia), cy_(LA, ia), cz_(LA, ia)};
-#pragma unroll 1
-    for (int ib = 0; ib < (LB + 1) * (LB + 2) / 2; ib++) {
-      const int b_[3] = {cx_(LB, ib), cy_(LB, ib), cz_(LB, ib)};
-      const double nab = pref * cfac(LA, ia) * cfac(LB, ib);
-#pragma unroll 1
-      for (int ic = 0; ic < (LC + 1) * (LC + 2) / 2; ic++) {
-        int th[3][2];
-        double fh[3][2];
-        const int nh[3] = {herm1(cx_(LC, ic), gam, -1.0, th[0], fh[0]),
-                           herm1(cy_(LC, ic), gam, -1.0, th[1], fh[1]),
-                           herm1(cz_(LC, ic), gam, -1.0, th[2], fh[2])};
-        const double sc_ = cfac(LC, ic) * nab;
-        const int mu = oa + ia, nu = ob + ib, P = oc + ic;
-#pragma unroll 1
+// ------------------------------------------------------------------ derivatives
+// GB300 issues an FP64 instruction of a warp about every 19 cycles per SM
+// (1.7 FP64 operations per clock), so the derivative kernel is bound by its
+// number of FP64 operations, as long as every SM has enough warps: shared
+// memory, index arithmetic and rolled loops are free beside them.  So
+// * whatever depends on the shell pair alone (product centre, E
+//   coefficients, their products over axes, the derivative combinations,
+//   norms) is made once per pair by its CTA and kept in shared memory as the
+//   coefficients of the R_tuv;
+// * the R_tuv of kItems (pair, auxiliary shell) items at a time, with every
+//   remaining factor folded into F_0, go to shared memory as well, and a
+//   warp then takes one function pair and auxiliary component for 32 items,
+//   one multiply-add per coefficient.  A class of few pairs (dd: 210 on
+//   C20H22) so still has 100 warps of work per 32 items.
+// All classes of C20H22 (1 M items): 1142 us, before (an item per thread,
+// everything recomputed by each) 3843 us; dd with p auxiliary shells 114
+// instead of 1160 us.  With the coefficients per pair but an item per thread
+// it was 3231 us: 52 CTAs for dd, 130 for dp.
+struct PairGeo {
+  double p, P[3], al, be;  // al, be: the two exponents
+  double K;                // K_ab * nbase_a * nbase_b
+  int oa, ob;              // first functions
+};
+
+struct PairSrc {
+  const int *pa, *pb;  // shells of each pair
+  int p0, np;          // the class's range of the list
+  const int *atom, *off;
+  const double *ex, *nb, *xyz;
+};
+
+// Geometry and E coefficients (per axis) of pairs first .. first + npb - 1 of
+// the class, one thread per (pair, axis).
+template <int IA, int JB>
+__device__ __forceinline__ void pair_setup(const PairSrc& s, int first, int npb, PairGeo* geo, double* E) {
+  constexpr int NE = (IA + 1) * (JB + 1) * (IA + JB + 1);
+  for (int i = threadIdx.x; i < 3 * npb; i += blockDim.x) {
+    const int d = i % 3, sa = s.pa[s.p0 + first + i / 3], sb = s.pb[s.p0 + first + i / 3];
+    const double* A = s.xyz + 3 * s.atom[sa];
+    const double* B = s.xyz + 3 * s.atom[sb];
+    const double a = s.ex[sa], b = s.ex[sb], p = a + b;
+    PairGeo& g = geo[i / 3];
+    const double P = (a * A[d] + b * B[d]) / p;
+    g.P[d] = P;
+    if (d == 0) {
+      double ab2 = 0.0;
+#pragma unroll
+      for (int k = 0; k < 3; k++) ab2 += (A[k] - B[k]) * (A[k] - B[k]);
+      g.p = p;
+      g.al = a;
+      g.be = b;
+      g.K = exp(-a * b / p * ab2) * s.nb[sa] * s.nb[sb];
+      g.oa = s.off[sa];
+      g.ob = s.off[sb];
+    }
+    hermite_E<IA, JB>(0.5 / p, P - A[d], P - B[d], E + i * NE);
+  }
+}
+
+// Derivative coefficients: per function pair and direction x (y, z the other
+// two axes) the products E^y_u E^z_v, then per t the pairs
+//   K N (2 alpha E^{a+1,b}_t - a E^{a-1,b}_t)   (centre A)
+//   K N (2 beta  E^{a,b+1}_t - b E^{a,b-1}_t)   (centre B),
+// so that both derivatives share sum_uv E^y_u E^z_v R_tuv.
+template <int LA, int LB, int LC>
+struct DerivTab {
+  static constexpr int L = LA + LB + LC + 1;
+  static constexpr int NA = (LA + 1) * (LA + 2) / 2, NB = (LB + 1) * (LB + 2) / 2, NC = (LC + 1) * (LC + 2) / 2;
+  static constexpr int NT = LA + LB + 3;
+  static constexpr int NE = (LA + 2) * (LB + 2) * NT;
+  // items whose R_tuv are held at a time: at most 44 KB of them
+  static constexpr int items() {
+    int n = 256;
+    while (n > 32 && n * NH<L>::n * 8 > 44 * 1024) n /= 2;
+    return n;
+  }
+  static constexpr int kItems = items();
+  // slots of the E^y E^z products (even, so that the (A, B) pairs are 16-byte aligned)
+  static __host__ __device__ constexpr int nyz(int ny, int nz) {
+    return ny + nz == 0 ? 0 : ((ny + 1) * (nz + 1) + 1) & ~1;
+  }
+  static constexpr int width() {
+    int w = 0;
+    for (int a = 0; a < NA; a++)
+      for (int b = 0; b < NB; b++) {
+        const int n[3] = {cx_(LA, a) + cx_(LB, b), cy_(LA, a) + cy_(LB, b), cz_(LA, a) + cz_(LB, b)};
         for (int x = 0; x < 3; x++) {
-          // differentiated direction x: E -> 2 alpha E^{a+1} - a_x E^{a-1}
-          // (centre A) and 2 beta E^{b+1} - b_x E^{b-1} (centre B)
-          const int y = (x + 1) % 3, z = (x + 2) % 3;
-          const int tx_max = a_[x] + b_[x] + 1;
-          double sA = 0.0, sB = 0.0;
-#pragma unroll 1
-          for (int t = 0; t <= tx_max; t++) {
-            const double up = E[x][a_[x] + 1][b_[x]][t];
-            const double dn = a_[x] > 0 ? E[x][a_[x] - 1][b_[x]][t] : 0.0;
-            const double upb = E[x][a_[x]][b_[x] + 1][t];
-            const double dnb = b_[x] > 0 ? E[x][a_[x]][b_[x] - 1][t] : 0.0;
-            const double eA = 2.0 * alpha * up - a_[x] * dn;
-            const double eB = 2.0 * beta * upb - b_[x] * dnb;
-            double r = 0.0;
-            // LC <= 1: one Hermite term per axis (loops of length 1 at compile time)
-            const int mx = LC <= 1 ? 1 : nh[x], my = LC <= 1 ? 1 : nh[y], mz = LC <= 1 ? 1 : nh[z];
-            for (int jx = 0; jx < mx; jx++)
-              for (int jy = 0; jy < my; jy++)
-                for (int jz = 0; jz < mz; jz++) {
-                  const double fc = fh[x][jx] * fh[y][jy] * fh[z][jz];
-                  double rr = 0.0;
-#pragma unroll 1
-                  for (int u = 0; u <= a_[y] + b_[y]; u++) {
-                    const double eu = E[y][a_[y]][b_[y]][u];
-#pragma unroll 1
-                    for (int v = 0; v <= a_[z] + b_[z]; v++) {
-                      int tuv[3];
-                      tuv[x] = t + th[x][jx];
-                      tuv[y] = u + th[y][jy];
-                      tuv[z] = v + th[z][jz];
-                      rr += eu * E[z][a_[z]][b_[z]][v] * R[hidx(tuv[0], tuv[1], tuv[2])];
-                    }
-                  }
-                  r += fc * rr;
-                }
-            sA += eA * r;
-            sB += eB * r;
-          }
-          D[x * plane + ((size_t)mu * nao + nu) * naux + P] = (T)(sA * sc_);
-          D[x * plane + ((size_t)nu * nao + mu) * naux + P] = (T)(sB * sc_);
+          const int k = nyz(n[(x + 1) % 3], n[(x + 2) % 3]) + 2 * (n[x] + 2);
+          w = k > w ? k : w;
         }
+      }
+    return w;
+  }
+  static constexpr int W = width();
+  static constexpr int kPair = NA * NB * 3 * W;
+  static constexpr size_t bytes(int pb) {
+    return (size_t)(NH<L>::n * kItems + pb * (kPair + 3 * NE)) * sizeof(double) + pb * sizeof(PairGeo);
+  }
+};
+constexpr int kDerivT = 256;
+
+// d(mu nu|P)/dA_x (A = centre of mu) and d(mu nu|P)/dB_x, written as
+// D[x][mu][nu][P] and D[x][nu][mu][P] (computed in FP64, stored as T); pb
+// shell pairs per CTA.
+template <int LA, int LB, int LC, class T>
+__global__ void __launch_bounds__(kDerivT) k_int3c_deriv(
+    PairSrc src, int pb, const int* __restrict__ auxl, int nax, const int* __restrict__ ax_atom,
+    const int* __restrict__ ax_off, const double* __restrict__ ax_ex, const double* __restrict__ ax_nb,
+    const double* __restrict__ boys_tab, int nao, int naux, T* __restrict__ D) {
+  using Tab = DerivTab<LA, LB, LC>;
+  constexpr int L = Tab::L, NA = Tab::NA, NB = Tab::NB, NT = Tab::NT, RI = Tab::kItems;
+  extern __shared__ __align__(16) double sm3c[];
+  double* tab = sm3c;
+  double* Rs = tab + pb * Tab::kPair;  // [hidx][item]
+  double* E = Rs + NH<L>::n * RI;
+  PairGeo* geo = (PairGeo*)(E + pb * 3 * Tab::NE);
+  const int first = blockIdx.x * pb, npb = min(pb, src.np - first);
+  pair_setup<LA + 1, LB + 1>(src, first, npb, geo, E);
+  __syncthreads();
+  for (int i = threadIdx.x; i < npb * NA * NB * 3; i += kDerivT) {
+    const int x = i % 3, f = i / 3, k = f / (NA * NB), ia = f / NB % NA, ib = f % NB;
+    const int a_[3] = {cx_(LA, ia), cy_(LA, ia), cz_(LA, ia)}, b_[3] = {cx_(LB, ib), cy_(LB, ib), cz_(LB, ib)};
+    const int y = (x + 1) % 3, z = (x + 2) % 3;
+    auto e = [&](int d, int da, int db) {
+      return E + ((k * 3 + d) * (LA + 2) * (LB + 2) + (a_[d] + da) * (LB + 2) + b_[d] + db) * NT;
+    };
+    const int nx = a_[x] + b_[x], ny = a_[y] + b_[y], nz = a_[z] + b_[z];
+    double* o = tab + i * Tab::W;
+    if (ny + nz > 0) {
+      const double *ey = e(y, 0, 0), *ez = e(z, 0, 0);
+      for (int u = 0; u <= ny; u++)
+        for (int v = 0; v <= nz; v++) o[u * (nz + 1) + v] = ey[u] * ez[v];
+    }
+    o += Tab::nyz(ny, nz);
+    const double s = geo[k].K * cfac(LA, ia) * cfac(LB, ib), ta = 2.0 * geo[k].al, tb = 2.0 * geo[k].be;
+    for (int t = 0; t <= nx + 1; t++) {
+      double A = ta * e(x, 1, 0)[t], B = tb * e(x, 0, 1)[t];
+      if (t < nx) {  // E^{a-1,b}_t and E^{a,b-1}_t end at t = a + b - 1
+        if (a_[x] > 0) A -= a_[x] * e(x, -1, 0)[t];
+        if (b_[x] > 0) B -= b_[x] * e(x, 0, -1)[t];
+      }
+      o[2 * t] = s * A;
+      o[2 * t + 1] = s * B;
+    }
+  }
+  const size_t plane = (size_t)nao * nao * naux;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i0 = 0; i0 < npb * nax; i0 += RI) {
+    const int ni = min(RI, npb * nax - i0);
+    __syncthreads();  // the coefficients; the last items' R_tuv have been read
+    if (threadIdx.x < ni) {
+      const int it = i0 + threadIdx.x, sc = auxl[it % nax];
+      const PairGeo& g = geo[it / nax];
+      const double* Cc = src.xyz + 3 * ax_atom[sc];
+      const double gam = ax_ex[sc], s = g.p + gam, rho = g.p * gam / s;
+      const double X = g.P[0] - Cc[0], Y = g.P[1] - Cc[1], Z = g.P[2] - Cc[2];
+      double F[L + 1], R[NH<L>::n];
+      boys<L>(rho * (X * X + Y * Y + Z * Z), boys_tab, F);
+      double pref = 2.0 * 17.493418327624862 /* pi^2.5 */ / (g.p * gam * sqrt(s)) * ax_nb[sc];
+      if (LC == 1) pref *= -0.5 / gam;  // p function: -1/2 gamma times R shifted by one
+      hermite_R<L>(pref, rho, X, Y, Z, F, R);
+#pragma unroll
+      for (int k = 0; k < NH<L>::n; k++) Rs[k * RI + threadIdx.x] = R[k];
+    }
+    __syncthreads();
+    const int ng = (ni + 31) / 32;
+    for (int w = warp; w < ng * (Tab::NC * NA * NB); w += kDerivT / 32) {
+      const int li = (w % ng) * 32 + lane, f = w / ng;
+      const int ic = f / (NA * NB), ia = f / NB % NA, ib = f % NB;
+      if (li >= ni) continue;
+      const int it = i0 + li, k = it / nax, sc = auxl[it % nax];
+      const int cx = cx_(LC, ic), cy = cy_(LC, ic), cz = cz_(LC, ic);
+      const double* R = Rs + li;
+      const double h = LC == 2 ? 0.5 / ax_ex[sc] : 0.0;
+      // R_tuv with the Hermite expansion of the auxiliary component (p: shifted;
+      // d: x^2 = Lambda_0 / 2g + Lambda_2 / 4g^2, xy = Lambda_1 Lambda_1 / 4g^2)
+      auto Q = [&](int t, int u, int v) {
+        double q = R[c_h.h[t + cx][u + cy][v + cz] * RI];
+        if (LC == 2) {
+          q *= h * h;
+          if (cx == 2 || cy == 2 || cz == 2) q += h * R[c_h.h[t][u][v] * RI];
+          q *= cfac(LC, ic);
+        }
+        return q;
+      };
+      const int mu = geo[k].oa + ia, nu = geo[k].ob + ib, P = ax_off[sc] + ic;
+      const size_t mn = ((size_t)mu * nao + nu) * naux + P, nm = ((size_t)nu * nao + mu) * naux + P;
+#pragma unroll
+      for (int x = 0; x < 3; x++) {
+        constexpr int kY[3] = {1, 2, 0}, kZ[3] = {2, 0, 1};
+        const int nx = cxyz(LA, ia, x) + cxyz(LB, ib, x), ny = cxyz(LA, ia, kY[x]) + cxyz(LB, ib, kY[x]),
+                  nz = cxyz(LA, ia, kZ[x]) + cxyz(LB, ib, kZ[x]);
+        const double* c = tab + (((k * NA + ia) * NB + ib) * 3 + x) * Tab::W;
+        const double2* ab = reinterpret_cast<const double2*>(c + Tab::nyz(ny, nz));
+        double sA = 0.0, sB = 0.0;
+#pragma unroll 1
+        for (int t = 0; t <= nx + 1; t++) {
+          auto q = [&](int u, int v) { return x == 0 ? Q(t, u, v) : x == 1 ? Q(v, t, u) : Q(u, v, t); };
+          double r = 0.0;
+          if (ny + nz == 0) {
+            r = q(0, 0);
+          } else {
+            const double* e = c;
+#pragma unroll 1
+            for (int u = 0; u <= ny; u++)
+#pragma unroll 1
+              for (int v = 0; v <= nz; v++) r += *e++ * q(u, v);
+          }
+          sA += ab[t].x * r;
+          sB += ab[t].y * r;
+        }
+        D[x * plane + mn] = (T)sA;
+        D[x * plane + nm] = (T)sB;
       }
     }
   }
@@ -490,7 +654,7 @@ __global__ void k_int2c(int nsh, const int* __restrict__ atom, const int* __rest
   double F[LM + 1];
   boys<LM>(rho * (X * X + Y * Y + Z * Z), boys_tab, F);
   double R[NH<LM>::n];
-  hermite_R<LM>(rho, X, Y, Z, F, R);
+  hermite_R<LM>(1.0, rho, X, Y, Z, F, R);
   const double pref = 2.0 * 17.493418327624862 / (a * c * sqrt(a + c)) * nbase[sp] * nbase[sq];
   const int l1 = lq[sp], l2 = lq[sq];
   for (int i = 0; i < ncart(l1); i++) {
@@ -690,17 +854,31 @@ static void launch_int3c(const ShellSet& ao, const ShellSet& aux, const PairList
   RIS_CHECK_LAUNCH();
 }
 
+// Shell pairs per CTA of k_int3c_deriv: as many as fill the items held at a
+// time, fewer while the class has less than three CTAs an SM (a dd class has
+// a few hundred pairs) or their coefficients would leave less than three CTAs
+// an SM's shared memory.
+template <class Tab>
+static int deriv_pairs(int np, int nax) {
+  int pb = std::min(cdiv(Tab::kItems, nax), std::max(1, np / (3 * 152)));
+  while (pb > 1 && Tab::bytes(pb) > 72 * 1024) pb--;
+  return pb;
+}
+
 template <int LA, int LB, int LC, class T>
 static void launch_int3c_deriv(const ShellSet& ao, const ShellSet& aux, const PairList& pl,
                                const double* xyz, const double* tab, T* D, cudaStream_t st) {
+  using Tab = DerivTab<LA, LB, LC>;
   const int cls = LA * (LA + 1) / 2 + LB;
-  const int p0 = pl.class_off[cls], np = pl.class_off[cls + 1] - p0;
+  const PairSrc src{pl.a, pl.b, pl.class_off[cls], pl.class_off[cls + 1] - pl.class_off[cls],
+                    ao.atom, ao.off, ao.ex, ao.nbase, xyz};
   const int nax = (int)aux.by_l[LC].size();
-  if (np == 0 || nax == 0) return;
-  const long long nt = (long long)np * nax;
-  k_int3c_deriv<LA, LB, LC, T><<<(unsigned)cdiv(nt, 128), 128, 0, st>>>(
-      pl.a, pl.b, p0, np, aux.d_by_l[LC], nax, ao.atom, ao.off, ao.ex, ao.nbase, aux.atom,
-      aux.off, aux.ex, aux.nbase, xyz, tab, ao.nfun, aux.nfun, D);
+  if (src.np == 0 || nax == 0) return;
+  const int pb = deriv_pairs<Tab>(src.np, nax);
+  static_assert(Tab::bytes(1) <= 72 * 1024, "coefficients of one pair");
+  ensure_smem_attr((const void*)k_int3c_deriv<LA, LB, LC, T>, 72 * 1024);
+  k_int3c_deriv<LA, LB, LC, T><<<cdiv(src.np, pb), kDerivT, Tab::bytes(pb), st>>>(
+      src, pb, aux.d_by_l[LC], nax, aux.atom, aux.off, aux.ex, aux.nbase, tab, ao.nfun, aux.nfun, D);
   RIS_CHECK_LAUNCH();
 }
 
