@@ -7,12 +7,19 @@
 // about FP32 accuracy at tensor-core rates.
 //
 // Kernel structure (one 128 x 128 output tile per CTA, 128 threads):
-//   warp 0 / lane 0 : TMA producer, 3-stage ring of (A_hi, A_lo, B_hi, B_lo)
-//                     tiles of 128 rows x 32 FP32 (128-byte swizzle)
+//   warp 0 / lane 0 : TMA producer, ring of (A_hi, A_lo, B_hi, B_lo) tiles of
+//                     128 rows x 16 FP32 (64-byte swizzle), 32 KB a stage
 //   warp 1          : allocates 128 TMEM columns; lane 0 issues
 //                     tcgen05.mma.kind::tf32 (M=128, N=128, K=8) and commits
 //                     each stage back to the producer through an mbarrier
 //   warps 0-3       : epilogue, tcgen05.ld of TMEM lanes 32w..32w+31
+// The contractions are short (K = 71 ... 441 on C20H22), so that a tile's
+// start (TMEM, barriers, first loads) and its epilogue (about 3000 cycles for
+// 128 x 128 stored as hi/lo) weigh as much as its products: a ring of three
+// stages takes 97 KB and leaves room for a second CTA on the SM, whose
+// products run meanwhile.  Grids of at most one CTA per SM take six stages
+// instead (exchange products of 18 C20H22 vectors
+// 254 -> 224 us; a mixed C20H22 evaluation's 170 launches 4474 -> 4156 us.)
 // All mbarrier waits are bounded (about one second of clock64 cycles); a
 // timeout sets the error flag, drains what this CTA has in flight and frees
 // its TMEM before returning.
@@ -31,12 +38,13 @@ namespace ris {
 namespace {
 using namespace tcx;
 
-constexpr int BM = 128, BN = 128, BK = 32, STAGES = 3;
-constexpr int TILE_BYTES = BM * BK * 4;                      // 16 KB
+constexpr int BM = 128, BN = 128, BK = 16;
+constexpr int KB = 32;  // slices of a split contraction are multiples of this
+constexpr int TILE_BYTES = BM * BK * 4;                      // 8 KB
 constexpr int STAGE_BYTES = 4 * TILE_BYTES;                  // hi/lo of A and B
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr int smem_bytes(int stages) { return stages * STAGE_BYTES + 1024 + 256; }
 
-// 3-D map {K, rows, batch} of FP32, box {32, 128, 1}, 128-byte swizzle.
+// 3-D map {K, rows, batch} of FP32, box {16, 128, 1}, 64-byte swizzle.
 CUtensorMap make_map(const float* base, int K, int rows, int ld, long long bstride, int nb) {
   RIS_REQUIRE(base != nullptr, RIS_ERR_ARG, "tc_gemm: null operand");
   RIS_REQUIRE(((uintptr_t)base & 15) == 0, RIS_ERR_ARG, "tc_gemm: operand not 16-byte aligned");
@@ -48,19 +56,19 @@ CUtensorMap make_map(const float* base, int K, int rows, int ld, long long bstri
   cuuint32_t box[3] = {BK, BM, 1};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)base, dims, strides, box, es,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   RIS_REQUIRE(r == CUDA_SUCCESS, RIS_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
   return m;
 }
 
-// K-major operand tile of 128 rows x 128 bytes with 128-byte swizzle:
-// start address, leading offset unused (1), stride 1024 B between 8-row
-// groups, descriptor version 1, layout type 2 (SWIZZLE_128B).
-__device__ __forceinline__ uint64_t desc_sw128(const void* p) {
+// K-major operand tile of 128 rows x 64 bytes with 64-byte swizzle: start
+// address, leading offset unused (1), stride 512 B between 8-row groups,
+// descriptor version 1, layout type 4 (SWIZZLE_64B).
+__device__ __forceinline__ uint64_t desc_sw64(const void* p) {
   const uint64_t a = sa(p);
-  return ((a & 0x3FFFFull) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
-         (2ull << 61);
+  return ((a & 0x3FFFFull) >> 4) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) |
+         (4ull << 61);
 }
 
 // kind::tf32 instruction descriptor: D FP32 (bit 4), A and B TF32 (2 at bits
@@ -105,7 +113,8 @@ struct TcArgs {
   int* err;
 };
 
-__global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUtensorMap mAh,
+template <int STAGES>
+__global__ void __launch_bounds__(128, 2) k_tc_gemm(const __grid_constant__ CUtensorMap mAh,
                                                      const __grid_constant__ CUtensorMap mAl,
                                                      const __grid_constant__ CUtensorMap mBh,
                                                      const __grid_constant__ CUtensorMap mBl,
@@ -124,7 +133,8 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
     ks = z;
     z = 0;
   }
-  const int kb0 = ks * args.kb_per, kb1 = min(args.nkb, kb0 + args.kb_per);
+  const int kb0 = ks * args.kb_per * (KB / BK);  // blocks of BK
+  const int kb1 = min((args.K + BK - 1) / BK, kb0 + args.kb_per * (KB / BK));
   const int zA = args.nbA > 1 ? z : 0, zB = args.nbB > 1 ? z : 0;
 
   if (threadIdx.x == 0) {
@@ -180,8 +190,8 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       uint8_t* st = smem + s * STAGE_BYTES;
-      const uint64_t ah = desc_sw128(st), al = desc_sw128(st + TILE_BYTES);
-      const uint64_t bh = desc_sw128(st + 2 * TILE_BYTES), bl = desc_sw128(st + 3 * TILE_BYTES);
+      const uint64_t ah = desc_sw64(st), al = desc_sw64(st + TILE_BYTES);
+      const uint64_t bh = desc_sw64(st + 2 * TILE_BYTES), bl = desc_sw64(st + 3 * TILE_BYTES);
 #pragma unroll
       for (int kk = 0; kk < BK / 8; kk++) {
         const uint64_t off = (uint64_t)((kk * 32) >> 4);  // 32 bytes per K=8 step
@@ -373,7 +383,6 @@ void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb
   }
   RIS_REQUIRE(A.rows >= M && B.rows >= N, RIS_ERR_ARG, "tc_gemm: operand rows");
   RIS_REQUIRE(nb <= 65535, RIS_ERR_ARG, "tc_gemm: batch too large");
-  ensure_smem_attr((const void*)k_tc_gemm, SMEM_BYTES);
   const CUtensorMap mAh = make_map(A.hi, K, M, A.ld, A.bstride, A.nb);
   const CUtensorMap mAl = make_map(A.lo, K, M, A.ld, A.bstride, A.nb);
   const CUtensorMap mBh = make_map(B.hi, K, N, B.ld, B.bstride, B.nb);
@@ -382,7 +391,7 @@ void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb
   a.M = M;
   a.N = N;
   a.K = K;
-  a.nkb = cdiv(K, BK);
+  a.nkb = cdiv(K, KB);
   a.nbA = A.nb;
   a.nbB = B.nb;
   a.ep = ep;
@@ -416,7 +425,11 @@ void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb
   }
   dim3 grid(cdiv(N, BN), cdiv(M, BM), a.ksplit > 1 ? a.ksplit : nb);
   prof_begin(kProfTcGemm, st);
-  k_tc_gemm<<<grid, 128, SMEM_BYTES, st>>>(mAh, mAl, mBh, mBl, a);
+  const bool deep = (long long)grid.x * grid.y * grid.z <= 152;
+  const auto kern = deep ? k_tc_gemm<6> : k_tc_gemm<3>;
+  const int smem = smem_bytes(deep ? 6 : 3);
+  ensure_smem_attr((const void*)kern, smem);
+  kern<<<grid, 128, smem, st>>>(mAh, mAl, mBh, mBl, a);
   RIS_CHECK_LAUNCH();
   if (a.ksplit > 1) {
     k_tc_reduce<<<cdiv((long long)M * N, 32), 256, 0, st>>>(M, N, a.ksplit, part, ep.alpha, ep.beta,
