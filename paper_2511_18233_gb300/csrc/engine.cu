@@ -30,6 +30,7 @@
 #include <map>
 #include <mutex>
 #include <set>
+#include <type_traits>
 
 #include "engine.cuh"
 #include "gemm_ff.cuh"
@@ -767,11 +768,11 @@ __host__ __device__ inline void slice_range(int nao, int nslice, int s, int& lo,
   hi = (int)((long long)nao * (s + 1) / nslice);
 }
 
-// State densities regrouped for the contraction: DRt[batch][mu][nu][b] =
-// DR_{8 batch + b}[mu][nu] (zero past the last state), so that a partner's
-// eight weights are two (FP32) or four (FP64) vector loads.
+// State densities regrouped for the contraction, `per` states a batch:
+// DRt[batch][mu][nu][b] = DR_{per batch + b}[mu][nu] (rows of kCBatch, zero
+// past the last state), so that a partner's weights are vector loads.
 template <class T>
-__global__ void k_states_t(const double* __restrict__ DR, int nsu, int nao, T* __restrict__ out) {
+__global__ void k_states_t(const double* __restrict__ DR, int nsu, int per, int nao, T* __restrict__ out) {
   const long long nn2 = (long long)nao * nao;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nn2) return;
@@ -779,21 +780,27 @@ __global__ void k_states_t(const double* __restrict__ DR, int nsu, int nao, T* _
   T v[kCBatch];
 #pragma unroll
   for (int b = 0; b < kCBatch; b++) {
-    const int s = batch * kCBatch + b;
-    v[b] = s < nsu ? (T)DR[(size_t)s * nn2 + t] : (T)0;
+    const int s = batch * per + b;
+    v[b] = b < per && s < nsu ? (T)DR[(size_t)s * nn2 + t] : (T)0;
   }
   T* o = out + ((size_t)batch * nn2 + t) * kCBatch;
 #pragma unroll
   for (int b = 0; b < kCBatch; b++) o[b] = v[b];
 }
 
-__device__ __forceinline__ void load_w8(const float* p, float (&w)[kCBatch]) {
-  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
-  w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
-}
-__device__ __forceinline__ void load_w8(const double* p, double (&w)[kCBatch]) {
+// NS weights (and what else their last vector holds)
+template <int NS>
+__device__ __forceinline__ void load_w(const float* p, float (&w)[kCBatch]) {
 #pragma unroll
-  for (int h = 0; h < 4; h++) {
+  for (int h = 0; h < (NS + 3) / 4; h++) {
+    const float4 a = *reinterpret_cast<const float4*>(p + 4 * h);
+    w[4 * h] = a.x; w[4 * h + 1] = a.y; w[4 * h + 2] = a.z; w[4 * h + 3] = a.w;
+  }
+}
+template <int NS>
+__device__ __forceinline__ void load_w(const double* p, double (&w)[kCBatch]) {
+#pragma unroll
+  for (int h = 0; h < (NS + 1) / 2; h++) {
     const double2 a = *reinterpret_cast<const double2*>(p + 2 * h);
     w[2 * h] = a.x;
     w[2 * h + 1] = a.y;
@@ -802,11 +809,16 @@ __device__ __forceinline__ void load_w8(const double* p, double (&w)[kCBatch]) {
 
 // Coulomb part, per state (the pair densities are linear in the per-state
 // transition densities): part[slice][b][x][mu][P] = sum_{nu in slice}
-// D[x][mu][nu][P] DRt[mu][nu][b], b < ns <= kCBatch, DRt the batch's
-// symmetrised state densities regrouped by k_states_t.
-template <class T>
+// D[x][mu][nu][P] DRt[mu][nu][b], b < NS <= kCBatch, DRt the batch's
+// symmetrised state densities regrouped by k_states_t.  One instance per
+// number of states: the running sums of eight states hold 96 and more
+// registers whatever their use, which left a single state's pass with a
+// third of the warps, waiting for its loads (C24H12, FP64, one state: 382 ->
+// 158 us; ten C20H22 states, as 5 + 5 instead of 8 + 2: 926 -> 804 us, where
+// the FP64 pipe bounds them).
+template <class T, int NS>
 __global__ void __launch_bounds__(128) k_contract_states(const T* __restrict__ D,
-                                                         const T* __restrict__ DRt, int ns,
+                                                         const T* __restrict__ DRt,
                                                          int nao, int nU, int nslice,
                                                          const int* __restrict__ nbPtr,
                                                          const int* __restrict__ nbCol,
@@ -820,10 +832,10 @@ __global__ void __launch_bounds__(128) k_contract_states(const T* __restrict__ D
   q1 += nbPtr[mu];
   const size_t nn2 = (size_t)nao * nao;
   const size_t plane = nn2 * nU;
-  double y[kCBatch][3];
-  T c[kCBatch][3];
+  double y[NS][3];
+  T c[NS][3];
 #pragma unroll
-  for (int b = 0; b < kCBatch; b++)
+  for (int b = 0; b < NS; b++)
 #pragma unroll
     for (int x = 0; x < 3; x++) y[b][x] = 0.0, c[b][x] = (T)0;
   const T* dr = DRt + (size_t)mu * nao * kCBatch;
@@ -837,35 +849,36 @@ __global__ void __launch_bounds__(128) k_contract_states(const T* __restrict__ D
       const size_t a = ((size_t)mu * nao + nu) * nU + P;
       const T d0 = D[a], d1 = D[plane + a], d2 = D[2 * plane + a];
       T w[kCBatch];
-      load_w8(dr + (size_t)nu * kCBatch, w);
+      load_w<NS>(dr + (size_t)nu * kCBatch, w);
 #pragma unroll
-      for (int b = 0; b < kCBatch; b++) {
-        if (b >= ns) break;
+      for (int b = 0; b < NS; b++) {
         c[b][0] += d0 * w[b];
         c[b][1] += d1 * w[b];
         c[b][2] += d2 * w[b];
       }
     }
 #pragma unroll
-    for (int b = 0; b < kCBatch; b++)
+    for (int b = 0; b < NS; b++)
 #pragma unroll
       for (int x = 0; x < 3; x++) y[b][x] += (double)c[b][x], c[b][x] = (T)0;
   }
-  double* ps = part + (size_t)blockIdx.y * ns * 3 * nao * nU;
+  double* ps = part + (size_t)blockIdx.y * NS * 3 * nao * nU;
 #pragma unroll
-  for (int b = 0; b < kCBatch; b++) {
-    if (b >= ns) break;
+  for (int b = 0; b < NS; b++) {
 #pragma unroll
     for (int x = 0; x < 3; x++) ps[(((size_t)b * 3 + x) * nao + mu) * nU + P] = y[b][x];
   }
 }
 
-// Exchange part, per pair of a batch (nb <= kCBatch), P < nK:
+// Exchange part, per pair of a batch of NB <= kCBatch, P < nK:
 //   part[slice][g][x][mu][P] = sum_{nu in slice} D[x][mu][nu][P]
 //                              (GK_g[mu][nu][P] + GK_g[nu][mu][P]) / 2
-template <class T, class G>
+// (the half is applied to the sum: a power of two, the same bits with one
+// FP64 operation in five less; the FP64 form is bound by those: ten C20H22
+// pairs 912 -> 490 us, FP32 489 -> 201 us).
+template <class T, class G, int NB>
 __global__ void __launch_bounds__(128) k_contract_exchange(const T* __restrict__ D,
-                                                           const G* __restrict__ GK, int nb,
+                                                           const G* __restrict__ GK,
                                                            int nao, int nU, int nK, int nslice,
                                                            const int* __restrict__ nbPtr,
                                                            const int* __restrict__ nbCol,
@@ -880,10 +893,10 @@ __global__ void __launch_bounds__(128) k_contract_exchange(const T* __restrict__
   const size_t nn2 = (size_t)nao * nao;
   const size_t plane = nn2 * nU;
   const size_t gk = nn2 * nK;
-  double s[kCBatch][3];
-  T c[kCBatch][3];
+  double s[NB][3];
+  T c[NB][3];
 #pragma unroll
-  for (int b = 0; b < kCBatch; b++)
+  for (int b = 0; b < NB; b++)
 #pragma unroll
     for (int x = 0; x < 3; x++) s[b][x] = 0.0, c[b][x] = (T)0;
   for (int qc = q0; qc < q1; qc += kChunk) {
@@ -896,26 +909,53 @@ __global__ void __launch_bounds__(128) k_contract_exchange(const T* __restrict__
       const T d0 = D[a], d1 = D[plane + a], d2 = D[2 * plane + a];
       const size_t k1 = mn * nK + P, k2 = ((size_t)nu * nao + mu) * nK + P;
 #pragma unroll
-      for (int b = 0; b < kCBatch; b++) {
-        if (b >= nb) break;
-        const T g = (T)0.5 * ((T)GK[b * gk + k1] + (T)GK[b * gk + k2]);
+      for (int b = 0; b < NB; b++) {
+        const T g = (T)GK[b * gk + k1] + (T)GK[b * gk + k2];
         c[b][0] += d0 * g;
         c[b][1] += d1 * g;
         c[b][2] += d2 * g;
       }
     }
 #pragma unroll
-    for (int b = 0; b < kCBatch; b++)
+    for (int b = 0; b < NB; b++)
 #pragma unroll
       for (int x = 0; x < 3; x++) s[b][x] += (double)c[b][x], c[b][x] = (T)0;
   }
-  double* ps = part + (size_t)blockIdx.y * nb * 3 * nao * nK;
+  double* ps = part + (size_t)blockIdx.y * NB * 3 * nao * nK;
 #pragma unroll
-  for (int b = 0; b < kCBatch; b++) {
-    if (b >= nb) break;
+  for (int b = 0; b < NB; b++) {
 #pragma unroll
-    for (int x = 0; x < 3; x++) ps[(((size_t)b * 3 + x) * nao + mu) * nK + P] = s[b][x];
+    for (int x = 0; x < 3; x++) ps[(((size_t)b * 3 + x) * nao + mu) * nK + P] = 0.5 * s[b][x];
   }
+}
+
+// The instance for n <= kCBatch states or pairs: f(std::integral_constant).
+template <class F>
+static void with_batch(int n, F&& f) {
+  switch (n) {
+    case 1: return f(std::integral_constant<int, 1>());
+    case 2: return f(std::integral_constant<int, 2>());
+    case 3: return f(std::integral_constant<int, 3>());
+    case 4: return f(std::integral_constant<int, 4>());
+    case 5: return f(std::integral_constant<int, 5>());
+    case 6: return f(std::integral_constant<int, 6>());
+    case 7: return f(std::integral_constant<int, 7>());
+    default: return f(std::integral_constant<int, 8>());
+  }
+}
+template <class T>
+static void contract_states(dim3 grid, cudaStream_t st, const T* D, const T* DRt, int ns, int nao, int nU,
+                            int nslice, const int* nbPtr, const int* nbCol, double* part) {
+  with_batch(ns, [&](auto n) {
+    k_contract_states<T, n.value><<<grid, 128, 0, st>>>(D, DRt, nao, nU, nslice, nbPtr, nbCol, part);
+  });
+}
+template <class T, class G>
+static void contract_exchange(dim3 grid, cudaStream_t st, const T* D, const G* GK, int nb, int nao, int nU,
+                              int nK, int nslice, const int* nbPtr, const int* nbCol, double* part) {
+  with_batch(nb, [&](auto n) {
+    k_contract_exchange<T, G, n.value><<<grid, 128, 0, st>>>(D, GK, nao, nU, nK, nslice, nbPtr, nbCol, part);
+  });
 }
 
 // out[i] = sum_s part[s][i], i < n (fixed order)
@@ -2964,26 +3004,26 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   SBuf<double> Yst((size_t)nsu * 3 * nn * nU, st);
   prof_begin(kProfContract, st);
   const double dbytes = mixed ? 4.0 : 8.0;  // derivative integrals in FP32 / FP64
-  const int nbat = cdiv(nsu, kCBatch);
+  const int nbat = cdiv(nsu, kCBatch), per = cdiv(nsu, nbat);  // states per batch
   const size_t dtb = (size_t)nn * nn * kCBatch;  // one batch of regrouped densities
   SBuf<float> DRf(mixed ? nbat * dtb : 1, st);
   SBuf<double> DRd(mixed ? 1 : nbat * dtb, st);
   if (mixed)
-    k_states_t<float><<<dim3(cdiv((long long)nn * nn, 256), nbat), 256, 0, st>>>(DR.p, nsu, nn, DRf.p);
+    k_states_t<float><<<dim3(cdiv((long long)nn * nn, 256), nbat), 256, 0, st>>>(DR.p, nsu, per, nn, DRf.p);
   else
-    k_states_t<double><<<dim3(cdiv((long long)nn * nn, 256), nbat), 256, 0, st>>>(DR.p, nsu, nn, DRd.p);
+    k_states_t<double><<<dim3(cdiv((long long)nn * nn, 256), nbat), 256, 0, st>>>(DR.p, nsu, per, nn, DRd.p);
   RIS_CHECK_LAUNCH();
   const int slJ = pick_slices((long long)nn * nU, nbAvg);
   SBuf<double> partJ((size_t)slJ * std::min(nsu, kCBatch) * 3 * nn * nU, st);
-  for (int s0 = 0; s0 < nsu; s0 += kCBatch) {
-    const int ns = std::min(kCBatch, nsu - s0);
+  for (int s0 = 0; s0 < nsu; s0 += per) {
+    const int ns = std::min(per, nsu - s0);
     const dim3 grid(cdiv((long long)nn * nU, 128), slJ);
-    const size_t bo = (size_t)(s0 / kCBatch) * dtb;
+    const size_t bo = (size_t)(s0 / per) * dtb;
     if (mixed)
-      k_contract_states<float><<<grid, 128, 0, st>>>(Df.p, DRf.p + bo, ns, nn, nU, slJ, nbPtr.p,
+      contract_states<float>(grid, st, Df.p, DRf.p + bo, ns, nn, nU, slJ, nbPtr.p,
                                                      nbCol.p, partJ.p);
     else
-      k_contract_states<double><<<grid, 128, 0, st>>>(D.p, DRd.p + bo, ns, nn, nU, slJ, nbPtr.p,
+      contract_states<double>(grid, st, D.p, DRd.p + bo, ns, nn, nU, slJ, nbPtr.p,
                                                       nbCol.p, partJ.p);
     RIS_CHECK_LAUNCH();
     const long long cnt = (long long)ns * 3 * nn * nU;
@@ -2995,7 +3035,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
                                   8.0 * (nsu * (double)nn * nn + 3.0 * nsu * nn * nU));
   // exchange part: pairs in batches sharing one pass over the derivative
   // integrals; G^K[mu][nu][P < nK] and Omega are formed per pair
-  const int NB = std::min(npair, kCBatch);
+  const int NB = cdiv(npair, cdiv(npair, kCBatch));  // pairs per batch
   const size_t gk = (size_t)nn * nn * nK;
   // G^K in FP32 when every term of it comes from the tensor cores (mixed TDA)
   const bool gk32 = mixed && !rpa;
@@ -3126,13 +3166,13 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
     prof_begin(kProfContract, st);
     const dim3 gridK(cdiv((long long)nn * nK, 128), slK);
     if (gk32)
-      k_contract_exchange<float, float><<<gridK, 128, 0, st>>>(Df.p, GK32.p, nb, nn, nU, nK, slK,
+      contract_exchange<float, float>(gridK, st, Df.p, GK32.p, nb, nn, nU, nK, slK,
                                                               nbPtr.p, nbCol.p, partK.p);
     else if (mixed)
-      k_contract_exchange<float, double><<<gridK, 128, 0, st>>>(Df.p, GK.p, nb, nn, nU, nK, slK,
+      contract_exchange<float, double>(gridK, st, Df.p, GK.p, nb, nn, nU, nK, slK,
                                                                nbPtr.p, nbCol.p, partK.p);
     else
-      k_contract_exchange<double, double><<<gridK, 128, 0, st>>>(D.p, GK.p, nb, nn, nU, nK, slK,
+      contract_exchange<double, double>(gridK, st, D.p, GK.p, nb, nn, nU, nK, slK,
                                                                 nbPtr.p, nbCol.p, partK.p);
     RIS_CHECK_LAUNCH();
     const long long cntK = (long long)nb * 3 * nn * nK;
@@ -3682,14 +3722,14 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
   k_symmetrize_sq<<<cdiv((long long)nsu * nn * nn, 256), 256, 0, st>>>(DR.p, nn, nsu);
   RIS_CHECK_LAUNCH();
   // state densities regrouped [batch][mu][nu][b] for the contraction
-  const int nbat = cdiv(nsu, kCBatch);
+  const int nbat = cdiv(nsu, kCBatch), per = cdiv(nsu, nbat);  // states per batch
   const size_t dtb = (size_t)nn * nn * kCBatch;
   SBuf<double> DRd(mixed ? 1 : nbat * dtb, st);
   if (mixed) {
     DRf.ensure(nbat * dtb, st);
-    k_states_t<float><<<dim3(cdiv((long long)nn * nn, 256), nbat), 256, 0, st>>>(DR.p, nsu, nn, DRf.p);
+    k_states_t<float><<<dim3(cdiv((long long)nn * nn, 256), nbat), 256, 0, st>>>(DR.p, nsu, per, nn, DRf.p);
   } else {
-    k_states_t<double><<<dim3(cdiv((long long)nn * nn, 256), nbat), 256, 0, st>>>(DR.p, nsu, nn, DRd.p);
+    k_states_t<double><<<dim3(cdiv((long long)nn * nn, 256), nbat), 256, 0, st>>>(DR.p, nsu, per, nn, DRd.p);
   }
   RIS_CHECK_LAUNCH();
   SBuf<double> cU((size_t)nsu * nU, st, true);
@@ -3703,7 +3743,7 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
     LiTl.ensure((size_t)nK * ldK, st, true);
     split_f64_t(LKinv.p, nK, nK, nK, LiTh.p, LiTl.p, ldK, st);
   }
-  const int NB = std::min(npair, kCBatch);
+  const int NB = cdiv(npair, cdiv(npair, kCBatch));
   int wmaxU = 1, wmaxK = 1;
   for (size_t k = 0; k < blkW.size(); k++) {
     wmaxU = std::max(wmaxU, blkW[k]);
@@ -3800,15 +3840,15 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
       prof_begin(kProfContract, st);
       double bytes = 0.0;
       if (g0 == 0) {  // Coulomb part: Y_s[x][mu][u0 + p] for every state
-        for (int s0 = 0; s0 < nsu; s0 += kCBatch) {
-          const int ns = std::min(kCBatch, nsu - s0);
+        for (int s0 = 0; s0 < nsu; s0 += per) {
+          const int ns = std::min(per, nsu - s0);
           const dim3 grid(cdiv((long long)nn * w, 128), slJ);
-          const size_t bo = (size_t)(s0 / kCBatch) * dtb;
+          const size_t bo = (size_t)(s0 / per) * dtb;
           if (mixed)
-            k_contract_states<float><<<grid, 128, 0, st>>>(D32.p, DRf.p + bo, ns, nn, w, slJ, nbPtr.p,
+            contract_states<float>(grid, st, D32.p, DRf.p + bo, ns, nn, w, slJ, nbPtr.p,
                                                            nbCol.p, partJ.p);
           else
-            k_contract_states<double><<<grid, 128, 0, st>>>(D64.p, DRd.p + bo, ns, nn, w, slJ, nbPtr.p,
+            contract_states<double>(grid, st, D64.p, DRd.p + bo, ns, nn, w, slJ, nbPtr.p,
                                                             nbCol.p, partJ.p);
           RIS_CHECK_LAUNCH();
           const long long rows = (long long)ns * 3 * nn;
@@ -3872,10 +3912,10 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
         }
         const dim3 gridK(cdiv((long long)nn * wK, 128), slK);
         if (mixed)
-          k_contract_exchange<float, float><<<gridK, 128, 0, st>>>(D32.p, Gam32.p, nb, nn, w, wK, slK,
+          contract_exchange<float, float>(gridK, st, D32.p, Gam32.p, nb, nn, w, wK, slK,
                                                                    nbPtr.p, nbCol.p, partK.p);
         else
-          k_contract_exchange<double, double><<<gridK, 128, 0, st>>>(D64.p, Gam64.p, nb, nn, w, wK, slK,
+          contract_exchange<double, double>(gridK, st, D64.p, Gam64.p, nb, nn, w, wK, slK,
                                                                      nbPtr.p, nbCol.p, partK.p);
         RIS_CHECK_LAUNCH();
         const long long rows = (long long)nb * 3 * nn;
