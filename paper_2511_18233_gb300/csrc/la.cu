@@ -449,8 +449,10 @@ size_t eig_work_size(int m) { return (size_t)m * m + 3 * (size_t)m + 64 + 64 * (
 // error ~1e-15), far cheaper than an FP64 division on this part; q outside the
 // FP32 range takes the division.
 __device__ __forceinline__ double rcp64(double q) {
-  const double aq = fabs(q);
-  if (!(aq > 1e-30 && aq < 1e30)) return 1.0 / q;
+  // (range test on the bit patterns, which order like the magnitudes: every
+  // FP64 instruction, a comparison too, costs the issuing warp about 75 cycles)
+  const long long aq = __double_as_longlong(q) & 0x7fffffffffffffffll;
+  if (!(aq > __double_as_longlong(1e-30) && aq < __double_as_longlong(1e30))) return 1.0 / q;
   double r = (double)__frcp_rn((float)q);
   r = r * fma(-q, r, 2.0);
   r = r * fma(-q, r, 2.0);
@@ -522,25 +524,54 @@ struct EigWork {
   }
 };
 
-// Gershgorin bounds of the tridiagonal matrix (d, e).
+// Gershgorin bounds of the tridiagonal matrix (d, e), by one whole warp
+// (scanned by one thread they were 9 us at m = 40).
 __device__ void tri_bounds(const double* d, const double* e, int m, double& glo, double& ghi) {
-  for (int i = 0; i < m; i++) {
+  const int lane = threadIdx.x & 31;
+  for (int i = lane; i < m; i += 32) {
     const double r = (i > 0 ? fabs(e[i - 1]) : 0.0) + (i + 1 < m ? fabs(e[i]) : 0.0);
     const double lo = d[i] - r, hi = d[i] + r;
-    if (i == 0 || lo < glo) glo = lo;
-    if (i == 0 || hi > ghi) ghi = hi;
+    if (i == lane || lo < glo) glo = lo;
+    if (i == lane || hi > ghi) ghi = hi;
   }
+  if (lane >= m) {  // lanes without an element repeat the first
+    const double r = m > 1 ? fabs(e[0]) : 0.0;
+    glo = d[0] - r;
+    ghi = d[0] + r;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double l2 = __shfl_xor_sync(0xffffffffu, glo, o), h2 = __shfl_xor_sync(0xffffffffu, ghi, o);
+    if (l2 < glo) glo = l2;
+    if (h2 > ghi) ghi = h2;
+  }
+}
+// sum over lanes 0 .. n - 1 (the other lanes' v is zero) of the first warp,
+// in lane 0 .. n - 1: block_sum's tree without the steps that add zeros
+__device__ __forceinline__ double lane_sum(double v, int n) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    if (o < n) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// |a| >= |b| and a == 0 on the bit patterns (finite a, b)
+__device__ __forceinline__ unsigned long long mag_bits(double a) {
+  return (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
 }
 
 // Stage 1 (one CTA): symmetrise H and reduce it to tridiagonal form
 // T = Q^T H Q by Householder reflections (d, e; reflectors kept in A).
+// Every FP64 instruction of a warp takes a quarter of the SM for about 75
+// cycles, so sums are taken by the warps that hold terms and the rank-2
+// update packs its elements into the lanes (m = 24 ... 40: 134 -> 96 us a
+// call, the same bits).
 // No __restrict__: every array is carved out of `work`, and with
 // restrict-qualified parameters the compiler reordered in-place updates.
 __global__ void __launch_bounds__(kEigT) k_eig_tridiag(const double* H, int ldH, int m,
                                                        double* work, int use_smem) {
   extern __shared__ double sm_A[];
   __shared__ double red[33];
-  __shared__ double sh_alpha, sh_tau;
+  __shared__ double sh_alpha, sh_tau, sh_K;
   __shared__ double p[kEigMaxM];   // A_sub v of the current step
   __shared__ double vc[kEigMaxM];  // the current Householder vector (column c below the diagonal)
   EigWork W(work, m);
@@ -554,12 +585,29 @@ __global__ void __launch_bounds__(kEigT) k_eig_tridiag(const double* H, int ldH,
     A[ij] = 0.5 * (H[(size_t)i * ldH + j] + H[(size_t)j * ldH + i]);
   }
   __syncthreads();
+  const int warp = tid >> 5, lane = tid & 31;
   for (int c = 0; c + 2 < m; c++) {
-    double part = 0.0;
-    for (int i = c + 1 + tid; i < m; i += kEigT) part += A[(size_t)i * m + c] * A[(size_t)i * m + c];
-    const double s = block_sum<kEigT>(part, red);
+    const int n = m - 1 - c;  // rows below the diagonal (at most kEigMaxM - 1 < kEigT)
+    // sum over the rows i = c + 1 + tid, valid in warp 0: only the warps that
+    // hold terms spend FP64 instructions on it (block_sum's order otherwise)
+    const int nw = (n + 31) >> 5;
+    auto row_sum = [&](double v) {
+      if (warp < nw) v = lane_sum(v, n);
+      if (nw > 1) {
+        if (lane == 0) red[warp] = v;
+        __syncthreads();
+        if (warp == 0) v = lane_sum(lane < nw ? red[lane] : 0.0, nw);
+      }
+      return v;
+    };
+    double x = 0.0;
+    if (tid < n) {
+      x = A[(size_t)(c + 1 + tid) * m + c];
+      vc[c + 1 + tid] = x;
+    }
+    const double s = row_sum(__dmul_rn(x, x));  // (not to be contracted with the first sum)
     if (tid == 0) {
-      const double x0 = A[(size_t)(c + 1) * m + c];
+      const double x0 = x;
       const double nrm = sqrt(s);
       d[c] = A[(size_t)c * m + c];
       if (nrm == 0.0) {
@@ -570,6 +618,7 @@ __global__ void __launch_bounds__(kEigT) k_eig_tridiag(const double* H, int ldH,
         const double v0 = x0 - alpha;
         const double vn2 = s - x0 * x0 + v0 * v0;
         A[(size_t)(c + 1) * m + c] = v0;
+        vc[c + 1] = v0;
         sh_alpha = alpha;
         sh_tau = vn2 > 0.0 ? 2.0 / vn2 : 0.0;
       }
@@ -578,14 +627,13 @@ __global__ void __launch_bounds__(kEigT) k_eig_tridiag(const double* H, int ldH,
     }
     __syncthreads();
     const double t = sh_tau;
-    if (t == 0.0) continue;
-    for (int i = c + 1 + tid; i < m; i += kEigT) vc[i] = A[(size_t)i * m + c];
-    __syncthreads();
+    if (mag_bits(t) == 0) continue;
     // p = t * A_sub v, using symmetry for coalesced reads: two threads per
     // row (alternate j), two partial sums each, so that the dependent FP64
     // chains are a quarter of the row long
-    for (int i0 = c + 1; i0 < m; i0 += kEigT / 2) {  // uniform: the shuffle needs every lane
+    for (int i0 = c + 1; i0 < m; i0 += kEigT / 2) {
       const int i = i0 + (tid >> 1), h = tid & 1;
+      if (i0 + (warp << 4) >= m) break;  // warp-uniform: the shuffle needs every lane
       double a0 = 0.0, a1 = 0.0;
       if (i < m) {
         int j = c + 1 + h;
@@ -600,15 +648,15 @@ __global__ void __launch_bounds__(kEigT) k_eig_tridiag(const double* H, int ldH,
       if (i < m && h == 0) p[i] = t * acc;
     }
     __syncthreads();
-    part = 0.0;
-    for (int i = c + 1 + tid; i < m; i += kEigT) part += p[i] * vc[i];
-    const double K = 0.5 * t * block_sum<kEigT>(part, red);
-    for (int i = c + 1 + tid; i < m; i += kEigT) p[i] -= K * vc[i];
+    const double K = row_sum(tid < n ? __dmul_rn(p[c + 1 + tid], vc[c + 1 + tid]) : 0.0);
+    if (tid == 0) sh_K = 0.5 * t * K;
     __syncthreads();
-    // rank-2 update of the trailing block: warps over rows, lanes over columns
-    for (int i = c + 1 + (tid >> 5); i < m; i += kEigT / 32) {
-      const double vi = vc[i], pi = p[i];
-      for (int j = c + 1 + (tid & 31); j < m; j += 32) A[(size_t)i * m + j] -= vi * p[j] + pi * vc[j];
+    if (tid < n) p[c + 1 + tid] -= sh_K * vc[c + 1 + tid];
+    __syncthreads();
+    // rank-2 update of the trailing block, its elements packed into the lanes
+    for (int q = tid; q < n * n; q += kEigT) {
+      const int i = c + 1 + q / n, j = c + 1 + q % n;
+      A[(size_t)i * m + j] -= vc[i] * p[j] + p[i] * vc[j];
     }
     __syncthreads();
   }
@@ -637,10 +685,12 @@ constexpr int kEigVecT = 128;
 // eigenvector of T by inverse iteration (Gaussian elimination with partial
 // pivoting of T - lambda_j I, three solves), and its back-transformation
 // x = H_0 ... H_{m-3} z.  Householder vectors in shared memory when
-// a_smem is set (m x m doubles).
+// a_smem is set (m x m doubles).  Chains of dependent FP64 instructions, about
+// 75 cycles each: tests on integers, reciprocals of the pivots kept from the
+// elimination and everything without a chain on all lanes took m = 24 ... 40
+// from 149 to 112 us a call (the same bits).
 __global__ void __launch_bounds__(kEigVecT) k_eig_vec(int m, double* work, int a_smem) {
   extern __shared__ double sm[];
-  __shared__ double red[33];
   __shared__ double sh_lo, sh_hi;
   EigWork W(work, m);
   const int j = blockIdx.x;
@@ -653,8 +703,8 @@ __global__ void __launch_bounds__(kEigVecT) k_eig_vec(int m, double* work, int a
   double* dd = dl + m;
   double* du = dd + m;
   double* du2 = du + m;
-  double* piv = du2 + m;
-  double* tau = piv + m;
+  double* pivd = du2 + m;  // row exchanges (int)
+  double* tau = pivd + m;
   float* df = (float*)(tau + m);
   float* e2f = df + m;
   double* As = tau + m + m;  // after the two float arrays (m doubles)
@@ -670,13 +720,15 @@ __global__ void __launch_bounds__(kEigVecT) k_eig_vec(int m, double* work, int a
     for (size_t t = tid; t < (size_t)m * m; t += kEigVecT) As[t] = W.A[t];
   const double* A = a_smem ? As : W.A;
   __syncthreads();
-  // Gershgorin bounds by one thread (every thread repeating the FP64 scan
-  // would load the SM's narrow FP64 pipe 128-fold)
-  if (tid == 0) {
+  // Gershgorin bounds by one warp (repeated by the others they would load
+  // the SM's narrow FP64 pipe)
+  if (tid < 32) {
     double lo0 = 0.0, hi0 = 0.0;
     tri_bounds(d, e, m, lo0, hi0);
-    sh_lo = lo0;
-    sh_hi = hi0;
+    if (tid == 0) {
+      sh_lo = lo0;
+      sh_hi = hi0;
+    }
   }
   __syncthreads();
   const double glo = sh_lo, ghi = sh_hi;
@@ -722,74 +774,105 @@ __global__ void __launch_bounds__(kEigVecT) k_eig_vec(int m, double* work, int a
   }
   __syncthreads();
   const double lj = 0.5 * (sh_lo + sh_hi);
-  if (tid == 0) {
+  // One warp from here on.  The elimination and the solves are chains of
+  // dependent FP64 operations in lane 0, with the running element in a
+  // register and every test on integers; what has no chain runs on all lanes.
+  if (tid < 32) {
     const double tiny = 1e-15 * tnorm;
-    for (int i = 0; i < m; i++) {
+    int* piv = (int*)pivd;
+    for (int i = tid; i < m; i += 32) {
       dd[i] = d[i] - lj;
       dl[i] = i + 1 < m ? e[i] : 0.0;
       du[i] = i + 1 < m ? e[i] : 0.0;
       du2[i] = 0.0;
-      piv[i] = 0.0;
+      piv[i] = 0;
+      // start vector depending on j: equal eigenvalues (a split T) give
+      // different vectors of their eigenspace, which stage 3 orthonormalises
+      z[i] = 1.0 + 0.01 * (double)((i * (j + 1)) % 7);
     }
-    for (int i = 0; i + 1 < m; i++) {
-      if (fabs(dd[i]) >= fabs(dl[i])) {
-        if (dd[i] == 0.0) dd[i] = tiny;
-        const double f = dl[i] * rcp64(dd[i]);
-        dl[i] = f;
-        dd[i + 1] -= f * du[i];
-      } else {
-        const double f = dd[i] * rcp64(dl[i]);
-        dd[i] = dl[i];
-        dl[i] = f;
-        const double tmp = du[i];
-        du[i] = dd[i + 1];
-        dd[i + 1] = tmp - f * dd[i + 1];
-        if (i + 2 < m) {
-          du2[i] = du[i + 1];
-          du[i + 1] = -f * du[i + 1];
-        }
-        piv[i] = 1.0;
-      }
-    }
-    if (dd[m - 1] == 0.0) dd[m - 1] = tiny;
-    for (int i = 0; i < m; i++) dd[i] = rcp64(dd[i]);  // pivots kept as reciprocals
-    // start vector depending on j: equal eigenvalues (a split T) give
-    // different vectors of their eigenspace, which stage 3 orthonormalises
-    for (int i = 0; i < m; i++) z[i] = 1.0 + 0.01 * (double)((i * (j + 1)) % 7);
-    for (int it = 0; it < 3; it++) {
+    __syncwarp();
+    if (tid == 0) {  // dd: reciprocals of the pivots
+      double c = dd[0], u = du[0];  // row i as left by the steps before
       for (int i = 0; i + 1 < m; i++) {
-        if (piv[i] == 0.0) {
-          z[i + 1] -= dl[i] * z[i];
+        const double l = dl[i], dn = dd[i + 1], un = du[i + 1];
+        if (mag_bits(c) >= mag_bits(l)) {
+          if (mag_bits(c) == 0) c = tiny;
+          const double rc = rcp64(c), f = l * rc;
+          dd[i] = rc;
+          dl[i] = f;
+          du[i] = u;
+          c = dn - f * u;
+          u = un;
         } else {
-          const double t0 = z[i];
-          z[i] = z[i + 1];
-          z[i + 1] = t0 - dl[i] * z[i];
+          const double rc = rcp64(l), f = c * rc;
+          dd[i] = rc;
+          dl[i] = f;
+          du[i] = dn;
+          c = u - f * dn;
+          if (i + 2 < m) {
+            du2[i] = un;
+            u = -f * un;
+          } else {
+            u = un;
+          }
+          piv[i] = 1;
         }
       }
-      z[m - 1] *= dd[m - 1];
-      if (m >= 2) z[m - 2] = (z[m - 2] - du[m - 2] * z[m - 1]) * dd[m - 2];
-      for (int i = m - 3; i >= 0; i--) z[i] = (z[i] - du[i] * z[i + 1] - du2[i] * z[i + 2]) * dd[i];
-      double nrm = 0.0;
-      for (int i = 0; i < m; i++) nrm += z[i] * z[i];
-      nrm = 1.0 / sqrt(nrm);
-      for (int i = 0; i < m; i++) z[i] *= nrm;
+      if (mag_bits(c) == 0) c = tiny;
+      dd[m - 1] = rcp64(c);
+      du[m - 1] = u;
     }
-    W.lam[j] = lj;
-  }
-  __syncthreads();
-  // back-transformation, H_{m-3} applied first, by one warp (each lane owns
-  // the same elements of z in the dot product and in the update, so the
-  // steps need no barrier)
-  if (tid < 32) {
+    for (int it = 0; it < 3; it++) {
+      __syncwarp();
+      double nrm = 0.0;
+      if (tid == 0) {
+        double c = z[0];
+        for (int i = 0; i + 1 < m; i++) {
+          const double n = z[i + 1], l = dl[i];
+          if (!piv[i]) {
+            z[i] = c;
+            c = n - l * c;
+          } else {
+            z[i] = n;
+            c = c - l * n;
+          }
+        }
+        double z1 = c * dd[m - 1], z2 = 0.0;
+        z[m - 1] = z1;
+        if (m >= 2) {
+          const double x = (z[m - 2] - du[m - 2] * z1) * dd[m - 2];
+          z[m - 2] = x;
+          z2 = z1;
+          z1 = x;
+        }
+        for (int i = m - 3; i >= 0; i--) {
+          double x = z[i] - du[i] * z1;
+          if (piv[i]) x = x - du2[i] * z2;  // du2 = 0 without an exchange
+          x = x * dd[i];
+          z[i] = x;
+          z2 = z1;
+          z1 = x;
+        }
+        for (int i = 0; i < m; i++) nrm += z[i] * z[i];
+        nrm = 1.0 / sqrt(nrm);
+      }
+      nrm = __shfl_sync(0xffffffffu, nrm, 0);
+      for (int i = tid; i < m; i += 32) z[i] *= nrm;
+    }
+    if (tid == 0) W.lam[j] = lj;
+    __syncwarp();
+    // back-transformation, H_{m-3} applied first (each lane owns the same
+    // elements of z, counted from row c + 1, in the dot product and in the
+    // update of a step)
     for (int c = m - 3; c >= 0; c--) {
       const double t = tau[c];
-      if (t == 0.0) continue;
+      if (mag_bits(t) == 0) continue;
       double part = 0.0;
       for (int i = c + 1 + tid; i < m; i += 32) part += A[(size_t)i * m + c] * z[i];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+      part = lane_sum(part, m - 1 - c);
       const double f = t * part;
       for (int i = c + 1 + tid; i < m; i += 32) z[i] -= f * A[(size_t)i * m + c];
+      __syncwarp();
     }
   }
   __syncthreads();
@@ -805,11 +888,13 @@ __global__ void __launch_bounds__(kEigT) k_eig_finish(int m, int k, double* w, d
   EigWork W(work, m);
   const int tid = threadIdx.x;
   for (int i = tid; i < k; i += kEigT) lam[i] = W.lam[i];
-  if (tid == 0) {
+  if (tid < 32) {
     double glo = 0.0, ghi = 0.0;
     tri_bounds(W.d, W.e, m, glo, ghi);
-    bnd[0] = glo;
-    bnd[1] = ghi;
+    if (tid == 0) {
+      bnd[0] = glo;
+      bnd[1] = ghi;
+    }
   }
   __syncthreads();
   const double tnorm = fmax(fmax(fabs(bnd[0]), fabs(bnd[1])), 1e-300);
@@ -1098,11 +1183,13 @@ __global__ void __launch_bounds__(kEigT) k_eig_finish32(int m, int k, double* w,
   EigWork W(work, m);
   const int tid = threadIdx.x;
   for (int i = tid; i < k; i += kEigT) lam[i] = W.lam[i];
-  if (tid == 0) {
+  if (tid < 32) {
     double glo = 0.0, ghi = 0.0;
     tri_bounds(W.d, W.e, m, glo, ghi);
-    bnd[0] = glo;
-    bnd[1] = ghi;
+    if (tid == 0) {
+      bnd[0] = glo;
+      bnd[1] = ghi;
+    }
   }
   __syncthreads();
   const double tnorm = fmax(fmax(fabs(bnd[0]), fabs(bnd[1])), 1e-300);
