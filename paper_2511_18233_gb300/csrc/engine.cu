@@ -589,11 +589,21 @@ __global__ void __launch_bounds__(32) k_cholqr_small(const double* G, int nt, do
 
 // FP64 GEMM, or the double-FP32 one (gemm_ff.cu) when ff is set and the
 // shape is one of its skinny forms.
-static void gemm_sub(bool ff, bool ta, bool tb, int m, int n, int k, double alpha, const double* A,
-                     int lda, const double* B, int ldb, double beta, double* C, int ldc,
-                     cudaStream_t st) {
+void Engine::gemm_sub(bool ff, bool ta, bool tb, int m, int n, int k, double alpha, const double* A,
+                      int lda, const double* B, int ldb, double beta, double* C, int ldc,
+                      cudaStream_t st) {
   if (!(ff && ffgemm(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, st)))
-    dgemm(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, st);
+    gemm(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, st);
+}
+
+// The FP64 form splits short contractions finely.  The mixed form keeps
+// slices of 256 and more: its Davidson stops at a residual of 1e-6, so that
+// another summation order would move its vectors by 1e-5.
+void Engine::gemm(bool ta, bool tb, int m, int n, int k, double alpha, const double* A, int lda,
+                  const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s,
+                  GemmBatch bt) {
+  bt.fine = opt.precision == RIS_FP64;
+  dgemm(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, s, bt);
 }
 
 static void cholqr_small(const double* G, int nt, double drop, double* P, int* nkeep,
@@ -1484,12 +1494,12 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   if (emuJ) {
     coulomb_emu(fJ, w2.p, w3.p);
   } else {
-    dgemm(true, false, o, n * nJ, n, 1.0, Co, nmo, TJ.p, n * nJ, 0.0, w2.p, n * nJ, st);
+    gemm(true, false, o, n * nJ, n, 1.0, Co, nmo, TJ.p, n * nJ, 0.0, w2.p, n * nJ, st);
     GemmBatch bt;
     bt.nb1 = o;
     bt.sB1 = (long long)n * nJ;
     bt.sC1 = (long long)v * nJ;
-    dgemm(true, false, v, nJ, n, 1.0, Cv, nmo, w2.p, nJ, 0.0, w3.p, nJ, st, bt);
+    gemm(true, false, v, nJ, n, 1.0, Cv, nmo, w2.p, nJ, 0.0, w3.p, nJ, st, bt);
   }
   BJ.ensure((size_t)nov * nJ, st);
   if (emuJ) {  // B[(i,a)][R] = sum_P W[(i,a)][P] L_J^-1[R][P]
@@ -1497,7 +1507,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     e.c64 = BJ.p; e.rs = nJ; e.cs = 1;
     emu_abt(fJ, (int)nov, nJ, nJ, w3.p, nJ, 1, LJinv.p, nJ, 1, e);
   } else {
-    dgemm(false, true, (int)nov, nJ, nJ, 1.0, w3.p, nJ, LJinv.p, nJ, 0.0, BJ.p, nJ, st);
+    gemm(false, true, (int)nov, nJ, nJ, 1.0, w3.p, nJ, LJinv.p, nJ, 0.0, BJ.p, nJ, st);
   }
   // exchange: oo and ov from C_o^T T^K, vv from C_v^T T^K
   const double* HK = w2.p;
@@ -1509,7 +1519,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     RIS_CHECK_LAUNCH();
     HK = w5.p;
   } else {
-    dgemm(true, false, o, n * nK, n, 1.0, Co, nmo, TK.p, n * nK, 0.0, w2.p, n * nK, st);
+    gemm(true, false, o, n * nK, n, 1.0, Co, nmo, TK.p, n * nK, 0.0, w2.p, n * nK, st);
   }
   release_emu_ops();
   if (emu_exchange()) {
@@ -1525,22 +1535,22 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     bt.nb1 = o;
     bt.sB1 = (long long)n * nK;
     bt.sC1 = (long long)o * nK;
-    dgemm(true, false, o, nK, n, 1.0, Co, nmo, HK, nK, 0.0, w3.p, nK, st, bt);
+    gemm(true, false, o, nK, n, 1.0, Co, nmo, HK, nK, 0.0, w3.p, nK, st, bt);
   }
   BKoo.ensure((size_t)o * o * nK, st);
-  dgemm(false, true, o * o, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, BKoo.p, nK, st);
+  gemm(false, true, o * o, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, BKoo.p, nK, st);
   cKoo.ensure((size_t)o * o * nK, st);
-  dgemm(false, false, o * o, nK, nK, 1.0, BKoo.p, nK, LKinv.p, nK, 0.0, cKoo.p, nK, st);
+  gemm(false, false, o * o, nK, nK, 1.0, BKoo.p, nK, LKinv.p, nK, 0.0, cKoo.p, nK, st);
   if (opt.rpa) {
     GemmBatch bt;
     bt.nb1 = o;
     bt.sB1 = (long long)n * nK;
     bt.sC1 = (long long)v * nK;
-    dgemm(true, false, v, nK, n, 1.0, Cv, nmo, HK, nK, 0.0, w3.p, nK, st, bt);
+    gemm(true, false, v, nK, n, 1.0, Cv, nmo, HK, nK, 0.0, w3.p, nK, st, bt);
     w4.ensure((size_t)nov * nK, st);
-    dgemm(false, true, (int)nov, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, w4.p, nK, st);  // [i][a][R]
+    gemm(false, true, (int)nov, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, w4.p, nK, st);  // [i][a][R]
     cKov.ensure((size_t)nov * nK, st);
-    dgemm(false, false, (int)nov, nK, nK, 1.0, w4.p, nK, LKinv.p, nK, 0.0, cKov.p, nK, st);
+    gemm(false, false, (int)nov, nK, nK, 1.0, w4.p, nK, LKinv.p, nK, 0.0, cKov.p, nK, st);
     BKovR.ensure((size_t)nov * nK, st);
     transpose_last2(w4.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]
     cKovP.ensure((size_t)nov * nK, st);
@@ -1551,14 +1561,14 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     build_Kvv_tc(w4.p);  // B[a][b][R]
   } else {
     w2.ensure((size_t)v * n * nK, st);
-    dgemm(true, false, v, n * nK, n, 1.0, Cv, nmo, TK.p, n * nK, 0.0, w2.p, n * nK, st);
+    gemm(true, false, v, n * nK, n, 1.0, Cv, nmo, TK.p, n * nK, 0.0, w2.p, n * nK, st);
     w3.ensure((size_t)v * v * nK, st);
     GemmBatch bt;
     bt.nb1 = v;
     bt.sB1 = (long long)n * nK;
     bt.sC1 = (long long)v * nK;
-    dgemm(true, false, v, nK, n, 1.0, Cv, nmo, w2.p, nK, 0.0, w3.p, nK, st, bt);
-    dgemm(false, true, v * v, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, w4.p, nK, st);  // B[a][b][R]
+    gemm(true, false, v, nK, n, 1.0, Cv, nmo, w2.p, nK, 0.0, w3.p, nK, st, bt);
+    gemm(false, true, v * v, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, w4.p, nK, st);  // B[a][b][R]
   }
   cKvv.ensure((size_t)v * v * nK, st);
   if (emu) {  // c[(a,b)][Q] = sum_R B[(a,b)][R] L_K^-1[R][Q]
@@ -1566,7 +1576,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     e.c64 = cKvv.p; e.rs = nK; e.cs = 1;
     emu_abt(kEmu10x6, v * v, nK, nK, w4.p, nK, 1, LKinv.p, 1, nK, e);
   } else {
-    dgemm(false, false, v * v, nK, nK, 1.0, w4.p, nK, LKinv.p, nK, 0.0, cKvv.p, nK, st);
+    gemm(false, false, v * v, nK, nK, 1.0, w4.p, nK, LKinv.p, nK, 0.0, cKvv.p, nK, st);
   }
   BKvvD.ensure((size_t)v * v * nK, st);
   transpose_last2(w4.p, v, v, nK, BKvvD.p, st);  // [b][R][a]
@@ -2020,8 +2030,8 @@ void Engine::apply_A_tda(const double* Xin, int nvec, double* out) {
   const int o = nocc, v = nvir;
   const long long nov = (long long)o * v;
   w5.ensure((size_t)nvec * std::max(nJ, 1), st);
-  dgemm(false, false, nvec, nJ, (int)nov, 1.0, Xin, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
-  dgemm(false, true, nvec, (int)nov, nJ, 2.0, w5.p, nJ, BJ.p, nJ, 0.0, out, (int)nov, st);
+  gemm(false, false, nvec, nJ, (int)nov, 1.0, Xin, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
+  gemm(false, true, nvec, (int)nov, nJ, 2.0, w5.p, nJ, BJ.p, nJ, 0.0, out, (int)nov, st);
   if (emu_exchange()) {
     exchange_emu(Xin, nvec, out, -opt.cx, 1.0, nullptr);
     k_add_diag<<<cdiv(nov * nvec, 256), 256, 0, st>>>(de.p, Xin, nov, nvec, out);
@@ -2034,14 +2044,14 @@ void Engine::apply_A_tda(const double* Xin, int nvec, double* out) {
     bt.nb1 = nvec;
     bt.sA1 = nov;
     bt.sC1 = (long long)o * nK * v;
-    dgemm(false, false, o, nK * v, v, 1.0, Xin, v, BKvvD.p, nK * v, 0.0, w6.p, nK * v, st, bt);
+    gemm(false, false, o, nK * v, v, 1.0, Xin, v, BKvvD.p, nK * v, 0.0, w6.p, nK * v, st, bt);
   }
   {
     GemmBatch bt;
     bt.nb1 = nvec;
     bt.sB1 = (long long)o * nK * v;
     bt.sC1 = nov;
-    dgemm(false, false, o, v, o * nK, -opt.cx, BKoo.p, o * nK, w6.p, v, 1.0, out, v, st, bt);
+    gemm(false, false, o, v, o * nK, -opt.cx, BKoo.p, o * nK, w6.p, v, 1.0, out, v, st, bt);
   }
   k_add_diag<<<cdiv(nov * nvec, 256), 256, 0, st>>>(de.p, Xin, nov, nvec, out);
   RIS_CHECK_LAUNCH();
@@ -2087,12 +2097,12 @@ void Engine::exchange_terms(const double* Z, int nvec, double* K1, double* K2, b
     bt.nb1 = nvec;
     bt.sA1 = nov;
     bt.sC1 = (long long)o * nK * v;
-    dgemm(false, false, o, nK * v, v, 1.0, Z, v, BKvvD.p, nK * v, 0.0, w6.p, nK * v, st, bt);
+    gemm(false, false, o, nK * v, v, 1.0, Z, v, BKvvD.p, nK * v, 0.0, w6.p, nK * v, st, bt);
     GemmBatch b2;
     b2.nb1 = nvec;
     b2.sB1 = (long long)o * nK * v;
     b2.sC1 = nov;
-    dgemm(false, false, o, v, o * nK, 1.0, BKoo.p, o * nK, w6.p, v, 0.0, K1, v, st, b2);
+    gemm(false, false, o, v, o * nK, 1.0, BKoo.p, o * nK, w6.p, v, 0.0, K1, v, st, b2);
   }
   // Y1[n][i][R][j] = sum_b B^K_ib,R Z_n[j][b];  K2_n = Y1_n . B^K as [(R,j)][a]
   SBuf<double> Y1((size_t)nvec * o * nK * o, st);
@@ -2105,20 +2115,20 @@ void Engine::exchange_terms(const double* Z, int nvec, double* K1, double* K2, b
   bt.sB2 = 0;
   bt.sC1 = (long long)o * nK * o;
   bt.sC2 = o;
-  dgemm(false, true, o, o, v, 1.0, BKovR.p, v, Z, v, 0.0, Y1.p, nK * o, st, bt);
+  gemm(false, true, o, o, v, 1.0, BKovR.p, v, Z, v, 0.0, Y1.p, nK * o, st, bt);
   GemmBatch b2;
   b2.nb1 = nvec;
   b2.sA1 = (long long)o * nK * o;
   b2.sC1 = nov;
-  dgemm(false, false, o, v, nK * o, 1.0, Y1.p, nK * o, BKovR.p, v, 0.0, K2, v, st, b2);
+  gemm(false, false, o, v, nK * o, 1.0, Y1.p, nK * o, BKovR.p, v, 0.0, K2, v, st, b2);
 }
 
 void Engine::apply_ApB_AmB(const double* Z, int nvec, double* outP, double* outM) {
   const long long nov = (long long)nocc * nvir;
   const bool mixed = opt.precision == RIS_MIXED;
   w5.ensure((size_t)nvec * std::max(nJ, 1), st);
-  dgemm(false, false, nvec, nJ, (int)nov, 1.0, Z, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
-  dgemm(false, true, nvec, (int)nov, nJ, 1.0, w5.p, nJ, BJ.p, nJ, 0.0, outP, (int)nov, st);
+  gemm(false, false, nvec, nJ, (int)nov, 1.0, Z, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
+  gemm(false, true, nvec, (int)nov, nJ, 1.0, w5.p, nJ, BJ.p, nJ, 0.0, outP, (int)nov, st);
   SBuf<double> K1((size_t)nvec * nov, st), K2((size_t)nvec * nov, st);
   exchange_terms(Z, nvec, K1.p, K2.p, mixed);
   k_rpa_combine<<<cdiv(nov * nvec, 256), 256, 0, st>>>(de.p, Z, K1.p, K2.p, nov, nvec, opt.cx, outP, outM);
@@ -2219,7 +2229,7 @@ void CoulPrecond::setup(Engine& e, bool shifted, double f_, int nmax) {
       tcg(nJ, nJ, (int)nr, capBh.p, capBl.p, lr, capWh.p, capWl.p, lr, 0, 1,
           ep_f64(cap.p, nJ, 0, f, r0 == 0 ? 0.0 : 1.0), e.d_tcerr, st);
     } else {
-      dgemm(true, false, nJ, nJ, (int)nr, f, e.BJ.p + (size_t)r0 * nJ, nJ, W.p, nJ, r0 == 0 ? 0.0 : 1.0,
+      e.gemm(true, false, nJ, nJ, (int)nr, f, e.BJ.p + (size_t)r0 * nJ, nJ, W.p, nJ, r0 == 0 ? 0.0 : 1.0,
             cap.p, nJ, st);
     }
   }
@@ -2227,7 +2237,7 @@ void CoulPrecond::setup(Engine& e, bool shifted, double f_, int nmax) {
   RIS_CHECK_LAUNCH();
   cholesky(cap.p, nJ, info.p, st);
   tri_inverse(cap.p, Li.p, nJ, st);
-  dgemm(true, false, nJ, nJ, nJ, 1.0, Li.p, nJ, Li.p, nJ, 0.0, capinv.p, nJ, st);
+  e.gemm(true, false, nJ, nJ, nJ, 1.0, Li.p, nJ, Li.p, nJ, 0.0, capinv.p, nJ, st);
   // mixed precision: 3xTF32 applications when the splits of B^J stay small
   // (a preconditioner only changes the number of iterations)
   tc = use_tc && (double)n * (ld4(nJ) + nJ) * 8.0 < 4.0e9;
@@ -2262,13 +2272,13 @@ void CoulPrecond::apply(Engine& e, const double* R, const int* idx, int nt, doub
     const int ln = ld4((int)n), lj = ld4(nJ);
     split_f64(T, nt, (int)n, n, Th.p, Tl.p, ln, st);
     tcg(nt, nJ, (int)n, Th.p, Tl.p, ln, BTh.p, BTl.p, ln, 0, 1, ep_f64(pY.p, nJ), e.d_tcerr, st);
-    dgemm(false, false, nt, nJ, nJ, 1.0, pY.p, nJ, capinv.p, nJ, 0.0, pZ.p, nJ, st);
+    e.gemm(false, false, nt, nJ, nJ, 1.0, pY.p, nJ, capinv.p, nJ, 0.0, pZ.p, nJ, st);
     split_f64(pZ.p, nt, nJ, nJ, Zh.p, Zl.p, lj, st);
     tcg(nt, (int)n, nJ, Zh.p, Zl.p, lj, Bh.p, Bl.p, lj, 0, 1, ep_f64(pP.p, n), e.d_tcerr, st);
   } else {
-    dgemm(false, false, nt, nJ, (int)n, 1.0, T, (int)n, e.BJ.p, nJ, 0.0, pY.p, nJ, st);
-    dgemm(false, false, nt, nJ, nJ, 1.0, pY.p, nJ, capinv.p, nJ, 0.0, pZ.p, nJ, st);
-    dgemm(false, true, nt, (int)n, nJ, 1.0, pZ.p, nJ, e.BJ.p, nJ, 0.0, pP.p, (int)n, st);
+    e.gemm(false, false, nt, nJ, (int)n, 1.0, T, (int)n, e.BJ.p, nJ, 0.0, pY.p, nJ, st);
+    e.gemm(false, false, nt, nJ, nJ, 1.0, pY.p, nJ, capinv.p, nJ, 0.0, pZ.p, nJ, st);
+    e.gemm(false, true, nt, (int)n, nJ, 1.0, pZ.p, nJ, e.BJ.p, nJ, 0.0, pP.p, (int)n, st);
   }
   k_precond_update<<<cdiv(n * nt, 256), 256, 0, st>>>(T, pP.p, dinv.p, n, nt, f);
   RIS_CHECK_LAUNCH();
@@ -2353,14 +2363,14 @@ void Engine::dav_core(int ns, const double* guess, int nguess, bool mixed, doubl
       row_norms(V.p, m, n, G0.p, st);
       k_scale_rows<<<cdiv(n * m, 256), 256, 0, st>>>(V.p, n, m, G0.p);
       RIS_CHECK_LAUNCH();
-      dgemm(false, true, m, m, (int)n, 1.0, V.p, (int)n, V.p, (int)n, 0.0, G0.p, m, st);
+      gemm(false, true, m, m, (int)n, 1.0, V.p, (int)n, V.p, (int)n, 0.0, G0.p, m, st);
       cholqr_small(G0.p, m, 1e-10, P0.p, (int*)(P0.p + m * m), st);
       int nk2 = 0;
       RIS_CUDA(cudaMemcpyAsync(&nk2, P0.p + m * m, sizeof(int), cudaMemcpyDeviceToHost, st));
       RIS_CUDA(cudaStreamSynchronize(st));
       RIS_REQUIRE(nk2 >= ns && (augment || nk2 == m), RIS_ERR_ARG,
                   "initial Davidson block is linearly dependent");
-      dgemm(false, false, nk2, (int)n, m, 1.0, P0.p, m, V.p, (int)n, 0.0, tmp.p, (int)n, st);
+      gemm(false, false, nk2, (int)n, m, 1.0, P0.p, m, V.p, (int)n, 0.0, tmp.p, (int)n, st);
       RIS_CUDA(cudaMemcpyAsync(V.p, tmp.p, sizeof(double) * nk2 * n, cudaMemcpyDeviceToDevice, st));
       m = nk2;
     }
@@ -2372,7 +2382,7 @@ void Engine::dav_core(int ns, const double* guess, int nguess, bool mixed, doubl
   }
   product(V.p, m, AV.p);
   int nprod = m;
-  dgemm(false, true, m, m, (int)n, 1.0, V.p, (int)n, AV.p, (int)n, 0.0, Hs.p, maxsp, st);
+  gemm(false, true, m, m, (int)n, 1.0, V.p, (int)n, AV.p, (int)n, 0.0, Hs.p, maxsp, st);
   std::vector<double> rn(ns);
   std::vector<double> rhist;
   bool converged = false;
@@ -2423,21 +2433,21 @@ void Engine::dav_core(int ns, const double* guess, int nguess, bool mixed, doubl
       if (s32) {
         // FP32 Ritz vectors are orthogonal only to FP32 level: orthonormalise
         // them in FP64 (CholQR) and project H on them instead of taking diag(w)
-        dgemm(false, true, keep, keep, m, 1.0, S.p, m, S.p, m, 0.0, G2.p, keep, st);
+        gemm(false, true, keep, keep, m, 1.0, S.p, m, S.p, m, 0.0, G2.p, keep, st);
         cholqr_small(G2.p, keep, 1e-10, P2.p, (int*)(P2.p + keep * keep), st);
         int nk2 = 0;
         RIS_CUDA(cudaMemcpyAsync(&nk2, P2.p + keep * keep, sizeof(int), cudaMemcpyDeviceToHost, st));
         RIS_CUDA(cudaStreamSynchronize(st));
         RIS_REQUIRE(nk2 >= ns, RIS_ERR_NOT_CONVERGED, "Davidson restart lost Ritz vectors");
         keep = nk2;
-        dgemm(false, false, keep, m, keep, 1.0, P2.p, keep, S.p, m, 0.0, S2.p, m, st);
-        dgemm(false, false, keep, m, m, 1.0, S2.p, m, Hs.p, maxsp, 0.0, T1.p, m, st);
-        dgemm(false, true, keep, keep, m, 1.0, T1.p, m, S2.p, m, 0.0, G2.p, keep, st);
+        gemm(false, false, keep, m, keep, 1.0, P2.p, keep, S.p, m, 0.0, S2.p, m, st);
+        gemm(false, false, keep, m, m, 1.0, S2.p, m, Hs.p, maxsp, 0.0, T1.p, m, st);
+        gemm(false, true, keep, keep, m, 1.0, T1.p, m, S2.p, m, 0.0, G2.p, keep, st);
         Sk = S2.p;
       }
-      dgemm(false, false, keep, (int)n, m, 1.0, Sk, m, V.p, (int)n, 0.0, tmp.p, (int)n, st);
+      gemm(false, false, keep, (int)n, m, 1.0, Sk, m, V.p, (int)n, 0.0, tmp.p, (int)n, st);
       RIS_CUDA(cudaMemcpyAsync(V.p, tmp.p, sizeof(double) * keep * n, cudaMemcpyDeviceToDevice, st));
-      dgemm(false, false, keep, (int)n, m, 1.0, Sk, m, AV.p, (int)n, 0.0, tmp.p, (int)n, st);
+      gemm(false, false, keep, (int)n, m, 1.0, Sk, m, AV.p, (int)n, 0.0, tmp.p, (int)n, st);
       RIS_CUDA(cudaMemcpyAsync(AV.p, tmp.p, sizeof(double) * keep * n, cudaMemcpyDeviceToDevice, st));
       if (s32) {
         RIS_CUDA(cudaMemcpy2DAsync(Hs.p, sizeof(double) * maxsp, G2.p, sizeof(double) * keep,
@@ -2462,12 +2472,12 @@ void Engine::dav_core(int ns, const double* guess, int nguess, bool mixed, doubl
     std::vector<double> hinfo(2 + 2 * (size_t)ns);
     row_norms(T.p, nt, n, info + 2, st);
     for (int pass = 0; pass < 2 && nkeep > 0; pass++) {
-      dgemm(false, true, nt, m, (int)n, 1.0, T.p, (int)n, V.p, (int)n, 0.0, Cc.p, m, st);
-      dgemm(false, false, nt, (int)n, m, -1.0, Cc.p, m, V.p, (int)n, 1.0, T.p, (int)n, st);
+      gemm(false, true, nt, m, (int)n, 1.0, T.p, (int)n, V.p, (int)n, 0.0, Cc.p, m, st);
+      gemm(false, false, nt, (int)n, m, -1.0, Cc.p, m, V.p, (int)n, 1.0, T.p, (int)n, st);
       row_norms(T.p, nt, n, info + 2 + ns, st);
       k_scale_rows<<<cdiv(n * nt, 256), 256, 0, st>>>(T.p, n, nt, info + 2 + ns);
       RIS_CHECK_LAUNCH();
-      dgemm(false, true, nt, nt, (int)n, 1.0, T.p, (int)n, T.p, (int)n, 0.0, G.p, nt, st);
+      gemm(false, true, nt, nt, (int)n, 1.0, T.p, (int)n, T.p, (int)n, 0.0, G.p, nt, st);
       cholqr_small(G.p, nt, drop, Pm.p, (int*)info, st, info + 1);
       RIS_CUDA(cudaMemcpyAsync(hinfo.data(), info, sizeof(double) * (2 + 2 * (size_t)ns),
                                cudaMemcpyDeviceToHost, st));
@@ -2476,7 +2486,7 @@ void Engine::dav_core(int ns, const double* guess, int nguess, bool mixed, doubl
       if (nkeep == 0) break;
       bool one_pass = mixed && pass == 0 && nkeep == nt && hinfo[1] >= 1e-4;
       for (int j = 0; j < nt && one_pass; j++) one_pass = hinfo[2 + ns + j] >= 0.25 * hinfo[2 + j];
-      dgemm(false, false, nkeep, (int)n, nt, 1.0, Pm.p, nt, T.p, (int)n, 0.0, tmp.p, (int)n, st);
+      gemm(false, false, nkeep, (int)n, nt, 1.0, Pm.p, nt, T.p, (int)n, 0.0, tmp.p, (int)n, st);
       RIS_CUDA(cudaMemcpyAsync(T.p, tmp.p, sizeof(double) * nkeep * n, cudaMemcpyDeviceToDevice, st));
       nt = nkeep;
       if (one_pass) break;
@@ -2486,7 +2496,7 @@ void Engine::dav_core(int ns, const double* guess, int nguess, bool mixed, doubl
                              cudaMemcpyDeviceToDevice, st));
     product(T.p, nt, AV.p + (size_t)m * n);
     nprod += nt;
-    dgemm(false, true, nt, m + nt, (int)n, 1.0, V.p + (size_t)m * n, (int)n, AV.p, (int)n, 0.0,
+    gemm(false, true, nt, m + nt, (int)n, 1.0, V.p + (size_t)m * n, (int)n, AV.p, (int)n, 0.0,
           Hs.p + (size_t)m * maxsp, maxsp, st);
     k_mirror<<<cdiv((long long)nt * m + 1, 256), 256, 0, st>>>(Hs.p, maxsp, m, m + nt);
     RIS_CHECK_LAUNCH();
@@ -2594,18 +2604,18 @@ void Engine::davidson_rpa(int ns) {
     int nkeep = nt;
     for (int pass = 0; pass < 2 && nkeep > 0; pass++) {
       if (m > 0) {
-        dgemm(false, true, nt, m, (int)n, 1.0, T.p, (int)n, V.p, (int)n, 0.0, Cc.p, m, st);
-        dgemm(false, false, nt, (int)n, m, -1.0, Cc.p, m, V.p, (int)n, 1.0, T.p, (int)n, st);
+        gemm(false, true, nt, m, (int)n, 1.0, T.p, (int)n, V.p, (int)n, 0.0, Cc.p, m, st);
+        gemm(false, false, nt, (int)n, m, -1.0, Cc.p, m, V.p, (int)n, 1.0, T.p, (int)n, st);
       }
       row_norms(T.p, nt, n, G.p, st);
       k_scale_rows<<<cdiv(n * nt, 256), 256, 0, st>>>(T.p, n, nt, G.p);
       RIS_CHECK_LAUNCH();
-      dgemm(false, true, nt, nt, (int)n, 1.0, T.p, (int)n, T.p, (int)n, 0.0, G.p, nt, st);
+      gemm(false, true, nt, nt, (int)n, 1.0, T.p, (int)n, T.p, (int)n, 0.0, G.p, nt, st);
       cholqr_small(G.p, nt, 1e-10, Pm.p, (int*)(Pm.p + nt * nt), st);
       RIS_CUDA(cudaMemcpyAsync(&nkeep, Pm.p + nt * nt, sizeof(int), cudaMemcpyDeviceToHost, st));
       RIS_CUDA(cudaStreamSynchronize(st));
       if (nkeep == 0) break;
-      dgemm(false, false, nkeep, (int)n, nt, 1.0, Pm.p, nt, T.p, (int)n, 0.0, tmp.p, (int)n, st);
+      gemm(false, false, nkeep, (int)n, nt, 1.0, Pm.p, nt, T.p, (int)n, 0.0, tmp.p, (int)n, st);
       RIS_CUDA(cudaMemcpyAsync(T.p, tmp.p, sizeof(double) * nkeep * n, cudaMemcpyDeviceToDevice, st));
       nt = nkeep;
     }
@@ -2613,9 +2623,9 @@ void Engine::davidson_rpa(int ns) {
   };
   auto subspace_rows = [&](int m0, int m1) {
     // rows m0..m1 of a+ and a-, mirrored
-    dgemm(false, true, m1 - m0, m1, (int)n, 1.0, V.p + (size_t)m0 * n, (int)n, PV.p, (int)n, 0.0,
+    gemm(false, true, m1 - m0, m1, (int)n, 1.0, V.p + (size_t)m0 * n, (int)n, PV.p, (int)n, 0.0,
           Ap.p + (size_t)m0 * maxsp, maxsp, st);
-    dgemm(false, true, m1 - m0, m1, (int)n, 1.0, V.p + (size_t)m0 * n, (int)n, MV.p, (int)n, 0.0,
+    gemm(false, true, m1 - m0, m1, (int)n, 1.0, V.p + (size_t)m0 * n, (int)n, MV.p, (int)n, 0.0,
           Am.p + (size_t)m0 * maxsp, maxsp, st);
     if (m0 > 0) {
       k_mirror<<<cdiv((long long)(m1 - m0) * m0 + 1, 256), 256, 0, st>>>(Ap.p, maxsp, m0, m1);
@@ -2642,8 +2652,8 @@ void Engine::davidson_rpa(int ns) {
     cholesky(Lc.p, m, d_info, st);
     int info = 0;
     RIS_CUDA(cudaMemcpyAsync(&info, d_info, sizeof(int), cudaMemcpyDeviceToHost, st));
-    dgemm(false, false, m, m, m, 1.0, Ap.p, maxsp, Lc.p, m, 0.0, Ht.p, m, st);
-    dgemm(true, false, m, m, m, 1.0, Lc.p, m, Ht.p, m, 0.0, Hm.p, m, st);
+    gemm(false, false, m, m, m, 1.0, Ap.p, maxsp, Lc.p, m, 0.0, Ht.p, m, st);
+    gemm(true, false, m, m, m, 1.0, Lc.p, m, Ht.p, m, 0.0, Hm.p, m, st);
     const int nk = std::min(m, ns);
     sym_eig_lowest(Hm.p, m, m, nk, w2.p, S.p, ework.p, st);
     RIS_CUDA(cudaStreamSynchronize(st));
@@ -2651,15 +2661,15 @@ void Engine::davidson_rpa(int ns) {
     k_rpa_omega<<<cdiv(ns * m, 256), 256, 0, st>>>(w2.p, ns, om.p, S.p, m);
     RIS_CHECK_LAUNCH();
     // R_sub = y L^T, L_sub = R_sub a+ / omega
-    dgemm(false, true, ns, m, m, 1.0, S.p, m, Lc.p, m, 0.0, Rs.p, m, st);
-    dgemm(false, false, ns, m, m, 1.0, Rs.p, m, Ap.p, maxsp, 0.0, Ls.p, m, st);
+    gemm(false, true, ns, m, m, 1.0, S.p, m, Lc.p, m, 0.0, Rs.p, m, st);
+    gemm(false, false, ns, m, m, 1.0, Rs.p, m, Ap.p, maxsp, 0.0, Ls.p, m, st);
     k_rowcomb<<<cdiv((long long)ns * m, 256), 256, 0, st>>>(Ls.p, nullptr, om.p, 1.0, 0.0, -1, m, ns, Ls.p);
     RIS_CHECK_LAUNCH();
-    dgemm(false, false, ns, (int)n, m, 1.0, Rs.p, m, V.p, (int)n, 0.0, Rf.p, (int)n, st);
-    dgemm(false, false, ns, (int)n, m, 1.0, Ls.p, m, V.p, (int)n, 0.0, Lf.p, (int)n, st);
+    gemm(false, false, ns, (int)n, m, 1.0, Rs.p, m, V.p, (int)n, 0.0, Rf.p, (int)n, st);
+    gemm(false, false, ns, (int)n, m, 1.0, Ls.p, m, V.p, (int)n, 0.0, Lf.p, (int)n, st);
     // residuals: (A+B)R - omega L and (A-B)L - omega R
-    dgemm(false, false, ns, (int)n, m, 1.0, Rs.p, m, PV.p, (int)n, 0.0, rR.p, (int)n, st);
-    dgemm(false, false, ns, (int)n, m, 1.0, Ls.p, m, MV.p, (int)n, 0.0, rL.p, (int)n, st);
+    gemm(false, false, ns, (int)n, m, 1.0, Rs.p, m, PV.p, (int)n, 0.0, rR.p, (int)n, st);
+    gemm(false, false, ns, (int)n, m, 1.0, Ls.p, m, MV.p, (int)n, 0.0, rL.p, (int)n, st);
     k_rowcomb<<<cdiv(n * ns, 256), 256, 0, st>>>(Lf.p, rR.p, om.p, -1.0, 1.0, 1, n, ns, rR.p);
     RIS_CHECK_LAUNCH();
     k_rowcomb<<<cdiv(n * ns, 256), 256, 0, st>>>(Rf.p, rL.p, om.p, -1.0, 1.0, 1, n, ns, rL.p);
@@ -2831,7 +2841,7 @@ struct GammaEmu {
       e.emu97(o * nK, n, coo.op, QT[c].op.sub((long long)sI * n8, n),
               emu_out(m + (size_t)o * nK, 1, kP));
       // Omega[P][Q] += w sum_ij c^oo_ij,P G_ij,Q   (K functions are union 0..nK-1)
-      dgemm(true, false, nK, nK, o * o, w, e.cKoo.p, nK, G.p, nK, 1.0, Om, nU, st);
+      e.gemm(true, false, nK, nK, o * o, w, e.cKoo.p, nK, G.p, nK, 1.0, Om, nU, st);
     }
     if (nc == 2) {
       const size_t oo = (size_t)o * nK, on = (size_t)o * n;
@@ -2849,7 +2859,7 @@ struct GammaEmu {
         RIS_CHECK_LAUNCH();
         k_pick_E<<<nt, 256, 0, st>>>(EE.p, o, 4 * o, 2 * c * o, nK, true, e1.p);
         RIS_CHECK_LAUNCH();
-        dgemm(false, true, nK, nK, o * o, sg * w, e2.p, o * o, e1.p, o * o, 1.0, Om, nU, st);
+        e.gemm(false, true, nK, nK, o * o, sg * w, e2.p, o * o, e1.p, o * o, 1.0, Om, nU, st);
       }
       gs.slice(f, kEmuRowsA, emu_src(EE.p, 1, nK, nK, 4LL * o * nK), (long long)o * nK, 4 * o, st);  // (k,P) over k'
       qs.slice(f, emu_cols(n), emu_src(QW.p, 1, n), n, 4 * o, st);                                     // mu over k'
@@ -2975,7 +2985,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
         r.slice(kEmu9x7, emu_cols(nsu * o), emu_src(u, v, 1), (long long)nsu * o, v, st);
         emu97(nn, nsu * o, c.op, r.op, emu_out(q, 1, nn));
       } else {
-        dgemm(false, true, nsu * o, nn, v, 1.0, u, v, Cv, nmo, 0.0, q, nn, st);
+        gemm(false, true, nsu * o, nn, v, 1.0, u, v, Cv, nmo, 0.0, q, nn, st);
       }
     }
     if (emu) {  // rows (s,nu) over i, columns mu
@@ -2987,12 +2997,12 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
       bt.nb1 = nsu;
       bt.sB1 = (long long)o * nn;
       bt.sC1 = (long long)nn * nn;
-      dgemm(false, false, nn, nn, o, 1.0, Co, nmo, QR.p, nn, 0.0, DR.p, nn, st, bt);
+      gemm(false, false, nn, nn, o, 1.0, Co, nmo, QR.p, nn, 0.0, DR.p, nn, st, bt);
     }
   }
   // u_s = R_s . B^J (nJ), c_s = u_s L^-1 (row vector)
-  dgemm(false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
-  dgemm(false, false, nsu, nJ, nJ, 1.0, w5.p, nJ, LJinv.p, nJ, 0.0, cJ.p, nJ, st);
+  gemm(false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
+  gemm(false, false, nsu, nJ, nJ, 1.0, w5.p, nJ, LJinv.p, nJ, 0.0, cJ.p, nJ, st);
   // Coulomb part of every pair density from per-state data: symmetrised
   // D^R and c^J on the union index (the contraction forms G^J on the fly)
   k_symmetrize_sq<<<cdiv((long long)nsu * nn * nn, 256), 256, 0, st>>>(DR.p, nn, nsu);
@@ -3098,18 +3108,18 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
         const double* QU = (cmb == 0 ? QR.p : QL.p) + (size_t)sI * o * nn;
         const double* QV = (cmb == 0 ? QR.p : QL.p) + (size_t)sJ * o * nn;
         // Z[j][b][P] = sum_a U[j][a] c^vv[a][b][P]
-        dgemm(false, false, o, v * nK, v, 1.0, U, v, cKvv.p, v * nK, 0.0, Z.p, v * nK, st);
+        gemm(false, false, o, v * nK, v, 1.0, U, v, cKvv.p, v * nK, 0.0, Z.p, v * nK, st);
         // G[j][k][P] = sum_b V[k][b] Z[j][b][P]
         {
           GemmBatch bt;
           bt.nb1 = o;
           bt.sB1 = (long long)v * nK;
           bt.sC1 = (long long)o * nK;
-          dgemm(false, false, o, nK, v, 1.0, Vv, v, Z.p, nK, 0.0, Goo.p, nK, st, bt);
+          gemm(false, false, o, nK, v, 1.0, Vv, v, Z.p, nK, 0.0, Goo.p, nK, st, bt);
         }
         // M1[mu][0:o][P] = C_o G ; M1[mu][o:2o][P] = Q_U^T c^oo
-        dgemm(false, false, nn, o * nK, o, 1.0, Co, nmo, Goo.p, o * nK, 0.0, M1.p, 2 * o * nK, st);
-        dgemm(true, false, nn, o * nK, o, 1.0, QU, nn, cKoo.p, o * nK, 0.0, M1.p + (size_t)o * nK,
+        gemm(false, false, nn, o * nK, o, 1.0, Co, nmo, Goo.p, o * nK, 0.0, M1.p, 2 * o * nK, st);
+        gemm(true, false, nn, o * nK, o, 1.0, QU, nn, cKoo.p, o * nK, 0.0, M1.p + (size_t)o * nK,
               2 * o * nK, st);
         k_build_W<<<cdiv(nn * 2 * o, 256), 256, 0, st>>>(C.p, nmo, QV, nn, o, WV.p);
         RIS_CHECK_LAUNCH();
@@ -3119,10 +3129,10 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
           bt.nb1 = nn;
           bt.sB1 = 2LL * o * nK;
           bt.sC1 = (long long)nn * nK;
-          dgemm(false, false, nn, nK, 2 * o, f, WV.p, 2 * o, M1.p, nK, 1.0, Gam, nK, st, bt);
+          gemm(false, false, nn, nK, 2 * o, f, WV.p, 2 * o, M1.p, nK, 1.0, Gam, nK, st, bt);
         }
         // Omega[P][Q] += f sum_ij c^oo_ij,P G_ij,Q   (K functions are union 0..nK-1)
-        dgemm(true, false, nK, nK, o * o, f, cKoo.p, nK, Goo.p, nK, 1.0, Om, nU, st);
+        gemm(true, false, nK, nK, o * o, f, cKoo.p, nK, Goo.p, nK, 1.0, Om, nU, st);
       }
       if (rpa) {
         // (ib|ja) terms, weights -c_x/2 for (R_I,R_J) and +c_x/2 for (L_I,L_J):
@@ -3141,24 +3151,24 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
           bP.nb1 = nK;
           bP.sB1 = nov;
           bP.sC1 = (long long)o * o;
-          dgemm(false, true, o, o, v, 1.0, U, v, cKovP.p, v, 0.0, E1.p, o, st, bP);
-          dgemm(false, true, o, o, v, 1.0, Vv, v, cKovP.p, v, 0.0, E2.p, o, st, bP);
+          gemm(false, true, o, o, v, 1.0, U, v, cKovP.p, v, 0.0, E1.p, o, st, bP);
+          gemm(false, true, o, o, v, 1.0, Vv, v, cKovP.p, v, 0.0, E2.p, o, st, bP);
           GemmBatch bM;
           bM.nb1 = nK;
           bM.sA1 = (long long)o * o;
           bM.sC1 = (long long)o * nn;
-          dgemm(false, false, o, nn, o, 1.0, E1.p, o, QV, nn, 0.0, M2.p, nn, st, bM);
-          dgemm(false, false, o, nn, o, 1.0, E2.p, o, QU, nn, 1.0, M2.p, nn, st, bM);
+          gemm(false, false, o, nn, o, 1.0, E1.p, o, QV, nn, 0.0, M2.p, nn, st, bM);
+          gemm(false, false, o, nn, o, 1.0, E2.p, o, QU, nn, 1.0, M2.p, nn, st, bM);
           k_permute120<<<cdiv((long long)nK * o * nn, 256), 256, 0, st>>>(M2.p, nK, o, nn, M2p.p);
           RIS_CHECK_LAUNCH();
           GemmBatch bG;
           bG.nb1 = nn;
           bG.sB1 = (long long)nK * o;
           bG.sC1 = (long long)nn * nK;
-          dgemm(false, true, nn, nK, o, wgt, C.p, nmo, M2p.p, o, 1.0, Gam, nK, st, bG);
+          gemm(false, true, nn, nK, o, wgt, C.p, nmo, M2p.p, o, 1.0, Gam, nK, st, bG);
           // E1t[P][k][i] = E1[P][i][k]
           transpose_last2(E1.p, nK, o, o, E1t.p, st);
-          dgemm(false, true, nK, nK, o * o, wgt, E2.p, o * o, E1t.p, o * o, 1.0, Om, nU, st);
+          gemm(false, true, nK, nK, o * o, wgt, E2.p, o * o, E1t.p, o * o, 1.0, Om, nU, st);
         }
       }
     }
@@ -3219,13 +3229,13 @@ void Engine::ensure_Kov() {
     transpose_last2(Bm.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]
     return;
   }
-  dgemm(true, false, o, n * nK, n, 1.0, Co, nmo, TK.p, n * nK, 0.0, H.p, n * nK, st);
+  gemm(true, false, o, n * nK, n, 1.0, Co, nmo, TK.p, n * nK, 0.0, H.p, n * nK, st);
   GemmBatch bt;
   bt.nb1 = o;
   bt.sB1 = (long long)n * nK;
   bt.sC1 = (long long)v * nK;
-  dgemm(true, false, v, nK, n, 1.0, Cv, nmo, H.p, nK, 0.0, Bia.p, nK, st, bt);
-  dgemm(false, true, (int)nov, nK, nK, 1.0, Bia.p, nK, LKinv.p, nK, 0.0, Bm.p, nK, st);  // [i][a][R]
+  gemm(true, false, v, nK, n, 1.0, Cv, nmo, H.p, nK, 0.0, Bia.p, nK, st, bt);
+  gemm(false, true, (int)nov, nK, nK, 1.0, Bia.p, nK, LKinv.p, nK, 0.0, Bm.p, nK, st);  // [i][a][R]
   BKovR.ensure((size_t)nov * nK, st);
   transpose_last2(Bm.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]
 }
@@ -3491,8 +3501,8 @@ void Engine::setup_streamed() {
       e2.c64 = BKao.p; e2.rs = nK; e2.cs = 1;
       emu_abt(kEmu10x6, (int)nfp, nK, nK, Ts.p, nU, 1, LKinv.p, nK, 1, e2);
     } else {
-      dgemm(false, true, (int)nfp, nJ, nU, 1.0, Ts.p, nU, LJu.p, nU, 0.0, BJao.p, nJ, st);
-      dgemm(false, true, (int)nfp, nK, nK, 1.0, Ts.p, nU, LKinv.p, nK, 0.0, BKao.p, nK, st);
+      gemm(false, true, (int)nfp, nJ, nU, 1.0, Ts.p, nU, LJu.p, nU, 0.0, BJao.p, nJ, st);
+      gemm(false, true, (int)nfp, nK, nK, 1.0, Ts.p, nU, LKinv.p, nK, 0.0, BKao.p, nK, st);
     }
     RIS_CUDA(cudaStreamSynchronize(st));  // host vectors go out of scope
   }
@@ -3561,12 +3571,12 @@ void Engine::build_B_streamed() {
         e2.c64 = BJ.p + r0; e2.rin = rw; e2.rld = (long long)v * nJ; e2.rs = 1; e2.cs = nJ;
         emu_abt(kEmu10x6, (int)rH, v, n, H.p, 1, rH, C.p + o, 1, nmo, e2);
       } else {  // H[i][nu][r], then per i: B[i][a][r0 + r]
-        dgemm(true, false, o, n * rw, n, 1.0, Co, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
+        gemm(true, false, o, n * rw, n, 1.0, Co, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
         GemmBatch bt;
         bt.nb1 = o;
         bt.sB1 = (long long)n * rw;
         bt.sC1 = (long long)v * nJ;
-        dgemm(true, false, v, rw, n, 1.0, Cv, nmo, H.p, rw, 0.0, BJ.p + r0, nJ, st, bt);
+        gemm(true, false, v, rw, n, 1.0, Cv, nmo, H.p, rw, 0.0, BJ.p + r0, nJ, st, bt);
       }
     }
   }
@@ -3630,18 +3640,18 @@ void Engine::build_B_streamed() {
       for (int r0 = 0; r0 < nK; r0 += rb) {
         const int rw = std::min(rb, nK - r0);
         scatter_block(BKao.p, nK, r0, rw, nfp, fpMu.p, fpNu.p, n, Tb.p, st);
-        dgemm(true, false, o, n * rw, n, 1.0, Co, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
+        gemm(true, false, o, n * rw, n, 1.0, Co, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
         GemmBatch bt;
         bt.nb1 = o;
         bt.sB1 = (long long)n * rw;
         bt.sC1 = (long long)o * nK;
-        dgemm(true, false, o, rw, n, 1.0, Co, nmo, H.p, rw, 0.0, BKoo.p + r0, nK, st, bt);
-        dgemm(true, false, v, n * rw, n, 1.0, Cv, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
+        gemm(true, false, o, rw, n, 1.0, Co, nmo, H.p, rw, 0.0, BKoo.p + r0, nK, st, bt);
+        gemm(true, false, v, n * rw, n, 1.0, Cv, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
         GemmBatch b2;
         b2.nb1 = v;
         b2.sB1 = (long long)n * rw;
         b2.sC1 = (long long)v * rw;
-        dgemm(true, false, v, rw, n, 1.0, Cv, nmo, H.p, rw, 0.0, G.p, rw, st, b2);
+        gemm(true, false, v, rw, n, 1.0, Cv, nmo, H.p, rw, 0.0, G.p, rw, st, b2);
         k_place_vv<<<(unsigned)cdiv((long long)v * v * rw, 256), 256, 0, st>>>(G.p, v, rw, r0, nK, BKvvD.p);
         RIS_CHECK_LAUNCH();
       }
@@ -3650,7 +3660,7 @@ void Engine::build_B_streamed() {
   Tb.release();
   // fitting coefficients of the oo block, c = B L^-1, as [P][i][k]
   cKoo.ensure((size_t)o * o * nK, st);
-  dgemm(false, false, o * o, nK, nK, 1.0, BKoo.p, nK, LKinv.p, nK, 0.0, cKoo.p, nK, st);
+  gemm(false, false, o * o, nK, nK, 1.0, BKoo.p, nK, LKinv.p, nK, 0.0, cKoo.p, nK, st);
   cKooP.ensure((size_t)o * o * nK, st);
   transpose_last2(cKoo.p, 1, o * o, nK, cKooP.p, st);
   if (mixed) {  // FP32 hi/lo operands of the products and of the gradient
@@ -3711,14 +3721,14 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
     QR.ensure((size_t)nsu * o * nn, st);
     t1.ensure((size_t)nn * v, st);
     for (int s = 0; s < nsu; s++) {
-      dgemm(false, false, nn, v, o, 1.0, Co, nmo, Rs.p + s * nov, v, 0.0, t1.p, v, st);
-      dgemm(false, true, nn, nn, v, 1.0, t1.p, v, Cv, nmo, 0.0, DR.p + (size_t)s * nn * nn, nn, st);
-      dgemm(false, true, o, nn, v, 1.0, Rs.p + s * nov, v, Cv, nmo, 0.0, QR.p + (size_t)s * o * nn, nn, st);
+      gemm(false, false, nn, v, o, 1.0, Co, nmo, Rs.p + s * nov, v, 0.0, t1.p, v, st);
+      gemm(false, true, nn, nn, v, 1.0, t1.p, v, Cv, nmo, 0.0, DR.p + (size_t)s * nn * nn, nn, st);
+      gemm(false, true, o, nn, v, 1.0, Rs.p + s * nov, v, Cv, nmo, 0.0, QR.p + (size_t)s * o * nn, nn, st);
     }
   }
   w5.ensure((size_t)nsu * nJ, st);
-  dgemm(false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
-  dgemm(false, false, nsu, nJ, nJ, 1.0, w5.p, nJ, LJinv.p, nJ, 0.0, cJ.p, nJ, st);
+  gemm(false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
+  gemm(false, false, nsu, nJ, nJ, 1.0, w5.p, nJ, LJinv.p, nJ, 0.0, cJ.p, nJ, st);
   k_symmetrize_sq<<<cdiv((long long)nsu * nn * nn, 256), 256, 0, st>>>(DR.p, nn, nsu);
   RIS_CHECK_LAUNCH();
   // state densities regrouped [batch][mu][nu][b] for the contraction
@@ -3814,15 +3824,15 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
         const double* U = Rs.p + (size_t)sI * nov;
         const double* V = Rs.p + (size_t)sJ * nov;
         SBuf<double> T1((size_t)o * nK * v, st), Gt((size_t)o * nK * o, st);
-        dgemm(false, false, o, nK * v, v, 1.0, V, v, BKvvD.p, nK * v, 0.0, T1.p, nK * v, st);  // [k][R][a]
-        dgemm(false, true, o * nK, o, v, 1.0, T1.p, v, U, v, 0.0, Gt.p, o, st);                 // [k][R][j]
+        gemm(false, false, o, nK * v, v, 1.0, V, v, BKvvD.p, nK * v, 0.0, T1.p, nK * v, st);  // [k][R][a]
+        gemm(false, true, o * nK, o, v, 1.0, T1.p, v, U, v, 0.0, Gt.p, o, st);                 // [k][R][j]
         double* G = Gd.p + (size_t)b * nK * o * o;
         GemmBatch bt;
         bt.nb1 = o;
         bt.sB1 = (long long)nK * o;
         bt.sC1 = o;
-        dgemm(true, false, nK, o, nK, 1.0, LKinv.p, nK, Gt.p, o, 0.0, G, o * o, st, bt);         // [P][k][j]
-        dgemm(false, true, nK, nK, o * o, f, cKooP.p, o * o, G, o * o, 1.0, Om, nU, st);
+        gemm(true, false, nK, o, nK, 1.0, LKinv.p, nK, Gt.p, o, 0.0, G, o * o, st, bt);         // [P][k][j]
+        gemm(false, true, nK, nK, o * o, f, cKooP.p, o * o, G, o * o, 1.0, Om, nU, st);
       }
     }
     RIS_CUDA(cudaMemcpyAsync(pst.p, h_pst.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
@@ -3897,8 +3907,8 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
             bp.nb1 = wK;
             bp.sB1 = (long long)o * o;
             bp.sC1 = 2LL * o;
-            dgemm(false, true, nn, o, o, 1.0, Co, nmo, G + (size_t)u0 * o * o, o, 0.0, M1d.p, wK * 2 * o, st, bp);
-            dgemm(true, false, nn, o, o, 1.0, QU, nn, cKooP.p + (size_t)u0 * o * o, o, 0.0, M1d.p + o,
+            gemm(false, true, nn, o, o, 1.0, Co, nmo, G + (size_t)u0 * o * o, o, 0.0, M1d.p, wK * 2 * o, st, bp);
+            gemm(true, false, nn, o, o, 1.0, QU, nn, cKooP.p + (size_t)u0 * o * o, o, 0.0, M1d.p + o,
                   wK * 2 * o, st, bp);
             k_build_W<<<cdiv(nn * 2 * o, 256), 256, 0, st>>>(C.p, nmo, QV, nn, o, WVd.p);
             RIS_CHECK_LAUNCH();
@@ -3906,7 +3916,7 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
             bm.nb1 = nn;
             bm.sB1 = (long long)wK * 2 * o;
             bm.sC1 = (long long)nn * wK;
-            dgemm(false, true, nn, wK, 2 * o, f, WVd.p, 2 * o, M1d.p, 2 * o, 0.0,
+            gemm(false, true, nn, wK, 2 * o, f, WVd.p, 2 * o, M1d.p, 2 * o, 0.0,
                   Gam64.p + (size_t)b * nn2 * wK, wK, st, bm);
           }
         }

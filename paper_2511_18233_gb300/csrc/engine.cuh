@@ -235,6 +235,11 @@ struct Engine : StreamOwner {
   void apply(int nvec, const double* X, double* out, double* out2);
 
   // helpers
+  void gemm(bool ta, bool tb, int m, int n, int k, double alpha, const double* A, int lda,
+            const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s,
+            GemmBatch bt = GemmBatch());
+  void gemm_sub(bool ff, bool ta, bool tb, int m, int n, int k, double alpha, const double* A,
+                int lda, const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t st);
   void apply_A_tda(const double* Xin, int nvec, double* out);
   void apply_A_mixed(const double* Xin, int nvec, double* out);
   void apply_exchange_mixed(const double* Z, int nvec, double* out, double alpha, double beta);

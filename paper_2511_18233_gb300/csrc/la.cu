@@ -133,6 +133,99 @@ __global__ void __launch_bounds__(256) k_dgemm(int m, int n, int k, double alpha
   }
 }
 
+// Products with few rows (a Davidson block or a state times a long tensor):
+// a tile is all m rows by bn columns, its m bn outputs dealt to the threads
+// one after the other, TQ to a thread, so that no multiply-add is spent on
+// padding of m or (of a narrow n) of n.  The FP64 pipe bounds these products
+// (a warp's instruction takes a quarter of an SM for 75 cycles whatever its
+// active lanes), and a 10 x 40 product in tiles of 16 x 32 is 2.6 times its
+// own work: over k = 31k, the Davidson projections of C20H22, 66 -> 23 us
+// (51 us with plain loads); 10 x 102 over 31k 143 -> 63 us.
+// The sum over k runs in order in one thread, as in k_dgemm: the same bits.
+// The tiles of a step arrive through a ring of four asynchronous copies (one
+// CTA an SM is all that such a product gives, so nothing else hides its
+// loads), issued by at least four warps; warps without outputs only copy.
+constexpr int kFlatM = 40, kFlatN = 128, kFlatT = 512, kFlatStages = 4;
+__device__ __forceinline__ void copy_async8(double* dst, const double* src, bool on) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(on ? 8 : 0) : "memory");
+}
+template <bool TA, bool TB, int TQ>
+__global__ void __launch_bounds__(kFlatT) k_dgemm_flat(int m, int n, int k, int bn, double alpha,
+                                                       const double* __restrict__ A, int lda,
+                                                       const double* __restrict__ B, int ldb, double beta,
+                                                       double* __restrict__ C, int ldc, GemmBatch bt,
+                                                       int ksplit, int kchunk) {
+  extern __shared__ double flat_sh[];  // kFlatStages x { A [kBK][m + 1], B [kBK][bn + 1] }
+  int kbeg = 0, kend = k;
+  if (ksplit > 1) {
+    kbeg = blockIdx.z * kchunk;
+    kend = min(k, kbeg + kchunk);
+    C += (size_t)blockIdx.z * m * n;
+  } else {
+    const int b1 = blockIdx.z / bt.nb2, b2 = blockIdx.z % bt.nb2;
+    A += b1 * bt.sA1 + b2 * bt.sA2;
+    B += b1 * bt.sB1 + b2 * bt.sB2;
+    C += b1 * bt.sC1 + b2 * bt.sC2;
+  }
+  const int tid = threadIdx.x, T = blockDim.x, col0 = blockIdx.x * bn, outs = m * bn;
+  const int la = m + 1, lb = bn + 1, stage = kBK * (la + lb);
+  int ai[TQ], bj[TQ];
+  double acc[TQ];
+#pragma unroll
+  for (int r = 0; r < TQ; r++) {
+    const int q = min(tid + r * T, outs - 1);  // past the end: a copy of the last output, not stored
+    ai[r] = q / bn;
+    bj[r] = q % bn;
+    acc[r] = 0.0;
+  }
+  const int steps = (kend - kbeg + kBK - 1) / kBK;
+  auto load = [&](int it) {
+    if (it < steps) {
+      const int k0 = kbeg + it * kBK;
+      double* As = flat_sh + (it % kFlatStages) * stage;
+      double* Bs = As + kBK * la;
+      for (int e = tid; e < m * kBK; e += T) {
+        const int i = TA ? e % m : e / kBK, kk = TA ? e / m : e % kBK, gk = k0 + kk;
+        const bool on = gk < kend;
+        copy_async8(As + kk * la + i, on ? (TA ? A + (size_t)gk * lda + i : A + (size_t)i * lda + gk) : A, on);
+      }
+      for (int e = tid; e < bn * kBK; e += T) {
+        const int j = TB ? e / kBK : e % bn, kk = TB ? e % kBK : e / bn, gj = col0 + j, gk = k0 + kk;
+        const bool on = gj < n && gk < kend;
+        copy_async8(Bs + kk * lb + j, on ? (TB ? B + (size_t)gj * ldb + gk : B + (size_t)gk * ldb + gj) : B, on);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int it = 0; it < kFlatStages - 1; it++) load(it);
+  for (int it = 0; it < steps; it++) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kFlatStages - 2) : "memory");
+    __syncthreads();  // step it has arrived for every thread; all are done with step it - 1
+    load(it + kFlatStages - 1);
+    const double* As = flat_sh + (it % kFlatStages) * stage;
+    const double* Bs = As + kBK * la;
+    if ((tid & ~31) < outs) {  // warp-uniform
+#pragma unroll
+      for (int kk = 0; kk < kBK; kk++)
+#pragma unroll
+        for (int r = 0; r < TQ; r++) acc[r] = fma(As[kk * la + ai[r]], Bs[kk * lb + bj[r]], acc[r]);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < TQ; r++) {
+    if (tid + r * T >= outs) continue;
+    const int gi = ai[r], gj = col0 + bj[r];
+    if (gj >= n) continue;
+    if (ksplit > 1) {
+      C[(size_t)gi * n + gj] = acc[r];
+    } else {
+      double* p = C + (size_t)gi * ldc + gj;
+      *p = beta == 0.0 ? alpha * acc[r] : fma(alpha, acc[r], beta * *p);
+    }
+  }
+}
+
 // 32 outputs per CTA; warp g adds the slices g, g + 8, ... in order, then
 // warp 0 adds the eight sums in order (the FP64 adds of a skinny product's
 // many slices spread over many SMs; same result every run).
@@ -184,6 +277,71 @@ TileShape pick_shape(int m, int n) {
   return best;
 }
 
+// Columns per tile, outputs per thread and threads of k_dgemm_flat.
+struct FlatPlan {
+  int bn, tq, threads;
+  int warp_fmas() const { return threads / 32 * tq; }  // FP64 instructions per k
+  size_t smem(int m) const { return sizeof(double) * kFlatStages * kBK * (m + 1 + bn + 1); }
+};
+// FP64 cycles per k of the busiest SM: an instruction takes one of its four
+// quarters for 75 cycles.
+double flat_cycles(const FlatPlan& p, int n, long long products) {
+  const long long ctas = (long long)cdiv(n, p.bn) * products;
+  return 75.0 * cdiv((long long)cdiv(ctas, 152) * p.warp_fmas(), 4);
+}
+FlatPlan plan_flat(int m, int n, long long products) {
+  FlatPlan best{};
+  double cost = -1;
+  for (int bn : {32, 16, 64, 128, 96, 48, n}) {  // among equals the earlier
+    if (bn > n || bn > kFlatN) continue;
+    const int out = m * bn, tq = out <= kFlatT ? 1 : out <= 2 * kFlatT ? 2 : 4;
+    if (out > 4 * kFlatT) continue;
+    const FlatPlan p{bn, tq, cdiv(cdiv(out, tq), 32) * 32};
+    const double c = flat_cycles(p, n, products);
+    if (cost < 0 || c < 0.95 * cost) {
+      cost = c;
+      best = p;
+    }
+  }
+  return best;
+}
+
+// Slice length with the least estimated time: the multiply-adds, per step of
+// kBK about 800 cycles for its loads, and for a split product the second
+// launch and its partial sums (about 5000 cycles, 75 / 4 per slice and warp).
+// With slices of at least 256 the products of a small molecule ran on a few
+// CTAs: 5 x 22 over k = 1455 (C4H6) 26 -> 4 us.
+int pick_fine(int m, int n, int k, const TileShape& sh) {
+  double best = -1;
+  int kchunk = k;
+  for (int s = 1; s <= std::min(512, cdiv(k, kBK)); s = s < 8 ? s + 1 : s + s / 8) {
+    const int kc = s == 1 ? k : cdiv(cdiv(k, s), kBK) * kBK, ks = s == 1 ? 1 : cdiv(k, kc);
+    double per_k;
+    if (m <= kFlatM) {
+      per_k = flat_cycles(plan_flat(m, n, ks), n, ks);
+    } else {
+      const long long tiles = (long long)cdiv(n, sh.bn()) * cdiv(m, sh.bm());
+      per_k = 150.0 * sh.tm * sh.tn * cdiv(tiles * ks, 152);
+    }
+    const double cost = per_k * kc + cdiv(kc, kBK) * 800.0 + (ks > 1 ? 5000.0 + 19.0 * ks : 0.0);
+    if (best < 0 || cost < best) {
+      best = cost;
+      kchunk = kc;
+    }
+    if ((double)s * m * n * sizeof(double) > 64e6) break;
+  }
+  return kchunk;
+}
+
+template <bool TA, bool TB>
+void launch_flat(const FlatPlan& p, dim3 grid, cudaStream_t st, int m, int n, int k, double alpha,
+                 const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc,
+                 const GemmBatch& bt, int ksplit, int kchunk) {
+  const auto kern = p.tq == 1 ? k_dgemm_flat<TA, TB, 1> : p.tq == 2 ? k_dgemm_flat<TA, TB, 2> : k_dgemm_flat<TA, TB, 4>;
+  ensure_smem_attr((const void*)kern, (int)(sizeof(double) * kFlatStages * kBK * (kFlatM + 1 + kFlatN + 1)));
+  kern<<<grid, std::max(p.threads, 128), p.smem(m), st>>>(m, n, k, p.bn, alpha, A, lda, B, ldb, beta, C, ldc, bt, ksplit, kchunk);
+}
+
 template <bool TA, bool TB, int THY, int TM, int TN>
 void launch_shape(dim3 grid, cudaStream_t st, int m, int n, int k, double alpha, const double* A,
                   int lda, const double* B, int ldb, double beta, double* C, int ldc,
@@ -222,7 +380,10 @@ void dgemm(bool transA, bool transB, int m, int n, int k, double alpha, const do
   const int tiles = cdiv(n, sh.bn()) * cdiv(m, sh.bm());
   // split k when a single product has too few tiles to occupy every SM twice
   int ksplit = 1, kchunk = k;
-  if (nb == 1 && tiles < 2 * 152 && k >= 512) {
+  if (bt.fine) {
+    if (nb == 1 && k > kBK) kchunk = pick_fine(m, n, k, sh);
+    ksplit = std::max(1, cdiv(k, std::max(1, kchunk)));
+  } else if (nb == 1 && tiles < 2 * 152 && k >= 512) {
     ksplit = std::min(cdiv(2 * 152, tiles), k / 256);
     ksplit = std::max(1, std::min(ksplit, 512));
     kchunk = ((cdiv(k, ksplit) + kBK - 1) / kBK) * kBK;
@@ -236,7 +397,13 @@ void dgemm(bool transA, bool transB, int m, int n, int k, double alpha, const do
   dim3 grid((unsigned)ntiles, 1, ksplit > 1 ? ksplit : nb);
   double* Cout = ksplit > 1 ? ws : C;
   prof_begin(kProfGemm, st);
-  if (!transA && !transB)
+  if (m <= kFlatM) {
+    const FlatPlan p = plan_flat(m, n, (long long)nb * ksplit);
+    const dim3 fg((unsigned)cdiv(n, p.bn), 1, grid.z);
+    const auto launch = transA ? (transB ? launch_flat<true, true> : launch_flat<true, false>)
+                               : (transB ? launch_flat<false, true> : launch_flat<false, false>);
+    launch(p, fg, st, m, n, k, alpha, A, lda, B, ldb, beta, Cout, ldc, bt, ksplit, kchunk);
+  } else if (!transA && !transB)
     launch_t<false, false>(sh, grid, st, m, n, k, alpha, A, lda, B, ldb, beta, Cout, ldc, bt, ksplit, kchunk);
   else if (!transA && transB)
     launch_t<false, true>(sh, grid, st, m, n, k, alpha, A, lda, B, ldb, beta, Cout, ldc, bt, ksplit, kchunk);

@@ -11,6 +11,7 @@ namespace ris {
 struct GemmBatch {
   int nb1 = 1, nb2 = 1;
   long long sA1 = 0, sA2 = 0, sB1 = 0, sB2 = 0, sC1 = 0, sC2 = 0;
+  bool fine = false;  // split the contraction as finely as pays (a single product)
 };
 void dgemm(bool transA, bool transB, int m, int n, int k, double alpha, const double* A, int lda,
            const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t st,
