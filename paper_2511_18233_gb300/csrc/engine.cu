@@ -714,13 +714,14 @@ __global__ void k_expand_cJ(const double* __restrict__ cJ, const int* __restrict
   cU[(size_t)s * nU + jU[Q]] = cJ[t];
 }
 
-// Omega[jU[P]][jU[Q]] = f cI[P] cJ[Q]   (whole matrix zeroed first by caller)
-__global__ void k_omega_J(const double* __restrict__ cI, const double* __restrict__ cJ,
+// Omega[jU[P]][jU[Q]] = f cI[P] cJ[Q] for every pair g = (I, J) of a batch
+// (blockIdx.y; the matrices zeroed first by the caller), c [state][nJ]
+__global__ void k_omega_J(const double* __restrict__ c, const int* __restrict__ pst,
                           const int* __restrict__ jU, int nJ, int nU, double f, double* __restrict__ O) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, g = blockIdx.y;
   if (t >= nJ * nJ) return;
   const int P = t / nJ, Q = t % nJ;
-  O[(size_t)jU[P] * nU + jU[Q]] += f * cI[P] * cJ[Q];
+  O[((size_t)g * nU + jU[P]) * nU + jU[Q]] += f * c[(size_t)pst[2 * g] * nJ + P] * c[(size_t)pst[2 * g + 1] * nJ + Q];
 }
 
 // W_V[nu][k] = C_o[nu][k] (k < o), Q[k-o][nu] (k >= o)
@@ -1799,6 +1800,11 @@ static void tcg(int M, int N, int K, const float* ah, const float* al, int lda, 
   B.nb = (nb > 1 && bsb != 0) ? nb : 1;  // bsb == 0: one B shared by every batch
   tc_gemm(M, N, K, A, B, nb, e, err, st);
 }
+static TcOperand tco(const float* h, const float* l, int rows, int ld, long long bs = 0, int nb = 1) {
+  TcOperand o;
+  o.hi = h; o.lo = l; o.rows = rows; o.ld = ld; o.bstride = bs; o.nb = nb;
+  return o;
+}
 static TcEpilogue ep_split(float* h, float* l, long long rs, long long cs = 1, long long bsc = 0) {
   TcEpilogue e;
   e.mode = kOutSplit; e.chi = h; e.clo = l; e.rs = rs; e.cs = cs; e.bsc = bsc;
@@ -1894,54 +1900,89 @@ void Engine::build_Kvv_tc(double* out) {
   (void)o;
 }
 
-void Engine::gamma_K_mixed(const float* USh, const float* USl, const float* VSh, const float* VSl,
-                           const float* WUh, const float* WUl, const float* WVh, const float* WVl,
-                           double f, double* Gam, float* Gam32, double* Om) {
+// Pairs share launches (the products of one pair are 24 to 700 tiles, so that
+// a pair at a time left the last wave of each of its six products half
+// empty, and U's 71 rows filled half of their only tile row): Z for runs of
+// consecutive states as one product, the others batched over the pairs
+// through the operands' batch maps (with the sums over unneeded padding no
+// longer zeroed: nine C20H22 couplings 2772 -> 2161 us a call).
+void Engine::gamma_K_mixed(int np, const int* sI, const int* sJ, int nsu, const float* Ush, const float* Usl,
+                           const float* Wh, const float* Wl, double f, double* Gam, float* Gam32, double* Om) {
   const int o = nocc, v = nvir, nn = nao;
   const int lv4 = ld4(v), lo4 = ld4(o), kp = ld4(2 * o);
-  // Z[P][j][b] = sum_a U[j][a] c^vv[P][b][a]   (one GEMM, columns (P, b))
-  SBuf<float> ZH((size_t)nK * o * lv4, st, true), ZL((size_t)nK * o * lv4, st, true);
-  {
-    TcEpilogue e = ep_split(ZH.p, ZL.p, lv4);
-    e.cin = v;
-    e.cld = (long long)o * lv4;
-    tcg(o, nK * v, v, USh, USl, lv4, cvvH.p, cvvL.p, lv4, 0, 1, e, d_tcerr, st);
-  }
-  // G[P][k][j] = sum_b V[k][b] Z[P][j][b]   (batch P, coalesced rows)
-  SBuf<float> GH((size_t)nK * o * lo4, st, true), GL((size_t)nK * o * lo4, st, true);
-  tcg(o, o, v, VSh, VSl, lv4, ZH.p, ZL.p, lv4, (long long)o * lv4, nK,
-      ep_split(GH.p, GL.p, lo4, 1, (long long)o * lo4), d_tcerr, st);
-  // M1[mu][P][k'] : k' < o  sum_i Q_U[i][mu] c^oo[P][i][k]
-  //                 k' >= o sum_j C_o[mu][j] G[P][k][j]
-  // each one GEMM over the columns (P, k)
-  SBuf<float> MH((size_t)nn * nK * kp, st, true), ML((size_t)nn * nK * kp, st, true);
-  {
-    TcEpilogue e = ep_split(MH.p, ML.p, (long long)nK * kp);
-    e.cin = o;
-    e.cld = kp;
-    tcg(nn, nK * o, o, WUh, WUl, kp, cooH.p, cooL.p, lo4, 0, 1, e, d_tcerr, st);
-    e.chi = MH.p + o;
-    e.clo = ML.p + o;
-    tcg(nn, nK * o, o, CoH.p, CoL.p, lo4, GH.p, GL.p, lo4, 0, 1, e, d_tcerr, st);
-  }
-  // Gamma[mu][nu][P] += f sum_k' W_V[nu][k'] M1[mu][P][k']: one GEMM, rows nu,
-  // columns (mu, P)
-  {
-    TcEpilogue e = Gam32 ? TcEpilogue() : ep_f64(Gam, nK, 0, f, 1.0);
-    if (Gam32) {  // sole writer of the FP32 G^K: plain stores, no read-modify-write
-      e.mode = kOutF32;
-      e.c32 = Gam32;
-      e.alpha = f;
-      e.beta = 0.0;
+  const long long su = (long long)o * lv4, sw = (long long)nn * kp, sz = nK * su, sg = (long long)nK * o * lo4,
+                  sm = nn * (long long)nK * kp, gk = (long long)nn * nn * nK;
+  // pairs at a time: about 2 GB of work space
+  const int per = (int)std::max(1LL, std::min({(long long)np, 8LL, (1LL << 28) / (sz + sg + sm), 65535LL / nK}));
+  // (padding of Z and M is never read: the products' K extents end before it;
+  // G's enters Omega's contraction and is zeroed)
+  SBuf<float> ZH((size_t)per * sz, st), ZL((size_t)per * sz, st), GH((size_t)per * sg, st, true),
+      GL((size_t)per * sg, st, true), MH((size_t)per * sm, st), ML((size_t)per * sm, st);
+  for (int p0 = 0; p0 < np; p0 += per) {
+    const int n = std::min(per, np - p0);
+    TcBatchMap mI, mJ, mV, mZ;  // products z: pairs (mI, mJ), or (pair, P) with V (mV) and Z (mZ)
+    mI.per = mJ.per = 1;
+    mV.per = mZ.per = nK;
+    mV.fixed = true;  // V is the pair's whatever P
+    int nz = 0, last = -1;  // slots of Z, the last slot's state
+    // Z[slot][P][j][b] = sum_a U[j][a] c^vv[P][b][a]   (columns (P, b))
+    for (int q = 0; q < n;) {
+      if (sI[p0 + q] == last) {  // as the pair before
+        mZ.b[q++] = (nz - 1) * nK;
+        continue;
+      }
+      const int q0 = q, s0 = sI[p0 + q], z0 = nz;
+      while (q < n && sI[p0 + q] == s0 + q - q0) mZ.b[q++] = nz++ * nK;
+      last = sI[p0 + q - 1];
+      TcEpilogue e = ep_split(ZH.p + z0 * sz, ZL.p + z0 * sz, lv4);
+      e.rin = o;
+      e.rld = sz;
+      e.cin = v;
+      e.cld = su;
+      tcg((nz - z0) * o, nK * v, v, Ush + s0 * su, Usl + s0 * su, lv4, cvvH.p, cvvL.p, lv4, 0, 1, e, d_tcerr, st);
     }
-    e.rs = nK;
-    e.cin = nK;
-    e.cld = (long long)nn * nK;
-    tcg(nn, nn * nK, 2 * o, WVh, WVl, kp, MH.p, ML.p, kp, 0, 1, e, d_tcerr, st);
+    for (int q = 0; q < n; q++) {
+      mI.b[q] = sI[p0 + q];
+      mJ.b[q] = mV.b[q] = sJ[p0 + q];
+    }
+    // G[pair][P][k][j] = sum_b V[k][b] Z[P][j][b]
+    tc_gemm(o, o, v, tco(Ush, Usl, o, lv4, su, nsu), tco(ZH.p, ZL.p, o, lv4, su, nz * nK), n * nK,
+            ep_split(GH.p, GL.p, lo4, 1, (long long)o * lo4), d_tcerr, st, nullptr, 0, true, mV, mZ);
+    // M[pair][mu][P][k'] : k' < o  sum_i Q_U[i][mu] c^oo[P][i][k]
+    //                      k' >= o sum_j C_o[mu][j] G[P][k][j]
+    // over the columns (P, k)
+    {
+      TcEpilogue e = ep_split(MH.p, ML.p, (long long)nK * kp, 1, sm);
+      e.cin = o;
+      e.cld = kp;
+      tc_gemm(nn, nK * o, o, tco(Wh, Wl, nn, kp, sw, nsu), tco(cooH.p, cooL.p, nK * o, lo4), n, e, d_tcerr, st,
+              nullptr, 0, true, mI);
+      e.chi = MH.p + o;
+      e.clo = ML.p + o;
+      tc_gemm(nn, nK * o, o, tco(CoH.p, CoL.p, nn, lo4), tco(GH.p, GL.p, nK * o, lo4, sg, n), n, e, d_tcerr, st);
+    }
+    // Gamma[pair][mu][nu][P] += f sum_k' W_V[nu][k'] M[mu][P][k']: rows nu,
+    // columns (mu, P)
+    {
+      TcEpilogue e = Gam32 ? TcEpilogue() : ep_f64(Gam + p0 * gk, nK, gk, f, 1.0);
+      if (Gam32) {  // sole writer of the FP32 G^K: plain stores, no read-modify-write
+        e.mode = kOutF32;
+        e.c32 = Gam32 + p0 * gk;
+        e.alpha = f;
+        e.beta = 0.0;
+        e.bsc = gk;
+      }
+      e.rs = nK;
+      e.cin = nK;
+      e.cld = (long long)nn * nK;
+      tc_gemm(nn, nn * nK, 2 * o, tco(Wh, Wl, nn, kp, sw, nsu), tco(MH.p, ML.p, nn * nK, kp, sm, n), n, e, d_tcerr,
+              st, nullptr, 0, true, mJ);
+    }
+    // Omega[pair][A][B] += f sum_{k,j} c^oo[A][k][j] G[B][k][j]
+    for (int q = 0; q < n; q++)
+      tcg(nK, nK, o * lo4, cooH.p, cooL.p, o * lo4, GH.p + q * sg, GL.p + q * sg, o * lo4, 0, 1,
+          ep_f64(Om + (size_t)(p0 + q) * nU * nU, nU, 0, f, 1.0), d_tcerr, st);
   }
-  // Omega[A][B] += f sum_{k,j} c^oo[A][k][j] G[B][k][j]
-  tcg(nK, nK, o * lo4, cooH.p, cooL.p, o * lo4, GH.p, GL.p, o * lo4, 0, 1, ep_f64(Om, nU, 0, f, 1.0),
-      d_tcerr, st);
 }
 
 // out = alpha * K1 + beta * out with K1 the (ij|ab) exchange contraction of
@@ -3069,40 +3110,31 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
     // (in mixed TDA and in the emulated form one exchange GEMM writes every element of G^K)
     if (!gk32 && !emu) RIS_CUDA(cudaMemsetAsync(GK.p, 0, sizeof(double) * nb * gk, st));
     RIS_CUDA(cudaMemsetAsync(OmB.p, 0, sizeof(double) * nb * nU * nU, st));
-    std::vector<int> h_pst(2 * nb);
+    std::vector<int> h_pst(2 * nb), hI(nb), hJ(nb);
     for (int b = 0; b < nb; b++) {
-      const int g = g0 + b;
-      const int sI = slot[pairs[2 * g]], sJ = slot[pairs[2 * g + 1]];
-      h_pst[2 * b] = sI;
-      h_pst[2 * b + 1] = sJ;
+      h_pst[2 * b] = hI[b] = slot[pairs[2 * (g0 + b)]];
+      h_pst[2 * b + 1] = hJ[b] = slot[pairs[2 * (g0 + b) + 1]];
+    }
+    RIS_CUDA(cudaMemcpyAsync(pst.p, h_pst.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
+    k_omega_J<<<dim3(cdiv(nJ * nJ, 256), nb), 256, 0, st>>>(cJ.p, pst.p, d_jU, nJ, nU, 2.0, OmB.p);
+    RIS_CHECK_LAUNCH();
+    // exchange (ij|ab) for (R_I,R_J) and (L_I,L_J), each with weight -c_x/2;
+    // with Y = 0 both combinations coincide, so one pass with -c_x.
+    for (int cmb = 0; mixed && cmb < (rpa ? 2 : 1); cmb++)
+      gamma_K_mixed(nb, hI.data(), hJ.data(), nsu, cmb == 0 ? RSh.p : LSh.p, cmb == 0 ? RSl.p : LSl.p,
+                    cmb == 0 ? WRh.p : WLh.p, cmb == 0 ? WRl.p : WLl.p, rpa ? -0.5 * cx : -cx, GK.p,
+                    gk32 ? GK32.p : nullptr, OmB.p);
+    for (int b = 0; b < nb; b++) {
+      const int sI = hI[b], sJ = hJ[b];
       double* Gam = gk32 ? nullptr : GK.p + (size_t)b * gk;
-      float* Gam32 = gk32 ? GK32.p + (size_t)b * gk : nullptr;
       double* Om = OmB.p + (size_t)b * nU * nU;
-      k_omega_J<<<cdiv(nJ * nJ, 256), 256, 0, st>>>(cJ.p + (size_t)sI * nJ, cJ.p + (size_t)sJ * nJ,
-                                                     d_jU, nJ, nU, 2.0, Om);
-      RIS_CHECK_LAUNCH();
       if (emu) {
         ge.pair(*this, sI, sJ, Gam, Om);
         continue;
       }
-      // exchange (ij|ab) for (R_I,R_J) and (L_I,L_J), each with weight -c_x/2;
-      // with Y = 0 both combinations coincide, so one pass with -c_x.
-      const int ncomb = rpa ? 2 : 1;
+      const int ncomb = mixed ? 0 : rpa ? 2 : 1;
       for (int cmb = 0; cmb < ncomb; cmb++) {
         const double f = rpa ? -0.5 * cx : -cx;
-        if (mixed) {
-          const size_t so = (size_t)o * lv4, sw = (size_t)nn * kp;
-          const float* USh = (cmb == 0 ? RSh.p : LSh.p) + sI * so;
-          const float* USl = (cmb == 0 ? RSl.p : LSl.p) + sI * so;
-          const float* VSh = (cmb == 0 ? RSh.p : LSh.p) + sJ * so;
-          const float* VSl = (cmb == 0 ? RSl.p : LSl.p) + sJ * so;
-          const float* WUh = (cmb == 0 ? WRh.p : WLh.p) + sI * sw;
-          const float* WUl = (cmb == 0 ? WRl.p : WLl.p) + sI * sw;
-          const float* WVh = (cmb == 0 ? WRh.p : WLh.p) + sJ * sw;
-          const float* WVl = (cmb == 0 ? WRl.p : WLl.p) + sJ * sw;
-          gamma_K_mixed(USh, USl, VSh, VSl, WUh, WUl, WVh, WVl, f, Gam, Gam32, Om);
-          continue;
-        }
         const double* U = (cmb == 0 ? Rs.p : Ls.p) + (size_t)sI * nov;
         const double* Vv = (cmb == 0 ? Rs.p : Ls.p) + (size_t)sJ * nov;
         const double* QU = (cmb == 0 ? QR.p : QL.p) + (size_t)sI * o * nn;
@@ -3172,7 +3204,6 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
         }
       }
     }
-    RIS_CUDA(cudaMemcpyAsync(pst.p, h_pst.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
     prof_begin(kProfContract, st);
     const dim3 gridK(cdiv((long long)nn * nK, 128), slK);
     if (gk32)
@@ -3777,15 +3808,13 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
     const int nb = std::min(NB, npair - g0);
     RIS_CUDA(cudaMemsetAsync(OmB.p, 0, sizeof(double) * nb * nU * nU, st));
     std::vector<int> h_pst(2 * nb);
+    for (int q = 0; q < 2 * nb; q++) h_pst[q] = slot.at(pairs[2 * g0 + q]);
+    RIS_CUDA(cudaMemcpyAsync(pst.p, h_pst.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
+    k_omega_J<<<dim3(cdiv(nJ * nJ, 256), nb), 256, 0, st>>>(cJ.p, pst.p, d_jU, nJ, nU, 2.0, OmB.p);
+    RIS_CHECK_LAUNCH();
     for (int b = 0; b < nb; b++) {
-      const int g = g0 + b;
-      const int sI = slot.at(pairs[2 * g]), sJ = slot.at(pairs[2 * g + 1]);
-      h_pst[2 * b] = sI;
-      h_pst[2 * b + 1] = sJ;
+      const int sI = h_pst[2 * b], sJ = h_pst[2 * b + 1];
       double* Om = OmB.p + (size_t)b * nU * nU;
-      k_omega_J<<<cdiv(nJ * nJ, 256), 256, 0, st>>>(cJ.p + (size_t)sI * nJ, cJ.p + (size_t)sJ * nJ, d_jU,
-                                                    nJ, nU, 2.0, Om);
-      RIS_CHECK_LAUNCH();
       // G~[k][R][j] = sum_ab V_kb B_ab,R U_ja, then G[P][k][j] = sum_R L^-1_RP G~[k][R][j]
       if (mixed) {
         const float* USh = RSh.p + (size_t)sI * o * lv4;
@@ -3835,7 +3864,6 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
         gemm(false, true, nK, nK, o * o, f, cKooP.p, o * o, G, o * o, 1.0, Om, nU, st);
       }
     }
-    RIS_CUDA(cudaMemcpyAsync(pst.p, h_pst.data(), sizeof(int) * 2 * nb, cudaMemcpyHostToDevice, st));
     // auxiliary blocks: derivative integrals regenerated and contracted at once
     for (size_t k = 0; k < auxBlk.size(); k++) {
       const int u0 = blkU0[k], w = blkW[k], wK = blkWK[k];

@@ -260,13 +260,13 @@ struct Engine : StreamOwner {
   void build_K_emu(const double* HK, double* Bvv);
   // K1 (alpha, beta into out) and, when K2 is given, K2 of exchange_terms
   void exchange_emu(const double* Z, int nvec, double* K1, double alpha, double beta, double* K2);
-  // exchange part of Gamma / Omega for one (U,V) pair with weight f (3xTF32);
-  // US/VS: splits of U, V [i][a]; WU/WV: [Q^T | C_o] splits of U and V;
-  // Gamma accumulated in FP64 (Gam) or, when Gam32 is given, written in FP32
-  // (overwritten: the caller's only exchange term)
-  void gamma_K_mixed(const float* USh, const float* USl, const float* VSh, const float* VSl,
-                     const float* WUh, const float* WUl, const float* WVh, const float* WVl,
-                     double f, double* Gam, float* Gam32, double* Om);
+  // exchange parts of Gamma / Omega for np <= 8 pairs (U, V) = (state sI[p],
+  // state sJ[p]) of nsu states with weight f (3xTF32); Us: splits of U [s][i][a];
+  // W: [Q^T | C_o] splits [s][nu][k']; Gamma accumulated in FP64 (Gam) or,
+  // when Gam32 is given, written in FP32 (overwritten: the caller's only
+  // exchange term), pair p at p nao^2 nK; Omega at p nU^2
+  void gamma_K_mixed(int np, const int* sI, const int* sJ, int nsu, const float* Ush, const float* Usl,
+                     const float* Wh, const float* Wl, double f, double* Gam, float* Gam32, double* Om);
   // ok != nullptr: a mixed-precision run that stalls above the tolerance
   // returns its current vectors with *ok = false instead of failing
   void dav_core(int ns, const double* guess, int nguess, bool mixed, double tol,

@@ -108,6 +108,7 @@ __device__ __forceinline__ float to_tf32(float x) {
 struct TcArgs {
   int M, N, K, nkb, ksplit, kb_per;
   int nbA, nbB;
+  TcBatchMap mapA, mapB;
   TcEpilogue ep;
   float* partial;  // split-K workspace [ksplit][M][N] (FP32) or null
   int* err;
@@ -135,7 +136,7 @@ __global__ void __launch_bounds__(128, 2) k_tc_gemm(const __grid_constant__ CUte
   }
   const int kb0 = ks * args.kb_per * (KB / BK);  // blocks of BK
   const int kb1 = min((args.K + BK - 1) / BK, kb0 + args.kb_per * (KB / BK));
-  const int zA = args.nbA > 1 ? z : 0, zB = args.nbB > 1 ? z : 0;
+  const int zA = args.mapA.at(z, args.nbA), zB = args.mapB.at(z, args.nbB);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; s++) {
@@ -365,7 +366,8 @@ void split_f64_t(const double* src, int rows, int cols, long long lds, float* hi
 constexpr int kTcKChunk = 16384;
 
 void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb, const TcEpilogue& ep,
-             int* d_err, cudaStream_t st, float* ws, size_t ws_floats, bool allow_alloc) {
+             int* d_err, cudaStream_t st, float* ws, size_t ws_floats, bool allow_alloc,
+             const TcBatchMap& mapA, const TcBatchMap& mapB) {
   if (M <= 0 || N <= 0 || nb <= 0) return;
   RIS_REQUIRE(K > 0, RIS_ERR_ARG, "tc_gemm: K must be positive");
   if (ep.mode == kOutF64 && K > kTcKChunk) {
@@ -377,7 +379,7 @@ void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb
       b.lo += k0;
       TcEpilogue e = ep;
       if (k0 > 0) e.beta = 1.0;
-      tc_gemm(M, N, std::min(kTcKChunk, K - k0), a, b, nb, e, d_err, st, ws, ws_floats, allow_alloc);
+      tc_gemm(M, N, std::min(kTcKChunk, K - k0), a, b, nb, e, d_err, st, ws, ws_floats, allow_alloc, mapA, mapB);
     }
     return;
   }
@@ -394,6 +396,8 @@ void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb
   a.nkb = cdiv(K, KB);
   a.nbA = A.nb;
   a.nbB = B.nb;
+  a.mapA = mapA;
+  a.mapB = mapB;
   a.ep = ep;
   a.err = d_err;
   a.partial = nullptr;

@@ -18,6 +18,18 @@ struct TcOperand {
   int nb = 1;
 };
 
+// Which matrix of a batched operand a product z takes: when per > 0 (up to
+// eight groups of `per` products) b[z / per], plus z % per unless `fixed`;
+// else matrix z.
+struct TcBatchMap {
+  int per = 0;
+  bool fixed = false;
+  int b[8] = {0};
+  __host__ __device__ int at(int z, int nb) const {
+    return per > 0 ? b[z / per] + (fixed ? 0 : z % per) : nb > 1 ? z : 0;
+  }
+};
+
 // Epilogue: element (i, j) of batch z, i < M, j < N, is stored at
 //   z * bsc + rpos(i) + cpos(j),
 // rpos(i) = (i / rin) * rld + (i % rin) * rs when rin > 0 (row blocks of rin
@@ -54,7 +66,8 @@ struct TcEpilogue {
 // only when ws is large enough).
 void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb,
              const TcEpilogue& ep, int* d_err, cudaStream_t st, float* ws = nullptr,
-             size_t ws_floats = 0, bool allow_alloc = true);
+             size_t ws_floats = 0, bool allow_alloc = true,
+             const TcBatchMap& mapA = TcBatchMap(), const TcBatchMap& mapB = TcBatchMap());
 
 // Split FP64 -> (hi, lo) FP32 with a row-major source [rows][cols] (leading
 // dimension lds) into [rows][ldd] (padding columns zero-filled).
