@@ -60,10 +60,12 @@ __device__ __forceinline__ void ff_store(double* p, float s, float c, double alp
 constexpr int kRowsKG = 4;  // warps per CTA, each a quarter of k
 
 // Shared memory: A split [k][RM] (float2); with TB the CTA's 32 rows of B
-// split and transposed, hi and lo [k][33]; the k-group partial sums
-// [kRowsKG - 1][RM][32] (float2).
+// split and transposed, hi and lo [k][33].  The k-group partial sums
+// [kRowsKG - 1][RM][32] (float2) take the operands' place once all warps are
+// done with them: 43 instead of 58 KB at 18 rows and k = 102, so five CTAs an
+// SM instead of three cover each other's loads (75 -> 60 us for 31k columns).
 inline size_t rows_smem(int RM, bool TB, int k) {
-  return (size_t)k * RM * 8 + (TB ? (size_t)k * 33 * 8 : 0) + (size_t)(kRowsKG - 1) * RM * 32 * 8;
+  return std::max((size_t)k * RM * 8 + (TB ? (size_t)k * 33 * 8 : 0), (size_t)(kRowsKG - 1) * RM * 32 * 8);
 }
 
 template <int RM, bool TB>
@@ -76,7 +78,7 @@ __global__ void __launch_bounds__(32 * kRowsKG) k_ff_rows(int m, int n, int k, d
   float2* sA = ff_sh;
   float* sBh = (float*)(sA + (size_t)k * RM);
   float* sBl = sBh + (TB ? (size_t)k * 33 : 0);
-  float2* sR = (float2*)(sBl + (TB ? (size_t)k * 33 : 0));
+  float2* sR = ff_sh;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int j0 = blockIdx.x * 32, j = j0 + lane;
   for (int e = threadIdx.x; e < k * RM; e += 32 * kRowsKG) {
@@ -136,6 +138,7 @@ __global__ void __launch_bounds__(32 * kRowsKG) k_ff_rows(int m, int n, int k, d
       for (int r = 0; r < RM; r++) ff_renorm(s[r], c[r]);
     }
   }
+  __syncthreads();
   if (w > 0) {
 #pragma unroll
     for (int r = 0; r < RM; r++) sR[((w - 1) * RM + r) * 32 + lane] = make_float2(s[r], c[r]);
@@ -156,28 +159,29 @@ __global__ void __launch_bounds__(32 * kRowsKG) k_ff_rows(int m, int n, int k, d
 }
 
 // ------------------------------------------------------------------ long k
-// Grid (n tiles of 32*TN columns, k chunks); CTA of 256 threads: warp w owns
-// output rows w, w + 8, ... (RW of them, m <= 8 RW), each lane TN columns,
-// so that all eight warps stage the operands whatever m is.  ws[chunk][m][n]
-// receives the chunk's (S, C) pairs.
+// Grid (n tiles of 32 columns, k chunks); CTA of 256 threads: warp w owns
+// output rows w, w + 8, ... (RW of them, m <= 8 RW), each lane a column, so
+// that all eight warps stage the operands whatever m is.  ws[chunk][m][n]
+// receives the chunk's (S, C) pairs.  A CTA's loads, splits and sums follow
+// one another, so small CTAs (17 KB, up to eight an SM) that cover each other
+// do as well as tiles of 128 columns with a quarter of A's splits (8, 10 and
+// 18 rows: 28, 50 and 77 us against 32, 52 and 75).
 constexpr int kLongT = 256;
-template <int TN, int RW, bool TB>
+template <int RW, bool TB>
 __global__ void __launch_bounds__(kLongT) k_ff_long(int m, int n, int k, int kchunk,
                                                     const double* __restrict__ A, int lda,
                                                     const double* __restrict__ B, int ldb,
                                                     float2* __restrict__ ws) {
-  constexpr int BN = 32 * TN;
+  constexpr int BN = 32;
   __shared__ float2 sA[32][33];      // [k][row]
   __shared__ float sBh[32][BN + 1];  // [k][column]
   __shared__ float sBl[32][BN + 1];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c0 = blockIdx.x * BN;
   const int kb = blockIdx.y * kchunk, ke = min(k, kb + kchunk);
-  float S[RW][TN], Cc[RW][TN];
+  float S[RW], Cc[RW];
 #pragma unroll
-  for (int i = 0; i < RW; i++)
-#pragma unroll
-    for (int t = 0; t < TN; t++) S[i][t] = Cc[i][t] = 0.f;
+  for (int i = 0; i < RW; i++) S[i] = Cc[i] = 0.f;
   for (int k0 = kb; k0 < ke; k0 += 32) {
     const int kn = min(32, ke - k0);
     __syncthreads();
@@ -218,41 +222,27 @@ __global__ void __launch_bounds__(kLongT) k_ff_long(int m, int n, int k, int kch
       }
     }
     __syncthreads();
-    float s[RW][TN], c[RW][TN];
+    float s[RW], c[RW];
 #pragma unroll
-    for (int i = 0; i < RW; i++)
-#pragma unroll
-      for (int t = 0; t < TN; t++) s[i][t] = c[i][t] = 0.f;
+    for (int i = 0; i < RW; i++) s[i] = c[i] = 0.f;
 #pragma unroll 2
     for (int kk = 0; kk < 32; kk++) {  // rows past kn are zero
-      float bh[TN], bl[TN];
-#pragma unroll
-      for (int t = 0; t < TN; t++) {
-        bh[t] = sBh[kk][lane + 32 * t];
-        bl[t] = sBl[kk][lane + 32 * t];
-      }
+      const float bh = sBh[kk][lane], bl = sBl[kk][lane];
 #pragma unroll
       for (int i = 0; i < RW; i++) {
         if (w + 8 * i < m) {  // warp-uniform
           const float2 a = sA[kk][w + 8 * i];
-#pragma unroll
-          for (int t = 0; t < TN; t++) ff_term(a.x, a.y, bh[t], bl[t], s[i][t], c[i][t]);
+          ff_term(a.x, a.y, bh, bl, s[i], c[i]);
         }
       }
     }
 #pragma unroll
-    for (int i = 0; i < RW; i++)
-#pragma unroll
-      for (int t = 0; t < TN; t++) ff_add(S[i][t], Cc[i][t], s[i][t], c[i][t]);
+    for (int i = 0; i < RW; i++) ff_add(S[i], Cc[i], s[i], c[i]);
   }
 #pragma unroll
   for (int i = 0; i < RW; i++) {
-    const int r = w + 8 * i;
-#pragma unroll
-    for (int t = 0; t < TN; t++) {
-      const int col = c0 + lane + 32 * t;
-      if (r < m && col < n) ws[((size_t)blockIdx.y * m + r) * n + col] = make_float2(S[i][t], Cc[i][t]);
-    }
+    const int r = w + 8 * i, col = c0 + lane;
+    if (r < m && col < n) ws[((size_t)blockIdx.y * m + r) * n + col] = make_float2(S[i], Cc[i]);
   }
 }
 
@@ -305,27 +295,11 @@ void rows_dispatch(int m, int n, int k, double alpha, const double* A, int lda, 
 #undef RIS_FF_RM
 }
 
-template <int TN, int RW, bool TB>
-void launch_long(dim3 grid, int m, int n, int k, int kchunk, const double* A, int lda,
-                 const double* B, int ldb, float2* ws, cudaStream_t st) {
-  k_ff_long<TN, RW, TB><<<grid, kLongT, 0, st>>>(m, n, k, kchunk, A, lda, B, ldb, ws);
-}
-
-template <int TN, bool TB>
-void long_rows(dim3 grid, int m, int n, int k, int kchunk, const double* A, int lda,
-               const double* B, int ldb, float2* ws, cudaStream_t st) {
-  if (m <= 8) return launch_long<TN, 1, TB>(grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
-  if (m <= 16) return launch_long<TN, 2, TB>(grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
-  return launch_long<TN, 4, TB>(grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
-}
-
 template <bool TB>
-void long_dispatch(int tn, dim3 grid, int m, int n, int k, int kchunk, const double* A, int lda,
+void long_dispatch(dim3 grid, int m, int n, int k, int kchunk, const double* A, int lda,
                    const double* B, int ldb, float2* ws, cudaStream_t st) {
-  if (tn == 1) return long_rows<1, TB>(grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
-  if (tn == 2) return long_rows<2, TB>(grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
-  if (tn == 3) return long_rows<3, TB>(grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
-  return long_rows<4, TB>(grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
+  const auto kern = m <= 8 ? k_ff_long<1, TB> : m <= 16 ? k_ff_long<2, TB> : k_ff_long<4, TB>;
+  kern<<<grid, kLongT, 0, st>>>(m, n, k, kchunk, A, lda, B, ldb, ws);
 }
 
 }  // namespace
@@ -349,20 +323,18 @@ bool ffgemm(bool transA, bool transB, int m, int n, int k, double alpha, const d
       rows_dispatch<false>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, st);
     RIS_CHECK_LAUNCH();
   } else {
-    const int tn = std::min(4, cdiv(n, 32));
-    const int ntile = cdiv(n, 32 * tn);
-    // about two CTAs per SM, chunks of at least 64 k
-    const int want = std::max(1, cdiv(2 * 152, ntile));
+    // about two chunks per SM and 128 columns, of at least 64 k
+    const int want = std::max(1, cdiv(2 * 152, cdiv(n, 32 * std::min(4, cdiv(n, 32)))));
     int kchunk = std::max(64, ((cdiv(k, want) + 31) / 32) * 32);
     const int nchunk = cdiv(k, kchunk);
     MemTrack* tr = nullptr;
     const size_t wsb = sizeof(float2) * (size_t)nchunk * m * n;
     float2* ws = (float2*)dev_alloc(wsb, st, &tr);
-    const dim3 grid((unsigned)ntile, (unsigned)nchunk);
+    const dim3 grid((unsigned)cdiv(n, 32), (unsigned)nchunk);
     if (transB)
-      long_dispatch<true>(tn, grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
+      long_dispatch<true>(grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
     else
-      long_dispatch<false>(tn, grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
+      long_dispatch<false>(grid, m, n, k, kchunk, A, lda, B, ldb, ws, st);
     RIS_CHECK_LAUNCH();
     k_ff_reduce<<<cdiv((long long)m * n, 32), 256, 0, st>>>(m, n, nchunk, ws, alpha, beta, C, ldc);
     RIS_CHECK_LAUNCH();
