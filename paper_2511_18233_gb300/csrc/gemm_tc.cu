@@ -6,11 +6,11 @@
 // in tensor memory (the lo.lo term is below FP32 resolution), which keeps
 // about FP32 accuracy at tensor-core rates.
 //
-// Kernel structure (one 128 x 128 output tile per CTA, 128 threads):
+// Kernel structure (one output tile of 128 x up to 128 per CTA, 128 threads):
 //   warp 0 / lane 0 : TMA producer, ring of (A_hi, A_lo, B_hi, B_lo) tiles of
 //                     128 rows x 16 FP32 (64-byte swizzle), 32 KB a stage
 //   warp 1          : allocates 128 TMEM columns; lane 0 issues
-//                     tcgen05.mma.kind::tf32 (M=128, N=128, K=8) and commits
+//                     tcgen05.mma.kind::tf32 (M=128, N <= 128, K=8) and commits
 //                     each stage back to the producer through an mbarrier
 //   warps 0-3       : epilogue, tcgen05.ld of TMEM lanes 32w..32w+31
 // The contractions are short (K = 71 ... 441 on C20H22), so that a tile's
@@ -44,8 +44,8 @@ constexpr int TILE_BYTES = BM * BK * 4;                      // 8 KB
 constexpr int STAGE_BYTES = 4 * TILE_BYTES;                  // hi/lo of A and B
 constexpr int smem_bytes(int stages) { return stages * STAGE_BYTES + 1024 + 256; }
 
-// 3-D map {K, rows, batch} of FP32, box {16, 128, 1}, 64-byte swizzle.
-CUtensorMap make_map(const float* base, int K, int rows, int ld, long long bstride, int nb) {
+// 3-D map {K, rows, batch} of FP32, box {16, box_rows, 1}, 64-byte swizzle.
+CUtensorMap make_map(const float* base, int K, int rows, int ld, long long bstride, int nb, int box_rows) {
   RIS_REQUIRE(base != nullptr, RIS_ERR_ARG, "tc_gemm: null operand");
   RIS_REQUIRE(((uintptr_t)base & 15) == 0, RIS_ERR_ARG, "tc_gemm: operand not 16-byte aligned");
   RIS_REQUIRE(ld % 4 == 0 && (nb == 1 || bstride % 4 == 0), RIS_ERR_ARG,
@@ -53,7 +53,7 @@ CUtensorMap make_map(const float* base, int K, int rows, int ld, long long bstri
   CUtensorMap m;
   cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)nb};
   cuuint64_t strides[2] = {(cuuint64_t)ld * 4, (cuuint64_t)(nb > 1 ? bstride : (long long)ld * rows) * 4};
-  cuuint32_t box[3] = {BK, BM, 1};
+  cuuint32_t box[3] = {BK, (cuuint32_t)box_rows, 1};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)base, dims, strides, box, es,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
@@ -73,14 +73,15 @@ __device__ __forceinline__ uint64_t desc_sw64(const void* p) {
 
 // kind::tf32 instruction descriptor: D FP32 (bit 4), A and B TF32 (2 at bits
 // 7 and 10), both K-major, N>>3 at bit 17, M>>4 at bit 24.
-constexpr uint32_t kIdesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                            ((uint32_t)(BM >> 4) << 24);
+__device__ __forceinline__ uint32_t idesc_tf32(int n) {
+  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+}
 
-__device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(kIdesc), "r"(acc)
+      "l"(a), "l"(b), "r"(idesc), "r"(acc)
       : "memory");
 }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
@@ -107,6 +108,7 @@ __device__ __forceinline__ float to_tf32(float x) {
 
 struct TcArgs {
   int M, N, K, nkb, ksplit, kb_per;
+  int bn;  // columns per tile
   int nbA, nbB;
   TcBatchMap mapA, mapB;
   TcEpilogue ep;
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(128, 2) k_tc_gemm(const __grid_constant__ CUte
   uint32_t* tmem_slot = (uint32_t*)(done + 1);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * BM;
+  const int bn = args.bn, n0 = blockIdx.x * bn, m0 = blockIdx.y * BM;
   int z = blockIdx.z, ks = 0;
   if (args.ksplit > 1) {
     ks = z;
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(128, 2) k_tc_gemm(const __grid_constant__ CUte
       if (*abort_flag) break;
       uint8_t* st = smem + s * STAGE_BYTES;
       const int kx = (kb0 + i) * BK;
-      mbar_expect_tx(&full[s], STAGE_BYTES);
+      mbar_expect_tx(&full[s], 2 * TILE_BYTES + 2 * bn * BK * 4);
       tma_load(st, &mAh, &full[s], kx, m0, zA);
       tma_load(st + TILE_BYTES, &mAl, &full[s], kx, m0, zA);
       tma_load(st + 2 * TILE_BYTES, &mBh, &full[s], kx, n0, zB);
@@ -183,6 +185,7 @@ __global__ void __launch_bounds__(128, 2) k_tc_gemm(const __grid_constant__ CUte
       mbar_wait(&full[i % STAGES], (i / STAGES) & 1);
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
+    const uint32_t idesc = idesc_tf32(bn);
     for (int i = 0; i < nk; i++) {
       const int s = i % STAGES;
       if (!mbar_wait(&full[s], (i / STAGES) & 1)) {
@@ -196,9 +199,9 @@ __global__ void __launch_bounds__(128, 2) k_tc_gemm(const __grid_constant__ CUte
 #pragma unroll
       for (int kk = 0; kk < BK / 8; kk++) {
         const uint64_t off = (uint64_t)((kk * 32) >> 4);  // 32 bytes per K=8 step
-        mma_tf32(tmem, ah + off, bl + off, (i > 0 || kk > 0) ? 1u : 0u);
-        mma_tf32(tmem, al + off, bh + off, 1u);
-        mma_tf32(tmem, ah + off, bh + off, 1u);
+        mma_tf32(tmem, ah + off, bl + off, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+        mma_tf32(tmem, al + off, bh + off, idesc, 1u);
+        mma_tf32(tmem, ah + off, bh + off, idesc, 1u);
       }
       mma_commit(&empty[s]);
     }
@@ -219,14 +222,14 @@ __global__ void __launch_bounds__(128, 2) k_tc_gemm(const __grid_constant__ CUte
   const TcEpilogue& ep = args.ep;
   float* tile = (float*)smem + warp * (32 * 33);
 #pragma unroll 1
-  for (int c0 = 0; c0 < BN; c0 += 32) {
+  for (int c0 = 0; c0 < bn; c0 += 32) {  // (columns past bn are not this tile's)
     float v[32];
     tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
     for (int j = 0; j < 32; j++) tile[lane * 33 + j] = v[j];
     __syncwarp();
     const int col = n0 + c0 + lane;
-    if (good && col < args.N) {
+    if (good && c0 + lane < bn && col < args.N) {
       const long long cpos = ep.cin > 0 ? (long long)(col / ep.cin) * ep.cld + (long long)(col % ep.cin) * ep.cs
                                         : (long long)col * ep.cs;
 #pragma unroll 4
@@ -385,11 +388,16 @@ void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb
   }
   RIS_REQUIRE(A.rows >= M && B.rows >= N, RIS_ERR_ARG, "tc_gemm: operand rows");
   RIS_REQUIRE(nb <= 65535, RIS_ERR_ARG, "tc_gemm: batch too large");
-  const CUtensorMap mAh = make_map(A.hi, K, M, A.ld, A.bstride, A.nb);
-  const CUtensorMap mAl = make_map(A.lo, K, M, A.ld, A.bstride, A.nb);
-  const CUtensorMap mBh = make_map(B.hi, K, N, B.ld, B.bstride, B.nb);
-  const CUtensorMap mBl = make_map(B.lo, K, N, B.ld, B.bstride, B.nb);
+  // the column tiles evenly wide (a multiple of 16), so that little of the
+  // last one is padding: N = 441 as four tiles of 112, 71 as one of 80
+  // (12% and 37% of the tensor time of such a product)
+  const int bn = cdiv(cdiv(N, cdiv(N, BN)), 16) * 16;
+  const CUtensorMap mAh = make_map(A.hi, K, M, A.ld, A.bstride, A.nb, BM);
+  const CUtensorMap mAl = make_map(A.lo, K, M, A.ld, A.bstride, A.nb, BM);
+  const CUtensorMap mBh = make_map(B.hi, K, N, B.ld, B.bstride, B.nb, bn);
+  const CUtensorMap mBl = make_map(B.lo, K, N, B.ld, B.bstride, B.nb, bn);
   TcArgs a;
+  a.bn = bn;
   a.M = M;
   a.N = N;
   a.K = K;
@@ -427,7 +435,7 @@ void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb
     }
     a.partial = part;
   }
-  dim3 grid(cdiv(N, BN), cdiv(M, BM), a.ksplit > 1 ? a.ksplit : nb);
+  dim3 grid(cdiv(N, bn), cdiv(M, BM), a.ksplit > 1 ? a.ksplit : nb);
   prof_begin(kProfTcGemm, st);
   const bool deep = (long long)grid.x * grid.y * grid.z <= 152;
   const auto kern = deep ? k_tc_gemm<6> : k_tc_gemm<3>;
