@@ -683,6 +683,18 @@ __global__ void k_axpby(long long n, double a, const double* __restrict__ x, dou
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n) z[t] = a * x[t] + (y ? b * y[t] : 0.0);
 }
+// R_s = X_s + Y_s and L_s = X_s - Y_s for the states listed in su (blockIdx.y;
+// Y null: zero), in one launch
+__global__ void k_states_RL(const double* __restrict__ X, const double* __restrict__ Y,
+                            const int* __restrict__ su, long long n, double* __restrict__ R,
+                            double* __restrict__ L) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const size_t i = (size_t)su[blockIdx.y] * n + t, o = (size_t)blockIdx.y * n + t;
+  const double x = X[i], y = Y ? Y[i] : 0.0;
+  R[o] = x + y;
+  L[o] = x - y;
+}
 static void axpby(long long n, double a, const double* x, double b, const double* y, double* z,
                   cudaStream_t st) {
   if (n <= 0) return;
@@ -998,15 +1010,17 @@ __device__ __forceinline__ double pair_w(const double* WKg, const double* YI, co
 
 // grad[g][A][x] = 2 sum_{mu in A, P} W_g - 2 sum_{P in A, mu} W_g
 //                 - sum_{P in A, Q} (O[P][Q] + O[Q][P]) dM[x][P][Q]
-// (block (A, g); the functions of atom A from the CSR lists)
+// (block (A, g, x); the functions of atom A from the CSR lists.  Bound by the
+// FP64 pipe and the strided reads of the second sum, both of which a block
+// per direction spreads over three times the CTAs: five C20H22 pairs 67 -> 34 us)
 __global__ void __launch_bounds__(128) k_grad_reduce_pairs(
     const double* __restrict__ WK, const double* __restrict__ Y, const double* __restrict__ cU,
     const int* __restrict__ pst, const double* __restrict__ O, const double* __restrict__ dM,
     const int* __restrict__ aoPtr, const int* __restrict__ aoList, const int* __restrict__ axPtr,
     const int* __restrict__ axList, int nao, int nU, int nK, int natm,
     double* __restrict__ grad) {
-  __shared__ double red[3][128];
-  const int A = blockIdx.x, g = blockIdx.y;
+  __shared__ double red[128];
+  const int A = blockIdx.x, g = blockIdx.y, x = blockIdx.z;
   const int sI = pst[2 * g], sJ = pst[2 * g + 1];
   const double* WKg = WK + (size_t)g * 3 * nao * nK;
   const double* YI = Y + (size_t)sI * 3 * nao * nU;
@@ -1014,33 +1028,29 @@ __global__ void __launch_bounds__(128) k_grad_reduce_pairs(
   const double* cI = cU + (size_t)sI * nU;
   const double* cJ = cU + (size_t)sJ * nU;
   const double* Og = O + (size_t)g * nU * nU;
-  double s[3] = {0.0, 0.0, 0.0};
+  double s = 0.0;
   const int a0 = aoPtr[A], na = aoPtr[A + 1] - a0;
   for (long long t = threadIdx.x; t < (long long)na * nU; t += 128) {
     const int mu = aoList[a0 + (int)(t / nU)], P = (int)(t % nU);
-#pragma unroll
-    for (int x = 0; x < 3; x++) s[x] += 2.0 * pair_w(WKg, YI, YJ, cI, cJ, x, mu, P, nao, nU, nK);
+    s += 2.0 * pair_w(WKg, YI, YJ, cI, cJ, x, mu, P, nao, nU, nK);
   }
   const int p0 = axPtr[A], np = axPtr[A + 1] - p0;
   for (long long t = threadIdx.x; t < (long long)np * nao; t += 128) {
     const int P = axList[p0 + (int)(t / nao)], mu = (int)(t % nao);
-#pragma unroll
-    for (int x = 0; x < 3; x++) s[x] -= 2.0 * pair_w(WKg, YI, YJ, cI, cJ, x, mu, P, nao, nU, nK);
+    s -= 2.0 * pair_w(WKg, YI, YJ, cI, cJ, x, mu, P, nao, nU, nK);
   }
   for (long long t = threadIdx.x; t < (long long)np * nU; t += 128) {
     const int P = axList[p0 + (int)(t / nU)], Q = (int)(t % nU);
     const double o = Og[(size_t)P * nU + Q] + Og[(size_t)Q * nU + P];
-#pragma unroll
-    for (int x = 0; x < 3; x++) s[x] -= o * dM[((size_t)x * nU + P) * nU + Q];
+    s -= o * dM[((size_t)x * nU + P) * nU + Q];
   }
-  for (int x = 0; x < 3; x++) red[x][threadIdx.x] = s[x];
+  red[threadIdx.x] = s;
   __syncthreads();
   for (int o = 64; o > 0; o >>= 1) {
-    if (threadIdx.x < o)
-      for (int x = 0; x < 3; x++) red[x][threadIdx.x] += red[x][threadIdx.x + o];
+    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
     __syncthreads();
   }
-  if (threadIdx.x < 3) grad[((size_t)g * natm + A) * 3 + threadIdx.x] = red[threadIdx.x][0];
+  if (threadIdx.x == 0) grad[((size_t)g * natm + A) * 3 + x] = red[0];
 }
 
 __global__ void k_divide_pairs(double* __restrict__ out, const double* __restrict__ num,
@@ -1103,32 +1113,44 @@ __global__ void k_cg_p(double* __restrict__ p, const double* __restrict__ z,
 // Phase of state blockIdx.x against the previous step: the overlap over the
 // five largest |X_prev| determinants (ties by index); a negative overlap
 // flips X (and Y) of the state.  sign[I] = +1 or -1.
-__global__ void __launch_bounds__(256) k_phase_align(double* __restrict__ X, double* __restrict__ Y,
+constexpr int kPhaseT = 512;
+__global__ void __launch_bounds__(kPhaseT) k_phase_align(double* __restrict__ X, double* __restrict__ Y,
                                                      const double* __restrict__ Xp, long long n,
                                                      int* __restrict__ sign) {
-  __shared__ unsigned long long bk[8];
-  __shared__ long long bi[8];
+  __shared__ unsigned long long bk[kPhaseT / 32];
+  __shared__ long long bi[kPhaseT / 32];
   __shared__ long long top[5];
   __shared__ double ov;
-  if (threadIdx.x < 5) top[threadIdx.x] = -1;
-  __syncthreads();
   const int I = blockIdx.x;
   const double* xp = Xp + (size_t)I * n;
   double* x = X + (size_t)I * n;
-  unsigned long long lastk = ~0ull;
-  long long lasti = -1;
-  for (int r = 0; r < 5; r++) {
-    // largest |xp| strictly after (lastk, lasti) in the order (|x| desc, index asc)
-    unsigned long long best = 0;
-    long long besti = -1;
-    for (long long i = threadIdx.x; i < n; i += 256) {
-      const unsigned long long k = (unsigned long long)__double_as_longlong(fabs(xp[i]));
-      const bool after = lasti < 0 || k < lastk || (k == lastk && i > lasti);
-      if (after && (besti < 0 || k > best || (k == best && i < besti))) {
-        best = k;
-        besti = i;
+  // the five largest |xp| in the order (|x| desc, index asc): every thread's
+  // own five in one pass, then five rounds over the threads' best remaining
+  // (five passes over the vector were 178 us at 15k amplitudes)
+  unsigned long long k5[5];
+  long long i5[5];
+#pragma unroll
+  for (int r = 0; r < 5; r++) k5[r] = 0, i5[r] = -1;
+  for (long long i = threadIdx.x; i < n; i += kPhaseT) {
+    unsigned long long k = (unsigned long long)__double_as_longlong(xp[i]) & 0x7fffffffffffffffull;
+    long long ix = i;
+    if (i5[4] >= 0 && k <= k5[4]) continue;  // (indices ascend: equal ones stay behind)
+    bool in = false;
+#pragma unroll
+    for (int r = 0; r < 5; r++)
+      if (in || i5[r] < 0 || k > k5[r]) {  // insert, the rest moves down
+        in = true;
+        const unsigned long long tk = k5[r];
+        const long long ti = i5[r];
+        k5[r] = k;
+        i5[r] = ix;
+        k = tk;
+        ix = ti;
       }
-    }
+  }
+  for (int r = 0; r < 5; r++) {
+    unsigned long long best = k5[0];
+    long long besti = i5[0];
     for (int o = 16; o > 0; o >>= 1) {
       const unsigned long long ok = __shfl_xor_sync(0xffffffffu, best, o);
       const long long oi = __shfl_xor_sync(0xffffffffu, besti, o);
@@ -1143,18 +1165,19 @@ __global__ void __launch_bounds__(256) k_phase_align(double* __restrict__ X, dou
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      for (int w = 1; w < 8; w++)
+      for (int w = 1; w < kPhaseT / 32; w++)
         if (bi[w] >= 0 && (bi[0] < 0 || bk[w] > bk[0] || (bk[w] == bk[0] && bi[w] < bi[0]))) {
           bk[0] = bk[w];
           bi[0] = bi[w];
         }
-      top[r] = bi[0];
+      top[r] = bi[0];  // -1: fewer than five elements
     }
     __syncthreads();
-    lastk = bk[0];
-    lasti = bi[0];
-    __syncthreads();
-    if (lasti < 0) break;  // fewer than five elements
+    if (top[r] >= 0 && i5[0] == top[r]) {  // its owner moves on
+#pragma unroll
+      for (int q = 0; q < 4; q++) k5[q] = k5[q + 1], i5[q] = i5[q + 1];
+      i5[4] = -1;
+    }
   }
   if (threadIdx.x == 0) {
     double s = 0.0;
@@ -1165,9 +1188,9 @@ __global__ void __launch_bounds__(256) k_phase_align(double* __restrict__ X, dou
   }
   __syncthreads();
   if (ov < 0.0) {
-    for (long long i = threadIdx.x; i < n; i += 256) x[i] = -x[i];
+    for (long long i = threadIdx.x; i < n; i += kPhaseT) x[i] = -x[i];
     if (Y)
-      for (long long i = threadIdx.x; i < n; i += 256) Y[(size_t)I * n + i] = -Y[(size_t)I * n + i];
+      for (long long i = threadIdx.x; i < n; i += kPhaseT) Y[(size_t)I * n + i] = -Y[(size_t)I * n + i];
   }
 }
 
@@ -2960,12 +2983,11 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   ensure_D();
   // per state: R, L, D^R = C_o R C_v^T, c^J, Q_R = R C_v^T, Q_L = L C_v^T
   SBuf<double> Rs((size_t)nsu * nov, st), Ls((size_t)nsu * nov, st), DR, cJ, QR, QL;
-  for (int s = 0; s < nsu; s++) {
-    const double* xs = Xa + (size_t)su[s] * nov;
-    const double* ys = rpa ? Ya + (size_t)su[s] * nov : nullptr;
-    axpby(nov, 1.0, xs, 1.0, ys, Rs.p + s * nov, st);
-    axpby(nov, 1.0, xs, -1.0, ys, Ls.p + s * nov, st);
-  }
+  SBuf<int> d_su(nsu, st);
+  // (pageable host-to-device copies are staged before the call returns)
+  RIS_CUDA(cudaMemcpyAsync(d_su.p, su.data(), sizeof(int) * nsu, cudaMemcpyHostToDevice, st));
+  k_states_RL<<<dim3(cdiv(nov, 256), nsu), 256, 0, st>>>(Xa, Ya, d_su.p, nov, Rs.p, Ls.p);
+  RIS_CHECK_LAUNCH();
   DR.ensure((size_t)nsu * nn * nn, st);
   cJ.ensure((size_t)nsu * nJ, st);
   w5.ensure((size_t)nsu * nJ, st);
@@ -3041,8 +3063,9 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
       gemm(false, false, nn, nn, o, 1.0, Co, nmo, QR.p, nn, 0.0, DR.p, nn, st, bt);
     }
   }
-  // u_s = R_s . B^J (nJ), c_s = u_s L^-1 (row vector)
-  gemm(false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
+  // u_s = R_s . B^J (nJ), c_s = u_s L^-1 (row vector); the long product in
+  // double-FP32 in the mixed form, like those of its Davidson
+  gemm_sub(mixed && opt.subspace_ff, false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
   gemm(false, false, nsu, nJ, nJ, 1.0, w5.p, nJ, LJinv.p, nJ, 0.0, cJ.p, nJ, st);
   // Coulomb part of every pair density from per-state data: symmetrised
   // D^R and c^J on the union index (the contraction forms G^J on the fly)
@@ -3222,7 +3245,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
     // algorithmic bytes: the P < nK part of D once, G^K twice per pair, W written
     prof_end(kProfContract, st,
              dbytes * 3.0 * nn * nn * nK + (gk32 ? 4.0 : 8.0) * 2.0 * nb * gk + 24.0 * nb * nn * nK);
-    k_grad_reduce_pairs<<<dim3(natm, nb), 128, 0, st>>>(WK.p, Yst.p, cU.p, pst.p, OmB.p, dMU.p,
+    k_grad_reduce_pairs<<<dim3(natm, nb, 3), 128, 0, st>>>(WK.p, Yst.p, cU.p, pst.p, OmB.p, dMU.p,
                                                         aoPtr.p, aoList.p, axPtr.p, axList.p, nn,
                                                         nU, nK, natm, out + (size_t)g0 * natm * 3);
     RIS_CHECK_LAUNCH();
@@ -3963,7 +3986,7 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
       }
       prof_end(kProfContract, st, bytes);
     }
-    k_grad_reduce_pairs<<<dim3(natm, nb), 128, 0, st>>>(WK.p, Yst.p, cU.p, pst.p, OmB.p, dMU.p, aoPtr.p,
+    k_grad_reduce_pairs<<<dim3(natm, nb, 3), 128, 0, st>>>(WK.p, Yst.p, cU.p, pst.p, OmB.p, dMU.p, aoPtr.p,
                                                         aoList.p, axPtr.p, axList.p, nn, nU, nK, natm,
                                                         out + (size_t)g0 * natm * 3);
     RIS_CHECK_LAUNCH();
@@ -4014,7 +4037,7 @@ void Engine::phase_align(int ns, const double* Xprev_in, int* sign_out, double* 
   SBuf<double> xp((size_t)ns * n, st);
   copy_in(xp.p, Xprev_in, (size_t)ns * n, st);
   SBuf<int> sg(ns, st);
-  k_phase_align<<<ns, 256, 0, st>>>(X.p, opt.rpa ? Y.p : nullptr, xp.p, n, sg.p);
+  k_phase_align<<<ns, kPhaseT, 0, st>>>(X.p, opt.rpa ? Y.p : nullptr, xp.p, n, sg.p);
   RIS_CHECK_LAUNCH();
   if (sign_out) {
     cudaPointerAttributes a;
