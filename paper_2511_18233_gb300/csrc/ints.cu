@@ -163,43 +163,6 @@ struct NH {
   static constexpr int n = (L + 1) * (L + 2) * (L + 3) / 6;
 };
 
-// E[d][i][j][t] for i <= IA, j <= JB.
-template <int IA, int JB>
-__device__ __forceinline__ void hermite_E(double p, const double (&PA)[3], const double (&PB)[3],
-                                          double (&E)[3][IA + 1][JB + 1][IA + JB + 1]) {
-  const double o2p = 0.5 / p;
-#pragma unroll
-  for (int d = 0; d < 3; d++) {
-#pragma unroll
-    for (int i = 0; i <= IA; i++)
-#pragma unroll
-      for (int j = 0; j <= JB; j++)
-#pragma unroll
-        for (int t = 0; t <= IA + JB; t++) E[d][i][j][t] = 0.0;
-    E[d][0][0][0] = 1.0;
-#pragma unroll
-    for (int i = 1; i <= IA; i++)
-#pragma unroll
-      for (int t = 0; t <= i; t++) {
-        double v = PA[d] * E[d][i - 1][0][t];
-        if (t > 0) v += o2p * E[d][i - 1][0][t - 1];
-        if (t + 1 <= i - 1) v += (t + 1) * E[d][i - 1][0][t + 1];
-        E[d][i][0][t] = v;
-      }
-#pragma unroll
-    for (int j = 1; j <= JB; j++)
-#pragma unroll
-      for (int i = 0; i <= IA; i++)
-#pragma unroll
-        for (int t = 0; t <= i + j; t++) {
-          double v = PB[d] * E[d][i][j - 1][t];
-          if (t > 0) v += o2p * E[d][i][j - 1][t - 1];
-          if (t + 1 <= i + j - 1) v += (t + 1) * E[d][i][j - 1][t + 1];
-          E[d][i][j][t] = v;
-        }
-  }
-}
-
 // E[i][j][t] of one axis for i <= IA, j <= JB (rows of IA + JB + 1; entries
 // past t = i + j are not written).
 template <int IA, int JB>
@@ -302,124 +265,9 @@ __device__ __forceinline__ int herm1(int k, double g, double sgn, int* tau, doub
   return 2;
 }
 
-struct PairGeom {
-  double p, PA[3], PB[3], P[3], pref_ab;  // pref_ab = K_ab * nbase_a * nbase_b
-};
-
-__device__ __forceinline__ void pair_geom(double a, const double* A, double b, const double* B,
-                                          double na, double nb, PairGeom& g) {
-  g.p = a + b;
-  double ab2 = 0.0;
-#pragma unroll
-  for (int d = 0; d < 3; d++) {
-    g.P[d] = (a * A[d] + b * B[d]) / g.p;
-    g.PA[d] = g.P[d] - A[d];
-    g.PB[d] = g.P[d] - B[d];
-    ab2 += (A[d] - B[d]) * (A[d] - B[d]);
-  }
-  g.pref_ab = exp(-a * b / g.p * ab2) * na * nb;
-}
-
 // ------------------------------------------------------------------ three-centre
-template <int LA, int LB, int LC>
-__global__ void __launch_bounds__(128) k_int3c(const int* __restrict__ pa, const int* __restrict__ pb,
-                                               int p0, int np, const int* __restrict__ auxl,
-                                               int nax, const int* __restrict__ sh_atom,
-                                               const int* __restrict__ sh_off,
-                                               const double* __restrict__ sh_ex,
-                                               const double* __restrict__ sh_nb,
-                                               const int* __restrict__ ax_atom,
-                                               const double* __restrict__ ax_ex,
-                                               const double* __restrict__ ax_nb,
-                                               const int* __restrict__ ax_jmap,
-                                               const int* __restrict__ ax_kmap,
-                                               const double* __restrict__ xyz,
-                                               const double* __restrict__ boys_tab, int nao,
-                                               int nJ, int nK, double* __restrict__ TJ,
-                                               double* __restrict__ TK,
-                                               const long long* __restrict__ poff,
-                                               const int* __restrict__ ax_off) {
-  constexpr int L = LA + LB + LC;
-  long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= (long long)np * nax) return;
-  const int ip = p0 + (int)(tid / nax);
-  const int sc = auxl[(int)(tid % nax)];
-  const int sa = pa[ip], sb = pb[ip];
-  const double* A = xyz + 3 * sh_atom[sa];
-  const double* B = xyz + 3 * sh_atom[sb];
-  const double* Cc = xyz + 3 * ax_atom[sc];
-  PairGeom g;
-  pair_geom(sh_ex[sa], A, sh_ex[sb], B, sh_nb[sa], sh_nb[sb], g);
-  const double gam = ax_ex[sc];
-  const double rho = g.p * gam / (g.p + gam);
-  const double X = g.P[0] - Cc[0], Y = g.P[1] - Cc[1], Z = g.P[2] - Cc[2];
-  double F[L + 1];
-  boys<L>(rho * (X * X + Y * Y + Z * Z), boys_tab, F);
-  double R[NH<L>::n];
-  hermite_R<L>(1.0, rho, X, Y, Z, F, R);
-  double E[3][LA + 1][LB + 1][LA + LB + 1];
-  hermite_E<LA, LB>(g.p, g.PA, g.PB, E);
-  const double pref = 2.0 * 17.493418327624862 /* pi^2.5 */ / (g.p * gam * sqrt(g.p + gam)) *
-                      g.pref_ab * ax_nb[sc];
-  const int oa = sh_off[sa], ob = sh_off[sb];
-  const int jm = ax_jmap[sc], km = ax_kmap[sc];
-#pragma unroll 1
-  for (int ia = 0; ia < (LA + 1) * (LA + 2) / 2; ia++) {
-    const int ax = cx_(LA, ia), ay = cy_(LA, ia), az = cz_(LA, ia);
-#pragma unroll 1
-    for (int ib = 0; ib < (LB + 1) * (LB + 2) / 2; ib++) {
-      const int bx = cx_(LB, ib), by = cy_(LB, ib), bz = cz_(LB, ib);
-      const double nab = pref * cfac(LA, ia) * cfac(LB, ib);
-#pragma unroll 1
-      for (int ic = 0; ic < (LC + 1) * (LC + 2) / 2; ic++) {
-        int tx[2], ty[2], tz[2];
-        double fx[2], fy[2], fz[2];
-        const int nx = herm1(cx_(LC, ic), gam, -1.0, tx, fx);
-        const int ny = herm1(cy_(LC, ic), gam, -1.0, ty, fy);
-        const int nz = herm1(cz_(LC, ic), gam, -1.0, tz, fz);
-        double s = 0.0;
-        const int mx = LC <= 1 ? 1 : nx, my = LC <= 1 ? 1 : ny, mz = LC <= 1 ? 1 : nz;
-        for (int jx = 0; jx < mx; jx++)
-          for (int jy = 0; jy < my; jy++)
-            for (int jz = 0; jz < mz; jz++) {
-              const int kx = tx[jx], ky = ty[jy], kz = tz[jz];
-              double sub = 0.0;
-#pragma unroll 1
-              for (int t = 0; t <= ax + bx; t++) {
-                const double et = E[0][ax][bx][t];
-#pragma unroll 1
-                for (int u = 0; u <= ay + by; u++) {
-                  const double eu = et * E[1][ay][by][u];
-#pragma unroll 1
-                  for (int v = 0; v <= az + bz; v++)
-                    sub += eu * E[2][az][bz][v] * R[hidx(t + kx, u + ky, v + kz)];
-                }
-              }
-              s += fx[jx] * fy[jy] * fz[jz] * sub;
-            }
-        s *= nab * cfac(LC, ic);
-        if (poff) {  // screened-pair storage: one row per function pair of this shell pair
-          constexpr int NB = (LB + 1) * (LB + 2) / 2;
-          TJ[(size_t)(poff[ip] + ia * NB + ib) * nJ + ax_off[sc] + ic] = s;
-          continue;
-        }
-        const int mu = oa + ia, nu = ob + ib;
-        if (jm >= 0) {
-          TJ[((size_t)mu * nao + nu) * nJ + jm + ic] = s;
-          TJ[((size_t)nu * nao + mu) * nJ + jm + ic] = s;
-        }
-        if (km >= 0) {
-          TK[((size_t)mu * nao + nu) * nK + km + ic] = s;
-          TK[((size_t)nu * nao + mu) * nK + km + ic] = s;
-        }
-      }
-    }
-  }
-}
-
-// ------------------------------------------------------------------ derivatives
 // GB300 issues an FP64 instruction of a warp about every 19 cycles per SM
-// (1.7 FP64 operations per clock), so the derivative kernel is bound by its
+// (1.7 FP64 operations per clock), so the kernels below are bound by their
 // number of FP64 operations, as long as every SM has enough warps: shared
 // memory, index arithmetic and rolled loops are free beside them.  So
 // * whatever depends on the shell pair alone (product centre, E
@@ -431,7 +279,7 @@ __global__ void __launch_bounds__(128) k_int3c(const int* __restrict__ pa, const
 //   warp then takes one function pair and auxiliary component for 32 items,
 //   one multiply-add per coefficient.  A class of few pairs (dd: 210 on
 //   C20H22) so still has 100 warps of work per 32 items.
-// All classes of C20H22 (1 M items): 1142 us, before (an item per thread,
+// Derivatives, all classes of C20H22 (1 M items): 1142 us, before (an item per thread,
 // everything recomputed by each) 3843 us; dd with p auxiliary shells 114
 // instead of 1160 us.  With the coefficients per pair but an item per thread
 // it was 3231 us: 52 CTAs for dd, 130 for dp.
@@ -476,6 +324,158 @@ __device__ __forceinline__ void pair_setup(const PairSrc& s, int first, int npb,
   }
 }
 
+// items whose R_tuv (n doubles each) are held at a time: at most 44 KB of them
+constexpr int items_held(int n) {
+  int k = 256;
+  while (k > 32 && k * n * 8 > 44 * 1024) k /= 2;
+  return k;
+}
+constexpr int kInt3cT = 256;
+
+// Coefficients of (ab|: per function pair (ia, ib) the products
+// (E^x_t E^y_u) E^z_v in the order of t, u, v (W slots per function pair).
+template <int LA, int LB, int LC>
+struct Int3cTab {
+  static constexpr int L = LA + LB + LC;
+  static constexpr int NA = (LA + 1) * (LA + 2) / 2, NB = (LB + 1) * (LB + 2) / 2, NC = (LC + 1) * (LC + 2) / 2;
+  static constexpr int NT = LA + LB + 1;
+  static constexpr int NE = (LA + 1) * (LB + 1) * NT;
+  static constexpr int kItems = items_held(NH<L>::n + 2);
+  static constexpr int width() {
+    int w = 0;
+    for (int a = 0; a < NA; a++)
+      for (int b = 0; b < NB; b++) {
+        const int k = (cx_(LA, a) + cx_(LB, b) + 1) * (cy_(LA, a) + cy_(LB, b) + 1) *
+                      (cz_(LA, a) + cz_(LB, b) + 1);
+        w = k > w ? k : w;
+      }
+    return w;
+  }
+  static constexpr int W = width();
+  static constexpr int kPair = NA * NB * W;
+  static constexpr size_t bytes(int pb) {
+    return (size_t)((NH<L>::n + 2) * kItems + pb * (kPair + 3 * NE)) * sizeof(double) + pb * sizeof(PairGeo);
+  }
+};
+
+// (mu nu|P), both orders of mu and nu, into T^J and T^K, or (poff given) into
+// the screened-pair storage; tiled like k_int3c_deriv below (all classes of
+// C20H22 857 -> 573 us; the same arithmetic per integral, the same bits).
+template <int LA, int LB, int LC>
+__global__ void __launch_bounds__(kInt3cT) k_int3c(PairSrc src, int pb, const int* __restrict__ auxl, int nax,
+                                                   const int* __restrict__ ax_atom,
+                                                   const double* __restrict__ ax_ex,
+                                                   const double* __restrict__ ax_nb,
+                                                   const int* __restrict__ ax_jmap,
+                                                   const int* __restrict__ ax_kmap,
+                                                   const double* __restrict__ boys_tab, int nao,
+                                                   int nJ, int nK, double* __restrict__ TJ,
+                                                   double* __restrict__ TK,
+                                                   const long long* __restrict__ poff,
+                                                   const int* __restrict__ ax_off) {
+  using Tab = Int3cTab<LA, LB, LC>;
+  constexpr int L = Tab::L, NA = Tab::NA, NB = Tab::NB, NT = Tab::NT, RI = Tab::kItems;
+  extern __shared__ __align__(16) double sm3c[];
+  double* tab = sm3c;
+  double* Rs = tab + pb * Tab::kPair;  // [hidx][item], then the item's prefactor and -1/2 gamma
+  double* E = Rs + (NH<L>::n + 2) * RI;
+  PairGeo* geo = (PairGeo*)(E + pb * 3 * Tab::NE);
+  const int first = blockIdx.x * pb, npb = min(pb, src.np - first);
+  pair_setup<LA, LB>(src, first, npb, geo, E);
+  __syncthreads();
+  for (int i = threadIdx.x; i < npb * NA * NB; i += kInt3cT) {
+    const int k = i / (NA * NB), ia = i / NB % NA, ib = i % NB;
+    auto e = [&](int d) {
+      return E + ((k * 3 + d) * (LA + 1) * (LB + 1) + cxyz(LA, ia, d) * (LB + 1) + cxyz(LB, ib, d)) * NT;
+    };
+    auto n = [&](int d) { return cxyz(LA, ia, d) + cxyz(LB, ib, d); };
+    double* o = tab + i * Tab::W;
+    for (int t = 0; t <= n(0); t++)
+      for (int u = 0; u <= n(1); u++) {
+        const double eu = e(0)[t] * e(1)[u];
+        for (int v = 0; v <= n(2); v++) *o++ = eu * e(2)[v];
+      }
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i0 = 0; i0 < npb * nax; i0 += RI) {
+    const int ni = min(RI, npb * nax - i0);
+    __syncthreads();  // the coefficients; the last items' R_tuv have been read
+    if (threadIdx.x < ni) {
+      const int it = i0 + threadIdx.x, sc = auxl[it % nax];
+      const PairGeo& g = geo[it / nax];
+      const double* Cc = src.xyz + 3 * ax_atom[sc];
+      const double gam = ax_ex[sc];
+      const double rho = g.p * gam / (g.p + gam);
+      const double X = g.P[0] - Cc[0], Y = g.P[1] - Cc[1], Z = g.P[2] - Cc[2];
+      double F[L + 1], R[NH<L>::n];
+      boys<L>(rho * (X * X + Y * Y + Z * Z), boys_tab, F);
+      hermite_R<L>(1.0, rho, X, Y, Z, F, R);
+#pragma unroll
+      for (int k = 0; k < NH<L>::n; k++) Rs[k * RI + threadIdx.x] = R[k];
+      Rs[NH<L>::n * RI + threadIdx.x] = 2.0 * 17.493418327624862 /* pi^2.5 */ /
+                                        (g.p * gam * sqrt(g.p + gam)) * g.K * ax_nb[sc];
+      if (LC == 1) Rs[(NH<L>::n + 1) * RI + threadIdx.x] = -0.5 / gam;
+    }
+    __syncthreads();
+    const int ng = (ni + 31) / 32;
+    for (int w = warp; w < ng * (Tab::NC * NA * NB); w += kInt3cT / 32) {
+      const int li = (w % ng) * 32 + lane, f = w / ng;
+      const int ic = f / (NA * NB), ia = f / NB % NA, ib = f % NB;
+      if (li >= ni) continue;
+      const int it = i0 + li, k = it / nax, sc = auxl[it % nax];
+      const double* R = Rs + li;
+      const double* tc = tab + ((k * NA + ia) * NB + ib) * Tab::W;
+      const int mx = cxyz(LA, ia, 0) + cxyz(LB, ib, 0), my = cxyz(LA, ia, 1) + cxyz(LB, ib, 1),
+                mz = cxyz(LA, ia, 2) + cxyz(LB, ib, 2);
+      auto sum = [&](int kx, int ky, int kz) {
+        const double* c = tc;
+        double s = 0.0;
+#pragma unroll 1
+        for (int t = 0; t <= mx; t++)
+#pragma unroll 1
+          for (int u = 0; u <= my; u++)
+#pragma unroll 1
+            for (int v = 0; v <= mz; v++) s += *c++ * R[c_h.h[t + kx][u + ky][v + kz] * RI];
+        return s;
+      };
+      double s = 0.0;
+      if (LC == 0) {
+        s = sum(0, 0, 0);
+      } else if (LC == 1) {
+        s = R[(NH<L>::n + 1) * RI] * sum(ic == 0, ic == 1, ic == 2);
+      } else {
+        int tx[2], ty[2], tz[2];
+        double fx[2], fy[2], fz[2];
+        const double gam = ax_ex[sc];
+        const int nx = herm1(cx_(LC, ic), gam, -1.0, tx, fx), ny = herm1(cy_(LC, ic), gam, -1.0, ty, fy),
+                  nz = herm1(cz_(LC, ic), gam, -1.0, tz, fz);
+        for (int jx = 0; jx < nx; jx++)
+          for (int jy = 0; jy < ny; jy++)
+            for (int jz = 0; jz < nz; jz++) s += fx[jx] * fy[jy] * fz[jz] * sum(tx[jx], ty[jy], tz[jz]);
+      }
+      // (the norms of all but xx, yy, zz are one)
+      double nab = R[NH<L>::n * RI];
+      if (cfac(LA, ia) != 1.0) nab *= cfac(LA, ia);
+      if (cfac(LB, ib) != 1.0) nab *= cfac(LB, ib);
+      if (cfac(LC, ic) != 1.0) nab *= cfac(LC, ic);
+      s *= nab;
+      if (poff) {  // screened-pair storage: one row per function pair of this shell pair
+        TJ[(size_t)(poff[src.p0 + first + k] + ia * NB + ib) * nJ + ax_off[sc] + ic] = s;
+        continue;
+      }
+      const int mu = geo[k].oa + ia, nu = geo[k].ob + ib, jm = ax_jmap[sc], km = ax_kmap[sc];
+      if (jm >= 0) {
+        TJ[((size_t)mu * nao + nu) * nJ + jm + ic] = s;
+        TJ[((size_t)nu * nao + mu) * nJ + jm + ic] = s;
+      }
+      if (km >= 0) {
+        TK[((size_t)mu * nao + nu) * nK + km + ic] = s;
+        TK[((size_t)nu * nao + mu) * nK + km + ic] = s;
+      }
+    }
+  }
+}
+
 // Derivative coefficients: per function pair and direction x (y, z the other
 // two axes) the products E^y_u E^z_v, then per t the pairs
 //   K N (2 alpha E^{a+1,b}_t - a E^{a-1,b}_t)   (centre A)
@@ -487,13 +487,7 @@ struct DerivTab {
   static constexpr int NA = (LA + 1) * (LA + 2) / 2, NB = (LB + 1) * (LB + 2) / 2, NC = (LC + 1) * (LC + 2) / 2;
   static constexpr int NT = LA + LB + 3;
   static constexpr int NE = (LA + 2) * (LB + 2) * NT;
-  // items whose R_tuv are held at a time: at most 44 KB of them
-  static constexpr int items() {
-    int n = 256;
-    while (n > 32 && n * NH<L>::n * 8 > 44 * 1024) n /= 2;
-    return n;
-  }
-  static constexpr int kItems = items();
+  static constexpr int kItems = items_held(NH<L>::n);
   // slots of the E^y E^z products (even, so that the (A, B) pairs are 16-byte aligned)
   static __host__ __device__ constexpr int nyz(int ny, int nz) {
     return ny + nz == 0 ? 0 : ((ny + 1) * (nz + 1) + 1) & ~1;
@@ -516,13 +510,11 @@ struct DerivTab {
     return (size_t)(NH<L>::n * kItems + pb * (kPair + 3 * NE)) * sizeof(double) + pb * sizeof(PairGeo);
   }
 };
-constexpr int kDerivT = 256;
-
 // d(mu nu|P)/dA_x (A = centre of mu) and d(mu nu|P)/dB_x, written as
 // D[x][mu][nu][P] and D[x][nu][mu][P] (computed in FP64, stored as T); pb
 // shell pairs per CTA.
 template <int LA, int LB, int LC, class T>
-__global__ void __launch_bounds__(kDerivT) k_int3c_deriv(
+__global__ void __launch_bounds__(kInt3cT) k_int3c_deriv(
     PairSrc src, int pb, const int* __restrict__ auxl, int nax, const int* __restrict__ ax_atom,
     const int* __restrict__ ax_off, const double* __restrict__ ax_ex, const double* __restrict__ ax_nb,
     const double* __restrict__ boys_tab, int nao, int naux, T* __restrict__ D) {
@@ -536,7 +528,7 @@ __global__ void __launch_bounds__(kDerivT) k_int3c_deriv(
   const int first = blockIdx.x * pb, npb = min(pb, src.np - first);
   pair_setup<LA + 1, LB + 1>(src, first, npb, geo, E);
   __syncthreads();
-  for (int i = threadIdx.x; i < npb * NA * NB * 3; i += kDerivT) {
+  for (int i = threadIdx.x; i < npb * NA * NB * 3; i += kInt3cT) {
     const int x = i % 3, f = i / 3, k = f / (NA * NB), ia = f / NB % NA, ib = f % NB;
     const int a_[3] = {cx_(LA, ia), cy_(LA, ia), cz_(LA, ia)}, b_[3] = {cx_(LB, ib), cy_(LB, ib), cz_(LB, ib)};
     const int y = (x + 1) % 3, z = (x + 2) % 3;
@@ -583,7 +575,7 @@ __global__ void __launch_bounds__(kDerivT) k_int3c_deriv(
     }
     __syncthreads();
     const int ng = (ni + 31) / 32;
-    for (int w = warp; w < ng * (Tab::NC * NA * NB); w += kDerivT / 32) {
+    for (int w = warp; w < ng * (Tab::NC * NA * NB); w += kInt3cT / 32) {
       const int li = (w % ng) * 32 + lane, f = w / ng;
       const int ic = f / (NA * NB), ia = f / NB % NA, ib = f % NB;
       if (li >= ni) continue;
@@ -839,45 +831,51 @@ void free_pairs(PairList& pl, cudaStream_t st) {
 }
 
 // ------------------------------------------------------------------ dispatch
+// Shell pairs per CTA: as many as fill the items held at a
+// time, fewer while the class has less than three CTAs an SM (a dd class has
+// a few hundred pairs) or their coefficients would leave less than three CTAs
+// an SM's shared memory.
+constexpr int kPairSmem = 72 * 1024;
+template <class Tab>
+static int pairs_per_cta(int np, int nax) {
+  int pb = std::min(cdiv(Tab::kItems, nax), std::max(1, np / (3 * 152)));
+  while (pb > 1 && Tab::bytes(pb) > kPairSmem) pb--;
+  return pb;
+}
+
+static PairSrc pair_src(const ShellSet& ao, const PairList& pl, int cls, const double* xyz) {
+  return {pl.a, pl.b, pl.class_off[cls], pl.class_off[cls + 1] - pl.class_off[cls],
+          ao.atom, ao.off, ao.ex, ao.nbase, xyz};
+}
+
 template <int LA, int LB, int LC>
 static void launch_int3c(const ShellSet& ao, const ShellSet& aux, const PairList& pl,
                          const double* xyz, const double* tab, int nJ, int nK, double* TJ,
                          double* TK, const long long* poff, cudaStream_t st) {
-  const int cls = LA * (LA + 1) / 2 + LB;
-  const int p0 = pl.class_off[cls], np = pl.class_off[cls + 1] - p0;
+  using Tab = Int3cTab<LA, LB, LC>;
+  const PairSrc src = pair_src(ao, pl, LA * (LA + 1) / 2 + LB, xyz);
   const int nax = (int)aux.by_l[LC].size();
-  if (np == 0 || nax == 0) return;
-  const long long nt = (long long)np * nax;
-  k_int3c<LA, LB, LC><<<(unsigned)cdiv(nt, 128), 128, 0, st>>>(
-      pl.a, pl.b, p0, np, aux.d_by_l[LC], nax, ao.atom, ao.off, ao.ex, ao.nbase, aux.atom, aux.ex,
-      aux.nbase, aux.jmap, aux.kmap, xyz, tab, ao.nfun, nJ, nK, TJ, TK, poff, aux.off);
+  if (src.np == 0 || nax == 0) return;
+  const int pb = pairs_per_cta<Tab>(src.np, nax);
+  static_assert(Tab::bytes(1) <= kPairSmem, "coefficients of one pair");
+  ensure_smem_attr((const void*)k_int3c<LA, LB, LC>, kPairSmem);
+  k_int3c<LA, LB, LC><<<cdiv(src.np, pb), kInt3cT, Tab::bytes(pb), st>>>(
+      src, pb, aux.d_by_l[LC], nax, aux.atom, aux.ex, aux.nbase, aux.jmap, aux.kmap, tab, ao.nfun, nJ,
+      nK, TJ, TK, poff, aux.off);
   RIS_CHECK_LAUNCH();
-}
-
-// Shell pairs per CTA of k_int3c_deriv: as many as fill the items held at a
-// time, fewer while the class has less than three CTAs an SM (a dd class has
-// a few hundred pairs) or their coefficients would leave less than three CTAs
-// an SM's shared memory.
-template <class Tab>
-static int deriv_pairs(int np, int nax) {
-  int pb = std::min(cdiv(Tab::kItems, nax), std::max(1, np / (3 * 152)));
-  while (pb > 1 && Tab::bytes(pb) > 72 * 1024) pb--;
-  return pb;
 }
 
 template <int LA, int LB, int LC, class T>
 static void launch_int3c_deriv(const ShellSet& ao, const ShellSet& aux, const PairList& pl,
                                const double* xyz, const double* tab, T* D, cudaStream_t st) {
   using Tab = DerivTab<LA, LB, LC>;
-  const int cls = LA * (LA + 1) / 2 + LB;
-  const PairSrc src{pl.a, pl.b, pl.class_off[cls], pl.class_off[cls + 1] - pl.class_off[cls],
-                    ao.atom, ao.off, ao.ex, ao.nbase, xyz};
+  const PairSrc src = pair_src(ao, pl, LA * (LA + 1) / 2 + LB, xyz);
   const int nax = (int)aux.by_l[LC].size();
   if (src.np == 0 || nax == 0) return;
-  const int pb = deriv_pairs<Tab>(src.np, nax);
-  static_assert(Tab::bytes(1) <= 72 * 1024, "coefficients of one pair");
-  ensure_smem_attr((const void*)k_int3c_deriv<LA, LB, LC, T>, 72 * 1024);
-  k_int3c_deriv<LA, LB, LC, T><<<cdiv(src.np, pb), kDerivT, Tab::bytes(pb), st>>>(
+  const int pb = pairs_per_cta<Tab>(src.np, nax);
+  static_assert(Tab::bytes(1) <= kPairSmem, "coefficients of one pair");
+  ensure_smem_attr((const void*)k_int3c_deriv<LA, LB, LC, T>, kPairSmem);
+  k_int3c_deriv<LA, LB, LC, T><<<cdiv(src.np, pb), kInt3cT, Tab::bytes(pb), st>>>(
       src, pb, aux.d_by_l[LC], nax, aux.atom, aux.off, aux.ex, aux.nbase, tab, ao.nfun, aux.nfun, D);
   RIS_CHECK_LAUNCH();
 }
