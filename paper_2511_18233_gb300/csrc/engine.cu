@@ -1066,21 +1066,40 @@ void divide_pairs(double* out, const double* num, const double* den, int npair, 
   RIS_CHECK_LAUNCH();
 }
 
-// out[j] = A_j . B_j (rows of length n), one block per row
-__global__ void k_row_dots(const double* __restrict__ A, const double* __restrict__ B, long long n,
-                           double* __restrict__ out) {
+// out[r] = sum_i A[r][i] B[r][i]: blockIdx.y = row, the row cut over
+// gridDim.x CTAs (one CTA a row had an SM's FP64 pipe to itself: 12.4 us at
+// 3 x 11k); the CTA of a row that finishes last adds the partial sums in
+// their order and resets the row's counter (part: gridDim.x a row).
+constexpr int kDotParts = 32;
+__global__ void __launch_bounds__(256) k_row_dots(const double* __restrict__ A, const double* __restrict__ B,
+                                                  long long n, double* __restrict__ part,
+                                                  int* __restrict__ count, double* __restrict__ out) {
   __shared__ double red[8];
-  const double* a = A + (size_t)blockIdx.x * n;
-  const double* b = B + (size_t)blockIdx.x * n;
+  __shared__ bool last;
+  const int r = blockIdx.y, np = gridDim.x;
+  const double* a = A + (size_t)r * n;
+  const double* b = B + (size_t)r * n;
+  const long long lo = n * blockIdx.x / np, hi = n * (blockIdx.x + 1) / np;
   double s = 0.0;
-  for (long long i = threadIdx.x; i < n; i += 256) s += a[i] * b[i];
+  for (long long i = lo + threadIdx.x; i < hi; i += 256) s += a[i] * b[i];
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < 8; w++) t += red[w];
-    out[blockIdx.x] = t;
+    part[(size_t)r * np + blockIdx.x] = t;
+    __threadfence();
+    last = atomicAdd(count + r, 1) == np - 1;
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return;
+  __threadfence();
+  s = threadIdx.x < np ? __ldcg(part + (size_t)r * np + threadIdx.x) : 0.0;
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (threadIdx.x == 0) {
+    out[r] = s;
+    count[r] = 0;
   }
 }
 
@@ -3311,7 +3330,13 @@ void Engine::zvector(int nr, const double* rhs_in, double* Z_out) {
   double* rzn = sc.p + 2 * nr;
   double* rr = sc.p + 3 * nr;
   double* bb = sc.p + 4 * nr;
-  SBuf<int> act(nr, st);
+  SBuf<int> act(nr, st), cnt(nr, st, true);
+  const int parts = (int)std::max(1LL, std::min<long long>(kDotParts, n / 512));
+  SBuf<double> part((size_t)nr * parts, st);
+  auto dots = [&](const double* u, const double* v, double* d) {
+    k_row_dots<<<dim3(parts, nr), 256, 0, st>>>(u, v, n, part.p, cnt.p, d);
+    RIS_CHECK_LAUNCH();
+  };
   copy_in(b.p, rhs_in, sz, st);
   RIS_CUDA(cudaMemcpyAsync(r.p, b.p, sizeof(double) * sz, cudaMemcpyDeviceToDevice, st));
   const bool mixed = opt.precision == RIS_MIXED;
@@ -3335,13 +3360,11 @@ void Engine::zvector(int nr, const double* rhs_in, double* Z_out) {
   if (cprec) cp.setup(*this, false, 4.0, nr);
   std::vector<int> h_act(nr, 1);
   std::vector<double> h_rr(nr), h_bb(nr);
-  k_row_dots<<<nr, 256, 0, st>>>(b.p, b.p, n, bb);
-  RIS_CHECK_LAUNCH();
+  dots(b.p, b.p, bb);
   RIS_CUDA(cudaMemcpyAsync(h_bb.data(), bb, sizeof(double) * nr, cudaMemcpyDeviceToHost, st));
   precondition(r.p, z.p);
   RIS_CUDA(cudaMemcpyAsync(p.p, z.p, sizeof(double) * sz, cudaMemcpyDeviceToDevice, st));
-  k_row_dots<<<nr, 256, 0, st>>>(r.p, z.p, n, rz);
-  RIS_CHECK_LAUNCH();
+  dots(r.p, z.p, rz);
   RIS_CUDA(cudaStreamSynchronize(st));
   for (int j = 0; j < nr; j++) h_act[j] = h_bb[j] > 0.0;
   int it = 0, nprod = 0;
@@ -3350,12 +3373,10 @@ void Engine::zvector(int nr, const double* rhs_in, double* Z_out) {
     RIS_CUDA(cudaMemcpyAsync(act.p, h_act.data(), sizeof(int) * nr, cudaMemcpyHostToDevice, st));
     apply_ApB_AmB(p.p, nr, q.p, nullptr);
     nprod += nr;
-    k_row_dots<<<nr, 256, 0, st>>>(p.p, q.p, n, pq);
-    RIS_CHECK_LAUNCH();
+    dots(p.p, q.p, pq);
     k_cg_xr<<<cdiv(n * nr, 256), 256, 0, st>>>(x.p, r.p, p.p, q.p, rz, pq, act.p, n, nr);
     RIS_CHECK_LAUNCH();
-    k_row_dots<<<nr, 256, 0, st>>>(r.p, r.p, n, rr);
-    RIS_CHECK_LAUNCH();
+    dots(r.p, r.p, rr);
     RIS_CUDA(cudaMemcpyAsync(h_rr.data(), rr, sizeof(double) * nr, cudaMemcpyDeviceToHost, st));
     RIS_CUDA(cudaStreamSynchronize(st));
     bool any = false;
@@ -3369,8 +3390,7 @@ void Engine::zvector(int nr, const double* rhs_in, double* Z_out) {
     }
     RIS_CUDA(cudaMemcpyAsync(act.p, h_act.data(), sizeof(int) * nr, cudaMemcpyHostToDevice, st));
     precondition(r.p, z.p);
-    k_row_dots<<<nr, 256, 0, st>>>(r.p, z.p, n, rzn);
-    RIS_CHECK_LAUNCH();
+    dots(r.p, z.p, rzn);
     k_cg_p<<<cdiv(n * nr, 256), 256, 0, st>>>(p.p, z.p, rzn, rz, act.p, n, nr);
     RIS_CHECK_LAUNCH();
     RIS_CUDA(cudaMemcpyAsync(rz, rzn, sizeof(double) * nr, cudaMemcpyDeviceToDevice, st));
