@@ -40,13 +40,15 @@
 //                     integers first and handed back, so that the next chunk
 //                     or tile runs on the tensor cores while the results are
 //                     rounded and stored
-// FP64 arithmetic is kept out of the epilogue (GB300 issues about 1.7 FP64
-// operations per clock per SM, so five per output would cost a 128 x 48 tile
-// 18k cycles, the time of 270 values of k): the result is rounded to FP64
-// with integer operations, bit for bit what the FP64 combination gives.
+// FP64 arithmetic is scarce in the epilogue (GB300 issues about 1.7 FP64
+// operations per clock per SM, so each per output costs a 128 x 48 tile 3.6k
+// cycles, the time of 55 values of k): a single conversion and FMA round the
+// result of up to eight chunks, longer sums are rounded with integer
+// operations, bit for bit the same.
 // Every mbarrier wait is bounded; a timeout sets the error flag, drains what
 // the CTA has in flight and frees its tensor memory.
 #include <algorithm>
+#include <cmath>
 
 #include "gemm_emu.cuh"
 #include "tc_ptx.cuh"
@@ -125,6 +127,8 @@ struct EmuArgs {
   longlong2* ws;   // split contraction: [slice][M][N] integer partial sums
   EmuEpilogue ep;
   int mode;        // 0: C = x, 1: C = alpha x, 2: C = alpha x + beta C
+  int ashift;      // x is taken times 2^ashift, negated if aneg (a power of two
+  int aneg;        // as alpha costs no FP64 operation)
   int* err;
 };
 
@@ -215,6 +219,7 @@ __device__ __forceinline__ long long emu_round53(long long lo) {
   return lo < 0 ? -(long long)a : (long long)a;
 }
 
+constexpr int kQuickK = 112;  // EmuAcc::quick from this contraction length on
 // Sum of one output over the chunks.
 template <class F>
 struct EmuAcc;
@@ -235,6 +240,27 @@ struct EmuAcc<Form9x7> {
     return emu_round(hi, lo, kShift, e - 2 * Form9x7::kFrac + 56);
   }
   __device__ __forceinline__ double result(int e) const { return value(hi, lo, e); }
+  // The same from at most kQuickChunks chunks (|hi + lo 2^-35| < 2^50) with two
+  // FP64 operations: lo's upper bits are carried into hi, which is turned into
+  // FP64 by its bit pattern and one subtraction, and one FMA adds the lower 35
+  // bits and rounds.  They enter as the bit pattern of 2^52 + bits, the 2^52
+  // having been taken from hi.  emu_round's hundred integer instructions in a
+  // row take longer (21504 x 512 over 142, an exchange density of C20H22: 165
+  // -> 148 us), but below kQuickK the products of a tile are done before its
+  // FP64 operations (2982 x 512 over 71: 27 -> 30 us), so it stays there.
+  static constexpr int kQuickChunks = 8;
+  __device__ __forceinline__ double quick(int e) const {
+    const long long h = hi + (lo >> kShift) - (1ll << 17);
+    const double lm = __longlong_as_double(0x4330000000000000ll | (lo & ((1ll << kShift) - 1)));
+    const double hd = __longlong_as_double(0x4338000000000000ll + h) - 6755399441055744.0;  // 1.5 2^52
+    const double x = fma(hd, 34359738368.0, lm);
+    const int sh = e - 2 * Form9x7::kFrac + 56;
+    const long long b = __double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7FF) + sh;
+    if ((b << 1) == 0) return x;
+    if (ex < 1 || ex > 2046) return ldexp(x, sh);
+    return __longlong_as_double(b + ((long long)sh << 52));
+  }
 };
 // 10 x 6: hi = V_0 2^12 + V_1 2^6 + V_2, lo = sum_{g>=3} V_g 2^(6(9-g)) < 2^61;
 // each chunk is fl(hi 2^42 + fl(lo)) (one conversion and one FMA in FP64),
@@ -256,6 +282,8 @@ struct EmuAcc<Form10x6> {
     s = first ? x : s + x;
   }
   __device__ __forceinline__ double result(int) const { return s; }
+  static constexpr int kQuickChunks = 0;
+  __device__ __forceinline__ double quick(int) const { return s; }
 };
 
 template <class F, int bn>
@@ -447,6 +475,8 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
       if (!good) break;
       double* prow = ep.c64 + emu_off(row, ep.rin, ep.rld, ep.rs);
       const int lrow = ep.lead ? ((row / ep.lrd) % ep.lrm) * ep.lrs : 0;
+      const bool quick = args.cps <= EmuAcc<F>::kQuickChunks && args.K >= kQuickK;
+      const bool bad = __any_sync(0xffffffffu, row_bad(lr) || row_bad(lc));
       const bool one_row = __all_sync(0xffffffffu, lrow == __shfl_sync(0xffffffffu, lrow, 0) && live);
       int lcur = -1, lmax = kEmuNoLead;
       auto flush = [&] {  // the running exponent of lead column lcur
@@ -466,7 +496,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
           const int jc = 4 * b + j;
           if (n0 + jc >= args.N) continue;  // warp-uniform
           const int lcj = __shfl_sync(0xffffffffu, lc, jc);
-          const long long cj = __shfl_sync(0xffffffffu, coff, jc);
+          const long long cj = ep.cin > 0 ? __shfl_sync(0xffffffffu, coff, jc) : (long long)(n0 + jc) * ep.cs;
           if constexpr (F::kBalanced) {
             if (args.ws) {  // one slice of the contraction: integer partial sums
               longlong2 s;
@@ -476,8 +506,10 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
               continue;
             }
           }
-          double x = acc[b][j].result(er + row_frame(lcj));
-          if (row_bad(lr) || row_bad(lcj)) x = __longlong_as_double(0x7ff8000000000000ll);
+          const int e = er + row_frame(lcj) + args.ashift;
+          double x = quick ? acc[b][j].quick(e) : acc[b][j].result(e);
+          if (args.aneg) x = __longlong_as_double(__double_as_longlong(x) ^ (1ll << 63));
+          if (bad && (row_bad(lr) || row_bad(lcj))) x = __longlong_as_double(0x7ff8000000000000ll);
           if (ep.lead) {
             const int li = __shfl_sync(0xffffffffu, lidx, jc);
             if (li != lcur) {
@@ -519,7 +551,8 @@ __global__ void __launch_bounds__(256) k_emu_finish(EmuArgs args, int nsplit) {
   }
   const int row = (int)(t / args.N), col = (int)(t % args.N);
   const int lr = args.ea[row], lc = args.eb[col];
-  double x = EmuAcc<Form9x7>::value(hi, lo, row_frame(lr) + row_frame(lc));
+  double x = EmuAcc<Form9x7>::value(hi, lo, row_frame(lr) + row_frame(lc) + args.ashift);
+  if (args.aneg) x = __longlong_as_double(__double_as_longlong(x) ^ (1ll << 63));
   if (row_bad(lr) || row_bad(lc)) x = __longlong_as_double(0x7ff8000000000000ll);
   const EmuEpilogue& ep = args.ep;
   if (ep.lead)
@@ -768,6 +801,13 @@ void gemm_pass(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
   a.ws = nullptr;
   a.ep = ep;
   a.mode = ep.beta != 0.0 ? 2 : ep.alpha != 1.0 ? 1 : 0;
+  a.ashift = a.aneg = 0;
+  int ax = 0;
+  if (F::kBalanced && a.mode == 1 && std::fabs(std::frexp(ep.alpha, &ax)) == 0.5 && std::abs(ax) < 256) {
+    a.mode = 0;
+    a.ashift = ax - 1;
+    a.aneg = ep.alpha < 0.0;
+  }
   a.err = d_err;
   const long long tiles = (long long)a.ntn * cdiv(M, EBM);
   RIS_REQUIRE(tiles * 64 < (1LL << 31), RIS_ERR_ARG, "emu_gemm: too many tiles");
