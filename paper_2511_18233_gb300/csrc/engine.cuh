@@ -256,7 +256,8 @@ struct Engine : StreamOwner {
   void ensure_emu_ops();
   void release_emu_ops();
   void check_tcerr();  // throws if a tensor-core pipeline wait timed out (synchronises)
-  void emu97(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep);
+  void emu97(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep,
+             const EmuBatch& bt = EmuBatch());
   void build_K_emu(const double* HK, double* Bvv);
   // K1 (alpha, beta into out) and, when K2 is given, K2 of exchange_terms
   void exchange_emu(const double* Z, int nvec, double* K1, double alpha, double beta, double* K2);

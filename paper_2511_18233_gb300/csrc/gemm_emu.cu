@@ -117,15 +117,16 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
 
 struct EmuArgs {
   int M, N, K;
-  int ntn, tiles;       // column tiles (fastest), all tiles
+  int ntn, tiles1, tiles;  // column tiles (fastest), tiles of a product, all tiles
   int nchunk, cps, ns;  // chunks of the contraction, chunks per slice of it, slices
   const __half* sa;     // digits; elements between K steps
   const __half* sb;
   long long pa, pb;
   const int* ea;
   const int* eb;
-  longlong2* ws;   // split contraction: [slice][M][N] integer partial sums
+  longlong2* ws;   // split contraction: [slice][product][M][N] integer partial sums
   EmuEpilogue ep;
+  EmuBatch bt;
   int mode;        // 0: C = x, 1: C = alpha x, 2: C = alpha x + beta C
   int ashift;      // x is taken times 2^ashift, negated if aneg (a power of two
   int aneg;        // as alpha costs no FP64 operation)
@@ -334,7 +335,8 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
     bool stop = false;  // warp-uniform
     for (int w = blockIdx.x; w < items && !stop; w += gridDim.x) {
       const int t = w % args.tiles, c0 = (w / args.tiles) * args.cps;
-      const int n0 = (t % args.ntn) * bn, m0 = (t / args.ntn) * EBM;
+      const int pr = t / args.tiles1, t1 = t - pr * args.tiles1;
+      const int n0 = (t1 % args.ntn) * bn + args.bt.b[pr], m0 = (t1 / args.ntn) * EBM + args.bt.a[pr];
       const int s0 = c0 * kSteps;
       const int s1 = min((args.K + EBK - 1) / EBK, (c0 + args.cps) * kSteps);
       const __half* ga = args.sa + (size_t)s0 * args.pa + (size_t)m0 * (16 * S);
@@ -428,14 +430,15 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
     for (int w = blockIdx.x; w < items && good; w += gridDim.x) {
       const int t = w % args.tiles, z = w / args.tiles, c0 = z * args.cps;
       const int nc = min(args.nchunk, c0 + args.cps) - c0;
-      const int n0 = (t % args.ntn) * bn + cg * ncol;
-      const int row = (t / args.ntn) * EBM + quad * 32 + lane;
+      const int pr = t / args.tiles1, t1 = t - pr * args.tiles1;
+      const int n0 = (t1 % args.ntn) * bn + cg * ncol;
+      const int row = (t1 / args.ntn) * EBM + quad * 32 + lane;
       const bool live = row < args.M;
-      const int lr = live ? args.ea[row] : kEmuNoLead;
+      const int lr = live ? args.ea[row + args.bt.a[pr]] : kEmuNoLead;
       const int er = row_frame(lr);
       // lane j < ncol holds column j's exponent and output offset
       const int mc = n0 + lane;
-      const int lc = (lane < ncol && mc < args.N) ? args.eb[mc] : kEmuNoLead;
+      const int lc = (lane < ncol && mc < args.N) ? args.eb[mc + args.bt.b[pr]] : kEmuNoLead;
       long long coff = 0;
       int lidx = 0;
       if (lane < ncol && mc < args.N) {
@@ -473,7 +476,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
         if (lane == 0) mbar_arrive(acc_empty);
       }
       if (!good) break;
-      double* prow = ep.c64 + emu_off(row, ep.rin, ep.rld, ep.rs);
+      double* prow = ep.c64 + args.bt.c[pr] + emu_off(row, ep.rin, ep.rld, ep.rs);
       const int lrow = ep.lead ? ((row / ep.lrd) % ep.lrm) * ep.lrs : 0;
       const bool quick = args.cps <= EmuAcc<F>::kQuickChunks && args.K >= kQuickK;
       const bool bad = __any_sync(0xffffffffu, row_bad(lr) || row_bad(lc));
@@ -502,7 +505,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
               longlong2 s;
               s.x = acc[b][j].hi;
               s.y = acc[b][j].lo;
-              if (live) args.ws[((size_t)z * args.M + row) * args.N + n0 + jc] = s;
+              if (live) args.ws[((size_t)(z * args.bt.n + pr) * args.M + row) * args.N + n0 + jc] = s;
               continue;
             }
           }
@@ -541,7 +544,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_emu_gemm(EmuArgs args) {
 // and rounds once.
 __global__ void __launch_bounds__(256) k_emu_finish(EmuArgs args, int nsplit) {
   const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
-  const long long mn = (long long)args.M * args.N;
+  const long long mn = (long long)args.M * args.N * args.bt.n;
   if (t >= mn) return;
   long long hi = 0, lo = 0;
   for (int z = 0; z < nsplit; z++) {
@@ -549,8 +552,10 @@ __global__ void __launch_bounds__(256) k_emu_finish(EmuArgs args, int nsplit) {
     hi += w.x;
     lo += w.y;
   }
-  const int row = (int)(t / args.N), col = (int)(t % args.N);
-  const int lr = args.ea[row], lc = args.eb[col];
+  const int pr = (int)(t / ((long long)args.M * args.N));
+  const long long q = t - (long long)pr * args.M * args.N;
+  const int row = (int)(q / args.N), col = (int)(q % args.N);
+  const int lr = args.ea[row + args.bt.a[pr]], lc = args.eb[col + args.bt.b[pr]];
   double x = EmuAcc<Form9x7>::value(hi, lo, row_frame(lr) + row_frame(lc) + args.ashift);
   if (args.aneg) x = __longlong_as_double(__double_as_longlong(x) ^ (1ll << 63));
   if (row_bad(lr) || row_bad(lc)) x = __longlong_as_double(0x7ff8000000000000ll);
@@ -558,7 +563,7 @@ __global__ void __launch_bounds__(256) k_emu_finish(EmuArgs args, int nsplit) {
   if (ep.lead)
     atomicMax(ep.lead + ((row / ep.lrd) % ep.lrm) * ep.lrs + ((col / ep.lcd) % ep.lcm) * ep.lcs,
               lead_exp(x));
-  double* p = ep.c64 + emu_off(row, ep.rin, ep.rld, ep.rs) + emu_off(col, ep.cin, ep.cld, ep.cs);
+  double* p = ep.c64 + args.bt.c[pr] + emu_off(row, ep.rin, ep.rld, ep.rs) + emu_off(col, ep.cin, ep.cld, ep.cs);
   store_out(p, x, args.mode, ep.alpha, ep.beta);
 }
 
@@ -647,7 +652,17 @@ __device__ __forceinline__ void put8(const double (&x)[8], int lead, __half* o, 
 
 __device__ __forceinline__ bool src_row(const EmuSource& src, int r, int rows, long long& off) {
   if (r >= rows) return false;
-  off = emu_off(r, src.rin, src.rld, src.rs);
+  long long base = 0;
+  if (src.bin > 0) {
+    const int blk = r / src.bin;
+    r -= blk * src.bin;
+    base = (long long)blk * src.bld;
+    if (r >= src.bvalid) {
+      off = base;
+      return false;
+    }
+  }
+  off = base + emu_off(r, src.rin, src.rld, src.rs);
   return src.rvalid == 0 || r % src.rin < src.rvalid;
 }
 
@@ -783,7 +798,7 @@ void slice_form(const EmuSource& src, int rows, int K, EmuOperand& op, cudaStrea
 
 template <class F>
 void gemm_pass(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep,
-               int* d_err, cudaStream_t st) {
+               int* d_err, cudaStream_t st, const EmuBatch& bt) {
   EmuArgs a;
   a.M = M;
   a.N = N;
@@ -809,7 +824,9 @@ void gemm_pass(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
     a.aneg = ep.alpha < 0.0;
   }
   a.err = d_err;
-  const long long tiles = (long long)a.ntn * cdiv(M, EBM);
+  a.bt = bt;
+  a.tiles1 = a.ntn * cdiv(M, EBM);
+  const long long tiles = (long long)a.ntn * cdiv(M, EBM) * bt.n;
   RIS_REQUIRE(tiles * 64 < (1LL << 31), RIS_ERR_ARG, "emu_gemm: too many tiles");
   a.tiles = (int)tiles;
   // slices of a long contraction: the number of chunk rounds of the busiest
@@ -820,7 +837,7 @@ void gemm_pass(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
     for (int s = 1; s <= std::min(a.nchunk, 64); s++) {
       const int cps = cdiv(a.nchunk, s);
       if (cdiv(a.nchunk, cps) != s) continue;
-      if (s > 1 && (double)s * M * N * sizeof(longlong2) > 1e9) break;
+      if (s > 1 && (double)s * M * N * bt.n * sizeof(longlong2) > 1e9) break;
       const long long cost = (long long)cdiv(tiles * s, 152) * (2 * cps + 1);
       if (best < 0 || cost < best) {
         best = cost;
@@ -831,14 +848,14 @@ void gemm_pass(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
   a.cps = cdiv(a.nchunk, ns);
   a.ns = ns;
   MemTrack* tr = nullptr;
-  const size_t wsb = (size_t)ns * M * N * sizeof(longlong2);
+  const size_t wsb = (size_t)ns * M * N * bt.n * sizeof(longlong2);
   if (ns > 1) a.ws = (longlong2*)dev_alloc(wsb, st, &tr);
   auto kern = bn == 48 ? k_emu_gemm<F, 48> : bn == 32 ? k_emu_gemm<F, 32> : k_emu_gemm<F, 16>;
   ensure_smem_attr((const void*)kern, Tile<F>::kSmem);
   kern<<<(unsigned)std::min<long long>(tiles * ns, 152), ETHREADS, Tile<F>::kSmem, st>>>(a);
   RIS_CHECK_LAUNCH();
   if (ns > 1) {
-    k_emu_finish<<<cdiv((long long)M * N, 256), 256, 0, st>>>(a, ns);
+    k_emu_finish<<<cdiv((long long)M * N * bt.n, 256), 256, 0, st>>>(a, ns);
     RIS_CHECK_LAUNCH();
     dev_free(a.ws, wsb, st, tr);
   }
@@ -849,7 +866,7 @@ void gemm_pass(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
 constexpr int kPassChunks = 512;
 template <class F>
 void gemm_form(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep,
-               int* d_err, cudaStream_t st) {
+               int* d_err, cudaStream_t st, const EmuBatch& bt) {
   prof_begin(kProfEmuGemm, st);
   constexpr int kPass = kPassChunks * F::kChunk;
   for (int k0 = 0; k0 < A.K; k0 += kPass) {
@@ -859,9 +876,9 @@ void gemm_form(int M, int N, const EmuOperand& A, const EmuOperand& B, const Emu
     b.s = B.s + (size_t)(k0 / EBK) * F::S * 16 * B.blocks * B.rb;
     a.K = b.K = std::min(kPass, A.K - k0);
     if (k0 > 0) e.beta = 1.0;
-    gemm_pass<F>(M, N, a, b, e, d_err, st);
+    gemm_pass<F>(M, N, a, b, e, d_err, st, bt);
   }
-  prof_end(kProfEmuGemm, st, 2.0 * M * N * (double)A.K);
+  prof_end(kProfEmuGemm, st, 2.0 * M * N * (double)A.K * bt.n);
 }
 
 }  // namespace
@@ -891,17 +908,21 @@ void emu_slice(EmuForm f, const EmuSource& src, int rows, int K, EmuOperand& op,
 }
 
 void emu_gemm(EmuForm f, int M, int N, const EmuOperand& A, const EmuOperand& B,
-              const EmuEpilogue& ep, int* d_err, cudaStream_t st) {
+              const EmuEpilogue& ep, int* d_err, cudaStream_t st, const EmuBatch& bt) {
   if (M <= 0 || N <= 0) return;
   RIS_REQUIRE(A.K == B.K && A.K > 0, RIS_ERR_ARG, "emu_gemm: contraction lengths differ");
-  RIS_REQUIRE(A.rows >= M && B.rows >= N, RIS_ERR_ARG, "emu_gemm: operand rows");
+  RIS_REQUIRE(bt.n >= 1 && bt.n <= 8 && (bt.n == 1 || !ep.lead), RIS_ERR_ARG, "emu_gemm: batch");
+  for (int p = 0; p < bt.n; p++) {
+    RIS_REQUIRE(A.rows - bt.a[p] >= M && B.rows - bt.b[p] >= N, RIS_ERR_ARG, "emu_gemm: operand rows");
+    RIS_REQUIRE(bt.a[p] % kEmuRowsA == 0 && bt.b[p] % B.rb == 0, RIS_ERR_ARG, "emu_gemm: batch rows");
+  }
   RIS_REQUIRE(A.rb == kEmuRowsA && (B.rb == 48 || B.rb == 32 || B.rb == 16), RIS_ERR_ARG,
               "emu_gemm: operand row blocks");
   RIS_REQUIRE(A.slices == emu_slices(f) && B.slices == A.slices, RIS_ERR_ARG, "emu_gemm: operand form");
   if (f == kEmu10x6)
-    gemm_form<Form10x6>(M, N, A, B, ep, d_err, st);
+    gemm_form<Form10x6>(M, N, A, B, ep, d_err, st, bt);
   else
-    gemm_form<Form9x7>(M, N, A, B, ep, d_err, st);
+    gemm_form<Form9x7>(M, N, A, B, ep, d_err, st, bt);
 }
 
 }  // namespace ris

@@ -41,14 +41,6 @@ struct EmuOperand {
   int rb = 0;
   long long blocks = 0;  // row blocks
   int slices = 0;
-  // rows r0 .. r0 + n - 1, r0 a multiple of rb
-  EmuOperand sub(long long r0, int n) const {
-    EmuOperand o = *this;
-    o.s += r0 * 16 * slices;
-    o.e += r0;
-    o.rows = n;
-    return o;
-  }
 };
 
 inline int emu_pad(int n, int rb) { return (n + rb - 1) / rb * rb; }
@@ -59,13 +51,17 @@ inline size_t emu_size(EmuForm f, long long rows, int K, int rb) {
 
 // Source placement: element (r, k) of an operand at src[row(r) + k * ks] with
 // row(r) = (r / rin) * rld + (r % rin) * rs (rin = 0: r * rs); rows with
-// r % rin >= rvalid are zero (rvalid = 0: none).
+// r % rin >= rvalid are zero (rvalid = 0: none).  With bin > 0 the rows come in
+// blocks of bin: block r / bin starts at (r / bin) * bld, its rows from bvalid
+// on are zero and the others are placed as above.
 struct EmuSource {
   const double* p = nullptr;
   long long rs = 0, ks = 1;
   int rin = 0;
   long long rld = 0;
   int rvalid = 0;
+  int bin = 0, bvalid = 0;
+  long long bld = 0;
 };
 
 // Slices src (rows x K) into op (op.rb set; op.s / op.e hold emu_size / rows
@@ -93,9 +89,18 @@ struct EmuEpilogue {
   void lead_cols(int d, int m, int s) { lcd = d; lcm = m; lcs = s; }
 };
 
+// Products that share a launch: product p takes A from row a[p] (a multiple of
+// kEmuRowsA), B from row b[p] (a multiple of its rb) and writes at c64 + c[p]
+// (without `lead`).
+struct EmuBatch {
+  int n = 1;
+  int a[8] = {0}, b[8] = {0};
+  long long c[8] = {0};
+};
+
 // C (M x N) = A (M x K) . B (N x K)^T from operands sliced in form f; *d_err
 // (device int) is set non-zero if a pipeline wait timed out.
 void emu_gemm(EmuForm f, int M, int N, const EmuOperand& A, const EmuOperand& B,
-              const EmuEpilogue& ep, int* d_err, cudaStream_t st);
+              const EmuEpilogue& ep, int* d_err, cudaStream_t st, const EmuBatch& bt = EmuBatch());
 
 }  // namespace ris

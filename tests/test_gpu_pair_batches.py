@@ -24,8 +24,9 @@ def ris_mod():
 @gpu
 @pytest.mark.parametrize("rpa", [0, 1])
 @pytest.mark.parametrize("precision", ["f64", "mixed"])
-def test_lists_of_pairs(ris_mod, precision, rpa):
-    mol = synth.chain_molecule(6, 31, True)
+@pytest.mark.parametrize("size", [6, 8])  # FP64 exchange densities on the FP64 pipe / emulated
+def test_lists_of_pairs(ris_mod, size, precision, rpa):
+    mol = synth.chain_molecule(size, 31, True)
     n = 11
     X = synth.random_amplitudes(n, mol.nocc, mol.nvir, seed=3)
     Y = 0.1 * synth.random_amplitudes(n, mol.nocc, mol.nvir, seed=4) if rpa else None
