@@ -463,12 +463,14 @@ def main():
     return 0
 
 
-def algorithmic_work(precision, d, nprod, npair, rpa=False, ff=True):
+def algorithmic_work(precision, d, nprod, npair, rpa=False, ff=True, emu=False):
     """The method's own work per evaluation and kernel class (scope-table
     counts, dense, no screening credit): flops for the GEMM classes (a
     3xTF32 or double-FP32 product counts once), bytes are reported by the
     library.  In the mixed form the Coulomb part of A.X runs as double-FP32
-    products (option subspace_ff, on by default)."""
+    products (option subspace_ff, on by default).  emu: the FP64 form with its
+    builds, exchange products and exchange densities as emulated FP64 products
+    (option emu_f64, on by default, systems above a size)."""
     n, o, v, nJ, nK = d["nao"], d["nocc"], d["nvir"], d["nJ"], d["nK"]
     nov = o * v
     coul_ax = 4.0 * nov * nJ * nprod * (2 if rpa else 1)
@@ -476,6 +478,8 @@ def algorithmic_work(precision, d, nprod, npair, rpa=False, ff=True):
     b_coul = 2.0 * o * n * n * nJ + 2.0 * o * v * n * nJ
     b_k = 2.0 * o * n * n * nK + 2.0 * o * o * n * nK + 2.0 * v * n * n * nK + 2.0 * v * v * n * nK
     gam = (2.0 * o * v * v * nK + 4.0 * n * n * o * nK) * npair
+    if precision == "fp64" and emu:
+        return {"dgemm_fp64": coul_ax, "emu_gemm_f64": exch_ax + b_coul + b_k + gam}
     if precision == "fp64":
         return {"dgemm_fp64": coul_ax + exch_ax + b_coul + b_k + gam}
     return {"dgemm_fp64": (0.0 if ff else coul_ax) + 2.0 * o * o * n * nK,
@@ -488,16 +492,18 @@ def classify(st, steps, step_ms_total, precision, dims, nprod, npair, workload="
     """Per kernel class: time share, executed and algorithmic work against
     the pipe's measured peak."""
     pk = peaks()
-    alg = algorithmic_work(precision, dims, nprod, npair)
+    f64emu = precision == "fp64" and st["emu_gemm_ms"] > 0
+    alg = algorithmic_work(precision, dims, nprod, npair, emu=f64emu)
     tf32x3 = pk["tf32_tflops"] / 3.0           # three TF32 passes per product
-    emu = pk["f16_tflops"] / 55.0               # 55 FP16 slice products per FP64 product
+    slices = 45 if f64emu else 55               # FP16 slice products per FP64 product (9 x 7 / 10 x 6 bits)
+    emu = pk["f16_tflops"] / slices
     ffx = pk["fp32_tflops"] / 12.0              # 12 FP32 instructions per double-FP32 multiply-add
     classes = {
         "tc_gemm_3xtf32": (st["tc_gemm_ms"], st["tc_gemm_flops"], "tensor (tf32)", tf32x3,
                            "TF32 tcgen05 probe / 3 passes"),
         "dgemm_fp64": (st["gemm_ms"], st["gemm_flops"], "fp64 fma", pk["fp64_tflops"], "FP64 FMA probe"),
         "emu_gemm_f64": (st["emu_gemm_ms"], st["emu_gemm_flops"], "tensor (f16)", emu,
-                         "FP16 tcgen05 probe / 55 slice products (FP64-equivalent)"),
+                         f"FP16 tcgen05 probe / {slices} slice products (FP64-equivalent)"),
         "ff_gemm_f64x": (st.get("ff_gemm_ms", 0.0), st.get("ff_gemm_flops", 0.0), "fp32 fma (double-FP32)",
                          ffx, "FP32 FMA probe / 12 instructions per multiply-add"),
         "contract": (st["contract_ms"], None, "hbm", None, "HBM copy"),
