@@ -7,19 +7,18 @@
 // about FP32 accuracy at tensor-core rates.
 //
 // Kernel structure (one output tile of 128 x up to 128 per CTA, 128 threads):
-//   warp 0 / lane 0 : TMA producer, ring of (A_hi, A_lo, B_hi, B_lo) tiles of
-//                     128 rows x 16 FP32 (64-byte swizzle), 32 KB a stage
+//   warp 0 / lane 0 : TMA producer, 3-stage ring of (A_hi, A_lo, B_hi, B_lo)
+//                     tiles of 128 rows x BK FP32 (swizzled over the row)
 //   warp 1          : allocates 128 TMEM columns; lane 0 issues
 //                     tcgen05.mma.kind::tf32 (M=128, N <= 128, K=8) and commits
 //                     each stage back to the producer through an mbarrier
 //   warps 0-3       : epilogue, tcgen05.ld of TMEM lanes 32w..32w+31
-// The contractions are short (K = 71 ... 441 on C20H22), so that a tile's
+// Many contractions are short (K = 71 ... 441 on C20H22), so that a tile's
 // start (TMEM, barriers, first loads) and its epilogue (about 3000 cycles for
-// 128 x 128 stored as hi/lo) weigh as much as its products: a ring of three
-// stages takes 97 KB and leaves room for a second CTA on the SM, whose
-// products run meanwhile.  Grids of at most one CTA per SM take six stages
-// instead (exchange products of 18 C20H22 vectors
-// 254 -> 224 us; a mixed C20H22 evaluation's 170 launches 4474 -> 4156 us.)
+// 128 x 128 stored as hi/lo) weigh as much as its products: with BK = 16 the
+// ring takes 97 KB and leaves room for a second CTA on the SM, whose products
+// run meanwhile; BK = 32 (193 KB) is the form of long contractions and small
+// grids (the rule and its figures stand at the launch).
 // All mbarrier waits are bounded (about one second of clock64 cycles); a
 // timeout sets the error flag, drains what this CTA has in flight and frees
 // its TMEM before returning.
@@ -38,14 +37,14 @@ namespace ris {
 namespace {
 using namespace tcx;
 
-constexpr int BM = 128, BN = 128, BK = 16;
+constexpr int BM = 128, BN = 128, STAGES = 3;
 constexpr int KB = 32;  // slices of a split contraction are multiples of this
-constexpr int TILE_BYTES = BM * BK * 4;                      // 8 KB
-constexpr int STAGE_BYTES = 4 * TILE_BYTES;                  // hi/lo of A and B
-constexpr int smem_bytes(int stages) { return stages * STAGE_BYTES + 1024 + 256; }
+constexpr int tile_bytes(int bk) { return BM * bk * 4; }
+constexpr int smem_bytes(int bk) { return STAGES * 4 * tile_bytes(bk) + 1024 + 256; }  // hi/lo of A and B
 
-// 3-D map {K, rows, batch} of FP32, box {16, box_rows, 1}, 64-byte swizzle.
-CUtensorMap make_map(const float* base, int K, int rows, int ld, long long bstride, int nb, int box_rows) {
+// 3-D map {K, rows, batch} of FP32, box {bk, box_rows, 1}, rows of a box
+// swizzled over their 64 (bk = 16) or 128 bytes.
+CUtensorMap make_map(const float* base, int K, int rows, int ld, long long bstride, int nb, int box_rows, int bk) {
   RIS_REQUIRE(base != nullptr, RIS_ERR_ARG, "tc_gemm: null operand");
   RIS_REQUIRE(((uintptr_t)base & 15) == 0, RIS_ERR_ARG, "tc_gemm: operand not 16-byte aligned");
   RIS_REQUIRE(ld % 4 == 0 && (nb == 1 || bstride % 4 == 0), RIS_ERR_ARG,
@@ -53,22 +52,23 @@ CUtensorMap make_map(const float* base, int K, int rows, int ld, long long bstri
   CUtensorMap m;
   cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)nb};
   cuuint64_t strides[2] = {(cuuint64_t)ld * 4, (cuuint64_t)(nb > 1 ? bstride : (long long)ld * rows) * 4};
-  cuuint32_t box[3] = {BK, (cuuint32_t)box_rows, 1};
+  cuuint32_t box[3] = {(cuuint32_t)bk, (cuuint32_t)box_rows, 1};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)base, dims, strides, box, es,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, bk == 16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   RIS_REQUIRE(r == CUDA_SUCCESS, RIS_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
   return m;
 }
 
-// K-major operand tile of 128 rows x 64 bytes with 64-byte swizzle: start
-// address, leading offset unused (1), stride 512 B between 8-row groups,
-// descriptor version 1, layout type 4 (SWIZZLE_64B).
-__device__ __forceinline__ uint64_t desc_sw64(const void* p) {
+// K-major operand tile of 128 rows x 4 BK bytes swizzled over its rows: start
+// address, leading offset unused (1), 8 rows between groups, descriptor
+// version 1, layout type 4 (SWIZZLE_64B) or 2 (SWIZZLE_128B).
+template <int BK>
+__device__ __forceinline__ uint64_t desc_sw(const void* p) {
   const uint64_t a = sa(p);
-  return ((a & 0x3FFFFull) >> 4) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) |
-         (4ull << 61);
+  return ((a & 0x3FFFFull) >> 4) | (1ull << 16) | ((uint64_t)(8 * BK * 4 >> 4) << 32) | (1ull << 46) |
+         ((BK == 16 ? 4ull : 2ull) << 61);
 }
 
 // kind::tf32 instruction descriptor: D FP32 (bit 4), A and B TF32 (2 at bits
@@ -116,12 +116,13 @@ struct TcArgs {
   int* err;
 };
 
-template <int STAGES>
+template <int BK>
 __global__ void __launch_bounds__(128, 2) k_tc_gemm(const __grid_constant__ CUtensorMap mAh,
                                                      const __grid_constant__ CUtensorMap mAl,
                                                      const __grid_constant__ CUtensorMap mBh,
                                                      const __grid_constant__ CUtensorMap mBl,
                                                      TcArgs args) {
+  constexpr int TILE_BYTES = tile_bytes(BK), STAGE_BYTES = 4 * TILE_BYTES;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + STAGES * STAGE_BYTES);
@@ -194,8 +195,8 @@ __global__ void __launch_bounds__(128, 2) k_tc_gemm(const __grid_constant__ CUte
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       uint8_t* st = smem + s * STAGE_BYTES;
-      const uint64_t ah = desc_sw64(st), al = desc_sw64(st + TILE_BYTES);
-      const uint64_t bh = desc_sw64(st + 2 * TILE_BYTES), bl = desc_sw64(st + 3 * TILE_BYTES);
+      const uint64_t ah = desc_sw<BK>(st), al = desc_sw<BK>(st + TILE_BYTES);
+      const uint64_t bh = desc_sw<BK>(st + 2 * TILE_BYTES), bl = desc_sw<BK>(st + 3 * TILE_BYTES);
 #pragma unroll
       for (int kk = 0; kk < BK / 8; kk++) {
         const uint64_t off = (uint64_t)((kk * 32) >> 4);  // 32 bytes per K=8 step
@@ -408,10 +409,6 @@ void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb
   // last one is padding: N = 441 as four tiles of 112, 71 as one of 80
   // (12% and 37% of the tensor time of such a product)
   const int bn = cdiv(cdiv(N, cdiv(N, BN)), 16) * 16;
-  const CUtensorMap mAh = make_map(A.hi, K, M, A.ld, A.bstride, A.nb, BM);
-  const CUtensorMap mAl = make_map(A.lo, K, M, A.ld, A.bstride, A.nb, BM);
-  const CUtensorMap mBh = make_map(B.hi, K, N, B.ld, B.bstride, B.nb, bn);
-  const CUtensorMap mBl = make_map(B.lo, K, N, B.ld, B.bstride, B.nb, bn);
   TcArgs a;
   a.bn = bn;
   a.M = M;
@@ -453,11 +450,23 @@ void tc_gemm(int M, int N, int K, const TcOperand& A, const TcOperand& B, int nb
   }
   dim3 grid(cdiv(N, bn), cdiv(M, BM), a.ksplit > 1 ? a.ksplit : nb);
   prof_begin(kProfTcGemm, st);
-  const bool deep = (long long)grid.x * grid.y * grid.z <= 152;
-  const auto kern = deep ? k_tc_gemm<6> : k_tc_gemm<3>;
-  const int smem = smem_bytes(deep ? 6 : 3);
-  ensure_smem_attr((const void*)kern, smem);
-  kern<<<grid, 128, smem, st>>>(mAh, mAl, mBh, mBl, a);
+  // Stages of 16 k let a second CTA onto the SM, which pays while a tile's start
+  // and epilogue matter and there is a second CTA: 2982 x 7056 over 72 156
+  // against 192 us, over 256 186 / 217, and with rows on 128-byte boundaries up
+  // to a few thousand (over 1024 316 / 341, 639 x 18522 200 / 232).  Otherwise
+  // their 64-byte rows cost more than they gain: grids of one CTA an SM 230
+  // against 156 us (512 x 2982 over 8192), rows across boundaries 179 / 155
+  // (639 x 18522 over 441) and twice the time on products of tens of GB.
+  const bool two = (long long)grid.x * grid.y * grid.z > 152 &&
+                   (K <= 256 || (K <= 4096 && A.ld % 32 == 0 && B.ld % 32 == 0));
+  const int bk = two ? 16 : 32;
+  const CUtensorMap mAh = make_map(A.hi, K, M, A.ld, A.bstride, A.nb, BM, bk);
+  const CUtensorMap mAl = make_map(A.lo, K, M, A.ld, A.bstride, A.nb, BM, bk);
+  const CUtensorMap mBh = make_map(B.hi, K, N, B.ld, B.bstride, B.nb, bn, bk);
+  const CUtensorMap mBl = make_map(B.lo, K, N, B.ld, B.bstride, B.nb, bn, bk);
+  const auto kern = bk == 16 ? k_tc_gemm<16> : k_tc_gemm<32>;
+  ensure_smem_attr((const void*)kern, smem_bytes(bk));
+  kern<<<grid, 128, smem_bytes(bk), st>>>(mAh, mAl, mBh, mBl, a);
   RIS_CHECK_LAUNCH();
   if (a.ksplit > 1) {
     const auto reduce = a.ksplit <= 8 ? k_tc_reduce<true> : k_tc_reduce<false>;
