@@ -114,9 +114,9 @@ typedef struct {
                          0: computed by the first derivative call */
   int emu_f64;        /* 1 (default): FP64-accurate products on the FP16 tensor cores by exact
                          operand splitting.  Mixed precision: the Coulomb B transforms (the
-                         two MO transforms of (mu nu|P)_J).  RIS_FP64: the exchange products
-                         (B^K build, the exchange part of the A products and of Gamma) of all
-                         but the smallest systems.  0: on the FP64 pipe */
+                         two MO transforms of (mu nu|P)_J).  RIS_FP64: the B build and the
+                         exchange products (the exchange part of the A products and of
+                         Gamma) of all but the smallest systems.  0: on the FP64 pipe */
   int eig_fp32;       /* mixed precision: 1 solves the Davidson subspace eigenproblem in FP32
                          (FP64 Rayleigh quotients, close pairs and restarts re-orthonormalised
                          in FP64, back to FP64 if the residuals stall); 0 (default): FP64 */

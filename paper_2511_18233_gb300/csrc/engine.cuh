@@ -250,7 +250,7 @@ struct Engine : StreamOwner {
   // FP64-accurate product on the tensor cores
   void emu_abt(EmuForm f, int M, int N, int K, const double* A, long long rsA, long long ksA, const double* B,
                long long rsB, long long ksB, const EmuEpilogue& ep);
-  // FP64 form: the exchange products (B^K build, A products, exchange
+  // FP64 form: the B build and the exchange products (A products, exchange
   // densities) as FP64-accurate products on the FP16 tensor cores
   bool emu_exchange() const;
   void ensure_emu_ops();
