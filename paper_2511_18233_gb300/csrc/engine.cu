@@ -1627,14 +1627,20 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   stage = 2;
 }
 
-// The FP64 form's exchange products run emulated on the tensor cores (option
-// emu_f64) unless the system is so small that the FP64 pipe finishes a
-// product before the emulation's extra passes (slicing, about ten launches)
-// would: kEmuMinFlops is the exchange work of one A product there.
-constexpr double kEmuMinFlops = 2.0e7;
+// The FP64 form's B build, exchange products and exchange densities run
+// emulated on the tensor cores (option emu_f64) from kEmuMinFlops of exchange
+// work per vector on.  At the line (C7H9) the build takes 374 instead of 651
+// us, five gradients 587 instead of 1195; below it the passes around the
+// products (slicing, about ten launches) outweigh them.  A block of vectors
+// needs kEmuMinProduct of work: one vector of C9H11 (5.4e7) 141 against 128
+// us, one of C10H12 (8.1e7) 146 against 163, eight of C7H9 142 against 273.
+constexpr double kEmuMinFlops = 2.0e7, kEmuMinProduct = 7.0e7;
 bool Engine::emu_exchange() const {
   return opt.precision == RIS_FP64 && opt.emu_f64 && !streamed &&
          2.0 * nocc * (double)nvir * nvir * nK >= kEmuMinFlops;
+}
+bool Engine::emu_product(int nvec) const {
+  return emu_exchange() && 2.0 * nvec * nocc * (double)nvir * nvir * nK >= kEmuMinProduct;
 }
 
 void Engine::emu97(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep,
@@ -2116,7 +2122,7 @@ void Engine::apply_A_tda(const double* Xin, int nvec, double* out) {
   w5.ensure((size_t)nvec * std::max(nJ, 1), st);
   gemm(false, false, nvec, nJ, (int)nov, 1.0, Xin, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
   gemm(false, true, nvec, (int)nov, nJ, 2.0, w5.p, nJ, BJ.p, nJ, 0.0, out, (int)nov, st);
-  if (emu_exchange()) {
+  if (emu_product(nvec)) {
     exchange_emu(Xin, nvec, out, -opt.cx, 1.0, nullptr);
     k_add_diag<<<cdiv(nov * nvec, 256), 256, 0, st>>>(de.p, Xin, nov, nvec, out);
     RIS_CHECK_LAUNCH();
@@ -2169,7 +2175,7 @@ void Engine::apply(int nvec, const double* Xh, double* out, double* out2) {
 void Engine::exchange_terms(const double* Z, int nvec, double* K1, double* K2, bool mixed) {
   const int o = nocc, v = nvir;
   const long long nov = (long long)o * v;
-  if (emu_exchange()) {
+  if (emu_product(nvec)) {
     exchange_emu(Z, nvec, K1, 1.0, 0.0, K2);
     return;
   }

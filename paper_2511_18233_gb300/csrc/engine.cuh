@@ -253,6 +253,7 @@ struct Engine : StreamOwner {
   // FP64 form: the B build and the exchange products (A products, exchange
   // densities) as FP64-accurate products on the FP16 tensor cores
   bool emu_exchange() const;
+  bool emu_product(int nvec) const;  // ... a product of nvec vectors
   void ensure_emu_ops();
   void release_emu_ops();
   void check_tcerr();  // throws if a tensor-core pipeline wait timed out (synchronises)
