@@ -606,6 +606,15 @@ void Engine::gemm(bool ta, bool tb, int m, int n, int k, double alpha, const dou
   dgemm(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, s, bt);
 }
 
+// The same for a product whose rounding the metric of set X (0: J, 1: K)
+// multiplies in the derivatives (kIllMetric): where that is much, its sums
+// stay in order.
+void Engine::gemm_set(int X, bool ta, bool tb, int m, int n, int k, double alpha, const double* A, int lda,
+                      const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s, GemmBatch bt) {
+  bt.fine = opt.precision == RIS_FP64 && !ill[X];
+  dgemm(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, s, bt);
+}
+
 static void cholqr_small(const double* G, int nt, double drop, double* P, int* nkeep,
                          cudaStream_t st, double* pivmin = nullptr) {
   RIS_REQUIRE(nt >= 1 && nt <= 64, RIS_ERR_ARG, "cholqr_small: block of 1..64 vectors");
@@ -1260,6 +1269,26 @@ void Engine::partners_from_host_pairs() {
   RIS_CUDA(cudaMemcpyAsync(nbCol.p, col.data(), sizeof(int) * col.size(), cudaMemcpyHostToDevice, st));
 }
 
+// Largest P of M_PP (M^-1)_PP (1 / (1 - the squared correlation of P with the
+// other functions), free of the functions' norms), M^-1 = Linv^T Linv with
+// Linv lower triangular; as the bits of a non-negative double.  32 columns a
+// CTA, a warp every eighth row; it runs beside the integrals.
+__global__ void __launch_bounds__(256) k_metric_inflation(const double* __restrict__ Linv, int n,
+                                                          const double* __restrict__ MU, int nU,
+                                                          const int* __restrict__ map,
+                                                          unsigned long long* __restrict__ out) {
+  __shared__ double red[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, P = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (P < n)
+    for (int R = P + w; R < n; R += 8) s += Linv[(size_t)R * n + P] * Linv[(size_t)R * n + P];
+  red[w][lane] = s;
+  __syncthreads();
+  if (w != 0 || P >= n) return;
+  for (int k = 1; k < 8; k++) s += red[k][lane];
+  atomicMax(out, (unsigned long long)__double_as_longlong(fabs(s * MU[(size_t)map[P] * nU + map[P]])));
+}
+
 void Engine::build_aux(int natm_, const double* coords, int nshell, const ris_shell* aos, int nJs,
                        const ris_shell* auxJ, int nKs, const ris_shell* auxK) {
   RIS_REQUIRE(natm_ > 0 && nshell > 0 && nJs > 0 && nKs > 0, RIS_ERR_ARG, "empty input");
@@ -1420,7 +1449,8 @@ void Engine::build_aux(int natm_, const double* coords, int nshell, const ris_sh
   // integrals (buffers allocated on st first)
   MU.ensure((size_t)nU * nU, st);
   dMU.ensure(3 * (size_t)nU * nU, st);
-  if (!d_info) RIS_ALLOC(cudaMallocAsync((void**)&d_info, sizeof(int) * 2, st));
+  if (!d_info) RIS_ALLOC(cudaMallocAsync((void**)&d_info, sizeof(MetricInfo), st));
+  RIS_CUDA(cudaMemsetAsync(d_info, 0, sizeof(MetricInfo), st));
   LJinv.ensure((size_t)nJ * nJ, st);
   LKinv.ensure((size_t)nK * nK, st);
   w1.ensure((size_t)std::max(nJ, nK) * std::max(nJ, nK), st);
@@ -1439,6 +1469,9 @@ void Engine::build_aux(int natm_, const double* coords, int nshell, const ris_sh
     RIS_CHECK_LAUNCH();
     cholesky(w1.p, n, d_info + set, st3);
     tri_inverse(w1.p, set == 0 ? LJinv.p : LKinv.p, n, st3);
+    k_metric_inflation<<<cdiv(n, 32), 256, 0, st3>>>(set == 0 ? LJinv.p : LKinv.p, n, MU.p, nU, map,
+                                                     ((MetricInfo*)d_info)->infl + set);
+    RIS_CHECK_LAUNCH();
   }
   RIS_CUDA(cudaEventRecord(evM, st3));
   // integrals: dense [mu][nu][P], or (streamed form) on the screened pairs
@@ -1462,12 +1495,17 @@ void Engine::build_aux(int natm_, const double* coords, int nshell, const ris_sh
   h_pa.assign(pin, pin + pl.npair);
   h_pb.assign(pin + pl.npair, pin + 2 * (size_t)pl.npair);
   partners_from_host_pairs();
-  int info[2];
-  RIS_CUDA(cudaMemcpyAsync(info, d_info, sizeof(info), cudaMemcpyDeviceToHost, st));
+  MetricInfo mi;
+  RIS_CUDA(cudaMemcpyAsync(&mi, d_info, sizeof(mi), cudaMemcpyDeviceToHost, st));
   RIS_CUDA(cudaStreamSynchronize(st));
-  RIS_REQUIRE(info[0] == 0 && info[1] == 0, RIS_ERR_METRIC_NOT_PD,
+  RIS_REQUIRE(mi.pivot[0] == 0 && mi.pivot[1] == 0, RIS_ERR_METRIC_NOT_PD,
               "auxiliary metric is not positive definite (pivot " +
-                  std::to_string(info[0] ? info[0] : info[1]) + ")");
+                  std::to_string(mi.pivot[0] ? mi.pivot[0] : mi.pivot[1]) + ")");
+  for (int set = 0; set < 2; set++) {
+    double f;
+    memcpy(&f, &mi.infl[set], sizeof(f));
+    ill[set] = !(f < kIllMetric);
+  }
   nao = nao_;
   if (streamed) setup_streamed();
   stage = 1;
@@ -1530,19 +1568,20 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   // Coulomb: H[i][nu][P] = sum_mu C_mu,i T[mu][nu][P]; B[i][a][P]; B L^-T
   // (mixed form: H as [nu][i][P], both transforms FP64-accurate on the
   // tensor cores)
-  const bool emu = opt.precision == RIS_MIXED && opt.emu_f64, emuJ = emu || emu_exchange();
+  const bool emu = opt.precision == RIS_MIXED && opt.emu_f64, emuJ = emu || (emu_exchange() && !ill[0]);
+  const bool emuK = emu_exchange() && !ill[1];
   const EmuForm fJ = emu ? kEmu10x6 : kEmu9x7;
   w2.ensure((size_t)o * n * std::max(nJ, nK), st);
   w3.ensure((size_t)std::max(nov, (long long)o * o) * std::max(nJ, nK), st);
   if (emuJ) {
     coulomb_emu(fJ, w2.p, w3.p);
   } else {
-    gemm(true, false, o, n * nJ, n, 1.0, Co, nmo, TJ.p, n * nJ, 0.0, w2.p, n * nJ, st);
+    gemm_set(0, true, false, o, n * nJ, n, 1.0, Co, nmo, TJ.p, n * nJ, 0.0, w2.p, n * nJ, st);
     GemmBatch bt;
     bt.nb1 = o;
     bt.sB1 = (long long)n * nJ;
     bt.sC1 = (long long)v * nJ;
-    gemm(true, false, v, nJ, n, 1.0, Cv, nmo, w2.p, nJ, 0.0, w3.p, nJ, st, bt);
+    gemm_set(0, true, false, v, nJ, n, 1.0, Cv, nmo, w2.p, nJ, 0.0, w3.p, nJ, st, bt);
   }
   BJ.ensure((size_t)nov * nJ, st);
   if (emuJ) {  // B[(i,a)][R] = sum_P W[(i,a)][P] L_J^-1[R][P]
@@ -1550,7 +1589,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     e.c64 = BJ.p; e.rs = nJ; e.cs = 1;
     emu_abt(fJ, (int)nov, nJ, nJ, w3.p, nJ, 1, LJinv.p, nJ, 1, e);
   } else {
-    gemm(false, true, (int)nov, nJ, nJ, 1.0, w3.p, nJ, LJinv.p, nJ, 0.0, BJ.p, nJ, st);
+    gemm_set(0, false, true, (int)nov, nJ, nJ, 1.0, w3.p, nJ, LJinv.p, nJ, 0.0, BJ.p, nJ, st);
   }
   // exchange: oo and ov from C_o^T T^K, vv from C_v^T T^K
   const double* HK = w2.p;
@@ -1562,10 +1601,10 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     RIS_CHECK_LAUNCH();
     HK = w5.p;
   } else {
-    gemm(true, false, o, n * nK, n, 1.0, Co, nmo, TK.p, n * nK, 0.0, w2.p, n * nK, st);
+    gemm_set(1, true, false, o, n * nK, n, 1.0, Co, nmo, TK.p, n * nK, 0.0, w2.p, n * nK, st);
   }
   release_emu_ops();
-  if (emu_exchange()) {
+  if (emuK) {
     w4.ensure((size_t)v * v * nK, st);
     build_K_emu(HK, w4.p);
     BKvvD.ensure((size_t)v * v * nK, st);
@@ -1578,22 +1617,22 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     bt.nb1 = o;
     bt.sB1 = (long long)n * nK;
     bt.sC1 = (long long)o * nK;
-    gemm(true, false, o, nK, n, 1.0, Co, nmo, HK, nK, 0.0, w3.p, nK, st, bt);
+    gemm_set(1, true, false, o, nK, n, 1.0, Co, nmo, HK, nK, 0.0, w3.p, nK, st, bt);
   }
   BKoo.ensure((size_t)o * o * nK, st);
-  gemm(false, true, o * o, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, BKoo.p, nK, st);
+  gemm_set(1, false, true, o * o, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, BKoo.p, nK, st);
   cKoo.ensure((size_t)o * o * nK, st);
-  gemm(false, false, o * o, nK, nK, 1.0, BKoo.p, nK, LKinv.p, nK, 0.0, cKoo.p, nK, st);
+  gemm_set(1, false, false, o * o, nK, nK, 1.0, BKoo.p, nK, LKinv.p, nK, 0.0, cKoo.p, nK, st);
   if (opt.rpa) {
     GemmBatch bt;
     bt.nb1 = o;
     bt.sB1 = (long long)n * nK;
     bt.sC1 = (long long)v * nK;
-    gemm(true, false, v, nK, n, 1.0, Cv, nmo, HK, nK, 0.0, w3.p, nK, st, bt);
+    gemm_set(1, true, false, v, nK, n, 1.0, Cv, nmo, HK, nK, 0.0, w3.p, nK, st, bt);
     w4.ensure((size_t)nov * nK, st);
-    gemm(false, true, (int)nov, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, w4.p, nK, st);  // [i][a][R]
+    gemm_set(1, false, true, (int)nov, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, w4.p, nK, st);  // [i][a][R]
     cKov.ensure((size_t)nov * nK, st);
-    gemm(false, false, (int)nov, nK, nK, 1.0, w4.p, nK, LKinv.p, nK, 0.0, cKov.p, nK, st);
+    gemm_set(1, false, false, (int)nov, nK, nK, 1.0, w4.p, nK, LKinv.p, nK, 0.0, cKov.p, nK, st);
     BKovR.ensure((size_t)nov * nK, st);
     transpose_last2(w4.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]
     cKovP.ensure((size_t)nov * nK, st);
@@ -1604,14 +1643,14 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     build_Kvv_tc(w4.p);  // B[a][b][R]
   } else {
     w2.ensure((size_t)v * n * nK, st);
-    gemm(true, false, v, n * nK, n, 1.0, Cv, nmo, TK.p, n * nK, 0.0, w2.p, n * nK, st);
+    gemm_set(1, true, false, v, n * nK, n, 1.0, Cv, nmo, TK.p, n * nK, 0.0, w2.p, n * nK, st);
     w3.ensure((size_t)v * v * nK, st);
     GemmBatch bt;
     bt.nb1 = v;
     bt.sB1 = (long long)n * nK;
     bt.sC1 = (long long)v * nK;
-    gemm(true, false, v, nK, n, 1.0, Cv, nmo, w2.p, nK, 0.0, w3.p, nK, st, bt);
-    gemm(false, true, v * v, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, w4.p, nK, st);  // B[a][b][R]
+    gemm_set(1, true, false, v, nK, n, 1.0, Cv, nmo, w2.p, nK, 0.0, w3.p, nK, st, bt);
+    gemm_set(1, false, true, v * v, nK, nK, 1.0, w3.p, nK, LKinv.p, nK, 0.0, w4.p, nK, st);  // B[a][b][R]
   }
   cKvv.ensure((size_t)v * v * nK, st);
   if (emu) {  // c[(a,b)][Q] = sum_R B[(a,b)][R] L_K^-1[R][Q]
@@ -1619,7 +1658,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     e.c64 = cKvv.p; e.rs = nK; e.cs = 1;
     emu_abt(kEmu10x6, v * v, nK, nK, w4.p, nK, 1, LKinv.p, 1, nK, e);
   } else {
-    gemm(false, false, v * v, nK, nK, 1.0, w4.p, nK, LKinv.p, nK, 0.0, cKvv.p, nK, st);
+    gemm_set(1, false, false, v * v, nK, nK, 1.0, w4.p, nK, LKinv.p, nK, 0.0, cKvv.p, nK, st);
   }
   BKvvD.ensure((size_t)v * v * nK, st);
   transpose_last2(w4.p, v, v, nK, BKvvD.p, st);  // [b][R][a]
@@ -3098,7 +3137,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   // Q_s[i][nu] = sum_a R_s[i][a] C_v[nu][a] for every state, and from it
   // D^R_s[mu][nu] = sum_i C_o[mu][i] Q_s[i][nu] (o n^2 multiply-adds; forming
   // C_o R_s first would take o n v + n^2 v)
-  const bool emu = emu_exchange();
+  const bool emu = emu_exchange(), emuG = emu && !ill[1];
   if (!mixed || rpa) {
     QR.ensure((size_t)nsu * o * nn, st);
     if (rpa) QL.ensure((size_t)nsu * o * nn, st);
@@ -3128,8 +3167,11 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   }
   // u_s = R_s . B^J (nJ), c_s = u_s L^-1 (row vector); the long product in
   // double-FP32 in the mixed form, like those of its Davidson
-  gemm_sub(mixed && opt.subspace_ff, false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
-  gemm(false, false, nsu, nJ, nJ, 1.0, w5.p, nJ, LJinv.p, nJ, 0.0, cJ.p, nJ, st);
+  if (mixed)
+    gemm_sub(opt.subspace_ff, false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
+  else
+    gemm_set(0, false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
+  gemm_set(0, false, false, nsu, nJ, nJ, 1.0, w5.p, nJ, LJinv.p, nJ, 0.0, cJ.p, nJ, st);
   // Coulomb part of every pair density from per-state data: symmetrised
   // D^R and c^J on the union index (the contraction forms G^J on the fly)
   k_symmetrize_sq<<<cdiv((long long)nsu * nn * nn, 256), 256, 0, st>>>(DR.p, nn, nsu);
@@ -3182,7 +3224,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   const int slK = pick_slices((long long)nn * nK, nbAvg);
   SBuf<double> partK((size_t)slK * NB * 3 * nn * nK, st);
   SBuf<int> pst(2 * NB, st);
-  if (opt.precision != RIS_MIXED && !emu) {
+  if (opt.precision != RIS_MIXED && !emuG) {
     Z.ensure((size_t)o * v * nK, st);
     Goo.ensure((size_t)o * o * nK, st);
     M1.ensure((size_t)nn * 2 * o * nK, st);
@@ -3190,11 +3232,11 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   }
   const double cx = opt.cx;
   GammaEmu ge;
-  if (emu) ge.setup(*this, nsu, Rs.p, rpa ? Ls.p : nullptr, QR.p, rpa ? QL.p : nullptr);
+  if (emuG) ge.setup(*this, nsu, Rs.p, rpa ? Ls.p : nullptr, QR.p, rpa ? QL.p : nullptr);
   for (int g0 = 0; g0 < npair; g0 += NB) {
     const int nb = std::min(NB, npair - g0);
     // (in mixed TDA and in the emulated form one exchange GEMM writes every element of G^K)
-    if (!gk32 && !emu) RIS_CUDA(cudaMemsetAsync(GK.p, 0, sizeof(double) * nb * gk, st));
+    if (!gk32 && !emuG) RIS_CUDA(cudaMemsetAsync(GK.p, 0, sizeof(double) * nb * gk, st));
     RIS_CUDA(cudaMemsetAsync(OmB.p, 0, sizeof(double) * nb * nU * nU, st));
     std::vector<int> h_pst(2 * nb), hI(nb), hJ(nb);
     for (int b = 0; b < nb; b++) {
@@ -3210,8 +3252,8 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
       gamma_K_mixed(nb, hI.data(), hJ.data(), nsu, cmb == 0 ? RSh.p : LSh.p, cmb == 0 ? RSl.p : LSl.p,
                     cmb == 0 ? WRh.p : WLh.p, cmb == 0 ? WRl.p : WLl.p, rpa ? -0.5 * cx : -cx, GK.p,
                     gk32 ? GK32.p : nullptr, OmB.p);
-    if (emu) ge.pairs(*this, nb, hI.data(), hJ.data(), GK.p, OmB.p);
-    for (int b = 0; b < nb && !emu; b++) {
+    if (emuG) ge.pairs(*this, nb, hI.data(), hJ.data(), GK.p, OmB.p);
+    for (int b = 0; b < nb && !emuG; b++) {
       const int sI = hI[b], sJ = hJ[b];
       double* Gam = gk32 ? nullptr : GK.p + (size_t)b * gk;
       double* Om = OmB.p + (size_t)b * nU * nU;
@@ -3223,18 +3265,18 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
         const double* QU = (cmb == 0 ? QR.p : QL.p) + (size_t)sI * o * nn;
         const double* QV = (cmb == 0 ? QR.p : QL.p) + (size_t)sJ * o * nn;
         // Z[j][b][P] = sum_a U[j][a] c^vv[a][b][P]
-        gemm(false, false, o, v * nK, v, 1.0, U, v, cKvv.p, v * nK, 0.0, Z.p, v * nK, st);
+        gemm_set(1, false, false, o, v * nK, v, 1.0, U, v, cKvv.p, v * nK, 0.0, Z.p, v * nK, st);
         // G[j][k][P] = sum_b V[k][b] Z[j][b][P]
         {
           GemmBatch bt;
           bt.nb1 = o;
           bt.sB1 = (long long)v * nK;
           bt.sC1 = (long long)o * nK;
-          gemm(false, false, o, nK, v, 1.0, Vv, v, Z.p, nK, 0.0, Goo.p, nK, st, bt);
+          gemm_set(1, false, false, o, nK, v, 1.0, Vv, v, Z.p, nK, 0.0, Goo.p, nK, st, bt);
         }
         // M1[mu][0:o][P] = C_o G ; M1[mu][o:2o][P] = Q_U^T c^oo
-        gemm(false, false, nn, o * nK, o, 1.0, Co, nmo, Goo.p, o * nK, 0.0, M1.p, 2 * o * nK, st);
-        gemm(true, false, nn, o * nK, o, 1.0, QU, nn, cKoo.p, o * nK, 0.0, M1.p + (size_t)o * nK,
+        gemm_set(1, false, false, nn, o * nK, o, 1.0, Co, nmo, Goo.p, o * nK, 0.0, M1.p, 2 * o * nK, st);
+        gemm_set(1, true, false, nn, o * nK, o, 1.0, QU, nn, cKoo.p, o * nK, 0.0, M1.p + (size_t)o * nK,
               2 * o * nK, st);
         k_build_W<<<cdiv(nn * 2 * o, 256), 256, 0, st>>>(C.p, nmo, QV, nn, o, WV.p);
         RIS_CHECK_LAUNCH();
@@ -3244,10 +3286,10 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
           bt.nb1 = nn;
           bt.sB1 = 2LL * o * nK;
           bt.sC1 = (long long)nn * nK;
-          gemm(false, false, nn, nK, 2 * o, f, WV.p, 2 * o, M1.p, nK, 1.0, Gam, nK, st, bt);
+          gemm_set(1, false, false, nn, nK, 2 * o, f, WV.p, 2 * o, M1.p, nK, 1.0, Gam, nK, st, bt);
         }
         // Omega[P][Q] += f sum_ij c^oo_ij,P G_ij,Q   (K functions are union 0..nK-1)
-        gemm(true, false, nK, nK, o * o, f, cKoo.p, nK, Goo.p, nK, 1.0, Om, nU, st);
+        gemm_set(1, true, false, nK, nK, o * o, f, cKoo.p, nK, Goo.p, nK, 1.0, Om, nU, st);
       }
       if (rpa) {
         // (ib|ja) terms, weights -c_x/2 for (R_I,R_J) and +c_x/2 for (L_I,L_J):
@@ -3266,24 +3308,24 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
           bP.nb1 = nK;
           bP.sB1 = nov;
           bP.sC1 = (long long)o * o;
-          gemm(false, true, o, o, v, 1.0, U, v, cKovP.p, v, 0.0, E1.p, o, st, bP);
-          gemm(false, true, o, o, v, 1.0, Vv, v, cKovP.p, v, 0.0, E2.p, o, st, bP);
+          gemm_set(1, false, true, o, o, v, 1.0, U, v, cKovP.p, v, 0.0, E1.p, o, st, bP);
+          gemm_set(1, false, true, o, o, v, 1.0, Vv, v, cKovP.p, v, 0.0, E2.p, o, st, bP);
           GemmBatch bM;
           bM.nb1 = nK;
           bM.sA1 = (long long)o * o;
           bM.sC1 = (long long)o * nn;
-          gemm(false, false, o, nn, o, 1.0, E1.p, o, QV, nn, 0.0, M2.p, nn, st, bM);
-          gemm(false, false, o, nn, o, 1.0, E2.p, o, QU, nn, 1.0, M2.p, nn, st, bM);
+          gemm_set(1, false, false, o, nn, o, 1.0, E1.p, o, QV, nn, 0.0, M2.p, nn, st, bM);
+          gemm_set(1, false, false, o, nn, o, 1.0, E2.p, o, QU, nn, 1.0, M2.p, nn, st, bM);
           k_permute120<<<cdiv((long long)nK * o * nn, 256), 256, 0, st>>>(M2.p, nK, o, nn, M2p.p);
           RIS_CHECK_LAUNCH();
           GemmBatch bG;
           bG.nb1 = nn;
           bG.sB1 = (long long)nK * o;
           bG.sC1 = (long long)nn * nK;
-          gemm(false, true, nn, nK, o, wgt, C.p, nmo, M2p.p, o, 1.0, Gam, nK, st, bG);
+          gemm_set(1, false, true, nn, nK, o, wgt, C.p, nmo, M2p.p, o, 1.0, Gam, nK, st, bG);
           // E1t[P][k][i] = E1[P][i][k]
           transpose_last2(E1.p, nK, o, o, E1t.p, st);
-          gemm(false, true, nK, nK, o * o, wgt, E2.p, o * o, E1t.p, o * o, 1.0, Om, nU, st);
+          gemm_set(1, false, true, nK, nK, o * o, wgt, E2.p, o * o, E1t.p, o * o, 1.0, Om, nU, st);
         }
       }
     }
@@ -3616,8 +3658,8 @@ void Engine::setup_streamed() {
       e2.c64 = BKao.p; e2.rs = nK; e2.cs = 1;
       emu_abt(kEmu10x6, (int)nfp, nK, nK, Ts.p, nU, 1, LKinv.p, nK, 1, e2);
     } else {
-      gemm(false, true, (int)nfp, nJ, nU, 1.0, Ts.p, nU, LJu.p, nU, 0.0, BJao.p, nJ, st);
-      gemm(false, true, (int)nfp, nK, nK, 1.0, Ts.p, nU, LKinv.p, nK, 0.0, BKao.p, nK, st);
+      gemm_set(0, false, true, (int)nfp, nJ, nU, 1.0, Ts.p, nU, LJu.p, nU, 0.0, BJao.p, nJ, st);
+      gemm_set(1, false, true, (int)nfp, nK, nK, 1.0, Ts.p, nU, LKinv.p, nK, 0.0, BKao.p, nK, st);
     }
     RIS_CUDA(cudaStreamSynchronize(st));  // host vectors go out of scope
   }
@@ -3686,12 +3728,12 @@ void Engine::build_B_streamed() {
         e2.c64 = BJ.p + r0; e2.rin = rw; e2.rld = (long long)v * nJ; e2.rs = 1; e2.cs = nJ;
         emu_abt(kEmu10x6, (int)rH, v, n, H.p, 1, rH, C.p + o, 1, nmo, e2);
       } else {  // H[i][nu][r], then per i: B[i][a][r0 + r]
-        gemm(true, false, o, n * rw, n, 1.0, Co, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
+        gemm_set(0, true, false, o, n * rw, n, 1.0, Co, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
         GemmBatch bt;
         bt.nb1 = o;
         bt.sB1 = (long long)n * rw;
         bt.sC1 = (long long)v * nJ;
-        gemm(true, false, v, rw, n, 1.0, Cv, nmo, H.p, rw, 0.0, BJ.p + r0, nJ, st, bt);
+        gemm_set(0, true, false, v, rw, n, 1.0, Cv, nmo, H.p, rw, 0.0, BJ.p + r0, nJ, st, bt);
       }
     }
   }
@@ -3755,18 +3797,18 @@ void Engine::build_B_streamed() {
       for (int r0 = 0; r0 < nK; r0 += rb) {
         const int rw = std::min(rb, nK - r0);
         scatter_block(BKao.p, nK, r0, rw, nfp, fpMu.p, fpNu.p, n, Tb.p, st);
-        gemm(true, false, o, n * rw, n, 1.0, Co, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
+        gemm_set(1, true, false, o, n * rw, n, 1.0, Co, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
         GemmBatch bt;
         bt.nb1 = o;
         bt.sB1 = (long long)n * rw;
         bt.sC1 = (long long)o * nK;
-        gemm(true, false, o, rw, n, 1.0, Co, nmo, H.p, rw, 0.0, BKoo.p + r0, nK, st, bt);
-        gemm(true, false, v, n * rw, n, 1.0, Cv, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
+        gemm_set(1, true, false, o, rw, n, 1.0, Co, nmo, H.p, rw, 0.0, BKoo.p + r0, nK, st, bt);
+        gemm_set(1, true, false, v, n * rw, n, 1.0, Cv, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
         GemmBatch b2;
         b2.nb1 = v;
         b2.sB1 = (long long)n * rw;
         b2.sC1 = (long long)v * rw;
-        gemm(true, false, v, rw, n, 1.0, Cv, nmo, H.p, rw, 0.0, G.p, rw, st, b2);
+        gemm_set(1, true, false, v, rw, n, 1.0, Cv, nmo, H.p, rw, 0.0, G.p, rw, st, b2);
         k_place_vv<<<(unsigned)cdiv((long long)v * v * rw, 256), 256, 0, st>>>(G.p, v, rw, r0, nK, BKvvD.p);
         RIS_CHECK_LAUNCH();
       }
@@ -3775,7 +3817,7 @@ void Engine::build_B_streamed() {
   Tb.release();
   // fitting coefficients of the oo block, c = B L^-1, as [P][i][k]
   cKoo.ensure((size_t)o * o * nK, st);
-  gemm(false, false, o * o, nK, nK, 1.0, BKoo.p, nK, LKinv.p, nK, 0.0, cKoo.p, nK, st);
+  gemm_set(1, false, false, o * o, nK, nK, 1.0, BKoo.p, nK, LKinv.p, nK, 0.0, cKoo.p, nK, st);
   cKooP.ensure((size_t)o * o * nK, st);
   transpose_last2(cKoo.p, 1, o * o, nK, cKooP.p, st);
   if (mixed) {  // FP32 hi/lo operands of the products and of the gradient
@@ -3842,8 +3884,8 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
     }
   }
   w5.ensure((size_t)nsu * nJ, st);
-  gemm(false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
-  gemm(false, false, nsu, nJ, nJ, 1.0, w5.p, nJ, LJinv.p, nJ, 0.0, cJ.p, nJ, st);
+  gemm_set(0, false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
+  gemm_set(0, false, false, nsu, nJ, nJ, 1.0, w5.p, nJ, LJinv.p, nJ, 0.0, cJ.p, nJ, st);
   k_symmetrize_sq<<<cdiv((long long)nsu * nn * nn, 256), 256, 0, st>>>(DR.p, nn, nsu);
   RIS_CHECK_LAUNCH();
   // state densities regrouped [batch][mu][nu][b] for the contraction
@@ -3937,15 +3979,15 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
         const double* U = Rs.p + (size_t)sI * nov;
         const double* V = Rs.p + (size_t)sJ * nov;
         SBuf<double> T1((size_t)o * nK * v, st), Gt((size_t)o * nK * o, st);
-        gemm(false, false, o, nK * v, v, 1.0, V, v, BKvvD.p, nK * v, 0.0, T1.p, nK * v, st);  // [k][R][a]
-        gemm(false, true, o * nK, o, v, 1.0, T1.p, v, U, v, 0.0, Gt.p, o, st);                 // [k][R][j]
+        gemm_set(1, false, false, o, nK * v, v, 1.0, V, v, BKvvD.p, nK * v, 0.0, T1.p, nK * v, st);  // [k][R][a]
+        gemm_set(1, false, true, o * nK, o, v, 1.0, T1.p, v, U, v, 0.0, Gt.p, o, st);                 // [k][R][j]
         double* G = Gd.p + (size_t)b * nK * o * o;
         GemmBatch bt;
         bt.nb1 = o;
         bt.sB1 = (long long)nK * o;
         bt.sC1 = o;
-        gemm(true, false, nK, o, nK, 1.0, LKinv.p, nK, Gt.p, o, 0.0, G, o * o, st, bt);         // [P][k][j]
-        gemm(false, true, nK, nK, o * o, f, cKooP.p, o * o, G, o * o, 1.0, Om, nU, st);
+        gemm_set(1, true, false, nK, o, nK, 1.0, LKinv.p, nK, Gt.p, o, 0.0, G, o * o, st, bt);         // [P][k][j]
+        gemm_set(1, false, true, nK, nK, o * o, f, cKooP.p, o * o, G, o * o, 1.0, Om, nU, st);
       }
     }
     // auxiliary blocks: derivative integrals regenerated and contracted at once
@@ -4019,8 +4061,8 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
             bp.nb1 = wK;
             bp.sB1 = (long long)o * o;
             bp.sC1 = 2LL * o;
-            gemm(false, true, nn, o, o, 1.0, Co, nmo, G + (size_t)u0 * o * o, o, 0.0, M1d.p, wK * 2 * o, st, bp);
-            gemm(true, false, nn, o, o, 1.0, QU, nn, cKooP.p + (size_t)u0 * o * o, o, 0.0, M1d.p + o,
+            gemm_set(1, false, true, nn, o, o, 1.0, Co, nmo, G + (size_t)u0 * o * o, o, 0.0, M1d.p, wK * 2 * o, st, bp);
+            gemm_set(1, true, false, nn, o, o, 1.0, QU, nn, cKooP.p + (size_t)u0 * o * o, o, 0.0, M1d.p + o,
                   wK * 2 * o, st, bp);
             k_build_W<<<cdiv(nn * 2 * o, 256), 256, 0, st>>>(C.p, nmo, QV, nn, o, WVd.p);
             RIS_CHECK_LAUNCH();
@@ -4028,7 +4070,7 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
             bm.nb1 = nn;
             bm.sB1 = (long long)wK * 2 * o;
             bm.sC1 = (long long)nn * wK;
-            gemm(false, true, nn, wK, 2 * o, f, WVd.p, 2 * o, M1d.p, 2 * o, 0.0,
+            gemm_set(1, false, true, nn, wK, 2 * o, f, WVd.p, 2 * o, M1d.p, 2 * o, 0.0,
                   Gam64.p + (size_t)b * nn2 * wK, wK, st, bm);
           }
         }

@@ -130,6 +130,25 @@ struct CoulPrecond {
   void apply(Engine& e, const double* R, const int* idx, int nt, double* T);
 };
 
+// What build_aux learns of the two metrics (J, K): the pivot at which the
+// factorisation failed (0: none) and the largest M_PP (M^-1)_PP (bits of a double).
+struct MetricInfo {
+  int pivot[2];
+  unsigned long long infl[2];
+};
+// The derivatives take c = M^-1 (rounding errors of the MO transforms), so a
+// rounding of the transforms and of B = W L^-T, or another order of their sums,
+// returns in FP64 gradients and couplings times the metric's inflation: against
+// sums in order, emulated transforms moved couplings by 2e-12 at an inflation
+// of 5e3 (chains of any length), 1e-10 at 1.3e5 (C24H12), 5e-10 at 6e5 (C42H18)
+// and 1.7e-9 at 1e6 (C54H18, relative 2-norm), and by a twentieth to a fiftieth
+// of that with these transforms alone summed in order.  From 3e4 on (5e-11 at
+// that rate) the FP64 form therefore keeps them on the FP64 pipe, in order (J:
+// the transforms, u = X B and c = u L^-1; K: these and the exchange densities).
+// The products with vectors, which take the metric's square root, and the
+// densities of a well-conditioned K set stay emulated.
+constexpr double kIllMetric = 3.0e4;
+
 struct Engine : StreamOwner {
   ris_options opt{};
   int device = 0;
@@ -158,7 +177,8 @@ struct Engine : StreamOwner {
   bool have_D = false;
   bool D_pending = false;             // D being computed on st2 (event evD)
   cudaEvent_t evA = nullptr, evD = nullptr;
-  int* d_info = nullptr;
+  int* d_info = nullptr;    // MetricInfo; its first int also serves other factorisations
+  bool ill[2] = {false, false};  // J, K metric: inflation of kIllMetric and more
 
   // MO data
   int nao = 0, nmo = 0, nocc = 0, nvir = 0;  // active sizes (after mo_window)
@@ -238,6 +258,9 @@ struct Engine : StreamOwner {
   void gemm(bool ta, bool tb, int m, int n, int k, double alpha, const double* A, int lda,
             const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s,
             GemmBatch bt = GemmBatch());
+  void gemm_set(int X, bool ta, bool tb, int m, int n, int k, double alpha, const double* A, int lda,
+                const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s,
+                GemmBatch bt = GemmBatch());
   void gemm_sub(bool ff, bool ta, bool tb, int m, int n, int k, double alpha, const double* A,
                 int lda, const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t st);
   void apply_A_tda(const double* Xin, int nvec, double* out);
