@@ -3165,12 +3165,9 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
       gemm(false, false, nn, nn, o, 1.0, Co, nmo, QR.p, nn, 0.0, DR.p, nn, st, bt);
     }
   }
-  // u_s = R_s . B^J (nJ), c_s = u_s L^-1 (row vector); the long product in
-  // double-FP32 in the mixed form, like those of its Davidson
-  if (mixed)
-    gemm_sub(opt.subspace_ff, false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
-  else
-    gemm_set(0, false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
+  // u_s = R_s . B^J (nJ), c_s = u_s L^-1 (row vector), FP64 in the mixed form
+  // too: L^-1 amplifies the rounding of u
+  gemm_set(0, false, false, nsu, nJ, (int)nov, 1.0, Rs.p, (int)nov, BJ.p, nJ, 0.0, w5.p, nJ, st);
   gemm_set(0, false, false, nsu, nJ, nJ, 1.0, w5.p, nJ, LJinv.p, nJ, 0.0, cJ.p, nJ, st);
   // Coulomb part of every pair density from per-state data: symmetrised
   // D^R and c^J on the union index (the contraction forms G^J on the fly)
