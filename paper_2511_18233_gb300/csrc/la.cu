@@ -794,7 +794,10 @@ __global__ void __launch_bounds__(kEigT) k_eig_tridiag(const double* H, int ldH,
     }
     __syncthreads();
     const double t = sh_tau;
-    if (mag_bits(t) == 0) continue;
+    if (mag_bits(t) == 0) {  // uniform; the next column's sh_tau waits until every thread has read this one
+      __syncthreads();
+      continue;
+    }
     // p = t * A_sub v, using symmetry for coalesced reads: two threads per
     // row (alternate j), two partial sums each, so that the dependent FP64
     // chains are a quarter of the row long
