@@ -1027,6 +1027,7 @@ __global__ void __launch_bounds__(kEigVecT) k_eig_vec(int m, double* work, int a
         nrm = 1.0 / sqrt(nrm);
       }
       nrm = __shfl_sync(0xffffffffu, nrm, 0);
+      __syncwarp();  // lane 0's z: a shuffle does not order memory
       for (int i = tid; i < m; i += 32) z[i] *= nrm;
     }
     if (tid == 0) W.lam[j] = lj;
