@@ -1548,6 +1548,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   C.ensure((size_t)n * nmo, st);
   eps.ensure(nmo, st);
   de.ensure(nov, st);
+  have_Kov = opt.rpa;  // the ov block is of these integrals and MOs: below for RPA, else on demand
   if (i0 == 0 && a1 == nmo_) {
     copy_in(C.p, Cin, (size_t)n * nmo, st);
     copy_in(eps.p, eps_in, nmo, st);
@@ -3361,7 +3362,7 @@ void Engine::ensure_Kov() {
   RIS_REQUIRE(!streamed, RIS_ERR_ARG, "the (ib|P) block is not available in the streamed form");
   const int o = nocc, v = nvir, n = nao;
   const long long nov = (long long)o * v;
-  if (BKovR.p && BKovR.n >= (size_t)nov * nK) return;
+  if (have_Kov) return;
   RIS_REQUIRE(TK.p, RIS_ERR_STATE, "three-centre integrals not available (trimmed context)");
   const double* Co = C.p;
   const double* Cv = C.p + o;
@@ -3380,6 +3381,7 @@ void Engine::ensure_Kov() {
     emu97((int)nov, nK, t.op, li.op, emu_out(Bm.p, nK, 1));
     BKovR.ensure((size_t)nov * nK, st);
     transpose_last2(Bm.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]
+    have_Kov = true;
     return;
   }
   gemm(true, false, o, n * nK, n, 1.0, Co, nmo, TK.p, n * nK, 0.0, H.p, n * nK, st);
@@ -3391,6 +3393,7 @@ void Engine::ensure_Kov() {
   gemm(false, true, (int)nov, nK, nK, 1.0, Bia.p, nK, LKinv.p, nK, 0.0, Bm.p, nK, st);  // [i][a][R]
   BKovR.ensure((size_t)nov * nK, st);
   transpose_last2(Bm.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]
+  have_Kov = true;
 }
 
 // Preconditioned conjugate gradients on (A+B)_ris Z = rhs (Eq. Z_vector with

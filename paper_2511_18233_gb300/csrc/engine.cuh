@@ -187,7 +187,8 @@ struct Engine : StreamOwner {
   DBuf BJ;        // [ov][RJ]
   DBuf BKoo;      // [i][j][R]
   DBuf BKvvD;     // [b][R][a] (Davidson layout)
-  DBuf BKovR;     // [R][i][a] (RPA)
+  DBuf BKovR;     // [R][i][a] (RPA, Z-vector)
+  bool have_Kov = false;  // BKovR holds the last B build's block
   DBuf cKovP;     // c^K_ov as [P][i][a] (RPA)
   DBuf cKoo, cKvv, cKov;  // fitting coefficients c = B L^-1, [p][q][P]
 
