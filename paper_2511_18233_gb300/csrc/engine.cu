@@ -1310,6 +1310,7 @@ void Engine::build_aux(int natm_, const double* coords, int nshell, const ris_sh
   check(auxJ, nJs, kMaxLAux, "J auxiliary shell");
   check(auxK, nKs, kMaxLAux, "K auxiliary shell");
   join_D();  // a previous geometry's derivative integrals may still read the shells
+  release_emu_ops();  // nothing of the last geometry's B tensors is used again
   stage = 0;
   have_D = false;
   natm = natm_;
@@ -1548,6 +1549,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   C.ensure((size_t)n * nmo, st);
   eps.ensure(nmo, st);
   de.ensure(nov, st);
+  release_emu_ops();   // digits of the last B build
   have_Kov = opt.rpa;  // the ov block is of these integrals and MOs: below for RPA, else on demand
   if (i0 == 0 && a1 == nmo_) {
     copy_in(C.p, Cin, (size_t)n * nmo, st);
@@ -1604,7 +1606,6 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   } else {
     gemm_set(1, true, false, o, n * nK, n, 1.0, Co, nmo, TK.p, n * nK, 0.0, w2.p, n * nK, st);
   }
-  release_emu_ops();
   if (emuK) {
     w4.ensure((size_t)v * v * nK, st);
     build_K_emu(HK, w4.p);

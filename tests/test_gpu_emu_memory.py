@@ -1,0 +1,39 @@
+"""Device memory of the FP64 form's emulated products."""
+import pytest
+
+from paper_2511_18233_gb300 import synth
+
+gpu = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ris_mod():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2511_18233_gb300 import build, ris
+    build.build()
+    return ris
+
+
+@gpu
+def test_digits_of_a_dense_geometry_go_with_it(ris_mod):
+    """A context that held a dense geometry with sliced B^K_vv (18 v^2 nK bytes) and
+    goes on to a streamed one holds no more than one that never sliced."""
+    small, large = synth.chain_molecule(20, 1, True), synth.chain_molecule(24, 1, True)
+    budget = int(3 * 1.2e9)  # the dense line at 1.2 GB: 0.94 (C20H22) and 1.6 GB (C24H26)
+    held = []
+    for emu in (1, 0):
+        c = ris_mod.Context(emu_f64=emu, mem_budget=budget)
+        for mol in (small, large):
+            c.build_aux(mol.coords, mol.shells, mol.aux_j, mol.aux_k)
+            c.build_B(mol.C, mol.mo_energy, mol.nocc)
+            X = synth.random_amplitudes(1, mol.nocc, mol.nvir, seed=2)
+            if mol is small:
+                c.apply(X)
+        with pytest.raises(ris_mod.RisError):  # the streamed form has no Z-vector
+            c.zvector(X)
+        held.append(c.stats()["bytes_held"])
+        c.close()
+    digits = 18 * small.nvir ** 2 * small.naux("K")
+    assert abs(held[0] - held[1]) < digits // 2, (held, digits)
