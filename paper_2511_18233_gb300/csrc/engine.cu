@@ -1270,14 +1270,19 @@ void Engine::partners_from_host_pairs() {
 }
 
 // Largest P of M_PP (M^-1)_PP (1 / (1 - the squared correlation of P with the
-// other functions), free of the functions' norms), M^-1 = Linv^T Linv with
-// Linv lower triangular; as the bits of a non-negative double.  32 columns a
-// CTA, a warp every eighth row; it runs beside the integrals.
-__global__ void __launch_bounds__(256) k_metric_inflation(const double* __restrict__ Linv, int n,
+// other functions), free of the functions' norms) of the J and the K metric
+// (blockIdx.y), M^-1 = Linv^T Linv with Linv lower triangular; as the bits of a
+// non-negative double.  32 columns a CTA, a warp every eighth row.
+__global__ void __launch_bounds__(256) k_metric_inflation(const double* __restrict__ LJ, int nJ,
+                                                          const int* __restrict__ mapJ,
+                                                          const double* __restrict__ LK, int nK,
+                                                          const int* __restrict__ mapK,
                                                           const double* __restrict__ MU, int nU,
-                                                          const int* __restrict__ map,
                                                           unsigned long long* __restrict__ out) {
   __shared__ double red[8][32];
+  const double* Linv = blockIdx.y ? LK : LJ;
+  const int* map = blockIdx.y ? mapK : mapJ;
+  const int n = blockIdx.y ? nK : nJ;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, P = blockIdx.x * 32 + lane;
   double s = 0.0;
   if (P < n)
@@ -1286,7 +1291,7 @@ __global__ void __launch_bounds__(256) k_metric_inflation(const double* __restri
   __syncthreads();
   if (w != 0 || P >= n) return;
   for (int k = 1; k < 8; k++) s += red[k][lane];
-  atomicMax(out, (unsigned long long)__double_as_longlong(fabs(s * MU[(size_t)map[P] * nU + map[P]])));
+  atomicMax(out + blockIdx.y, (unsigned long long)__double_as_longlong(fabs(s * MU[(size_t)map[P] * nU + map[P]])));
 }
 
 void Engine::build_aux(int natm_, const double* coords, int nshell, const ris_shell* aos, int nJs,
@@ -1470,10 +1475,10 @@ void Engine::build_aux(int natm_, const double* coords, int nshell, const ris_sh
     RIS_CHECK_LAUNCH();
     cholesky(w1.p, n, d_info + set, st3);
     tri_inverse(w1.p, set == 0 ? LJinv.p : LKinv.p, n, st3);
-    k_metric_inflation<<<cdiv(n, 32), 256, 0, st3>>>(set == 0 ? LJinv.p : LKinv.p, n, MU.p, nU, map,
-                                                     ((MetricInfo*)d_info)->infl + set);
-    RIS_CHECK_LAUNCH();
   }
+  k_metric_inflation<<<dim3(cdiv(std::max(nJ, nK), 32), 2), 256, 0, st3>>>(
+      LJinv.p, nJ, d_jU, LKinv.p, nK, d_kU, MU.p, nU, ((MetricInfo*)d_info)->infl);
+  RIS_CHECK_LAUNCH();
   RIS_CUDA(cudaEventRecord(evM, st3));
   // integrals: dense [mu][nu][P], or (streamed form) on the screened pairs
   // only, after the metric factors are known

@@ -139,15 +139,18 @@ struct MetricInfo {
 // The derivatives take c = M^-1 (rounding errors of the MO transforms), so a
 // rounding of the transforms and of B = W L^-T, or another order of their sums,
 // returns in FP64 gradients and couplings times the metric's inflation: against
-// sums in order, emulated transforms moved couplings by 2e-12 at an inflation
-// of 5e3 (chains of any length), 1e-10 at 1.3e5 (C24H12), 5e-10 at 6e5 (C42H18)
-// and 1.7e-9 at 1e6 (C54H18, relative 2-norm), and by a twentieth to a fiftieth
-// of that with these transforms alone summed in order.  From 3e4 on (5e-11 at
-// that rate) the FP64 form therefore keeps them on the FP64 pipe, in order (J:
-// the transforms, u = X B and c = u L^-1; K: these and the exchange densities).
-// The products with vectors, which take the metric's square root, and the
-// densities of a well-conditioned K set stay emulated.
-constexpr double kIllMetric = 3.0e4;
+// sums in order, emulated transforms moved them by 2e-12 at an inflation of 5e3
+// (chains of any length), by 1.5e-10 at most in 34 calls at 1.3e5 (C24H12), by
+// 7e-10 at 6e5 (C42H18) and 1.7e-9 at 1e6 (C54H18, relative 2-norm), and by a
+// twentieth of that with these transforms alone summed in order.  From 2e5 on
+// (2.5e-10 at that rate, a quarter of what FP64 results are held to) the FP64
+// form therefore keeps them on the FP64 pipe, in order (J: the transforms,
+// u = X B and c = u L^-1; K: these and the exchange densities), whatever that
+// costs: a geometry of C54H18 takes 191 ms instead of 36 (and 461 before any
+// emulation), one of C24H12 stays at what the emulated products give.  The
+// products with vectors, which take the metric's square root, and the densities
+// of a well-conditioned K set stay emulated.
+constexpr double kIllMetric = 2.0e5;
 
 struct Engine : StreamOwner {
   ris_options opt{};

@@ -59,7 +59,7 @@ def test_derivatives_of_ill_conditioned_metrics(ris_mod, radius, k_as_j):
 @pytest.mark.parametrize("kind,size,low,high", [("chain", 12, 4e3, 6e3), ("chain", 40, 4e3, 6e3),
                                                 ("flake", 4.0, 1.2e5, 1.4e5), ("flake", 6.2, 9e5, 1.1e6)])
 def test_inflation_of_the_workloads(oracle, kind, size, low, high):
-    """The figures that the library's line (3e4) was set by: max M_PP (M^-1)_PP of
+    """The figures that the library's line (2e5) was set by: max M_PP (M^-1)_PP of
     the Coulomb sets, on either side of it; the exchange sets are far below."""
     mol = (synth.chain_molecule(size, 1, True, False) if kind == "chain" else
            synth.flake_molecule(size, 1, False))
