@@ -1315,7 +1315,7 @@ void Engine::build_aux(int natm_, const double* coords, int nshell, const ris_sh
   check(auxJ, nJs, kMaxLAux, "J auxiliary shell");
   check(auxK, nKs, kMaxLAux, "K auxiliary shell");
   join_D();  // a previous geometry's derivative integrals may still read the shells
-  release_emu_ops();  // nothing of the last geometry's B tensors is used again
+  drop_emu_ops();  // digits of the last geometry's B tensors
   stage = 0;
   have_D = false;
   natm = natm_;
@@ -1495,6 +1495,7 @@ void Engine::build_aux(int natm_, const double* coords, int nshell, const ris_sh
     TK.release();
     D.release();
     Df.release();
+    release_emu_ops();
   }
   RIS_CUDA(cudaStreamWaitEvent(st, evM, 0));
   RIS_CUDA(cudaEventSynchronize(evC));
@@ -1554,7 +1555,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   C.ensure((size_t)n * nmo, st);
   eps.ensure(nmo, st);
   de.ensure(nov, st);
-  release_emu_ops();   // digits of the last B build
+  drop_emu_ops();
   have_Kov = opt.rpa;  // the ov block is of these integrals and MOs: below for RPA, else on demand
   if (i0 == 0 && a1 == nmo_) {
     copy_in(C.p, Cin, (size_t)n * nmo, st);
@@ -1595,7 +1596,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   if (emuJ) {  // B[(i,a)][R] = sum_P W[(i,a)][P] L_J^-1[R][P]
     EmuEpilogue e;
     e.c64 = BJ.p; e.rs = nJ; e.cs = 1;
-    emu_abt(fJ, (int)nov, nJ, nJ, w3.p, nJ, 1, LJinv.p, nJ, 1, e);
+    emu_abt(fJ, nov, nJ, nJ, w3.p, nJ, 1, LJinv.p, nJ, 1, e);
   } else {
     gemm_set(0, false, true, (int)nov, nJ, nJ, 1.0, w3.p, nJ, LJinv.p, nJ, 0.0, BJ.p, nJ, st);
   }
@@ -1663,7 +1664,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   if (emu) {  // c[(a,b)][Q] = sum_R B[(a,b)][R] L_K^-1[R][Q]
     EmuEpilogue e;
     e.c64 = cKvv.p; e.rs = nK; e.cs = 1;
-    emu_abt(kEmu10x6, v * v, nK, nK, w4.p, nK, 1, LKinv.p, 1, nK, e);
+    emu_abt(kEmu10x6, (long long)v * v, nK, nK, w4.p, nK, 1, LKinv.p, 1, nK, e);
   } else {
     gemm_set(1, false, false, v * v, nK, nK, 1.0, w4.p, nK, LKinv.p, nK, 0.0, cKvv.p, nK, st);
   }
@@ -1698,6 +1699,34 @@ void Engine::emu97(int M, int N, const EmuOperand& A, const EmuOperand& B, const
   emu_gemm(kEmu9x7, M, N, A, B, ep, d_tcerr, st, bt);
 }
 
+// Products of the rows of src (K long) with each operand of `to`, the rows cut
+// in blocks whose digits take 1 GB at most (2.25 times what they are cut from:
+// whole, T^J would take 3.8 GB on C40H42).  A block is still some thousand
+// tiles, and rows are cut one by one, so that blocks change neither time nor bits.
+void Engine::emu_rows(EmuForm f, const EmuSource& src, long long rows, int K, std::initializer_list<EmuTo> to) {
+  EmuMat& a = ebRows;
+  if (!d_tcerr) {
+    RIS_ALLOC(cudaMallocAsync((void**)&d_tcerr, sizeof(int), st));
+    RIS_CUDA(cudaMemsetAsync(d_tcerr, 0, sizeof(int), st));
+  }
+  auto place = [](long long r, int in, long long ld, long long rs) { return in > 0 ? r / in * ld : r * rs; };
+  int unit = std::max(1, src.rin);  // blocks start where a run of rows starts, in the source and in each result
+  for (const EmuTo& t : to) unit = std::max(unit, t.ep.rin);
+  const long long fit = (1LL << 30) / (32LL * emu_slices(f) * cdiv(K, 16));
+  const long long per = std::max(1LL, fit / unit) * unit;
+  for (long long r0 = 0; r0 < rows; r0 += per) {
+    const long long r = std::min(per, rows - r0);
+    EmuSource s = src;
+    s.p += place(r0, src.rin, src.rld, src.rs);
+    a.slice(f, kEmuRowsA, s, r, K, st);
+    for (const EmuTo& t : to) {
+      EmuEpilogue e = t.ep;
+      e.c64 += place(r0, e.rin, e.rld, e.rs);
+      emu_gemm(f, (int)r, t.N, a.op, *t.B, e, d_tcerr, st);
+    }
+  }
+}
+
 void Engine::check_tcerr() {
   if (!d_tcerr) return;
   int h_err = 0;
@@ -1706,9 +1735,15 @@ void Engine::check_tcerr() {
   RIS_REQUIRE(h_err == 0, RIS_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
 }
 
+// The digits are void; their storage stays for the next ones (to give 1 GB
+// back and take it again costs up to 1 ms each time).
+void Engine::drop_emu_ops() {
+  emu_ready = false;
+  for (EmuMat* m : {&ebBoo, &ebBvv, &ebBov, &ebBovT}) m->op = EmuOperand();
+}
 void Engine::release_emu_ops() {
   emu_ready = false;
-  for (EmuMat* m : {&ebBoo, &ebBvv, &ebBov, &ebBovT}) m->release();
+  for (EmuMat* m : {&ebBoo, &ebBvv, &ebBov, &ebBovT, &ebRows}) m->release();
 }
 
 static EmuSource emu_src(const double* p, long long rs, long long ks, int rin = 0, long long rld = 0,
@@ -1746,29 +1781,30 @@ void Engine::build_K_emu(const double* HK, double* Bvv) {
   const long long nov = (long long)o * v;
   const double* Cv = C.p + o;
   const EmuForm f = kEmu9x7;
-  EmuMat cv, co, li, lt, a;
+  EmuMat cv, co, li, lt;
   cv.slice(f, emu_cols(v), emu_src(Cv, 1, nmo), v, n, st);            // rows a over mu
+  co.slice(f, emu_cols(o), emu_src(C.p, 1, nmo), o, n, st);
   li.slice(f, emu_cols(nK), emu_src(LKinv.p, nK, 1), nK, nK, st);      // rows R over P
   lt.slice(f, emu_cols(nK), emu_src(LKinv.p, 1, nK), nK, nK, st);      // rows Q over R
   // [x][y][P] -> B = . L^-T -> c = B L^-1, rows (x, y)
   auto metric = [&](const double* g, long long rows, double* B, double* c) {
-    a.slice(f, kEmuRowsA, emu_src(g, nK, 1), rows, nK, st);
-    emu97((int)rows, nK, a.op, li.op, emu_out(B, nK, 1));
-    a.slice(f, kEmuRowsA, emu_src(B, nK, 1), rows, nK, st);
-    emu97((int)rows, nK, a.op, lt.op, emu_out(c, nK, 1));
+    emu_rows(f, emu_src(g, nK, 1), rows, nK, {{&li.op, nK, emu_out(B, nK, 1)}});
+    emu_rows(f, emu_src(B, nK, 1), rows, nK, {{&lt.op, nK, emu_out(c, nK, 1)}});
   };
   {  // rows (i,P) of HK over nu
-    EmuMat h;
-    h.slice(f, kEmuRowsA, emu_src(HK, 1, nK, nK, (long long)n * nK), (long long)o * nK, n, st);
-    co.slice(f, emu_cols(o), emu_src(C.p, 1, nmo), o, n, st);
+    SBuf<double> goo((size_t)o * o * nK, st), Bia;
     w3.ensure((size_t)std::max(nov, (long long)o * o) * nK, st);
-    emu97(o * nK, o, h.op, co.op, emu_out(w3.p, 1, nK, nK, (long long)o * nK));
+    const EmuSource h = emu_src(HK, 1, nK, nK, (long long)n * nK);
+    const EmuTo oo = {&co.op, o, emu_out(goo.p, 1, nK, nK, (long long)o * nK)};
+    if (opt.rpa)
+      emu_rows(f, h, (long long)o * nK, n, {oo, {&cv.op, v, emu_out(w3.p, 1, nK, nK, (long long)v * nK)}});
+    else
+      emu_rows(f, h, (long long)o * nK, n, {oo});
     BKoo.ensure((size_t)o * o * nK, st);
     cKoo.ensure((size_t)o * o * nK, st);
-    metric(w3.p, (long long)o * o, BKoo.p, cKoo.p);
+    metric(goo.p, (long long)o * o, BKoo.p, cKoo.p);
     if (opt.rpa) {
-      emu97(o * nK, v, h.op, cv.op, emu_out(w3.p, 1, nK, nK, (long long)v * nK));
-      SBuf<double> Bia((size_t)nov * nK, st);  // [i][a][R]
+      Bia.ensure((size_t)nov * nK, st);  // [i][a][R]
       cKov.ensure((size_t)nov * nK, st);
       metric(w3.p, nov, Bia.p, cKov.p);
       BKovR.ensure((size_t)nov * nK, st);
@@ -1778,13 +1814,10 @@ void Engine::build_K_emu(const double* HK, double* Bvv) {
   // rows (nu,P) over mu (T^K symmetric in mu, nu), then rows (a,P) over nu
   w2.ensure((size_t)v * n * nK, st);
   w3.ensure((size_t)v * v * nK, st);
-  {
-    EmuMat t;
-    t.slice(f, kEmuRowsA, emu_src(TK.p, 1, (long long)n * nK), (long long)n * nK, n, st);
-    emu97(n * nK, v, t.op, cv.op, emu_out(w2.p, 1, (long long)n * nK));  // H[a][nu][P]
-  }
-  a.slice(f, kEmuRowsA, emu_src(w2.p, 1, nK, nK, (long long)n * nK), (long long)v * nK, n, st);
-  emu97(v * nK, v, a.op, cv.op, emu_out(w3.p, 1, nK, nK, (long long)v * nK));  // [a][b][P]
+  emu_rows(f, emu_src(TK.p, 1, (long long)n * nK), (long long)n * nK, n,
+           {{&cv.op, v, emu_out(w2.p, 1, (long long)n * nK)}});  // H[a][nu][P]
+  emu_rows(f, emu_src(w2.p, 1, nK, nK, (long long)n * nK), (long long)v * nK, n,
+           {{&cv.op, v, emu_out(w3.p, 1, nK, nK, (long long)v * nK)}});  // [a][b][P]
   cKvv.ensure((size_t)v * v * nK, st);
   metric(w3.p, (long long)v * v, Bvv, cKvv.p);
 }
@@ -1923,31 +1956,21 @@ static TcEpilogue ep_f64(double* c, long long rs, long long bsc = 0, double alph
 void Engine::coulomb_emu(EmuForm f, double* H, double* W) {
   const int o = nocc, v = nvir, n = nao;
   const long long rT = (long long)n * nJ, rH = (long long)o * nJ;
-  // H[(nu,P)][i]: A[(nu,P)][mu] = T[mu][(nu,P)], B[i][mu] = C[mu][i]; blocks
-  // of nu, so that the digits of T stay below about 4 GB on any system
-  const int per = (int)std::max(1LL, std::min((long long)n, (1LL << 31) / ((long long)emu_slices(f) * n * nJ)));
-  for (int nu = 0; nu < n; nu += per) {
-    const int nn = std::min(per, n - nu);
-    EmuEpilogue e1;
-    e1.c64 = H + nu * rH; e1.rin = nJ; e1.rld = rH; e1.rs = 1; e1.cs = nJ;
-    emu_abt(f, nn * nJ, o, n, TJ.p + (long long)nu * nJ, 1, rT, C.p, 1, nmo, e1);
-  }
+  // H[(nu,P)][i]: A[(nu,P)][mu] = T[mu][(nu,P)], B[i][mu] = C[mu][i]
+  EmuEpilogue e1;
+  e1.c64 = H; e1.rin = nJ; e1.rld = rH; e1.rs = 1; e1.cs = nJ;
+  emu_abt(f, rT, o, n, TJ.p, 1, rT, C.p, 1, nmo, e1);
   // W[(i,P)][a]: A[(i,P)][nu] = H[nu][(i,P)], B[a][nu] = C[nu][o + a]
   EmuEpilogue e2;
   e2.c64 = W; e2.rin = nJ; e2.rld = (long long)v * nJ; e2.rs = 1; e2.cs = nJ;
-  emu_abt(f, (int)rH, v, n, H, 1, rH, C.p + o, 1, nmo, e2);
+  emu_abt(f, rH, v, n, H, 1, rH, C.p + o, 1, nmo, e2);
 }
 
-void Engine::emu_abt(EmuForm f, int M, int N, int K, const double* A, long long rsA, long long ksA,
+void Engine::emu_abt(EmuForm f, long long M, int N, int K, const double* A, long long rsA, long long ksA,
                      const double* B, long long rsB, long long ksB, const EmuEpilogue& ep) {
-  if (!d_tcerr) {
-    RIS_ALLOC(cudaMallocAsync((void**)&d_tcerr, sizeof(int), st));
-    RIS_CUDA(cudaMemsetAsync(d_tcerr, 0, sizeof(int), st));
-  }
-  EmuMat a, b;
-  a.slice(f, kEmuRowsA, emu_src(A, rsA, ksA), M, K, st);
+  EmuMat b;
   b.slice(f, emu_cols(N), emu_src(B, rsB, ksB), N, K, st);
-  emu_gemm(f, M, N, a.op, b.op, ep, d_tcerr, st);
+  emu_rows(f, emu_src(A, rsA, ksA), M, K, {{&b.op, N, ep}});
 }
 
 // Mixed precision: (ab|P)_K = sum_mu,nu C_mu,a C_nu,b (mu nu|P) by two
@@ -3375,16 +3398,15 @@ void Engine::ensure_Kov() {
   SBuf<double> H((size_t)o * n * nK, st), Bia((size_t)nov * nK, st), Bm((size_t)nov * nK, st);
   if (emu_exchange()) {
     const EmuForm f = kEmu9x7;
-    EmuMat t, c, li;
-    t.slice(f, kEmuRowsA, emu_src(TK.p, 1, (long long)n * nK), (long long)n * nK, n, st);  // rows (nu,P) over mu
+    EmuMat c, li;
     c.slice(f, emu_cols(o), emu_src(Co, 1, nmo), o, n, st);
-    emu97(n * nK, o, t.op, c.op, emu_out(H.p, 1, (long long)n * nK));  // H[i][nu][P]
-    t.slice(f, kEmuRowsA, emu_src(H.p, 1, nK, nK, (long long)n * nK), (long long)o * nK, n, st);
+    emu_rows(f, emu_src(TK.p, 1, (long long)n * nK), (long long)n * nK, n,
+             {{&c.op, o, emu_out(H.p, 1, (long long)n * nK)}});  // rows (nu,P) over mu: H[i][nu][P]
     c.slice(f, emu_cols(v), emu_src(Cv, 1, nmo), v, n, st);
-    emu97(o * nK, v, t.op, c.op, emu_out(Bia.p, 1, nK, nK, (long long)v * nK));  // [i][a][P]
-    t.slice(f, kEmuRowsA, emu_src(Bia.p, nK, 1), nov, nK, st);
+    emu_rows(f, emu_src(H.p, 1, nK, nK, (long long)n * nK), (long long)o * nK, n,
+             {{&c.op, v, emu_out(Bia.p, 1, nK, nK, (long long)v * nK)}});  // [i][a][P]
     li.slice(f, emu_cols(nK), emu_src(LKinv.p, nK, 1), nK, nK, st);
-    emu97((int)nov, nK, t.op, li.op, emu_out(Bm.p, nK, 1));
+    emu_rows(f, emu_src(Bia.p, nK, 1), nov, nK, {{&li.op, nK, emu_out(Bm.p, nK, 1)}});
     BKovR.ensure((size_t)nov * nK, st);
     transpose_last2(Bm.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]
     have_Kov = true;
@@ -3659,10 +3681,10 @@ void Engine::setup_streamed() {
     if (opt.precision == RIS_MIXED && opt.emu_f64) {
       EmuEpilogue e;
       e.c64 = BJao.p; e.rs = nJ; e.cs = 1;
-      emu_abt(kEmu10x6, (int)nfp, nJ, nU, Ts.p, nU, 1, LJu.p, nU, 1, e);
+      emu_abt(kEmu10x6, nfp, nJ, nU, Ts.p, nU, 1, LJu.p, nU, 1, e);
       EmuEpilogue e2;
       e2.c64 = BKao.p; e2.rs = nK; e2.cs = 1;
-      emu_abt(kEmu10x6, (int)nfp, nK, nK, Ts.p, nU, 1, LKinv.p, nK, 1, e2);
+      emu_abt(kEmu10x6, nfp, nK, nK, Ts.p, nU, 1, LKinv.p, nK, 1, e2);
     } else {
       gemm_set(0, false, true, (int)nfp, nJ, nU, 1.0, Ts.p, nU, LJu.p, nU, 0.0, BJao.p, nJ, st);
       gemm_set(1, false, true, (int)nfp, nK, nK, 1.0, Ts.p, nU, LKinv.p, nK, 0.0, BKao.p, nK, st);
@@ -3729,10 +3751,10 @@ void Engine::build_B_streamed() {
         const long long rT = (long long)n * rw, rH = (long long)o * rw;
         EmuEpilogue e1;
         e1.c64 = H.p; e1.rin = rw; e1.rld = rH; e1.rs = 1; e1.cs = rw;
-        emu_abt(kEmu10x6, (int)rT, o, n, Tb.p, 1, rT, C.p, 1, nmo, e1);
+        emu_abt(kEmu10x6, rT, o, n, Tb.p, 1, rT, C.p, 1, nmo, e1);
         EmuEpilogue e2;
         e2.c64 = BJ.p + r0; e2.rin = rw; e2.rld = (long long)v * nJ; e2.rs = 1; e2.cs = nJ;
-        emu_abt(kEmu10x6, (int)rH, v, n, H.p, 1, rH, C.p + o, 1, nmo, e2);
+        emu_abt(kEmu10x6, rH, v, n, H.p, 1, rH, C.p + o, 1, nmo, e2);
       } else {  // H[i][nu][r], then per i: B[i][a][r0 + r]
         gemm_set(0, true, false, o, n * rw, n, 1.0, Co, nmo, Tb.p, n * rw, 0.0, H.p, n * rw, st);
         GemmBatch bt;

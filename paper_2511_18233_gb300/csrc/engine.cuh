@@ -1,5 +1,6 @@
 // TDDFT-ris engine state and stages.
 #pragma once
+#include <initializer_list>
 #include <map>
 #include <string>
 #include <vector>
@@ -89,6 +90,13 @@ struct EmuMat {
     e.release();
     op = EmuOperand();
   }
+};
+
+// One of the products of a left operand: with B (N rows), to ep.
+struct EmuTo {
+  const EmuOperand* B;
+  int N;
+  EmuEpilogue ep;
 };
 
 // The context's stream; a base class so that it outlives every buffer
@@ -214,6 +222,7 @@ struct Engine : StreamOwner {
   EmuMat ebBoo;   // rows i over (j,R)
   EmuMat ebBov;   // rows (R,i) over b         (RPA and Z-vector products)
   EmuMat ebBovT;  // rows a over (R,j)
+  EmuMat ebRows;  // a block of the left operand of emu_rows
 
   // excitations
   int nstates = 0;
@@ -275,17 +284,19 @@ struct Engine : StreamOwner {
   void coulomb_emu(EmuForm f, double* H, double* W);  // H [nu][i][P], W [i][a][P]
   // C = A B^T, element (r, k) of A at A[r rsA + k ksA] (B likewise), as an
   // FP64-accurate product on the tensor cores
-  void emu_abt(EmuForm f, int M, int N, int K, const double* A, long long rsA, long long ksA, const double* B,
+  void emu_abt(EmuForm f, long long M, int N, int K, const double* A, long long rsA, long long ksA, const double* B,
                long long rsB, long long ksB, const EmuEpilogue& ep);
   // FP64 form: the B build and the exchange products (A products, exchange
   // densities) as FP64-accurate products on the FP16 tensor cores
   bool emu_exchange() const;
   bool emu_product(int nvec) const;  // ... a product of nvec vectors
   void ensure_emu_ops();
+  void drop_emu_ops();
   void release_emu_ops();
   void check_tcerr();  // throws if a tensor-core pipeline wait timed out (synchronises)
   void emu97(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep,
              const EmuBatch& bt = EmuBatch());
+  void emu_rows(EmuForm f, const EmuSource& src, long long rows, int K, std::initializer_list<EmuTo> to);
   void build_K_emu(const double* HK, double* Bvv);
   // K1 (alpha, beta into out) and, when K2 is given, K2 of exchange_terms
   void exchange_emu(const double* Z, int nvec, double* K1, double alpha, double beta, double* K2);

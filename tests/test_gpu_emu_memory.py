@@ -1,4 +1,5 @@
 """Device memory of the FP64 form's emulated products."""
+import numpy as np
 import pytest
 
 from paper_2511_18233_gb300 import synth
@@ -37,3 +38,29 @@ def test_digits_of_a_dense_geometry_go_with_it(ris_mod):
         c.close()
     digits = 18 * small.nvir ** 2 * small.naux("K")
     assert abs(held[0] - held[1]) < digits // 2, (held, digits)
+
+
+@gpu
+@pytest.mark.parametrize("rpa", [0, 1])
+def test_build_in_blocks_of_rows(ris_mod, rpa):
+    """C40H42, whose T^K digits (1.5 GB) and half-transformed digits (1.3 GB) take two
+    blocks: the peak of the build stays within one block (1.1 GB with the small operands)
+    of the FP64 pipe's, and products and gradients are those of the FP64 pipe (bars
+    of the smaller chains: 1e-12, 1e-10)."""
+    mol = synth.chain_molecule(40, 3, True)
+    X = synth.random_amplitudes(2, mol.nocc, mol.nvir, seed=6)
+    peak, got = [], []
+    for emu in (1, 0):
+        c = ris_mod.Context(emu_f64=emu, rpa=rpa, deriv_prefetch=0)
+        c.build_aux(mol.coords, mol.shells, mol.aux_j, mol.aux_k)
+        c.build_B(mol.C, mol.mo_energy, mol.nocc)
+        peak.append(c.stats()["bytes_peak"])
+        ax = c.apply(X)
+        got.append((list(ax) if rpa else [ax]) + [c.gradient([1], X=X, Y=0.1 * X if rpa else None)])
+        if not rpa:
+            got[-1].append(c.zvector(X[:1]))
+        c.close()
+    print("build peaks", peak)
+    assert peak[0] - peak[1] < 1.1 * 2 ** 30, peak
+    for a, b, bar in zip(got[0], got[1], [1e-12, 1e-12, 1e-10] if rpa else [1e-12, 1e-10, 1e-8]):
+        assert np.max(np.abs(a - b)) <= bar * np.max(np.abs(b))
