@@ -1704,7 +1704,7 @@ void Engine::emu97(int M, int N, const EmuOperand& A, const EmuOperand& B, const
 // whole, T^J would take 3.8 GB on C40H42).  A block is still some thousand
 // tiles, and rows are cut one by one, so that blocks change neither time nor bits.
 void Engine::emu_rows(EmuForm f, const EmuSource& src, long long rows, int K, std::initializer_list<EmuTo> to) {
-  EmuMat& a = ebRows;
+  EmuMat a;
   if (!d_tcerr) {
     RIS_ALLOC(cudaMallocAsync((void**)&d_tcerr, sizeof(int), st));
     RIS_CUDA(cudaMemsetAsync(d_tcerr, 0, sizeof(int), st));
@@ -1743,7 +1743,7 @@ void Engine::drop_emu_ops() {
 }
 void Engine::release_emu_ops() {
   emu_ready = false;
-  for (EmuMat* m : {&ebBoo, &ebBvv, &ebBov, &ebBovT, &ebRows}) m->release();
+  for (EmuMat* m : {&ebBoo, &ebBvv, &ebBov, &ebBovT}) m->release();
 }
 
 static EmuSource emu_src(const double* p, long long rs, long long ks, int rin = 0, long long rld = 0,

@@ -222,7 +222,6 @@ struct Engine : StreamOwner {
   EmuMat ebBoo;   // rows i over (j,R)
   EmuMat ebBov;   // rows (R,i) over b         (RPA and Z-vector products)
   EmuMat ebBovT;  // rows a over (R,j)
-  EmuMat ebRows;  // a block of the left operand of emu_rows
 
   // excitations
   int nstates = 0;
