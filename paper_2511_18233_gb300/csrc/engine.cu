@@ -1556,6 +1556,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
   eps.ensure(nmo, st);
   de.ensure(nov, st);
   drop_emu_ops();
+  have_cKovP = false;
   have_Kov = opt.rpa;  // the ov block is of these integrals and MOs: below for RPA, else on demand
   if (i0 == 0 && a1 == nmo_) {
     copy_in(C.p, Cin, (size_t)n * nmo, st);
@@ -1645,6 +1646,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
     transpose_last2(w4.p, 1, (int)nov, nK, BKovR.p, st);  // [R][ia]
     cKovP.ensure((size_t)nov * nK, st);
     transpose_last2(cKov.p, 1, (int)nov, nK, cKovP.p, st);  // [P][ia]
+    have_cKovP = true;
   }
   w4.ensure((size_t)v * v * nK, st);
   if (opt.precision == RIS_MIXED && !opt.refine) {
@@ -1687,7 +1689,27 @@ bool Engine::emu_exchange() const {
          2.0 * nocc * (double)nvir * nvir * nK >= kEmuMinFlops;
 }
 bool Engine::emu_product(int nvec) const {
-  return emu_exchange() && 2.0 * nvec * nocc * (double)nvir * nvir * nK >= kEmuMinProduct;
+  if (!emu_exchange() || 2.0 * nvec * nocc * (double)nvir * nvir * nK < kEmuMinProduct) return false;
+  // the digits that the products keep, where they are not held yet
+  const double digits = 18.0 * nK * ((double)nvir * nvir + (double)nocc * nocc + 2.0 * nocc * nvir);
+  return ebBvv.s.p || room(digits) >= digits;
+}
+
+// Bytes, up to `want`, that the context may still take: what mem_budget leaves
+// and, for a gigabyte and more (the query would cost a small call time), nine
+// tenths of what the device and its allocation pool have free.
+double Engine::room(double want) const {
+  double left = want;
+  if (opt.mem_budget) left = std::min(left, std::max(0.0, (double)opt.mem_budget - (double)mem.cur));
+  if (want < 1e9) return left;
+  size_t fr = 0, tot = 0;
+  uint64_t held = 0, used = 0;
+  cudaMemPool_t pool;
+  RIS_CUDA(cudaMemGetInfo(&fr, &tot));
+  RIS_CUDA(cudaDeviceGetDefaultMemPool(&pool, device));
+  RIS_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held));
+  RIS_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used));
+  return std::min(left, 0.9 * ((double)fr + (double)held - (double)used));
 }
 
 void Engine::emu97(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep,
@@ -2030,8 +2052,10 @@ void Engine::gamma_K_mixed(int np, const int* sI, const int* sJ, int nsu, const 
   const int lv4 = ld4(v), lo4 = ld4(o), kp = ld4(2 * o);
   const long long su = (long long)o * lv4, sw = (long long)nn * kp, sz = nK * su, sg = (long long)nK * o * lo4,
                   sm = nn * (long long)nK * kp, gk = (long long)nn * nn * nK;
-  // pairs at a time: about 2 GB of work space
-  const int per = (int)std::max(1LL, std::min({(long long)np, 8LL, (1LL << 28) / (sz + sg + sm), 65535LL / nK}));
+  // pairs at a time: up to 2 GB of work space, half of what is free
+  const double bytes = 8.0 * (sz + sg + sm), want = std::min(np, 8) * bytes;
+  const int fit = (int)(std::min(2147483648.0, want <= bytes ? want : 0.5 * room(2.0 * want)) / bytes);
+  const int per = (int)std::max(1LL, std::min({(long long)np, 8LL, (long long)fit, 65535LL / nK}));
   // (padding of Z and M is never read: the products' K extents end before it;
   // G's enters Omega's contraction and is zeroed)
   SBuf<float> ZH((size_t)per * sz, st), ZL((size_t)per * sz, st), GH((size_t)per * sg, st, true),
@@ -2946,6 +2970,20 @@ struct GammaEmu {
   int nc = 1, kw = 0, o8 = 0, n8 = 0;
   const double* Q[2] = {nullptr, nullptr};
 
+  // what setup and one pair take (bytes) is there
+  static bool fits(const Engine& e, int nsu, bool rpa) {
+    const double o = e.nocc, v = e.nvir, n = e.nao, nK = e.nK, kw = (rpa ? 5 : 2) * o, c = rpa ? 2 : 1;
+    const double keep = 18.0 * (nK * (v * v + o * o + (c - 1) * o * v) + n * o + nsu * (c * (o * v + n * o) + n * kw)) +
+                        8.0 * nsu * n * kw;
+    const double need = keep + pair_bytes(e, (int)kw);
+    return e.room(need) >= need;
+  }
+  static double pair_bytes(const Engine& e, int kw) {
+    const double o = e.nocc, v = e.nvir, n = e.nao, nK = e.nK;
+    return 8 * o * v * nK + 27.0 * emu_pad((int)(o * nK), kEmuRowsA) * v + 8 * n * kw * nK +
+           18.0 * emu_pad((int)(n * nK), kEmuRowsA) * kw;
+  }
+
   void setup(Engine& e, int nsu, const double* R, const double* L, const double* QR, const double* QL) {
     const int o = e.nocc, v = e.nvir, n = e.nao, nK = e.nK;
     const EmuForm f = kEmu9x7;
@@ -2983,10 +3021,12 @@ struct GammaEmu {
   // empty and one of its products a third of the device (ten C20H22
   // pairs: 3108 -> 2411 us in the products, 571 -> 328 us in the slicing).
   void pairs(Engine& e, int np, const int* sI, const int* sJ, double* Gam, double* Om) {
-    const long long o = e.nocc, v = e.nvir, n = e.nao, nK = e.nK;
-    const long long bytes = 8 * o * v * nK + 27 * emu_pad((int)(o * nK), kEmuRowsA) * v + 8 * n * kw * nK +
-                            18 * emu_pad((int)(n * nK), kEmuRowsA) * (long long)kw;
-    const int per = (int)std::max(1LL, std::min({(long long)np, 8LL, (6LL << 30) / bytes}));  // work space
+    const long long n = e.nao, nK = e.nK;
+    const double bytes = pair_bytes(e, kw);
+    // work space: up to 6 GB, half of what is free
+    const double want = std::min(np, 8) * bytes;
+    const double fit = std::min(6442450944.0, np == 1 ? want : 0.5 * e.room(2.0 * want));
+    const int per = (int)std::max(1LL, std::min({(long long)np, 8LL, (long long)(fit / bytes)}));
     for (int p = 0; p < np; p += per)
       batch(e, std::min(per, np - p), sI + p, sJ + p, Gam + p * n * n * nK, Om + (size_t)p * e.nU * e.nU);
   }
@@ -3167,7 +3207,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   // Q_s[i][nu] = sum_a R_s[i][a] C_v[nu][a] for every state, and from it
   // D^R_s[mu][nu] = sum_i C_o[mu][i] Q_s[i][nu] (o n^2 multiply-adds; forming
   // C_o R_s first would take o n v + n^2 v)
-  const bool emu = emu_exchange(), emuG = emu && !ill[1];
+  const bool emu = emu_exchange(), emuG = emu && !ill[1] && GammaEmu::fits(*this, nsu, rpa);
   if (!mixed || rpa) {
     QR.ensure((size_t)nsu * o * nn, st);
     if (rpa) QL.ensure((size_t)nsu * o * nn, st);
@@ -3258,6 +3298,11 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
     WV.ensure((size_t)nn * 2 * o, st);
   }
   const double cx = opt.cx;
+  if (rpa && !emuG && !have_cKovP) {
+    cKovP.ensure((size_t)nov * nK, st);
+    transpose_last2(cKov.p, 1, (int)nov, nK, cKovP.p, st);  // [P][ia]
+    have_cKovP = true;
+  }
   GammaEmu ge;
   if (emuG) ge.setup(*this, nsu, Rs.p, rpa ? Ls.p : nullptr, QR.p, rpa ? QL.p : nullptr);
   for (int g0 = 0; g0 < npair; g0 += NB) {

@@ -201,6 +201,7 @@ struct Engine : StreamOwner {
   DBuf BKovR;     // [R][i][a] (RPA, Z-vector)
   bool have_Kov = false;  // BKovR holds the last B build's block
   DBuf cKovP;     // c^K_ov as [P][i][a] (RPA)
+  bool have_cKovP = false;  // cKovP holds the last B build's block
   DBuf cKoo, cKvv, cKov;  // fitting coefficients c = B L^-1, [p][q][P]
 
   // mixed precision (3xTF32) operands: hi/lo FP32 splits
@@ -288,6 +289,7 @@ struct Engine : StreamOwner {
   // FP64 form: the B build and the exchange products (A products, exchange
   // densities) as FP64-accurate products on the FP16 tensor cores
   bool emu_exchange() const;
+  double room(double want) const;
   bool emu_product(int nvec) const;  // ... a product of nvec vectors
   void ensure_emu_ops();
   void drop_emu_ops();

@@ -64,3 +64,43 @@ def test_build_in_blocks_of_rows(ris_mod, rpa):
     assert peak[0] - peak[1] < 1.1 * 2 ** 30, peak
     for a, b, bar in zip(got[0], got[1], [1e-12, 1e-12, 1e-10] if rpa else [1e-12, 1e-10, 1e-8]):
         assert np.max(np.abs(a - b)) <= bar * np.max(np.abs(b))
+
+
+def _gradients(ris_mod, mol, X, rpa, **opt):
+    c = ris_mod.Context(rpa=rpa, **opt)
+    c.build_aux(mol.coords, mol.shells, mol.aux_j, mol.aux_k)
+    c.build_B(mol.C, mol.mo_energy, mol.nocc)
+    ax = c.apply(X)
+    g = c.gradient(range(len(X)), X=X, Y=0.1 * X if rpa else None)
+    s = c.stats()
+    c.close()
+    return list(ax) if rpa else [ax], g, s
+
+
+@gpu
+@pytest.mark.parametrize("rpa", [0, 1])
+def test_pair_batches_stay_within_the_budget(ris_mod, rpa):
+    """Eight gradients of C20H22 need 2.3 GB on the FP64 pipe; with eight pairs at a time
+    the emulated densities would take the context to 3.5 (TDA) and 4.8 GB (RPA).
+    With a budget of 3 GB fewer pairs share launches, with the same bits."""
+    mol = synth.chain_molecule(20, 1, True)
+    X = synth.random_amplitudes(8, mol.nocc, mol.nvir, seed=3)
+    _, free, _ = _gradients(ris_mod, mol, X, rpa)
+    _, g, s = _gradients(ris_mod, mol, X, rpa, mem_budget=int(3e9))
+    assert s["bytes_peak"] <= 3e9, s["bytes_peak"]
+    assert np.array_equal(g, free)
+
+
+@gpu
+@pytest.mark.parametrize("rpa", [0, 1])
+def test_without_room_products_and_densities_run_on_the_fp64_pipe(ris_mod, rpa):
+    """No room for digits: what needed none before still runs, on the FP64 pipe (bars
+    of the emulated form: 1e-12, 1e-10), and holds no more than with emu_f64 = 0."""
+    mol = synth.chain_molecule(12, 2, True)
+    X = synth.random_amplitudes(3, mol.nocc, mol.nvir, seed=3)
+    ax, g, s = _gradients(ris_mod, mol, X, rpa, mem_budget=1, stream=-1)
+    rx, rg, rs = _gradients(ris_mod, mol, X, rpa, emu_f64=0)
+    for a, b in zip(ax, rx):
+        assert np.max(np.abs(a - b)) <= 1e-12 * np.max(np.abs(b))
+    assert np.max(np.abs(g - rg)) <= 1e-10 * np.max(np.abs(rg))
+    assert s["bytes_held"] <= rs["bytes_held"] + 2 ** 20
