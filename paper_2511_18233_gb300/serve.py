@@ -55,6 +55,10 @@ def _ld4(n: int) -> int:
 
 # ---------------------------------------------------------------- footprint
 
+# exchange work of a product from which the library's FP64 form runs emulated
+EMU_MIN_WORK = 2.0e7
+
+
 def footprint_bytes(nao: int, nocc: int, nJ: int, nK: int, nU: int, nstates: int,
                     nstate_deriv: int, mixed: bool) -> int:
     """Upper estimate of the device bytes one request holds at its peak.
@@ -67,6 +71,10 @@ def footprint_bytes(nao: int, nocc: int, nJ: int, nK: int, nU: int, nstates: int
     parts of a batch of pair densities and per-state densities).  The
     derivative integrals d(mu nu|P)/dR (FP32 in mixed precision) are computed
     on a side stream from the auxiliary build on, so they count as persistent.
+    In FP64, systems above a size run their B build, exchange products and
+    exchange densities on digit slices of the operands (18 bytes an element):
+    a block of the build's, the kept B^K_vv and B^K_oo, the vectors' and their
+    intermediates', and a batch of pairs' are counted.
     """
     n, o = nao, nocc
     v = n - o
@@ -100,7 +108,21 @@ def footprint_bytes(nao: int, nocc: int, nJ: int, nK: int, nU: int, nstates: int
                  + 3 * s * n * nU + 4 * s * o * n + n * v + 2 * o * v * nK + 2 * n * o * nK)
     if mixed:
         deriv += f * 4 * s * (o * _ld4(v) + n * _ld4(2 * o))
-    total = aux + B + dint + d * 2 * ns * nov + max(dav, deriv)
+    build = keep = 0
+    if not mixed and 2 * o * v * v * nK >= EMU_MIN_WORK:
+        def digits(rows, K):
+            return 18 * ((rows + 127) // 128 * 128) * ((K + 15) // 16 * 16) + 4 * rows
+        block = max(digits(n * nJ, n), digits(o * nJ, n), digits(nov, nJ), digits(max(v, o) * nK, n),
+                    digits(v * v, nK))
+        build = min(block, 1 << 30) + digits(v, n) + digits(o, n) + 2 * digits(M, M)
+        keep = digits(nK * v, v) + digits(o, o * nK)
+        nb = max(1, min(nb0, 1280 // o + 1))  # vectors of one block of a product
+        dav += digits(nb * o, v) + digits(nb * v, o * nK)
+        pair = d * (o * v * nK + o * o * nK + 2 * o * n * nK) + digits(o * nK, v) + digits(o * nK, o) \
+            + digits(n * nK, 2 * o)
+        deriv += digits(v * nK, v) + digits(o * nK, o) + max(pair, min(nbp * pair, 6 << 30)) \
+            + s * (digits(o, v) + digits(n, o) + digits(n, 2 * o) + d * 2 * n * o)
+    total = aux + B + dint + keep + d * 2 * ns * nov + max(build, dav, deriv)
     return int(1.25 * total) + (32 << 20)
 
 
