@@ -1448,7 +1448,7 @@ void Engine::build_aux(int natm_, const double* coords, int nshell, const ris_sh
     if (pin) RIS_CUDA(cudaFreeHost(pin));
     pin = nullptr;
     pin_n = 2 * (size_t)std::max(pl.npair, 1);
-    RIS_ALLOC(cudaMallocHost((void**)&pin, sizeof(int) * pin_n));
+    RIS_ALLOC(cudaMallocHost((void**)&pin, sizeof(int) * (pin_n + 1)));
   }
   // the metric factors (two-centre integrals, Cholesky, inverse) depend on
   // the auxiliary shells only: they run on st3 beside the three-centre
@@ -1749,12 +1749,19 @@ void Engine::emu_rows(EmuForm f, const EmuSource& src, long long rows, int K, st
   }
 }
 
+// The pipelines' error flag: queued to the host (behind the pair list's pinned
+// copy), looked at after a synchronisation that the call makes anyway (one of
+// its own costs a call 13 us), or both at once.
+void Engine::post_tcerr() {
+  if (d_tcerr) RIS_CUDA(cudaMemcpyAsync(pin + pin_n, d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, st));
+}
+void Engine::test_tcerr() const {
+  RIS_REQUIRE(!d_tcerr || pin[pin_n] == 0, RIS_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
+}
 void Engine::check_tcerr() {
-  if (!d_tcerr) return;
-  int h_err = 0;
-  RIS_CUDA(cudaMemcpyAsync(&h_err, d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, st));
+  post_tcerr();
   RIS_CUDA(cudaStreamSynchronize(st));
-  RIS_REQUIRE(h_err == 0, RIS_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
+  test_tcerr();
 }
 
 // The digits are void; their storage stays for the next ones (to give 1 GB
@@ -2250,16 +2257,17 @@ void Engine::apply(int nvec, const double* Xh, double* out, double* out2) {
   if (opt.rpa) {
     z.ensure(n, st);
     apply_ApB_AmB(x.p, nvec, y.p, z.p);
-    if (emu_exchange()) check_tcerr();
     copy_out(out2, z.p, n, st);
   } else if (opt.precision == RIS_MIXED) {
     apply_A_mixed(x.p, nvec, y.p);
   } else {
     apply_A_tda(x.p, nvec, y.p);
   }
-  if (emu_exchange()) check_tcerr();
   copy_out(out, y.p, n, st);
+  const bool flag = emu_exchange();
+  if (flag) post_tcerr();
   RIS_CUDA(cudaStreamSynchronize(st));
+  if (flag) test_tcerr();
 }
 
 // (ij|ab) and (ib|ja) exchange contractions (Eqs. A_matrix, B_matrix):
@@ -3305,6 +3313,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
   }
   GammaEmu ge;
   if (emuG) ge.setup(*this, nsu, Rs.p, rpa ? Ls.p : nullptr, QR.p, rpa ? QL.p : nullptr);
+  const bool flag = mixed || emu;
   for (int g0 = 0; g0 < npair; g0 += NB) {
     const int nb = std::min(NB, npair - g0);
     // (in mixed TDA and in the emulated form one exchange GEMM writes every element of G^K)
@@ -3423,9 +3432,10 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
                                                         aoPtr.p, aoList.p, axPtr.p, axList.p, nn,
                                                         nU, nK, natm, out + (size_t)g0 * natm * 3);
     RIS_CHECK_LAUNCH();
+    if (flag) post_tcerr();
     RIS_CUDA(cudaStreamSynchronize(st));  // h_pst goes out of scope
   }
-  if (opt.precision == RIS_MIXED || emu_exchange()) check_tcerr();
+  if (flag) test_tcerr();
 }
 
 
@@ -4166,9 +4176,10 @@ void Engine::pair_derivs_streamed(int npair, const int* pairs, int nsu, const st
                                                         aoList.p, axPtr.p, axList.p, nn, nU, nK, natm,
                                                         out + (size_t)g0 * natm * 3);
     RIS_CHECK_LAUNCH();
+    if (mixed) post_tcerr();
     RIS_CUDA(cudaStreamSynchronize(st));  // h_pst goes out of scope
   }
-  if (mixed || emu_exchange()) check_tcerr();
+  if (mixed) test_tcerr();
 }
 
 // ------------------------------------------------------------------ time couplings

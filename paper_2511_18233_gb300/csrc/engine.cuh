@@ -110,7 +110,7 @@ struct StreamOwner {
   cudaEvent_t evC = nullptr;   // its host copy is done
   cudaEvent_t evM = nullptr;   // the metric factors are done (st3)
   int* pin = nullptr;          // pinned host copy of the pair list
-  size_t pin_n = 0;
+  size_t pin_n = 0;            // its ints; one more holds the error flag
   ~StreamOwner() {
     if (st3) cudaStreamSynchronize(st3);
     if (pin) cudaFreeHost(pin);
@@ -294,7 +294,9 @@ struct Engine : StreamOwner {
   void ensure_emu_ops();
   void drop_emu_ops();
   void release_emu_ops();
-  void check_tcerr();  // throws if a tensor-core pipeline wait timed out (synchronises)
+  void post_tcerr();
+  void test_tcerr() const;  // throws if a tensor-core pipeline wait timed out, as of the last post
+  void check_tcerr();       // post, synchronise, test
   void emu97(int M, int N, const EmuOperand& A, const EmuOperand& B, const EmuEpilogue& ep,
              const EmuBatch& bt = EmuBatch());
   void emu_rows(EmuForm f, const EmuSource& src, long long rows, int K, std::initializer_list<EmuTo> to);
