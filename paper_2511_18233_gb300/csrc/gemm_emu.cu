@@ -912,6 +912,9 @@ void emu_gemm(EmuForm f, int M, int N, const EmuOperand& A, const EmuOperand& B,
   if (M <= 0 || N <= 0) return;
   RIS_REQUIRE(A.K == B.K && A.K > 0, RIS_ERR_ARG, "emu_gemm: contraction lengths differ");
   RIS_REQUIRE(bt.n >= 1 && bt.n <= 8 && (bt.n == 1 || !ep.lead), RIS_ERR_ARG, "emu_gemm: batch");
+  // `lead` takes the exponents of A B^T itself, of one pass
+  RIS_REQUIRE(!ep.lead || (ep.alpha == 1.0 && ep.beta == 0.0 && A.K <= kPassChunks * Form9x7::kChunk), RIS_ERR_ARG,
+              "emu_gemm: row exponents of a scaled, summed or very long product");
   for (int p = 0; p < bt.n; p++) {
     RIS_REQUIRE(A.rows - bt.a[p] >= M && B.rows - bt.b[p] >= N, RIS_ERR_ARG, "emu_gemm: operand rows");
     RIS_REQUIRE(bt.a[p] % kEmuRowsA == 0 && bt.b[p] % B.rb == 0, RIS_ERR_ARG, "emu_gemm: batch rows");

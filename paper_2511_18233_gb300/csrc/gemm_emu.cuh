@@ -82,7 +82,7 @@ struct EmuEpilogue {
   // as one row, by atomic maximum into
   //   lead[((r / lrd) % lrm) * lrs + ((c / lcd) % lcm) * lcs]
   // (filled with kEmuNoLead before), so that slicing them needs no pass of its
-  // own for the row exponents
+  // own for the row exponents; alpha 1, beta 0 and K of one pass only (229376)
   int* lead = nullptr;
   int lrd = 1, lrm = 1, lrs = 0, lcd = 1, lcm = 1, lcs = 0;
   void lead_rows(int d, int m, int s) { lrd = d; lrm = m; lrs = s; }
