@@ -116,7 +116,16 @@ typedef struct {
                          operand splitting.  Mixed precision: the Coulomb B transforms (the
                          two MO transforms of (mu nu|P)_J).  RIS_FP64: the B build and the
                          exchange products (the exchange part of the A products and of
-                         Gamma) of all but the smallest systems.  0: on the FP64 pipe */
+                         Gamma) of all but the smallest systems, except the B build and
+                         Gamma of auxiliary sets whose metric is nearly singular (largest
+                         M_PP (M^-1)_PP of 2e5 and more: the derivatives amplify their
+                         rounding) and what the free memory or mem_budget has no room for.
+                         Errors are below FP64's relative to the largest elements of the
+                         operands' rows (see ris_debug_gemm_f64emu97); an element far below
+                         its row's largest keeps fewer than 53 bits (none beyond 2^-62), so
+                         results that depend on such elements alone are not accurate
+                         element by element, and a row with an infinity gives NaN.
+                         0: on the FP64 pipe */
   int eig_fp32;       /* mixed precision: 1 solves the Davidson subspace eigenproblem in FP32
                          (FP64 Rayleigh quotients, close pairs and restarts re-orthonormalised
                          in FP64, back to FP64 if the residuals stall); 0 (default): FP64 */

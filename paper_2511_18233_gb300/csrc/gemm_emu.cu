@@ -33,7 +33,7 @@
 //                     tcgen05.mma of N = (up to 256 / BN) BN multiplies A
 //                     slice p with several B slices at once: the 128-row A
 //                     slice is read from shared memory once per such group
-//                     instead of once per product (13 instructions a stage
+//                     instead of once per product (14 instructions a stage
 //                     instead of 45 at 9 x 7, BN = 48)
 //   warps 2-17      : epilogue, one output row and a quarter of the columns
 //                     per thread.  A chunk's accumulators are read into

@@ -16,7 +16,12 @@ namespace ris {
 //             rounded to nearest): the exchange products of the FP64 form.
 //             45 slice products instead of 55, and a frame 9 bits finer than
 //             an FP64 significand, so that a row's small elements beside one
-//             nine bits larger still keep FP64's relative precision
+//             nine bits larger still keep FP64's relative precision.  Below
+//             that an element keeps fewer than 53 bits (none from 2^-62 of the
+//             row's largest on), and products of digits p + q >= 9 are
+//             dropped: normwise, against max_k|A_rk| max_k|B_ck|, errors are
+//             below FP64's, element by element (a row whose large elements
+//             meet zeros) they are not
 enum EmuForm { kEmu10x6 = 0, kEmu9x7 = 1 };
 constexpr int emu_slices(EmuForm f) { return f == kEmu10x6 ? 10 : 9; }
 
