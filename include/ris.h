@@ -342,6 +342,14 @@ int ris_debug_dgemm(int transA, int transB, int m, int n, int k, double alpha, c
                     int lda, const double* B, int ldb, double beta, double* C, int ldc);
 
 /*
+ * Test hook: the same with the contraction split as finely as pays, as the
+ * FP64 form has it (another order of the sums).
+ */
+int ris_debug_dgemm_fine(int transA, int transB, int m, int n, int k, double alpha,
+                         const double* A, int lda, const double* B, int ldb, double beta, double* C,
+                         int ldc);
+
+/*
  * Test hook: lowest k (<= 64) eigenpairs of a symmetric m x m row-major
  * matrix with the device eigensolver of the Davidson subspace problem.
  * H: [m][m], w: [k] ascending, V: [k][m] (row j = eigenvector j); DEVICE

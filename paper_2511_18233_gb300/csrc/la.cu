@@ -1589,19 +1589,30 @@ void gemv_rows(const double* V, int nrow, long long ncol, const double* x, doubl
 
 // Test hook (declared in include/ris.h): lowest k eigenpairs of a symmetric
 // m x m matrix with the device subspace eigensolver; device pointers.
-extern "C" int ris_debug_dgemm(int transA, int transB, int m, int n, int k, double alpha,
-                               const double* A, int lda, const double* B, int ldb, double beta,
-                               double* C, int ldc) {
+static int debug_dgemm(int transA, int transB, int m, int n, int k, double alpha, const double* A, int lda,
+                       const double* B, int ldb, double beta, double* C, int ldc, bool fine) {
   using namespace ris;
   try {
     RIS_REQUIRE(m >= 0 && n >= 0 && k >= 0 && A && B && C, RIS_ERR_ARG, "bad dgemm arguments");
-    dgemm(transA != 0, transB != 0, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, 0);
+    GemmBatch bt;
+    bt.fine = fine;
+    dgemm(transA != 0, transB != 0, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, 0, bt);
     RIS_CUDA(cudaDeviceSynchronize());
     return 0;
   } catch (const Error& e) {
     fprintf(stderr, "ris_debug_dgemm: %s\n", e.msg.c_str());
     return (int)e.code;
   }
+}
+extern "C" int ris_debug_dgemm(int transA, int transB, int m, int n, int k, double alpha,
+                               const double* A, int lda, const double* B, int ldb, double beta,
+                               double* C, int ldc) {
+  return debug_dgemm(transA, transB, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, false);
+}
+extern "C" int ris_debug_dgemm_fine(int transA, int transB, int m, int n, int k, double alpha,
+                                    const double* A, int lda, const double* B, int ldb, double beta,
+                                    double* C, int ldc) {
+  return debug_dgemm(transA, transB, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, true);
 }
 
 extern "C" int ris_debug_sym_eig_f32(int m, int k, const double* H, double* w, double* V) {
