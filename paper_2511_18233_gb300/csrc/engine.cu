@@ -3120,6 +3120,7 @@ void Engine::pair_derivs(int npair, const int* pairs, int nx, const double* X_in
                          const double* Y_in, double* out) {
   RIS_REQUIRE(stage >= 2, RIS_ERR_STATE, "derivatives before ris_build_B");
   RIS_REQUIRE(npair >= 1 && pairs, RIS_ERR_ARG, "no pairs");
+  RIS_REQUIRE(!(X_in && Y_in) || opt.rpa, RIS_ERR_ARG, "Y amplitudes need a context made for RPA");
   const int o = nocc, v = nvir, nn = nao;
   const long long nov = (long long)o * v;
   const double* Xa;
