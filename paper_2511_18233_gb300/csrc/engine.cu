@@ -1690,9 +1690,11 @@ bool Engine::emu_exchange() const {
 }
 bool Engine::emu_product(int nvec) const {
   if (!emu_exchange() || 2.0 * nvec * nocc * (double)nvir * nvir * nK < kEmuMinProduct) return false;
-  // the digits that the products keep, where they are not held yet
-  const double digits = 18.0 * nK * ((double)nvir * nvir + (double)nocc * nocc + 2.0 * nocc * nvir);
-  return ebBvv.s.p || room(digits) >= digits;
+  if (emu_ready) return true;
+  // the digits that the products keep, beyond the storage that the last ones left
+  double digits = 18.0 * nK * ((double)nvir * nvir + (double)nocc * nocc + 2.0 * nocc * nvir);
+  for (const EmuMat* m : {&ebBvv, &ebBoo, &ebBov, &ebBovT}) digits -= 2.0 * m->s.n;
+  return digits <= 0.0 || room(digits) >= digits;
 }
 
 // Bytes, up to `want`, that the context may still take: what mem_budget leaves
