@@ -1678,7 +1678,7 @@ void Engine::build_B(int nao_, int nmo_, int nocc_, const double* Cin, const dou
 
 // The FP64 form's B build, exchange products and exchange densities run
 // emulated on the tensor cores (option emu_f64) from kEmuMinFlops of exchange
-// work per vector on.  At the line (C7H9) the build takes 374 instead of 651
+// work per vector on (build and densities up to kIllMetric).  At the line (C7H9) the build takes 374 instead of 651
 // us, five gradients 587 instead of 1195; below it the passes around the
 // products (slicing, about ten launches) outweigh them.  A block of vectors
 // needs kEmuMinProduct of work: one vector of C9H11 (5.4e7) 141 against 128
